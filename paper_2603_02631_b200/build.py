@@ -5,11 +5,13 @@ nvcc cross-compiles without a GPU, so this also runs on a CPU-only machine.
 """
 from __future__ import annotations
 
+import concurrent.futures
 import glob
 import os
 import shutil
 import subprocess
 import sys
+import tempfile
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
@@ -18,7 +20,7 @@ LIB_PATH = os.path.join(PKG_DIR, "libspf.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
-    "-Xcompiler", "-fPIC,-fvisibility=hidden", "--shared", "-Xptxas", "-v",
+    "-Xcompiler", "-fPIC,-fvisibility=hidden", "-Xptxas", "-v",
 ]
 
 
@@ -45,14 +47,23 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
     """Builds libspf.so if it is missing or older than its sources; returns its path."""
     if not force and not is_stale():
         return LIB_PATH
-    cmd = [_nvcc(), *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", LIB_PATH, *sources()]
-    proc = subprocess.run(cmd, capture_output=True, text=True)
-    if verbose or proc.returncode != 0:
-        sys.stderr.write(proc.stdout + proc.stderr)
-    if proc.returncode != 0:
-        raise RuntimeError("nvcc failed: " + " ".join(cmd))
+    include = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
+
+    def run(cmd):
+        proc = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or proc.returncode != 0:
+            sys.stderr.write(proc.stdout + proc.stderr)
+        if proc.returncode != 0:
+            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+        return proc.stdout + proc.stderr
+
+    with tempfile.TemporaryDirectory() as tmp:
+        objects = [os.path.join(tmp, os.path.basename(src) + ".o") for src in sources()]
+        with concurrent.futures.ThreadPoolExecutor(os.cpu_count() or 1) as pool:
+            log = "".join(pool.map(lambda so: run([_nvcc(), *NVCC_FLAGS, *include, "-c", so[0], "-o", so[1]]), zip(sources(), objects)))
+        run([_nvcc(), *NVCC_FLAGS, "--shared", "-o", LIB_PATH, *objects])
     with open(os.path.join(PKG_DIR, "libspf.ptxas.log"), "w") as f:
-        f.write(proc.stdout + proc.stderr)
+        f.write(log)
     return LIB_PATH
 
 

@@ -1,8 +1,10 @@
 // Host side of the C ABI: argument validation, error text, dispatch of spf_score.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "common.cuh"
 #include "score.cuh"
@@ -85,6 +87,50 @@ int32_t device_sm_count(int* out) {
   return SPF_OK;
 }
 
+// Scratch that a call with these prompts may use: the general path works on one prompt at a time, the fused path on up to
+// kFusedMaxBatch consecutive ones.
+size_t workspace_need(const ScoreProblem* p, int32_t n) {
+  size_t need = 0, window = 0;
+  for (int32_t i = 0; i < n; ++i) {
+    window += score_fused_workspace_bytes(p[i]);
+    if (i >= kFusedMaxBatch) window -= score_fused_workspace_bytes(p[i - kFusedMaxBatch]);
+    need = std::max(need, std::max(score_mma_workspace_bytes(p[i]), window));
+  }
+  return need;
+}
+
+int32_t check_workspace(const char* who, const ScoreProblem* p, int32_t n, const void* workspace, size_t workspace_bytes) {
+  const size_t need = workspace_need(p, n);
+  if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
+    return fail(SPF_ERR_WORKSPACE, "%s: workspace is null or not 256-byte aligned", who);
+  if (workspace_bytes < need) return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need);
+  return SPF_OK;
+}
+
+// Scores validated prompts: runs of consecutive prompts that the fused kernel takes go to it together, the others one by
+// one to the general kernels.
+int32_t score_problems(const char* who, const ScoreProblem* p, int32_t n, int path, void* workspace, size_t workspace_bytes,
+                       int32_t* dev_status, cudaStream_t stream) {
+  int32_t st = check_workspace(who, p, n, workspace, workspace_bytes);
+  if (st != SPF_OK) return st;
+  int sm_count = 0;
+  st = device_sm_count(&sm_count);
+  if (st != SPF_OK) return st;
+  for (int32_t i = 0; i < n;) {
+    int32_t j = i;
+    while (j < n && (path == 2 || (path == 0 && score_fused_supported(p[j], sm_count)))) ++j;
+    if (j > i) {
+      st = score_fused_launch(p + i, j - i, workspace, sm_count, dev_status, stream);
+      i = j;
+    } else {
+      st = score_mma_launch(p[i], workspace, sm_count, stream);
+      ++i;
+    }
+    if (st != SPF_OK) return st;
+  }
+  return SPF_OK;
+}
+
 }  // namespace
 
 int32_t fail(int32_t code, const char* fmt, ...) {
@@ -101,55 +147,41 @@ void clear_error() { g_error[0] = '\0'; }
 
 using namespace spf;
 
-extern "C" size_t spf_score_workspace_bytes(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts) {
+// The three forms of a prompt (contiguous, paged, 8-bit keys) differ in how they become a ScoreProblem; everything else is
+// shared.
+template <class Prompt, class Make>
+static int32_t make_problems(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n_prompts, Make make,
+                             std::vector<ScoreProblem>* out) {
   clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1) {
-    fail(SPF_ERR_INVALID_ARG, "spf_score_workspace_bytes: null argument or n_prompts < 1");
-    return 0;
-  }
-  size_t need = 0;
+  if (shape == nullptr || prompts == nullptr || n_prompts < 1)
+    return fail(SPF_ERR_INVALID_ARG, "%s: null argument or n_prompts < 1", who);
+  out->resize((size_t)n_prompts);
   for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    if (make_problem(shape, prompts[i], i, &p) != SPF_OK) return 0;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
+    const int32_t st = make(shape, prompts[i], i, &(*out)[i]);
+    if (st != SPF_OK) return st;
   }
-  return need;
+  return SPF_OK;
+}
+
+static int32_t make_flat_problem(const spf_shape* shape, const spf_prompt& pr, int32_t index, ScoreProblem* out) {
+  return make_problem(shape, pr, index, out);
+}
+
+extern "C" size_t spf_score_workspace_bytes(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts) {
+  std::vector<ScoreProblem> p;
+  if (make_problems("spf_score_workspace_bytes", shape, prompts, n_prompts, make_flat_problem, &p) != SPF_OK) return 0;
+  return workspace_need(p.data(), n_prompts);
 }
 
 static int32_t score_impl(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts, const float* const* extra_lse,
                           void* workspace, size_t workspace_bytes, int32_t* dev_status, void* cuda_stream, int path_override = -1) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1)
-    return fail(SPF_ERR_INVALID_ARG, "spf_score: null argument or n_prompts < 1");
-  // validate everything before the first launch
-  size_t need = 0;
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    const int32_t st = make_problem(shape, prompts[i], i, &p);
-    if (st != SPF_OK) return st;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
-  }
-  if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
-    return fail(SPF_ERR_WORKSPACE, "spf_score: workspace is null or not 256-byte aligned");
-  if (workspace_bytes < need)
-    return fail(SPF_ERR_WORKSPACE, "spf_score: workspace has %zu bytes, %zu needed", workspace_bytes, need);
-  int sm_count = 0;
-  {
-    const int32_t st = device_sm_count(&sm_count);
-    if (st != SPF_OK) return st;
-  }
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    make_problem(shape, prompts[i], i, &p);
-    if (extra_lse != nullptr) p.extra_lse = extra_lse[i];
-    const int path = path_override >= 0 ? path_override : g_score_path.load(std::memory_order_relaxed);
-    const bool fused = path == 2 || (path == 0 && score_fused_supported(p, sm_count));
-    const int32_t st = fused ? score_fused_launch(p, workspace, sm_count, dev_status, stream)
-                             : score_mma_launch(p, workspace, sm_count, stream);
-    if (st != SPF_OK) return st;
-  }
-  return SPF_OK;
+  std::vector<ScoreProblem> p;
+  const int32_t st = make_problems("spf_score", shape, prompts, n_prompts, make_flat_problem, &p);
+  if (st != SPF_OK) return st;
+  for (int32_t i = 0; i < n_prompts && extra_lse != nullptr; ++i) p[i].extra_lse = extra_lse[i];
+  const int path = path_override >= 0 ? path_override : g_score_path.load(std::memory_order_relaxed);
+  return score_problems("spf_score", p.data(), n_prompts, path, workspace, workspace_bytes, dev_status,
+                        static_cast<cudaStream_t>(cuda_stream));
 }
 
 namespace spf {
@@ -196,52 +228,18 @@ static int32_t make_paged_problem(const spf_shape* shape, const spf_paged_prompt
 }
 
 extern "C" size_t spf_score_paged_workspace_bytes(const spf_shape* shape, const spf_paged_prompt* prompts, int32_t n_prompts) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1) {
-    fail(SPF_ERR_INVALID_ARG, "spf_score_paged_workspace_bytes: null argument or n_prompts < 1");
-    return 0;
-  }
-  size_t need = 0;
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    if (make_paged_problem(shape, prompts[i], i, &p) != SPF_OK) return 0;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
-  }
-  return need;
+  std::vector<ScoreProblem> p;
+  if (make_problems("spf_score_paged_workspace_bytes", shape, prompts, n_prompts, make_paged_problem, &p) != SPF_OK) return 0;
+  return workspace_need(p.data(), n_prompts);
 }
 
 extern "C" int32_t spf_score_paged(const spf_shape* shape, const spf_paged_prompt* prompts, int32_t n_prompts, void* workspace,
                                    size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1)
-    return fail(SPF_ERR_INVALID_ARG, "spf_score_paged: null argument or n_prompts < 1");
-  int sm_count = 0;
-  {
-    const int32_t st = device_sm_count(&sm_count);
-    if (st != SPF_OK) return st;
-  }
-  size_t need = 0;
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    const int32_t st = make_paged_problem(shape, prompts[i], i, &p);
-    if (st != SPF_OK) return st;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
-  }
-  if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
-    return fail(SPF_ERR_WORKSPACE, "spf_score_paged: workspace is null or not 256-byte aligned");
-  if (workspace_bytes < need)
-    return fail(SPF_ERR_WORKSPACE, "spf_score_paged: workspace has %zu bytes, %zu needed", workspace_bytes, need);
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    make_paged_problem(shape, prompts[i], i, &p);
-    const int path = g_score_path.load(std::memory_order_relaxed);
-    const bool fused = path == 2 || (path == 0 && score_fused_supported(p, sm_count));
-    const int32_t st = fused ? score_fused_launch(p, workspace, sm_count, dev_status, stream)
-                             : score_mma_launch(p, workspace, sm_count, stream);
-    if (st != SPF_OK) return st;
-  }
-  return SPF_OK;
+  std::vector<ScoreProblem> p;
+  const int32_t st = make_problems("spf_score_paged", shape, prompts, n_prompts, make_paged_problem, &p);
+  if (st != SPF_OK) return st;
+  return score_problems("spf_score_paged", p.data(), n_prompts, g_score_path.load(std::memory_order_relaxed), workspace, workspace_bytes,
+                        dev_status, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // 8-bit key cache: described as a bf16 prompt over the same pointers (the checks are the same: strides count elements,
@@ -263,50 +261,18 @@ static int32_t make_fp8_problem(const spf_shape* shape, const spf_fp8_prompt& fp
 }
 
 extern "C" size_t spf_score_fp8_workspace_bytes(const spf_shape* shape, const spf_fp8_prompt* prompts, int32_t n_prompts) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1) {
-    fail(SPF_ERR_INVALID_ARG, "spf_score_fp8_workspace_bytes: null argument or n_prompts < 1");
-    return 0;
-  }
-  size_t need = 0;
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    if (make_fp8_problem(shape, prompts[i], i, &p) != SPF_OK) return 0;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
-  }
-  return need;
+  std::vector<ScoreProblem> p;
+  if (make_problems("spf_score_fp8_workspace_bytes", shape, prompts, n_prompts, make_fp8_problem, &p) != SPF_OK) return 0;
+  return workspace_need(p.data(), n_prompts);
 }
 
 extern "C" int32_t spf_score_fp8(const spf_shape* shape, const spf_fp8_prompt* prompts, int32_t n_prompts, void* workspace,
-                                 size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1)
-    return fail(SPF_ERR_INVALID_ARG, "spf_score_fp8: null argument or n_prompts < 1");
-  size_t need = 0;
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    const int32_t st = make_fp8_problem(shape, prompts[i], i, &p);
-    if (st != SPF_OK) return st;
-    need = std::max(need, std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p)));
-  }
-  if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
-    return fail(SPF_ERR_WORKSPACE, "spf_score_fp8: workspace is null or not 256-byte aligned");
-  if (workspace_bytes < need) return fail(SPF_ERR_WORKSPACE, "spf_score_fp8: workspace has %zu bytes, %zu needed", workspace_bytes, need);
-  int sm_count = 0;
-  {
-    const int32_t st = device_sm_count(&sm_count);
-    if (st != SPF_OK) return st;
-  }
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    ScoreProblem p;
-    make_fp8_problem(shape, prompts[i], i, &p);
-    const int path = g_score_path.load(std::memory_order_relaxed);
-    const bool fused = path == 2 || (path == 0 && score_fused_supported(p, sm_count));
-    const int32_t st = fused ? score_fused_launch(p, workspace, sm_count, dev_status, stream) : score_mma_launch(p, workspace, sm_count, stream);
-    if (st != SPF_OK) return st;
-  }
-  return SPF_OK;
+                                   size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
+  std::vector<ScoreProblem> p;
+  const int32_t st = make_problems("spf_score_fp8", shape, prompts, n_prompts, make_fp8_problem, &p);
+  if (st != SPF_OK) return st;
+  return score_problems("spf_score_fp8", p.data(), n_prompts, g_score_path.load(std::memory_order_relaxed), workspace, workspace_bytes,
+                        dev_status, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // Key-sharded scoring: the two sweeps of the general path as separate calls.
@@ -328,16 +294,14 @@ static int32_t score_shard(const spf_shape* shape, const spf_prompt* prompt, int
   if (st != SPF_OK) return st;
   if (phase == 1) p.importance = nullptr;
   if (phase == 2) p.lse_out = nullptr;
-  const size_t need = std::max(score_mma_workspace_bytes(p), score_fused_workspace_bytes(p));
-  if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
-    return fail(SPF_ERR_WORKSPACE, "%s: workspace is null or not 256-byte aligned", who);
-  if (workspace_bytes < need) return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need);
+  const int32_t ws = check_workspace(who, &p, 1, workspace, workspace_bytes);
+  if (ws != SPF_OK) return ws;
   int sm_count = 0;
   const int32_t sc = device_sm_count(&sm_count);
   if (sc != SPF_OK) return sc;
   const int path = g_score_path.load(std::memory_order_relaxed);
   if (allow_fused && (path == 2 || (path == 0 && score_fused_supported(p, sm_count))))
-    return score_fused_launch(p, workspace, sm_count, dev_status, static_cast<cudaStream_t>(cuda_stream), phase, lse_in);
+    return score_fused_launch(&p, 1, workspace, sm_count, dev_status, static_cast<cudaStream_t>(cuda_stream), phase, lse_in);
   return score_mma_launch_phase(p, workspace, sm_count, phase, lse_in, static_cast<cudaStream_t>(cuda_stream));
 }
 

@@ -1,0 +1,1108 @@
+// Token-importance scoring, fused path: ONE persistent kernel that reads the key cache once from HBM.
+//
+// Why logits are looked at twice.  The max over (layer, head) is taken over softmax PROBABILITIES, so a logit can only be
+// compared across heads after its row's log-sum-exp is known, and that needs all N keys of the row.  Each (layer, kv-head)
+// slab of keys is therefore visited twice:
+//   visit 1 ("sum")  accumulates  sum_s exp2(c * q.k - ref)  per query row;
+//   visit 2 ("max")  folds  max_{l,h} (c * q.k - lse)  into a running maximum per (lookahead i, key s).
+//
+// Two forms of the kernel, by what lies between the visits.
+//   Resident (template ONCE): the logits wait in tensor memory.  A tile's 128 x NCOLS accumulators are summed by the sum
+//   warps and stay where they are until the slab's log-sum-exps arrive; then the max warps fold them and free the columns.
+//   Keys are copied and multiplied once.  This needs room for a CTA's tiles of one slab plus those that arrive during the
+//   hand-over: up to 32 query rows, and prompts of up to a few hundred thousand tokens (see resident_tiles).
+//   Two-pass: the logits are recomputed.  The two visits are two independent pipelines (TMA warp -> key ring -> MMA warp ->
+//   tensor-memory ring -> epilogue warps) that share the SM and meet only in the log-sum-exps.  Visit 2 follows visit 1 over
+//   the same list of tiles as soon as a slab's log-sum-exps are there; visit 1 may be at most `lead` tiles ahead of it, so
+//   that the second read still finds its tiles in L2.  For 64 query rows, where tensor memory holds six tiles' logits.
+//
+// Work split.  A prompt has T tiles of 128 keys and S slabs.  Its CTAs form `parts` groups; group p takes the slabs s with
+// s % parts == p and its CTAs deal the T tiles out among themselves.  One group (parts = 1) is the plain split for long
+// prompts: a CTA owns its tiles for all slabs and writes their importance alone.  More groups are what keeps the chip busy
+// when there are fewer tiles than SMs, and what evens out a last round of tiles that would leave most SMs idle; the groups'
+// running maxima then meet in global memory (integer max on order-preserving bits, exact and independent of order), and the
+// last group to finish 32 keys turns them into importance.  Several prompts share one launch, each with CTAs of its own.
+//
+// Tensor-core tiles.  The operands in shared memory are 128 keys x d (TMA) and the slab's query rows x d (row j = i * G + g:
+// lookahead i, head g of the GQA group, the group padded to a power of two).  Resident, and visit 2 of the two-pass form:
+// keys are the tensor-memory lanes, so the max over the heads of a group is in-thread; the sum over keys ends every slab
+// with a 32-lane reduction of up to 32 columns.  Visit 1 of the two-pass form: query rows are the lanes (weight-stationary
+// instructions, which fill all 128 lanes with 32 or 64 rows), so the sum over keys stays inside a thread too; with 64
+// columns the reduction cost 1000 to 2900 cycles per slab and CTA.  The running maxima live in tensor memory next to the
+// accumulators.
+//
+// Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each).  4: fetches log-sum-exps
+// for visit 2.  5..7: publishers (add a slab's row sums of this CTA to the slab's totals; the CTA that completes a slab
+// converts the totals).  8..15: "sum" warps.  16..23: "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM
+// lane quadrant and the next bit the `set`: the two sets take turns at the tiles, so that one set's tensor-memory loads and
+// waits run while the other set computes.  (Splitting every tile's columns between the sets kept all eight warps in step,
+// all waiting or all computing.)
+//
+// Reference.  Visit 1 subtracts one reference per slab inside the exp2 argument: the SMALLEST logit of the slab's rows
+// against one fixed sample key, plus a margin of 60 (base-2 units).  Every row's largest logit is at least its own sample
+// logit, hence at least reference - 60, and ex2.approx.ftz only flushes terms below reference - 126, i.e. terms more than
+// 2^66 times smaller than the row's largest: no row can lose anything that matters, whatever the spread between the heads
+// of a group.  What can still go wrong is overflow: a row sum reaches 2^128 when some logit lies about 188 - log2(keys at
+// that level) base-2 units (157 at the very least, about 109 nats) above the slab's smallest sample logit.  That is
+// detected (the sum is inf) and reported as SPF_ERR_RANGE; the caller can then use the general path.
+//
+// Cross-CTA step.  All CTAs use the same reference for a slab, so their partial sums can simply be added.  To make the
+// total independent of the order in which CTAs arrive, the fp32 partial sums are added EXACTLY: each is split over two
+// 40-bit limbs of a 280-bit fixed-point accumulator per row (64-bit integer atomics, no carries needed), which covers every
+// finite fp32 value.  The CTA whose arrival completes a slab converts the accumulators to log-sum-exps and stores each as
+// one 64-bit word {value, 1}; the other CTAs poll those words, so no CTA repeats the conversion and no fence sits between
+// value and flag.  Results are bit-identical from run to run.  Visit 1 waits for other CTAs only through its lead over
+// visit 2, which covers at least one whole slab, so every slab's sums complete and the words always arrive.
+//
+// Every wait on a barrier, word or flag in this file is bounded: on expiry the kernel records SPF_ERR_TIMEOUT, drains and
+// returns normally.  The one wait that has no limit is the hardware's own: tcgen05.alloc blocks while another resident CTA
+// on the SM holds tensor memory (this kernel asks for all of it), i.e. until that CTA exits.
+#pragma once
+
+#include "score.cuh"
+#include "tc_ptx.cuh"
+
+namespace spf {
+
+constexpr int kFusedThreads = 768;
+constexpr int kVisitWarps = 8;         // epilogue warps per visit
+constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
+constexpr int kPublisherWarp0 = 5, kPublisherWarps = 3;
+constexpr int kLimbs = 7;              // 40-bit limbs of the exact row-sum accumulators (covers every finite fp32)
+constexpr int kLimbStride = 8;         // 64-bit words per row in the accumulator array
+constexpr int kMaxQStages = 4;         // query tiles in flight per visit (two-pass: 2)
+constexpr int kMaxKeyStages = 16;      // key tiles in flight per visit
+constexpr int kMaxTmemStages = 4;      // two-pass: accumulator stages per visit and set
+constexpr int kMaxResident = 32;       // resident: tiles in tensor memory
+constexpr int kTmemColsAll = 512;      // the CTA takes all of its SM's tensor memory
+constexpr int kOffSlots = 4;           // slabs whose log-sum-exps may be in shared memory at once
+constexpr int kSumSlots = 8;           // slabs whose row sums may be on their way to the publishers at once
+constexpr float kRefMargin = 60.f;     // base-2 units added to the sampled reference logit
+
+// Key rows are d bf16 (128 or 256 bytes) or d E4M3 bytes (64 or 128).  A tile is stored as sub-tiles of 128 keys x one
+// swizzle span: 128 bytes of the row (128-byte swizzle), or the whole row where it has only 64 bytes (64-byte swizzle).
+__host__ __device__ constexpr int row_bytes(int d, bool fp8) { return fp8 ? d : 2 * d; }
+__host__ __device__ constexpr int sub_row_bytes(int rowb) { return rowb > 128 ? 128 : rowb; }
+// Query rows of a visit-1 instruction (its M), and its accumulator columns per tile: 32 x 32 or 64 x 64.
+__host__ __device__ constexpr int sum_rows(int ncols) { return ncols <= 32 ? 32 : 64; }
+
+struct FusedPrompt {
+  const CUtensorMap* k_maps;   // [n_layers] (element of a sub-row, key, sub-tile, kv-head[, pool block])
+  const unsigned char* q_tiles;   // [slab] query operands as the tensor cores read them (swizzled, padding rows zero)
+  unsigned long long* limbs;   // [slab][NCOLS][kLimbStride] exact fixed-point sums of exp2(c*q.k - ref) over all keys
+  unsigned* counters;          // [slab] CTAs whose share of the slab's row sums is in the accumulators
+  unsigned long long* lse;     // [slab][NCOLS] {log-sum-exp in base-2 units, 1} once known
+  const float* refs;           // [slab] reference of visit 1
+  const float* slab_c;         // [slab] 8-bit keys: accumulated dot product -> base-2 logit; null: FusedArgs::c for all
+  unsigned* amax;              // [m][n_tiles * 128] order-preserving bits of the running maxima (parts > 1)
+  unsigned* finished;          // [n_tiles][4] arrivals at `amax` (parts > 1)
+  float* importance;           // [N]
+  float* lse_out;              // optional [L][Hq][m], natural log
+  const float* extra_lse;      // optional [L][Hq][m], natural log: what each row's denominator holds besides the prompt keys
+  const float* lse_in;         // visit 2 alone: row log-sum-exps supplied by the caller, natural log, [L][Hq][m]
+  const int32_t* block_table;  // paged key cache (block_tokens > 0): pool block of each logical block
+  int64_t n_tokens;
+  int block_tokens, n_tiles;
+  int cta0, parts, per_part;   // CTAs cta0 .. cta0 + parts * per_part - 1
+  int lead;                    // tiles that visit 1 may be ahead of visit 2
+};
+
+struct FusedArgs {
+  FusedPrompt prompt[kFusedMaxBatch];
+  int n_prompts, n_layers, n_kv_heads, group, n_lookahead;
+  int table_tiles;             // tiles per CTA for which there is a table (paged key cache), else 0
+  int mode;                    // 0: the whole computation; 1: visit 1 alone (row log-sum-exps of these keys); 2: visit 2 alone
+  int k_stages[2], t_stages[2];   // per visit: key tiles; accumulator stages per set (resident: [0] alone, tiles in tensor memory)
+  int max_tiles_per_stage;     // tiles per accumulator stage of visit 2 (visit 1: one)
+  float c;                     // softmax scale * log2(e)
+  int32_t* dev_status;         // optional
+};
+
+// Barrier addresses (8 bytes each): two visits' rings, the log-sum-exp slots, the row-sum slots.
+struct FusedBars {
+  uint32_t base;
+  static constexpr int kVisit = 2 * (kMaxKeyStages + kMaxQStages), kTmem = 2 * kVisit, kShared = kTmem + 2 * kMaxResident;
+  static constexpr int kCount = kShared + 2 * kOffSlots + 2 * kSumSlots + 2;
+  __device__ uint32_t k_full(int v, int s) const { return base + 8u * (v * kVisit + s); }
+  __device__ uint32_t k_empty(int v, int s) const { return base + 8u * (v * kVisit + kMaxKeyStages + s); }
+  __device__ uint32_t q_full(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + s); }
+  __device__ uint32_t q_empty(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + kMaxQStages + s); }
+  // two-pass: stage s of a visit's set; resident: stage s (v = set = 0)
+  __device__ uint32_t t_full(int v, int set, int s) const { return base + 8u * (kTmem + (v * 2 + set) * kMaxTmemStages + s); }
+  __device__ uint32_t t_empty(int v, int set, int s) const { return t_full(v, set, s) + 8u * kMaxResident; }
+  __device__ uint32_t off_ready(int x) const { return base + 8u * (kShared + x); }
+  __device__ uint32_t off_free(int x) const { return base + 8u * (kShared + kOffSlots + x); }
+  __device__ uint32_t sums_ready(int x) const { return base + 8u * (kShared + 2 * kOffSlots + x); }
+  __device__ uint32_t sums_free(int x) const { return base + 8u * (kShared + 2 * kOffSlots + kSumSlots + x); }
+  __device__ uint32_t mma_done(int v) const { return base + 8u * (kShared + 2 * kOffSlots + 2 * kSumSlots + v); }
+};
+static_assert(4 * kMaxTmemStages <= kMaxResident, "the two-pass stages use the same barriers");
+
+struct FusedSmem {
+  uint32_t k_off[2], q_off[2], sums_off, off_off, offc_off, bar_off, misc_off, tile_off, total;
+};
+
+__host__ __device__ inline FusedSmem fused_smem(int d, bool fp8, int ncols, bool once, int tiles, const int k_stages[2]) {
+  FusedSmem s;
+  uint32_t o = 0;
+  const uint32_t rowb = (uint32_t)row_bytes(d, fp8), q_rows = ncols < 32 ? 32 : ncols;
+  for (int v = 0; v < 2; ++v) { s.k_off[v] = o; o += (uint32_t)k_stages[v] * kTileKeys * rowb; }
+  for (int v = 0; v < 2; ++v) { s.q_off[v] = o; o += (uint32_t)(once ? (v == 0 ? kMaxQStages : 0) : 2) * (fp8 ? 2 : 1) * q_rows * rowb; }
+  s.sums_off = o;  o += kSumSlots * 256 * 4;            // [slot][set][quadrant][lane]
+  s.off_off = o;   o += kOffSlots * 64 * 4;
+  s.offc_off = o;  o += kOffSlots * 4;
+  s.bar_off = o;   o += FusedBars::kCount * 8;
+  s.misc_off = o;  o += 64;
+  s.tile_off = o;  o += tiles * 8;                      // paged key cache: row in the block and pool block of each tile
+  s.total = o;
+  return s;
+}
+
+struct Ring {
+  int stage = 0;
+  uint32_t phase = 0;
+  int n;
+  __device__ explicit Ring(int n_) : n(n_) {}
+  __device__ void advance() {
+    if (++stage == n) {
+      stage = 0;
+      phase ^= 1u;
+    }
+  }
+};
+
+// fp32 <-> unsigned bits whose integer order is the float order (0 is below every float).
+__device__ __forceinline__ unsigned order_bits(float x) {
+  const unsigned b = __float_as_uint(x);
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float from_order_bits(unsigned u) {
+  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+
+template <int D, int NCOLS, int G, bool FP8, bool ONCE>
+struct FusedTraits {
+  static constexpr int QS = ONCE ? kMaxQStages : 2;                // query tiles in flight per visit
+  static constexpr int SR = sum_rows(NCOLS);                       // two-pass visit 1: query rows per instruction = accumulator columns per tile
+  static constexpr int CW = NCOLS < 32 ? NCOLS : 32;               // visit 2: accumulators per tensor-memory load
+  static constexpr int NCH = NCOLS / CW;                           // loads per tile: 1 or 2
+  static constexpr int NI = NCOLS / G;                             // lookahead slots per key in the running-max columns
+  static constexpr int NIW = CW / G;                               // of which one load's accumulators hold
+  static constexpr int ROWB = row_bytes(D, FP8);                   // bytes per key row: 64, 128 or 256
+  static constexpr int SUBROW = sub_row_bytes(ROWB);               // the swizzle span: 128 bytes, or the whole 64-byte row
+  static constexpr int KSUB = ROWB / SUBROW;                       // sub-tiles per key tile
+  static constexpr int KSTEPS = SUBROW / 32;                       // tensor-core instructions per sub-tile (32 bytes of the row each)
+  static constexpr int XSUB = SUBROW / (FP8 ? 1 : 2);              // elements per sub-tile row
+  static constexpr int kSubTileBytes = kTileKeys * SUBROW;
+  static constexpr int kTileBytes = KSUB * kSubTileBytes;
+  static constexpr int QPARTS = FP8 ? 2 : 1;                       // 8-bit keys: the queries come as two E4M3 terms
+  static constexpr int kQSub = (NCOLS < 32 ? 32 : NCOLS) * SUBROW; // the weight-stationary form multiplies at least 32 rows; unused ones are zero
+  static constexpr int kQBytes = QPARTS * KSUB * kQSub;
+};
+
+// What every warp of a CTA knows about its share of the work.
+struct FusedShare {
+  const FusedPrompt* p;
+  int part, parts, first, step;   // this CTA's slabs are part, part + parts, ...; its tiles first, first + step, ...
+  int n_slabs, n_tiles;           // how many of each
+  __device__ int slab(int n) const { return part + n * parts; }
+  __device__ int tile(int lt) const { return first + lt * step; }
+};
+
+// Which set of epilogue warps takes local tile lt of the CTA's n-th slab.  The sums take turns from slab to slab too, so
+// that slabs of a single tile are shared out; a tile's maxima always belong to the same warps.
+__device__ __forceinline__ int fused_set(int v, int n, int lt) { return (v == 0 ? lt + n : lt) & 1; }
+
+// ---------------------------------------------------------------------------------------------- TMA producer of one visit
+template <class T, bool ONCE>
+__device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedShare& sh, int v, unsigned char* k_tiles, unsigned char* q_tiles,
+                                              const int2* tile_at, const FusedBars& bars, volatile int* visit2_issued, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  Ring kr(a.k_stages[v]), qr(T::QS);
+  const uint64_t policy = !ONCE && v == 0 ? l2_policy_keep() : l2_policy_drop();
+  const uint32_t k_smem = smem_u32(k_tiles), q_smem = smem_u32(q_tiles);
+  const CUtensorMap* const maps = p.k_maps;
+  const unsigned char* const q_src = p.q_tiles;
+  const bool paged = p.block_tokens > 0;
+  const int n_kv_heads = a.n_kv_heads;
+  const int lead = !ONCE && a.mode == 0 ? p.lead : 0x7fffffff;
+  // slab n is (layer, hk); from one slab of the CTA to the next both advance by a fixed step
+  int layer = sh.part / n_kv_heads, hk = sh.part - layer * n_kv_heads, issued = 0;
+  const int layer_step = sh.parts / n_kv_heads, hk_step = sh.parts - layer_step * n_kv_heads;
+  map_acquire(maps + layer);
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    const CUtensorMap* map = maps + layer;
+    if (!mbar_wait(bars.q_empty(v, qr.stage), qr.phase ^ 1u, ab)) return;
+    mbar_expect_tx(bars.q_full(v, qr.stage), (uint32_t)T::kQBytes);
+    bulk_load(q_smem + (uint32_t)(qr.stage * T::kQBytes), q_src + (int64_t)sh.slab(n) * T::kQBytes, (uint32_t)T::kQBytes,
+              bars.q_full(v, qr.stage));
+    qr.advance();
+    for (int lt = 0; lt < sh.n_tiles; ++lt, ++issued) {
+      if (!ONCE && v == 0) {
+        // never more than `lead` tiles ahead of visit 2
+        unsigned long long t0 = 0;
+        for (uint32_t it = 1; issued - *visit2_issued >= lead; ++it) {
+          if (give_up(it, t0, ab)) return;
+          __nanosleep(40);
+        }
+      }
+      if (!mbar_wait(bars.k_empty(v, kr.stage), kr.phase ^ 1u, ab)) return;
+      const uint32_t dst = k_smem + (uint32_t)(kr.stage * T::kTileBytes), bar = bars.k_full(v, kr.stage);
+      mbar_expect_tx(bar, (uint32_t)T::kTileBytes);
+      if (paged) {
+        const int2 at = tile_at[lt];
+        tma_load_5d(dst, map, 0, at.x, 0, hk, at.y, bar, policy);
+      } else {
+        tma_load_4d(dst, map, 0, sh.tile(lt) * kTileKeys, 0, hk, bar, policy);
+      }
+      kr.advance();
+      if (v == 1) *visit2_issued = issued + 1;
+    }
+    const int before = layer;
+    hk += hk_step;
+    layer += layer_step;
+    if (hk >= n_kv_heads) {
+      hk -= n_kv_heads;
+      ++layer;
+    }
+    if (layer != before && n + 1 < sh.n_slabs) map_acquire(maps + layer);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- MMA issuer of one visit
+// The whole warp walks the loop (addresses and descriptors stay warp-uniform); one elected lane issues.
+template <class T, int NCOLS, bool FP8, int V>
+__device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedShare& sh, const unsigned char* k_tiles,
+                                               const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
+  constexpr uint32_t idesc = V == 0 ? instr_desc(T::SR, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
+  constexpr int kTileCols = V == 0 ? T::SR : NCOLS;
+  const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
+  const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
+  const int tps = V == 0 ? 1 : a.max_tiles_per_stage, stages = a.t_stages[V];
+  Ring kr(a.k_stages[V]), qr(T::QS), tr0(stages), tr1(stages);
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    if (!mbar_wait_warp(bars.q_full(V, qr.stage), qr.phase, ab)) return;
+    const uint64_t qd0 = q_desc0 + (uint64_t)((qr.stage * T::kQBytes) >> 4);
+    int fill0 = 0, fill1 = 0;                                      // tiles in the sets' current stages
+    auto tile = [&](int lt, int set, Ring& tr, int& fill) -> bool {
+      if (fill == 0) {
+        if (!mbar_wait2_warp(bars.k_full(V, kr.stage), kr.phase, bars.t_empty(V, set, tr.stage), tr.phase ^ 1u, ab)) return false;
+      } else {
+        if (!mbar_wait_warp(bars.k_full(V, kr.stage), kr.phase, ab)) return false;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem + (uint32_t)(((set * stages + tr.stage) * tps + fill) * kTileCols);
+      const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
+      const bool last = ++fill == tps || lt + 2 >= sh.n_tiles;     // of this stage: it is full, or the set has no tile left
+      if (elect_one()) {
+        // 8-bit keys: the two query terms accumulate into the same columns
+#pragma unroll
+        for (int part = 0; part < T::QPARTS; ++part)
+#pragma unroll
+          for (int h = 0; h < T::KSUB; ++h)
+#pragma unroll
+            for (int ks = 0; ks < T::KSTEPS; ++ks) {
+              const uint64_t kd = kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks;
+              const uint64_t qd = qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks;
+              if constexpr (V == 0) tc_mma<FP8, true>(d_tmem, qd, kd, idesc, (uint32_t)((part | h | ks) != 0));
+              else tc_mma<FP8, false>(d_tmem, kd, qd, idesc, (uint32_t)((part | h | ks) != 0));
+            }
+        tc_commit(bars.k_empty(V, kr.stage));
+        if (last) tc_commit(bars.t_full(V, set, tr.stage));
+      }
+      __syncwarp();
+      kr.advance();
+      if (last) {
+        tr.advance();
+        fill = 0;
+      }
+      return true;
+    };
+    for (int lt = 0; lt < sh.n_tiles; ++lt)
+      if (!(fused_set(V, n, lt) == 0 ? tile(lt, 0, tr0, fill0) : tile(lt, 1, tr1, fill1))) return;
+    if (elect_one()) tc_commit(bars.q_empty(V, qr.stage));         // arrives once the slab's MMAs are done
+    __syncwarp();
+    qr.advance();
+  }
+  // leave only after everything issued has completed and signalled its barriers
+  if (elect_one()) tc_commit(bars.mma_done(V));
+  __syncwarp();
+  mbar_wait_warp(bars.mma_done(V), 0u, ab);
+}
+
+// ---------------------------------------------------------------------------------------------- visit 1: sums
+// A thread has one query row and, per tile, 32 or 64 of its keys (64 rows: lanes 64.. repeat the rows for the tile's second
+// half; 32 rows: a quarter of the keys per quadrant).  Bound by the exp2 unit (16 results a cycle and SM: 512 cycles per
+// tile of 64 rows; the loop alone with its MMAs takes 645).  One load of 32 columns at a time, computed before the next is
+// asked for: the other set's warps fill the gap, and keeping a load in flight across the arithmetic measured 8 to 15 % slower.
+template <class T, bool FP8>
+__device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
+                                          const FusedBars& bars, const Abort& ab) {
+  constexpr int NL = T::SR / 32;                                   // tensor-memory loads of 32 columns per tile
+  const FusedPrompt& p = *sh.p;
+  const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
+  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+  const float* const refs = p.refs;
+  const float* const slab_c = p.slab_c;
+  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * a.t_stages[0] * T::SR);
+  const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
+  const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - (T::SR == 64 ? (quad >> 1) * 64 : quad * 32);
+  Ring tr(a.t_stages[0]);
+  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
+  for (int n = 0; n < n_slabs; ++n) {
+    const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
+    if (n + 1 < n_slabs) {
+      next_ref = __ldg(refs + sh.slab(n + 1));
+      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
+    }
+    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int lt = fused_set(0, n, 0) == set ? 0 : 1; lt < n_tiles; lt += 2) {
+      if (!mbar_wait_warp(bars.t_full(0, set, tr.stage), tr.phase, ab)) return;
+      tc_fence_after();
+      const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * T::SR);
+      const uint32_t empty = bars.t_empty(0, set, tr.stage);
+      tr.advance();
+#pragma unroll
+      for (int load = 0; load < NL; ++load) {
+        uint32_t r[32];
+        tmem_issue<32>(taddr + (uint32_t)(32 * load), r);
+        tmem_load_wait();
+        tmem_ready<32>(r);
+        if (load + 1 == NL) {
+          // the stage can be overwritten: its last accumulators are in registers
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(empty);
+        }
+        if (sh.tile(lt) < full_tiles) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            float x, y;
+            unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
+            acc[j & 3] = add2(acc[j & 3], pack2(fast_exp2(x), fast_exp2(y)));
+          }
+        } else {
+          // the prompt's last, partial tile: keys beyond the end count nothing
+          const int left = tail_keys - load * 32;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            float x, y;
+            unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
+            acc[j & 3] = add2(acc[j & 3], pack2(2 * j < left ? fast_exp2(x) : 0.f, 2 * j + 1 < left ? fast_exp2(y) : 0.f));
+          }
+        }
+      }
+    }
+    const int slot = n % kSumSlots;
+    if (n >= kSumSlots)
+      if (!mbar_wait_warp(bars.sums_free(slot), (uint32_t)(n / kSumSlots - 1) & 1u, ab)) return;
+    float x, y;
+    unpack2(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), x, y);
+    sums[((slot * 2 + set) * 4 + quad) * 32 + lane] = x + y;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.sums_ready(slot));
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- publishers
+// Publisher w takes slabs w, w + 3, ...: adds the CTA's row sums to the slab's exact totals, then counts the CTA in.  A fence
+// and an atomic's round trip per slab: three warps keep up with slabs of a single tile.
+template <class T, int NCOLS, int G>
+__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums,
+                                              const FusedBars& bars, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  constexpr int RPL = NCOLS == 64 ? 2 : 1;                         // rows per lane
+  const unsigned expected = (unsigned)min(p.per_part, p.n_tiles);
+  for (int n = which; n < sh.n_slabs; n += kPublisherWarps) {
+    const int slot = n % kSumSlots, slab = sh.slab(n);
+    if (!mbar_wait_warp(bars.sums_ready(slot), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
+    const float* in = sums + slot * 256;
+    float tot[RPL];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      float t = 0.f;
+#pragma unroll
+      for (int set = 0; set < 2; ++set)
+#pragma unroll
+        for (int q = 0; q < 4 / RPL; ++q) t += in[(set * 4 + q * RPL + r) * 32 + lane];   // 64 rows: quadrants r and r + 2
+      tot[r] = t;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.sums_free(slot));
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const int row = lane + 32 * r;
+      if (row < NCOLS && row % G < a.group && row / G < a.n_lookahead) {
+        const uint32_t bits = __float_as_uint(tot[r]);
+        const uint32_t expo = bits >> 23;                          // sums are non-negative: no sign bit
+        if (expo >= 255u) {
+          if (a.dev_status != nullptr) atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
+        } else if (expo != 0u) {
+          // value = mantissa * 2^(pos - 149)
+          const unsigned long long mant = (unsigned long long)((bits & 0x7FFFFFu) | 0x800000u);
+          const uint32_t pos = expo - 1u, limb = pos / 40u, off = pos % 40u;
+          unsigned long long* acc = p.limbs + ((int64_t)slab * NCOLS + row) * kLimbStride + limb;
+          const unsigned long long lo = (mant << off) & ((1ull << 40) - 1ull), hi = mant >> (40u - off);
+          atomicAdd(acc, lo);
+          if (hi != 0ull) atomicAdd(acc + 1, hi);
+        }
+      }
+    }
+    // the warp's additions before the count, the count before the reads below: one release-acquire operation orders both
+    __syncwarp();
+    unsigned before = 0;
+    if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(p.counters + slab) : "memory");
+    before = __shfl_sync(0xffffffffu, before, 0);
+    __syncwarp();
+    if (before + 1u != expected) continue;
+    // this CTA completed the slab: the exact totals become log-sum-exps
+    const float ref = __ldg(p.refs + slab);
+    unsigned long long w[RPL][kLimbs];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const unsigned long long* acc = p.limbs + ((int64_t)slab * NCOLS + min(lane + 32 * r, NCOLS - 1)) * kLimbStride;
+#pragma unroll
+      for (int i = 0; i < kLimbs; ++i) w[r][i] = __ldcg(acc + i);
+    }
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const int row = lane + 32 * r;
+      if (row >= NCOLS) continue;
+      float lse2 = INFINITY;                                       // rows that do not exist: exp2(x - lse2) = 0
+      if (row % G < a.group && row / G < a.n_lookahead) {
+        double total = 0.0;                                        // sum of limb_i * 2^(40 i - 149), exact to 2^-53
+#pragma unroll
+        for (int i = kLimbs - 1; i >= 0; --i) total += __longlong_as_double((long long)(1023 + 40 * i - 149) << 52) * (double)w[r][i];
+        // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision
+        const long long tb = __double_as_longlong(total);
+        const int expo = (int)((tb >> 52) & 0x7ff) - 1023;
+        const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+        lse2 = ref + ((float)expo + log2f(mant));
+        if (!(total > 0.0) || expo == 1024) lse2 = INFINITY;       // an empty or overflowed row sum
+        const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
+        if (p.extra_lse != nullptr) {
+          // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
+          const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
+          const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
+          lse2 = hi + log2f(1.f + exp2f(lo - hi));
+        }
+        if (!(lse2 > -INFINITY && lse2 < INFINITY) && a.dev_status != nullptr)
+          atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
+        if (p.lse_out != nullptr) p.lse_out[out_idx] = lse2 * kLn2;
+      }
+      const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
+      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + row), "l"(word) : "memory");
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- log-sum-exps for visit 2
+// Fetches each slab's log-sum-exps in turn, kAhead slabs' words in flight, and hands them to the max warps through shared
+// memory (negated: what visit 2 adds).
+template <class T, int NCOLS, int G, bool FP8>
+__device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedShare& sh, int lane, float* off, float* off_c,
+                                                const FusedBars& bars, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  constexpr int RPL = NCOLS == 64 ? 2 : 1;
+  constexpr int kAhead = 4;
+  unsigned long long w[kAhead][RPL];
+  auto load = [&](unsigned long long (&dst)[RPL], int n) {
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const int row = min(lane + 32 * r, NCOLS - 1);
+      if (a.mode == 2) {
+        const bool real = row % G < a.group && row / G < a.n_lookahead;
+        const float v = real ? __ldg(p.lse_in + ((int64_t)sh.slab(n) * a.group + row % G) * a.n_lookahead + row / G) * kLog2e : INFINITY;
+        dst[r] = (1ull << 32) | __float_as_uint(v);
+      } else {
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(dst[r]) : "l"(p.lse + (int64_t)sh.slab(n) * NCOLS + row) : "memory");
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < kAhead; ++i)
+    if (i < sh.n_slabs) load(w[i], i);
+  for (int n0 = 0; n0 < sh.n_slabs; n0 += kAhead) {
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int n = n0 + i;
+      if (n < sh.n_slabs) {
+        unsigned long long t0 = 0;
+        for (uint32_t it = 1;; ++it) {
+          bool there = true;
+#pragma unroll
+          for (int r = 0; r < RPL; ++r) there = there && (w[i][r] >> 32) != 0ull;
+          if (__all_sync(0xffffffffu, there)) break;
+          if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
+          load(w[i], n);
+        }
+        float v[RPL];
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) v[r] = -__uint_as_float((unsigned)w[i][r]);
+        if (n + kAhead < sh.n_slabs) load(w[i], n + kAhead);
+        const int slot = n % kOffSlots;
+        if (n >= kOffSlots)
+          if (!mbar_wait_warp(bars.off_free(slot), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
+#pragma unroll
+        for (int r = 0; r < RPL; ++r)
+          if (lane + 32 * r < NCOLS) off[slot * 64 + lane + 32 * r] = v[r];
+        if constexpr (FP8) {
+          if (lane == 0) off_c[slot] = __ldg(p.slab_c + sh.slab(n));
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.off_ready(slot));
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- visit 2: maxima
+// Folds one load's accumulators into the running maxima over (layer, head) of the base-2 logits less their rows'
+// log-sum-exps (slots past n_lookahead hold padding and are never read).
+template <class T, int G>
+__device__ __forceinline__ void fold_maxima(const uint32_t (&r)[T::CW], uint32_t (&am)[T::NIW], const ulonglong2* off2, uint64_t cc) {
+  float z[T::CW];
+#pragma unroll
+  for (int j = 0; j < T::CW / 4; ++j) {
+    const ulonglong2 o = off2[j];
+    unpack2(fma2(pack2(r[4 * j], r[4 * j + 1]), cc, o.x), z[4 * j], z[4 * j + 1]);
+    unpack2(fma2(pack2(r[4 * j + 2], r[4 * j + 3]), cc, o.y), z[4 * j + 2], z[4 * j + 3]);
+  }
+#pragma unroll
+  for (int i = 0; i < T::NIW; ++i) {
+    float m = __uint_as_float(am[i]);
+    if constexpr (G == 1) {
+      m = fmaxf(m, z[i]);
+    } else {
+#pragma unroll
+      for (int g = 0; g < G; g += 2) m = max3(m, z[i * G + g], z[i * G + g + 1]);
+    }
+    am[i] = __float_as_uint(m);
+  }
+}
+
+// -inf in the running maxima of a set's tiles.
+template <class T>
+__device__ __forceinline__ void clear_maxima(uint32_t amax_addr, int set, int n_tiles) {
+  uint32_t ninf[T::NIW];
+#pragma unroll
+  for (int j = 0; j < T::NIW; ++j) ninf[j] = 0xff800000u;
+  for (int lt = set; lt < n_tiles; lt += 2)
+#pragma unroll
+    for (int ch = 0; ch < T::NCH; ++ch) tmem_store<T::NIW>(amax_addr + (uint32_t)(lt * T::NI + ch * T::NIW), ninf);
+}
+
+template <class T, int NCOLS, int G, bool FP8>
+__device__ __forceinline__ bool fused_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, uint32_t amax_tmem,
+                                          const float* off, const float* off_c, const FusedBars& bars, const Abort& ab) {
+  constexpr int CW = T::CW, NCH = T::NCH, NIW = T::NIW;
+  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
+  const int tps = a.max_tiles_per_stage, stages = a.t_stages[1];
+  const uint32_t lane_bits = (uint32_t)(quad * 32) << 16;
+  const uint32_t lane_addr = tmem + lane_bits + (uint32_t)(set * stages * tps * NCOLS);
+  const uint32_t amax_addr = amax_tmem + lane_bits;
+  Ring tr(stages);
+  clear_maxima<T>(amax_addr, set, sh.n_tiles);
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    const int slot = n % kOffSlots;
+    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return false;
+    const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
+    const float c = FP8 ? off_c[slot] : a.c;
+    const uint64_t cc = pack2(c, c);
+    for (int lt = set; lt < sh.n_tiles;) {
+      if (!mbar_wait_warp(bars.t_full(1, set, tr.stage), tr.phase, ab)) return false;
+      tc_fence_after();
+      tmem_store_wait();                                           // the maxima read below may be this warp's last stores
+      const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * tps * NCOLS);
+      const uint32_t empty = bars.t_empty(1, set, tr.stage);
+      tr.advance();
+      uint32_t r[CW], am[NIW];
+      if constexpr (NCOLS == 16) {
+        uint32_t r1[CW], am1[NIW];
+        const bool two = tps > 1 && lt + 2 < sh.n_tiles;
+        tmem_issue<CW>(taddr, r);
+        tmem_issue<NIW>(amax_addr + (uint32_t)(lt * T::NI), am);
+        if (two) {
+          tmem_issue<CW>(taddr + NCOLS, r1);
+          tmem_issue<NIW>(amax_addr + (uint32_t)((lt + 2) * T::NI), am1);
+        }
+        tmem_load_wait();
+        tmem_ready<CW>(r);
+        tmem_ready<NIW>(am);
+        tmem_ready<CW>(r1);
+        tmem_ready<NIW>(am1);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty);
+        fold_maxima<T, G>(r, am, off2, cc);
+        tmem_store<NIW>(amax_addr + (uint32_t)(lt * T::NI), am);
+        if (two) {
+          fold_maxima<T, G>(r1, am1, off2, cc);
+          tmem_store<NIW>(amax_addr + (uint32_t)((lt + 2) * T::NI), am1);
+        }
+        lt += 2 * tps;
+      } else {
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) {
+          const uint32_t am_addr = amax_addr + (uint32_t)(lt * T::NI + ch * NIW);
+          tmem_issue<CW>(taddr + (uint32_t)(ch * CW), r);
+          tmem_issue<NIW>(am_addr, am);
+          tmem_load_wait();
+          tmem_ready<CW>(r);
+          tmem_ready<NIW>(am);
+          if (ch + 1 == NCH) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty);
+          }
+          fold_maxima<T, G>(r, am, off2 + ch * (CW / 4), cc);
+          tmem_store<NIW>(am_addr, am);
+        }
+        lt += 2;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.off_free(slot));
+  }
+  tmem_store_wait();
+  return true;
+}
+
+// ---------------------------------------------------------------------------------------------- resident form
+// Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.
+struct ResidentRing {
+  int stage = 0, n;
+  uint32_t phase = 0;
+  __device__ explicit ResidentRing(int n_) : n(n_) {}
+  __device__ void advance(int by) {                                // by <= n
+    stage += by;
+    if (stage >= n) {
+      stage -= n;
+      phase ^= 1u;
+    }
+  }
+};
+
+template <class T, int NCOLS, bool FP8>
+__device__ __forceinline__ void resident_multiply(const FusedArgs& a, const FusedShare& sh, const unsigned char* k_tiles,
+                                                  const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
+  constexpr uint32_t idesc = instr_desc(kTileKeys, NCOLS, FP8);
+  const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
+  const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
+  Ring kr(a.k_stages[0]), qr(T::QS), tr(a.t_stages[0]);
+  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+  for (int n = 0; n < n_slabs; ++n) {
+    if (!mbar_wait_warp(bars.q_full(0, qr.stage), qr.phase, ab)) return;
+    const uint64_t qd0 = q_desc0 + (uint64_t)((qr.stage * T::kQBytes) >> 4);
+    for (int lt = 0; lt < n_tiles; ++lt) {
+      if (!mbar_wait2_warp(bars.k_full(0, kr.stage), kr.phase, bars.t_empty(0, 0, tr.stage), tr.phase ^ 1u, ab)) return;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem + (uint32_t)(tr.stage * NCOLS);
+      const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
+      if (elect_one()) {
+#pragma unroll
+        for (int part = 0; part < T::QPARTS; ++part)               // 8-bit keys: the two query terms accumulate into the same columns
+#pragma unroll
+          for (int h = 0; h < T::KSUB; ++h)
+#pragma unroll
+            for (int ks = 0; ks < T::KSTEPS; ++ks)
+              tc_mma<FP8, false>(d_tmem, kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks,
+                                 qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks, idesc, (uint32_t)((part | h | ks) != 0));
+        tc_commit(bars.k_empty(0, kr.stage));
+        tc_commit(bars.t_full(0, 0, tr.stage));
+      }
+      __syncwarp();
+      kr.advance();
+      tr.advance();
+    }
+    if (elect_one()) tc_commit(bars.q_empty(0, qr.stage));
+    __syncwarp();
+    qr.advance();
+  }
+  if (elect_one()) tc_commit(bars.mma_done(0));
+  __syncwarp();
+  mbar_wait_warp(bars.mma_done(0), 0u, ab);
+}
+
+// The sums.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it shares out over the
+// warp at the end of a slab.
+template <class T, int NCOLS, bool FP8>
+__device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
+                                             const FusedBars& bars, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
+  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+  const float* const refs = p.refs;
+  const float* const slab_c = p.slab_c;
+  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
+  const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
+  const int tail_lanes = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32;   // real keys of this quadrant in the last tile
+  const bool frees = a.mode == 1;                                  // no visit 2: nobody else frees the stages
+  ResidentRing tr(a.t_stages[0]);
+  tr.advance(set);
+  int lt = set;                                                    // this set's next tile, counted from the slab's first
+  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
+  for (int n = 0; n < n_slabs; ++n) {
+    const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
+    if (n + 1 < n_slabs) {
+      next_ref = __ldg(refs + sh.slab(n + 1));
+      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
+    }
+    uint64_t acc[NCOLS / 2];
+#pragma unroll
+    for (int j = 0; j < NCOLS / 2; ++j) acc[j] = 0ull;
+    const bool any = lt < n_tiles;
+    for (; lt < n_tiles; lt += 2) {
+      if (!mbar_wait_warp(bars.t_full(0, 0, tr.stage), tr.phase, ab)) return;
+      tc_fence_after();
+      uint32_t r[NCOLS];
+      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
+      tmem_load_wait();
+      tmem_ready<NCOLS>(r);
+      if (frees) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.t_empty(0, 0, tr.stage));
+      }
+      tr.advance(2);
+      if (sh.tile(lt) < full_tiles || lane < tail_lanes) {
+#pragma unroll
+        for (int j = 0; j < NCOLS / 2; ++j) {
+          float x, y;
+          unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
+          acc[j] = add2(acc[j], pack2(fast_exp2(x), fast_exp2(y)));
+        }
+      }
+    }
+    lt -= n_tiles;
+    // Sum over the warp's 32 keys: transposing butterfly steps, each of which halves the columns a lane holds, then (16
+    // columns) one plain step.  The publishers add up quadrants and sets.
+    float s[NCOLS];
+    s[0] = 0.f;
+    if (any) {
+#pragma unroll
+      for (int j = 0; j < NCOLS / 2; ++j) unpack2(acc[j], s[2 * j], s[2 * j + 1]);
+      int width = NCOLS;
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        if (width > 1) {
+          width >>= 1;
+          const bool upper = (lane & off) != 0;
+#pragma unroll
+          for (int j = 0; j < NCOLS / 2; ++j) {
+            if (j < width) {
+              const float send = upper ? s[j] : s[j + width];
+              const float keep = upper ? s[j + width] : s[j];
+              s[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+          }
+        } else {
+          s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
+        }
+      }
+    }
+    const int slot = n % kSumSlots;
+    if (n >= kSumSlots)
+      if (!mbar_wait_warp(bars.sums_free(slot), (uint32_t)(n / kSumSlots - 1) & 1u, ab)) return;
+    float* out = sums + ((slot * 2 + set) * 4 + quad) * 32;
+    if constexpr (NCOLS == 32) {
+      out[lane] = s[0];
+    } else {
+      if ((lane & 1) == 0) out[lane >> 1] = s[0];
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.sums_ready(slot));
+  }
+}
+
+// The maxima, once the slab's log-sum-exps are there.  A tile's maxima always belong to the same warps (lt mod 2 == set).
+template <class T, int NCOLS, int G, bool FP8>
+__device__ __forceinline__ bool resident_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem,
+                                             uint32_t amax_tmem, const float* off, const float* off_c, const FusedBars& bars,
+                                             const Abort& ab) {
+  constexpr int NI = T::NI;
+  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
+  const int n_tiles = sh.n_tiles;
+  const uint32_t lane_bits = (uint32_t)(quad * 32) << 16;
+  const uint32_t lane_addr = tmem + lane_bits, amax_addr = amax_tmem + lane_bits;
+  clear_maxima<T>(amax_addr, set, n_tiles);
+  ResidentRing first(a.t_stages[0]);                               // the stage of the slab's first tile
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    const int slot = n % kOffSlots;
+    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return false;
+    const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
+    const float c = FP8 ? off_c[slot] : a.c;
+    const uint64_t cc = pack2(c, c);
+    ResidentRing tr = first;
+    tr.advance(set);
+    for (int lt = set; lt < n_tiles; lt += 2) {
+      // complete long since (the log-sum-exps contain it), except where visit 2 runs alone
+      if (!mbar_wait_warp(bars.t_full(0, 0, tr.stage), tr.phase, ab)) return false;
+      tc_fence_after();
+      tmem_store_wait();                                           // the maxima read below may be this warp's last stores
+      uint32_t r[NCOLS], am[NI];
+      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
+      tmem_issue<NI>(amax_addr + (uint32_t)(lt * NI), am);
+      tmem_load_wait();
+      tmem_ready<NCOLS>(r);
+      tmem_ready<NI>(am);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bars.t_empty(0, 0, tr.stage));
+      tr.advance(2);
+      fold_maxima<T, G>(r, am, off2, cc);
+      tmem_store<NI>(amax_addr + (uint32_t)(lt * NI), am);
+    }
+    first.advance(n_tiles);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.off_free(slot));
+  }
+  tmem_store_wait();
+  return true;
+}
+
+// ---------------------------------------------------------------------------------------------- importance
+// Mean over the lookahead of exp2(running max).  One group of CTAs (parts = 1): straight from tensor memory.  Several: the
+// groups' maxima meet in global memory, and whichever warp brings the last contribution for 32 keys reads the result.
+template <class T, int NCOLS, int G>
+__device__ __forceinline__ void fused_finish(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t amax_tmem) {
+  constexpr int NI = T::NI, FC = NI < 16 ? NI : 16;
+  const FusedPrompt& p = *sh.p;
+  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
+  const uint32_t lane_addr = amax_tmem + ((uint32_t)(quad * 32) << 16);
+  const float inv_m = 1.f / (float)a.n_lookahead;
+  const bool meet = p.parts > 1;
+  const int64_t n_pad = (int64_t)p.n_tiles * kTileKeys;
+  for (int lt = set; lt < sh.n_tiles; lt += 2) {
+    const int tile = sh.tile(lt);
+    const int64_t key = (int64_t)tile * kTileKeys + quad * 32 + lane;
+    float sum = 0.f;
+#pragma unroll
+    for (int q = 0; q < NI / FC; ++q) {
+      uint32_t v[FC];
+      tmem_issue<FC>(lane_addr + (uint32_t)(lt * NI + q * FC), v);
+      tmem_load_wait();
+      tmem_ready<FC>(v);
+#pragma unroll
+      for (int j = 0; j < FC; ++j) {
+        const int i = q * FC + j;
+        if (i < a.n_lookahead) {
+          if (meet) atomicMax(p.amax + (int64_t)i * n_pad + key, order_bits(__uint_as_float(v[j])));
+          else sum += fast_exp2(__uint_as_float(v[j]));
+        }
+      }
+    }
+    if (meet) {
+      __threadfence();
+      __syncwarp();
+      unsigned before = 0;
+      if (lane == 0) before = atomicAdd(p.finished + tile * 4 + quad, 1u);
+      if (__shfl_sync(0xffffffffu, before, 0) + 1u != (unsigned)p.parts) continue;
+      __threadfence();
+#pragma unroll 8
+      for (int i = 0; i < a.n_lookahead; ++i) sum += fast_exp2(from_order_bits(__ldcg(p.amax + (int64_t)i * n_pad + key)));
+    }
+    if (key < p.n_tokens) p.importance[key] = sum * inv_m;
+  }
+}
+
+// ---------------------------------------------------------------------------------------------- kernel
+template <int D, int NCOLS, int G, bool FP8, bool ONCE>
+__global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __grid_constant__ FusedArgs a) {
+  using T = FusedTraits<D, NCOLS, G, FP8, ONCE>;
+  static_assert(T::CW % G == 0, "a load's accumulators must hold whole GQA groups");
+  extern __shared__ unsigned char smem_raw[];
+  // 1024-byte alignment by offsetting the shared array itself, so that the compiler still knows these are shared-memory
+  // addresses (a round trip through an integer would turn every access into a generic one)
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const FusedSmem lay = fused_smem(D, FP8, NCOLS, ONCE, a.table_tiles, a.k_stages);
+  float* sums = reinterpret_cast<float*>(smem + lay.sums_off);
+  float* off = reinterpret_cast<float*>(smem + lay.off_off);
+  float* off_c = reinterpret_cast<float*>(smem + lay.offc_off);
+  volatile int* misc = reinterpret_cast<volatile int*>(smem + lay.misc_off);  // [0] abort, [1] tensor-memory base, [2] tiles visit 2 has issued
+  const FusedBars bars{smem_u32(smem + lay.bar_off)};
+  const Abort ab{misc, a.dev_status};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  // ------------------------------------------------------------------ this CTA's share
+  FusedShare sh;
+  {
+    int pi = 0;
+    while (pi + 1 < a.n_prompts && (int)blockIdx.x >= a.prompt[pi + 1].cta0) ++pi;
+    const FusedPrompt& p = a.prompt[pi];
+    const int local = (int)blockIdx.x - p.cta0;
+    sh.p = &p;
+    sh.parts = p.parts;
+    sh.part = local % p.parts;
+    sh.first = local / p.parts;
+    sh.step = p.per_part;
+    const int slabs = a.n_layers * a.n_kv_heads;
+    sh.n_slabs = (slabs - sh.part + p.parts - 1) / p.parts;
+    sh.n_tiles = sh.first < min(p.per_part, p.n_tiles) ? (p.n_tiles - sh.first + sh.step - 1) / sh.step : 0;
+  }
+  if (sh.n_tiles == 0) return;
+
+  // ------------------------------------------------------------------ set-up
+  if (threadIdx.x == 0) {
+    misc[0] = 0;
+    misc[1] = 0;
+    misc[2] = 0;
+    for (int v = 0; v < (ONCE ? 1 : 2); ++v) {
+      for (int s = 0; s < a.k_stages[v]; ++s) {
+        mbar_init(bars.k_full(v, s), 1);
+        mbar_init(bars.k_empty(v, s), 1);
+      }
+      for (int s = 0; s < T::QS; ++s) {
+        mbar_init(bars.q_full(v, s), 1);
+        mbar_init(bars.q_empty(v, s), 1);
+      }
+      for (int set = 0; set < (ONCE ? 1 : 2); ++set)
+        for (int s = 0; s < a.t_stages[v]; ++s) {
+          mbar_init(bars.t_full(v, set, s), 1);
+          mbar_init(bars.t_empty(v, set, s), kVisitWarps / 2);
+        }
+      mbar_init(bars.mma_done(v), 1);
+    }
+    for (int x = 0; x < kOffSlots; ++x) {
+      mbar_init(bars.off_ready(x), 1);
+      mbar_init(bars.off_free(x), kVisitWarps);
+    }
+    for (int x = 0; x < kSumSlots; ++x) {
+      mbar_init(bars.sums_ready(x), kVisitWarps);
+      mbar_init(bars.sums_free(x), 1);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // paged key cache: a tile never straddles a block (blocks are multiples of 128 tokens): one lookup per tile for the whole kernel
+  int2* const tile_at = reinterpret_cast<int2*>(smem + lay.tile_off);
+  if (sh.p->block_tokens > 0) {
+    grid_wait();
+    for (int lt = threadIdx.x; lt < sh.n_tiles; lt += kFusedThreads) {
+      const int key0 = sh.tile(lt) * kTileKeys;
+      tile_at[lt] = make_int2(key0 % sh.p->block_tokens, __ldg(sh.p->block_table + key0 / sh.p->block_tokens));
+    }
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)&misc[1])),
+                 "r"(kTmemColsAll)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = (uint32_t)misc[1];
+  // tensor memory: the accumulator stages, then the running maxima, [local tile][NI] columns (lane = key)
+  const uint32_t tmem_v2 = tmem_base + (uint32_t)(2 * a.t_stages[0] * T::SR);
+  const uint32_t amax_tmem = ONCE ? tmem_base + (uint32_t)(a.t_stages[0] * NCOLS)
+                                  : tmem_v2 + (uint32_t)(2 * a.t_stages[1] * a.max_tiles_per_stage * NCOLS);
+  grid_wait();                                                     // what the preparing kernel wrote is visible from here on
+
+  // ------------------------------------------------------------------ roles
+  const bool visit1 = a.mode != 2, visit2 = a.mode != 1;
+  if (warp < 4) {
+    const int v = warp & 1;
+    if (ONCE ? v == 0 : (v == 0 ? visit1 : visit2)) {
+      unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
+      if (warp < 2) {
+        if (lane == 0) fused_produce<T, ONCE>(a, sh, v, k_tiles, q_tiles, tile_at, bars, misc + 2, ab);
+      } else if constexpr (ONCE) {
+        resident_multiply<T, NCOLS, FP8>(a, sh, k_tiles, q_tiles, tmem_base, bars, ab);
+      } else if (v == 0) {
+        fused_multiply<T, NCOLS, FP8, 0>(a, sh, k_tiles, q_tiles, tmem_base, bars, ab);
+      } else {
+        fused_multiply<T, NCOLS, FP8, 1>(a, sh, k_tiles, q_tiles, tmem_v2, bars, ab);
+      }
+    }
+  } else if (warp < kSumWarp0) {
+    if (warp < kPublisherWarp0) {
+      if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
+    } else {
+      if (visit1) fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
+    }
+  } else if (warp < kMaxWarp0) {
+    if (visit1) {
+      if constexpr (ONCE) resident_sum<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+      else fused_sum<T, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+    }
+  } else if (visit2) {
+    bool ok;
+    if constexpr (ONCE) ok = resident_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
+    else ok = fused_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_v2, amax_tmem, off, off_c, bars, ab);
+    if (ok && misc[0] == 0) fused_finish<T, NCOLS, G>(a, sh, warp, lane, amax_tmem);
+  }
+
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  if (misc[0] != 0) {
+    // a wait ran out somewhere: give copies and MMAs still in flight time to land before TMEM goes away
+    const unsigned long long t0 = global_timer();
+    while (global_timer() - t0 < 2000000ull) __nanosleep(1000);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemColsAll) : "memory");
+  }
+}
+
+// Launches the instantiation for this geometry (one translation unit per head dimension and key format).
+struct FusedLaunch {
+  int ncols, padded_group, n_cta, smem_bytes;
+  bool once;
+};
+int32_t fused_launch_d64(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream);
+int32_t fused_launch_d128(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream);
+int32_t fused_launch_d64_fp8(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream);
+int32_t fused_launch_d128_fp8(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream);
+
+// The kernel's cross-CTA hand-over needs every CTA of the grid on an SM at the same time.  The launch therefore asks the
+// runtime for exactly that guarantee (a cooperative launch; no grid-wide barrier is used): a grid that cannot be
+// co-resident -- fewer SMs available than the device reports, e.g. under MPS with a limited SM share -- is refused here
+// instead of spinning into the bounded waits.  SMs that are merely busy with other kernels delay the launch; they do not
+// break it.
+template <int D, int NCOLS, int G, bool FP8, bool ONCE>
+int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
+  auto kern = score_fused_kernel<D, NCOLS, G, FP8, ONCE>;
+  SPF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem_bytes));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)l.n_cta);
+  cfg.blockDim = dim3(kFusedThreads);
+  cfg.dynamicSmemBytes = (size_t)l.smem_bytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, args);
+  if (err == cudaErrorCooperativeLaunchTooLarge) {
+    (void)cudaGetLastError();
+    return fail(SPF_ERR_UNSUPPORTED, "spf_score: the %d CTAs of the fused kernel cannot all be resident on this device; use the general path",
+                l.n_cta);
+  }
+  SPF_CUDA_CHECK(err);
+  return SPF_OK;
+}
+
+template <int D, int NCOLS, bool FP8, bool ONCE>
+int32_t fused_launch_group(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
+  switch (l.padded_group) {
+    case 1: return fused_launch_one<D, NCOLS, 1, FP8, ONCE>(args, l, stream);
+    case 2: return fused_launch_one<D, NCOLS, 2, FP8, ONCE>(args, l, stream);
+    case 4: return fused_launch_one<D, NCOLS, 4, FP8, ONCE>(args, l, stream);
+    default: return fused_launch_one<D, NCOLS, 8, FP8, ONCE>(args, l, stream);
+  }
+}
+
+template <int D, bool FP8>
+int32_t fused_launch(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
+  switch (l.ncols) {
+    case 16: return l.once ? fused_launch_group<D, 16, FP8, true>(args, l, stream) : fused_launch_group<D, 16, FP8, false>(args, l, stream);
+    case 32: return l.once ? fused_launch_group<D, 32, FP8, true>(args, l, stream) : fused_launch_group<D, 32, FP8, false>(args, l, stream);
+    default: return fused_launch_group<D, 64, FP8, false>(args, l, stream);
+  }
+}
+
+}  // namespace spf

@@ -16,7 +16,7 @@ struct ScoreProblem {
   float* importance;
   float* lse_out;  // may be null
   // 8-bit key cache (k_scale != null): the layer pointers hold E4M3 bytes, strides count bytes, key (l, hk, s, j) has the
-  // value k_scale[l * Hkv + hk] * E4M3(byte); only the general path reads this format
+  // value k_scale[l * Hkv + hk] * E4M3(byte)
   const float* k_scale;
   const float* extra_lse;  // may be null: fp32 [L][Hq][m], natural log of what the row's denominator holds besides the prompt keys
   // paged key cache (block_tokens > 0): k.p[l] is layer l's block pool, bf16 [n_pool_blocks][Hkv][block_tokens][d];
@@ -36,16 +36,18 @@ int32_t score_mma_launch(const ScoreProblem& p, void* workspace, int sm_count, c
 int32_t score_mma_launch_phase(const ScoreProblem& p, void* workspace, int sm_count, int phase, const float* lse_in,
                                cudaStream_t stream);
 
-// Fused single-kernel path (tcgen05 + TMA, key cache read once from HBM).  Covers G in {1,2,4,8},
-// G*m <= 64, up to kFusedMaxLayers layers and prompt lengths whose per-CTA state fits shared memory.
+// Fused single-kernel path (tcgen05 + TMA, key cache read once from HBM).  Covers G <= 8 with G, padded to a power of two,
+// times m <= 64, up to kFusedMaxLayers layers and prompt lengths whose running maxima fit tensor memory.
 constexpr int kFusedMaxLayers = 64;
 constexpr int kFusedMaxCtas = 256;  // upper bound on the persistent grid
+constexpr int kFusedMaxBatch = 16;  // prompts per launch
 bool score_fused_supported(const ScoreProblem& p, int sm_count);
 size_t score_fused_workspace_bytes(const ScoreProblem& p);
 // mode 0: the whole computation; 1: first visit only: row log-sum-exps over the given keys to p.lse_out (p.importance unused);
 // 2: second visit only, with the rows' log-sum-exps `lse_in` (device, natural log, [L][Hq][m]) supplied by the caller
-int32_t score_fused_launch(const ScoreProblem& p, void* workspace, int sm_count, int32_t* dev_status, cudaStream_t stream, int mode = 0,
-                           const float* lse_in = nullptr);
+// The prompts share one geometry; each has its own score_fused_workspace_bytes of the workspace, one after the other.
+int32_t score_fused_launch(const ScoreProblem* p, int n_prompts, void* workspace, int sm_count, int32_t* dev_status, cudaStream_t stream,
+                           int mode = 0, const float* lse_in = nullptr);
 
 // spf_score with the kernel path given for this call only (0 automatic, 1 general, 2 fused) instead of the process-wide setting.
 int32_t score_on_path(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts, void* workspace, size_t workspace_bytes,
