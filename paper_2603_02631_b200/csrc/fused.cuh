@@ -32,8 +32,7 @@
 // accumulators.
 //
 // Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each).  4: fetches log-sum-exps
-// for visit 2.  5..7: publishers (add a slab's row sums of this CTA to the slab's totals; the CTA that completes a slab
-// converts the totals).  8..15: "sum" warps.  16..23: "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM
+// for visit 2.  5..7: publishers (store this CTA's row sums of a slab; add up all CTAs' sums of the rows this CTA owns).  8..15: "sum" warps.  16..23: "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM
 // lane quadrant and the next bit the `set`: the two sets take turns at the tiles, so that one set's tensor-memory loads and
 // waits run while the other set computes.  (Splitting every tile's columns between the sets kept all eight warps in step,
 // all waiting or all computing.)
@@ -46,13 +45,15 @@
 // that level) base-2 units (157 at the very least, about 109 nats) above the slab's smallest sample logit.  That is
 // detected (the sum is inf) and reported as SPF_ERR_RANGE; the caller can then use the general path.
 //
-// Cross-CTA step.  All CTAs use the same reference for a slab, so their partial sums can simply be added.  To make the
-// total independent of the order in which CTAs arrive, the fp32 partial sums are added EXACTLY: each is split over two
-// 40-bit limbs of a 280-bit fixed-point accumulator per row (64-bit integer atomics, no carries needed), which covers every
-// finite fp32 value.  The CTA whose arrival completes a slab converts the accumulators to log-sum-exps and stores each as
-// one 64-bit word {value, 1}; the other CTAs poll those words, so no CTA repeats the conversion and no fence sits between
-// value and flag.  Results are bit-identical from run to run.  Visit 1 waits for other CTAs only through its lead over
-// visit 2, which covers at least one whole slab, so every slab's sums complete and the words always arrive.
+// Cross-CTA step.  All CTAs use the same reference for a slab, so their partial sums can simply be added.  Each CTA stores
+// its sums as plain words, [slab][four rows][CTA of the group], zero meaning "not there yet".  Every four rows of a slab
+// have an owner among the CTAs, which reads everybody's words, adds them up in double in a fixed order and stores the
+// log-sum-exps as 64-bit words {value, 1}; every CTA polls those.  No atomics, no fences, no counters: two stores and two
+// polls, about 3 us from a slab's last sum to its log-sum-exps everywhere, and every run arrives at the same bits.  (Exact
+// atomic sums with an arrival counter took 5.4 us; every CTA reading everybody's sums 2 us, but 7 us of a slab's time.)
+// How far visit 2 trails visit 1 is what has to fit in L2, so this latency is what the split is built around.  Visit 1
+// waits for other CTAs only through its lead over visit 2, which covers at least one whole slab, so every slab's sums
+// complete and the words always arrive.
 //
 // Every wait on a barrier, word or flag in this file is bounded: on expiry the kernel records SPF_ERR_TIMEOUT, drains and
 // returns normally.  The one wait that has no limit is the hardware's own: tcgen05.alloc blocks while another resident CTA
@@ -67,9 +68,7 @@ namespace spf {
 constexpr int kFusedThreads = 768;
 constexpr int kVisitWarps = 8;         // epilogue warps per visit
 constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
-constexpr int kPublisherWarp0 = 5, kPublisherWarps = 3;
-constexpr int kLimbs = 7;              // 40-bit limbs of the exact row-sum accumulators (covers every finite fp32)
-constexpr int kLimbStride = 8;         // 64-bit words per row in the accumulator array
+constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
 constexpr int kMaxQStages = 4;         // query tiles in flight per visit (two-pass: 2)
 constexpr int kMaxKeyStages = 16;      // key tiles in flight per visit
 constexpr int kMaxTmemStages = 4;      // two-pass: accumulator stages per visit and set
@@ -89,8 +88,7 @@ __host__ __device__ constexpr int sum_rows(int ncols) { return ncols <= 32 ? 32 
 struct FusedPrompt {
   const CUtensorMap* k_maps;   // [n_layers] (element of a sub-row, key, sub-tile, kv-head[, pool block])
   const unsigned char* q_tiles;   // [slab] query operands as the tensor cores read them (swizzled, padding rows zero)
-  unsigned long long* limbs;   // [slab][NCOLS][kLimbStride] exact fixed-point sums of exp2(c*q.k - ref) over all keys
-  unsigned* counters;          // [slab] CTAs whose share of the slab's row sums is in the accumulators
+  float4* row_sums;            // [slab][NCOLS / 4][per_part] each CTA's sums of exp2(c*q.k - ref) for four rows; 0: not there yet
   unsigned long long* lse;     // [slab][NCOLS] {log-sum-exp in base-2 units, 1} once known
   const float* refs;           // [slab] reference of visit 1
   const float* slab_c;         // [slab] 8-bit keys: accumulated dot product -> base-2 logit; null: FusedArgs::c for all
@@ -405,94 +403,122 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
 }
 
 // ---------------------------------------------------------------------------------------------- publishers
-// Publisher w takes slabs w, w + 3, ...: adds the CTA's row sums to the slab's exact totals, then counts the CTA in.  A fence
-// and an atomic's round trip per slab: three warps keep up with slabs of a single tile.
+// Rows 4q .. 4q + 3 of a slab: adds up all CTAs' words and stores the log-sum-exps.
+template <class T, int NCOLS, int G>
+__device__ __forceinline__ bool reduce_rows(const FusedArgs& a, const FusedShare& sh, int slab, int q, int n_ctas, int lane, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  constexpr int Q = NCOLS / 4;
+  constexpr int MAXW = (kFusedMaxCtas + 31) / 32;                  // words per lane
+  const int per_part = p.per_part;
+  const float4* in = p.row_sums + ((int64_t)slab * Q + q) * per_part;
+  float4 v[MAXW];
+#pragma unroll
+  for (int i = 0; i < MAXW; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  unsigned long long t0 = 0;
+  for (uint32_t it = 1;; ++it) {
+    // whatever is not there yet is asked for again (a word may also be caught half written)
+#pragma unroll
+    for (int i = 0; i < MAXW; ++i)
+      if (lane + 32 * i < n_ctas && (v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f))
+        asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w)
+                     : "l"(in + lane + 32 * i)
+                     : "memory");
+    bool there = true;
+#pragma unroll
+    for (int i = 0; i < MAXW; ++i)
+      there = there && (lane + 32 * i >= n_ctas || !(v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f));
+    if (__all_sync(0xffffffffu, there)) break;
+    if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return false;
+    __nanosleep(100);
+  }
+  double t[4] = {0.0, 0.0, 0.0, 0.0};                            // the CTAs' shares are fp32: exact to 2^-53
+#pragma unroll
+  for (int i = 0; i < MAXW; ++i) {
+    t[0] += (double)v[i].x;
+    t[1] += (double)v[i].y;
+    t[2] += (double)v[i].z;
+    t[3] += (double)v[i].w;
+  }
+  // two transposing steps leave one row per eight lanes: row 4q + (lane >> 3 & 3), with the bits exchanged
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const double send = (lane & 16) ? t[e] : t[e + 2], keep = (lane & 16) ? t[e + 2] : t[e];
+    t[e] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+  {
+    const double send = (lane & 8) ? t[0] : t[1], keep = (lane & 8) ? t[1] : t[0];
+    t[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int off = 4; off >= 1; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
+  if ((lane & 7) == 0) {
+    const int row = 4 * q + (lane >> 3);                         // lane 8: t[1], lane 16: t[2], lane 24: t[3]
+    float lse2 = INFINITY;                                       // rows that do not exist: exp2(x - lse2) = 0
+    if (row % G < a.group && row / G < a.n_lookahead) {
+      // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision; an empty (below every
+      // normal number) or overflowed row sum has none
+      const long long tb = __double_as_longlong(t[0]);
+      const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+      lse2 = __ldg(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
+      if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
+      const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
+      if (p.extra_lse != nullptr) {
+        // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
+        const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
+        const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
+        lse2 = hi + log2f(1.f + exp2f(lo - hi));
+      }
+      if (!(lse2 > -INFINITY && lse2 < INFINITY) && a.dev_status != nullptr) atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
+      if (p.lse_out != nullptr) p.lse_out[out_idx] = lse2 * kLn2;
+    }
+    const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + row), "l"(word) : "memory");
+  }
+  __syncwarp();
+  return true;
+}
+
+// Publisher w takes slabs w, w + 3, ...: stores this CTA's row sums (a row that does not exist gets its meaningless sum
+// stored too: everybody waits for every word) and then adds up everybody's sums of the rows that this CTA owns.  Item
+// n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab, belongs to CTA (item mod CTAs).  Only now: polling for words that
+// cannot be there yet slowed the key copies down.
 template <class T, int NCOLS, int G>
 __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums,
                                               const FusedBars& bars, const Abort& ab) {
-  const FusedPrompt& p = *sh.p;
-  constexpr int RPL = NCOLS == 64 ? 2 : 1;                         // rows per lane
-  const unsigned expected = (unsigned)min(p.per_part, p.n_tiles);
+  constexpr int Q = NCOLS / 4;                                     // lane q has rows 4q .. 4q + 3
+  float4* const row_sums = sh.p->row_sums;
+  const int per_part = sh.p->per_part, n_ctas = min(per_part, sh.p->n_tiles);
   for (int n = which; n < sh.n_slabs; n += kPublisherWarps) {
-    const int slot = n % kSumSlots, slab = sh.slab(n);
+    const int slot = n % kSumSlots;
     if (!mbar_wait_warp(bars.sums_ready(slot), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
-    const float* in = sums + slot * 256;
-    float tot[RPL];
-#pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-      float t = 0.f;
+    float t[4] = {0.f, 0.f, 0.f, 0.f};
+    if (lane < Q) {
+      // [set][quadrant][lane]: 64 rows: quadrants 0 and 2 have rows 0..31, 1 and 3 rows 32..63; else every quadrant all rows
+      const float* in = sums + slot * 256 + (NCOLS == 64 ? (lane >> 3) * 32 + (lane & 7) * 4 : lane * 4);
 #pragma unroll
       for (int set = 0; set < 2; ++set)
 #pragma unroll
-        for (int q = 0; q < 4 / RPL; ++q) t += in[(set * 4 + q * RPL + r) * 32 + lane];   // 64 rows: quadrants r and r + 2
-      tot[r] = t;
+        for (int q = 0; q < (NCOLS == 64 ? 2 : 4); ++q) {
+          const float4 v = *reinterpret_cast<const float4*>(in + set * 128 + q * (NCOLS == 64 ? 64 : 32));
+          t[0] += v.x;
+          t[1] += v.y;
+          t[2] += v.z;
+          t[3] += v.w;
+        }
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.sums_free(slot));
+    if (lane < Q) {
+      unsigned w[4];
 #pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-      const int row = lane + 32 * r;
-      if (row < NCOLS && row % G < a.group && row / G < a.n_lookahead) {
-        const uint32_t bits = __float_as_uint(tot[r]);
-        const uint32_t expo = bits >> 23;                          // sums are non-negative: no sign bit
-        if (expo >= 255u) {
-          if (a.dev_status != nullptr) atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
-        } else if (expo != 0u) {
-          // value = mantissa * 2^(pos - 149)
-          const unsigned long long mant = (unsigned long long)((bits & 0x7FFFFFu) | 0x800000u);
-          const uint32_t pos = expo - 1u, limb = pos / 40u, off = pos % 40u;
-          unsigned long long* acc = p.limbs + ((int64_t)slab * NCOLS + row) * kLimbStride + limb;
-          const unsigned long long lo = (mant << off) & ((1ull << 40) - 1ull), hi = mant >> (40u - off);
-          atomicAdd(acc, lo);
-          if (hi != 0ull) atomicAdd(acc + 1, hi);
-        }
-      }
+      for (int e = 0; e < 4; ++e) w[e] = max(__float_as_uint(t[e]), 1u);   // never "not there yet"; 2^-149 is nothing to a row's sum
+      asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};"
+                   ::"l"(row_sums + ((int64_t)sh.slab(n) * Q + lane) * per_part + sh.first), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                   : "memory");
     }
-    // the warp's additions before the count, the count before the reads below: one release-acquire operation orders both
-    __syncwarp();
-    unsigned before = 0;
-    if (lane == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(p.counters + slab) : "memory");
-    before = __shfl_sync(0xffffffffu, before, 0);
-    __syncwarp();
-    if (before + 1u != expected) continue;
-    // this CTA completed the slab: the exact totals become log-sum-exps
-    const float ref = __ldg(p.refs + slab);
-    unsigned long long w[RPL][kLimbs];
-#pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-      const unsigned long long* acc = p.limbs + ((int64_t)slab * NCOLS + min(lane + 32 * r, NCOLS - 1)) * kLimbStride;
-#pragma unroll
-      for (int i = 0; i < kLimbs; ++i) w[r][i] = __ldcg(acc + i);
-    }
-#pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-      const int row = lane + 32 * r;
-      if (row >= NCOLS) continue;
-      float lse2 = INFINITY;                                       // rows that do not exist: exp2(x - lse2) = 0
-      if (row % G < a.group && row / G < a.n_lookahead) {
-        double total = 0.0;                                        // sum of limb_i * 2^(40 i - 149), exact to 2^-53
-#pragma unroll
-        for (int i = kLimbs - 1; i >= 0; --i) total += __longlong_as_double((long long)(1023 + 40 * i - 149) << 52) * (double)w[r][i];
-        // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision
-        const long long tb = __double_as_longlong(total);
-        const int expo = (int)((tb >> 52) & 0x7ff) - 1023;
-        const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-        lse2 = ref + ((float)expo + log2f(mant));
-        if (!(total > 0.0) || expo == 1024) lse2 = INFINITY;       // an empty or overflowed row sum
-        const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
-        if (p.extra_lse != nullptr) {
-          // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
-          const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
-          const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
-          lse2 = hi + log2f(1.f + exp2f(lo - hi));
-        }
-        if (!(lse2 > -INFINITY && lse2 < INFINITY) && a.dev_status != nullptr)
-          atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
-        if (p.lse_out != nullptr) p.lse_out[out_idx] = lse2 * kLn2;
-      }
-      const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + row), "l"(word) : "memory");
-    }
+    for (int q = (int)(((unsigned)(n + 1) * (unsigned)n_ctas * Q + sh.first - n * Q) % (unsigned)n_ctas); q < Q; q += n_ctas)
+      if (!reduce_rows<T, NCOLS, G>(a, sh, sh.slab(n), q, n_ctas, lane, ab)) return;
   }
 }
 
@@ -1015,10 +1041,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
       }
     }
   } else if (warp < kSumWarp0) {
-    if (warp < kPublisherWarp0) {
+    if (warp == kFetchWarp) {
       if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
-    } else {
-      if (visit1) fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
+    } else if (visit1) {
+      fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
     }
   } else if (warp < kMaxWarp0) {
     if (visit1) {

@@ -388,7 +388,8 @@ bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, 
 // ---------------------------------------------------------------------------------------------- workspace
 struct FusedWorkspace {
   size_t k_maps, refs, slab_c, q_tiles;              // written by the preparing kernel
-  size_t limbs, counters, lse, finished, amax;       // cleared by it: [limbs, finished), and the rest where groups meet
+  size_t row_sums, lse;                              // cleared by it, the sums as far as used
+  size_t finished, amax;                             // cleared by it where groups meet
   size_t total;
 };
 
@@ -406,8 +407,7 @@ FusedWorkspace fused_workspace(const ScoreProblem& p) {
   w.refs = take(n_slabs * sizeof(float));
   w.slab_c = take(p.k_scale != nullptr ? n_slabs * sizeof(float) : 0);
   w.q_tiles = take(n_slabs * 2 * ncols * (size_t)p.head_dim);     // bf16, or two 8-bit terms
-  w.limbs = take(n_slabs * ncols * kLimbStride * sizeof(unsigned long long));
-  w.counters = take(n_slabs * sizeof(unsigned));
+  w.row_sums = take(n_slabs * std::min<size_t>(n_tiles, kFusedMaxCtas) * ncols * sizeof(float));
   w.lse = take(n_slabs * ncols * sizeof(unsigned long long));
   w.finished = take(n_tiles * 4 * sizeof(unsigned));
   w.amax = take((size_t)p.n_lookahead * n_tiles * kTileKeys * sizeof(unsigned));
@@ -487,12 +487,11 @@ int32_t launch_group(const ScoreProblem* p, int n, const Geometry& g, const Spli
     for (int layer = 0; layer < q.n_layers; ++layer) pp.k_layers[layer] = q.k.p[layer];
     pp.q = q.q;
     pp.k_maps_out = reinterpret_cast<CUtensorMap*>(base + w.k_maps);
-    // the regions are laid out for 64 rows; the accumulators of a narrower geometry use (and clear) the front of theirs
-    const size_t rows = (size_t)g.n_slabs * g.ncols;
-    pp.clear[0] = reinterpret_cast<uint4*>(base + w.limbs);
-    pp.clear_words[0] = (int64_t)(rows * kLimbStride * sizeof(unsigned long long) / 16);
-    pp.clear[1] = reinterpret_cast<uint4*>(base + w.counters);
-    pp.clear_words[1] = (int64_t)(((meet ? w.total : w.finished) - w.counters) / 16);
+    // the sums of a narrower geometry, or of fewer CTAs, use (and clear) the front of their region
+    pp.clear[0] = reinterpret_cast<uint4*>(base + w.row_sums);
+    pp.clear_words[0] = (int64_t)g.n_slabs * split[i].per_part * g.ncols * (int64_t)sizeof(float) / 16;
+    pp.clear[1] = reinterpret_cast<uint4*>(base + w.lse);
+    pp.clear_words[1] = (int64_t)(((meet ? w.total : w.finished) - w.lse) / 16);
     pp.refs = reinterpret_cast<float*>(base + w.refs);
     pp.slab_c = reinterpret_cast<float*>(base + w.slab_c);
     pp.q_tiles = reinterpret_cast<unsigned char*>(base + w.q_tiles);
@@ -507,8 +506,7 @@ int32_t launch_group(const ScoreProblem* p, int n, const Geometry& g, const Spli
 
     fp.k_maps = pp.k_maps_out;
     fp.q_tiles = pp.q_tiles;
-    fp.limbs = reinterpret_cast<unsigned long long*>(base + w.limbs);
-    fp.counters = reinterpret_cast<unsigned*>(base + w.counters);
+    fp.row_sums = reinterpret_cast<float4*>(base + w.row_sums);
     fp.lse = reinterpret_cast<unsigned long long*>(base + w.lse);
     fp.refs = pp.refs;
     fp.slab_c = g.fp8 ? pp.slab_c : nullptr;
