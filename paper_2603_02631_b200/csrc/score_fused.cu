@@ -1,6 +1,7 @@
 // Host side of the fused scoring path (kernel: fused.cuh): the split of a batch over the SMs, workspace layout, tensor
 // maps, and the preparing kernel that runs in front of it.
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "fused.cuh"
@@ -199,24 +200,29 @@ int32_t launch_prep(const PrepArgs<N>& args, int d, bool fp8, int n_slabs, int n
 constexpr int kSmemBudget = 227 * 1024 - 1024;   // dynamic shared memory we may ask for, minus alignment slack
 // Key bytes between the first and the second read of a tile that still sit in L2 (126 MB, in two halves).
 constexpr double kL2KeyBytes = 80e6;
-// Key bytes an SM reads while a slab's sums travel to the other SMs and come back as log-sum-exps (about 3 us).
-constexpr int kHandoverBytes = 128 * 1024;
+// What an SM's share of the memory bandwidth brings in a microsecond (6.5 TB/s over 148 SMs).
+constexpr double kSmBytesPerUs = 44e3;
+// Microseconds from a slab's last key to its log-sum-exps having freed the slab's tiles; and what a tile of the next slab
+// takes when its keys are there already.
+constexpr double kHandoverUs = 5.5, kBurstUs = 0.3;
 
 struct Geometry {
   bool ok = false, fp8 = false, once = false;
   int ncols = 0, padded_group = 0, n_slabs = 0, tile_bytes = 0;
   int max_tiles = 0;      // tiles per CTA whose running maxima fit tensor memory next to the least number of stages
   int lead = 0;           // two-pass: tiles of lead over visit 2 that L2 holds
-  int handover = 0;       // tiles that arrive while a slab's sums travel to the other SMs and come back as log-sum-exps
+  int handover = 0;       // two-pass: tiles that arrive while a slab's sums travel to the other SMs and come back
   // Resident form: tiles whose logits fit tensor memory next to the running maxima of `tiles` tiles.
   int resident(int tiles) const {
     return std::min(kMaxResident, (kTmemColsAll - tiles * (ncols / padded_group)) / ncols);
   }
-  // Tiles that may lie between the two visits for CTAs with `tiles` tiles a slab.
-  int room(int tiles) const { return once ? resident(tiles) : lead; }
-  // Tiles that lie between the visits when neither waits: resident tiles are folded and freed in a burst when the
-  // log-sum-exps arrive, while a visit 2 that copies and multiplies again takes as long as visit 1.
-  int wanted(int tiles) const { return (once ? tiles : 2 * tiles) + handover; }
+  // Most tiles a CTA and slab that leave the two visits room to overlap.
+  int comfortable_tiles() const {
+    if (!once) return std::max(1, (lead - handover) / 2);           // visit 2 takes as long as visit 1
+    int t = 1;
+    while (2 * resident(t + 1) >= 3 * (t + 1)) ++t;
+    return t;
+  }
 };
 
 Geometry geometry(const ScoreProblem& p, int sm_count) {
@@ -238,10 +244,10 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
   g.n_slabs = p.n_layers * p.n_kv_heads;
   g.tile_bytes = kTileKeys * row_bytes(p.head_dim, g.fp8);
   g.lead = std::max(2, (int)(kL2KeyBytes / ((double)sm_count * g.tile_bytes)));
-  g.handover = std::max(2, kHandoverBytes / g.tile_bytes);
+  g.handover = std::max(2, (int)(3.0 * kSmBytesPerUs / g.tile_bytes));
   const int tiles = (int)std::min<int64_t>(ceil_div(ceil_div(p.n_tokens, kTileKeys), std::min(sm_count, kFusedMaxCtas)), 1 << 20);
   // the resident form wants a slab's tiles and a few more in tensor memory
-  g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + std::min(g.handover, 3);
+  g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + 3;
   g.max_tiles = (kTmemColsAll - 2 * (sum_rows(g.ncols) + g.ncols)) / (g.ncols / g.padded_group);
   g.ok = tiles <= g.max_tiles;
   return g;
@@ -249,92 +255,114 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
 
 struct Split {
   int parts = 1, per_part = 1, tiles = 1;   // `tiles` per CTA of a group
+  double cost = 0;                          // time, in tiles that an SM's share of the memory bandwidth brings
 };
 
-// The best split of T tiles x S slabs over at most `ctas` CTAs.  What counts is the CTA with the most tile visits; a slab
-// costs a CTA a fraction of a tile on top (its sums' hand-over), and meeting in global memory about half a tile per tile.
-// More groups mean more tiles a CTA and slab, which have to lie between the two visits: where there is no room for them
-// (and the CTA's whole work is more than that), one visit waits for the other.
-Split best_split(const Geometry& g, int64_t n_tiles, int ctas) {
+// Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 4k to 250k tokens.
+// Three things can bound it, and near a tie they add up:
+//   memory: half the CTA with the most tiles, half the average (a CTA with more than its share gets more bandwidth);
+//   latency (resident): a tile's place is taken until its slab's log-sum-exps are back, and there is room for `held` slabs;
+//   the sum warps, which every slab costs a reduction over the warp on top of its tiles.
+// Two-pass: the tiles, stretched where L2 does not hold the lead that the hand-over takes.
+double split_cost(const Geometry& g, int64_t n_tiles, int tiles, int parts, int per_part, int share) {
+  const int slabs = (g.n_slabs + parts - 1) / parts;
+  const double units = (double)tiles * slabs, fair = (double)n_tiles * g.n_slabs / share;
+  if (!g.once) {
+    const double stretch = units > g.lead ? std::max(1.0, (double)(2 * tiles + g.handover) / g.lead) : 1.0;
+    return units * stretch + 0.1 * slabs + 2.0 * tiles;
+  }
+  const double us = g.tile_bytes / kSmBytesPerUs, per_tile = (double)g.resident(tiles) / tiles;
+  const double held = std::max(1.0, 0.5 * (per_tile + std::floor(per_tile)));
+  const double memory = 0.5 * (units + fair);
+  const double latency = std::max(kHandoverUs / us + tiles, slabs / held * (kHandoverUs + tiles * kBurstUs) / us);
+  const double sums = slabs * (g.ncols == 32 ? 0.9 + 0.24 * ((tiles + 1) / 2) : 0.5 + 0.16 * ((tiles + 1) / 2)) / us;
+  return std::cbrt(memory * memory * memory + latency * latency * latency + sums * sums * sums) + 2.0 * tiles;
+}
+
+// The best split over at most `ctas` CTAs; cost < 0 if there is none.  `share`: CTAs among which the memory bandwidth is
+// divided, for this prompt's part of it.
+Split best_split(const Geometry& g, int64_t n_tiles, int ctas, int share) {
   Split best;
-  double best_cost = 1e30;
+  best.cost = -1;
   for (int parts = 1; parts <= std::min(ctas, g.n_slabs); ++parts) {
-    const int per_part = (int)std::min<int64_t>(ctas / parts, n_tiles);
-    const int tiles = (int)ceil_div(n_tiles, per_part), slabs = (g.n_slabs + parts - 1) / parts;
-    if (tiles > g.max_tiles) break;
-    if (g.once && g.resident(tiles) < tiles + 1) break;
-    double cost = (double)tiles * slabs;
-    if (tiles * slabs > g.room(tiles)) cost *= std::max(1.0, (double)g.wanted(tiles) / g.room(tiles));
-    cost += 0.25 * slabs + (parts > 1 ? 0.5 * tiles : 0.0);
-    if (cost < best_cost * 0.999) {
-      best_cost = cost;
+    const int most = (int)std::min<int64_t>(ctas / parts, n_tiles);
+    const int64_t tiles = ceil_div(n_tiles, most);
+    if (tiles > g.max_tiles || (g.once && g.resident((int)tiles) < tiles + 1)) break;
+    const int per_part = (int)ceil_div(n_tiles, tiles);              // no more CTAs than these tiles need
+    const double cost = split_cost(g, n_tiles, (int)tiles, parts, per_part, share);
+    if (best.cost < 0 || cost < best.cost * 0.999) {
       best.parts = parts;
       best.per_part = per_part;
-      best.tiles = tiles;
+      best.tiles = (int)tiles;
+      best.cost = cost;
     }
   }
   return best;
 }
 
-// The fewest CTAs that finish a prompt in at most `units` tile visits each.
-Split fewest_ctas(const Geometry& g, int64_t n_tiles, int units) {
-  Split best;
-  best.per_part = 1 << 20;
-  for (int parts = 1; parts <= std::min(g.n_slabs, 64); ++parts) {
-    const int slabs = (g.n_slabs + parts - 1) / parts;
-    int tiles = (int)std::min<int64_t>(std::min(units / slabs, g.max_tiles), n_tiles);
-    while (tiles >= 1 && ((units > g.room(tiles) && g.wanted(tiles) > g.room(tiles)) || (g.once && g.resident(tiles) < tiles + 1))) --tiles;
-    if (tiles < 1) continue;
-    const int per_part = (int)ceil_div(n_tiles, tiles);
-    if ((int64_t)parts * per_part < (int64_t)best.parts * best.per_part) {
-      best.parts = parts;
-      best.per_part = per_part;
-      best.tiles = (int)ceil_div(n_tiles, per_part);
-    }
-  }
-  return best;
-}
-
-// Splits a group of prompts over the SMs, each on CTAs of its own: the smallest number of tile visits per CTA for which the
-// prompts' CTAs fit (bisection: fewer visits never need fewer CTAs by more than the rounding of fewest_ctas).
+// Splits a group of prompts over the SMs, each on CTAs of its own: CTAs in proportion to the tiles, then a few moves from
+// the prompt that would be done first to the one that would be done last.
 bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count, Split* out) {
   if (n == 1) {
-    out[0] = best_split(g, n_tiles[0], sm_count);
-    return true;
+    out[0] = best_split(g, n_tiles[0], sm_count, sm_count);
+    return out[0].cost >= 0;
   }
   int64_t total = 0;
   for (int i = 0; i < n; ++i) total += n_tiles[i];
-  auto fits = [&](int units) {
-    int64_t ctas = 0;
-    for (int i = 0; i < n; ++i) {
-      out[i] = fewest_ctas(g, n_tiles[i], units);
-      ctas += (int64_t)out[i].parts * out[i].per_part;
-    }
-    return ctas <= sm_count;
+  int ctas[kFusedMaxBatch], left = sm_count;
+  for (int i = 0; i < n; ++i) left -= ctas[i] = std::max(1, (int)(n_tiles[i] * sm_count / total));
+  auto fit = [&](int i) {
+    out[i] = best_split(g, n_tiles[i], ctas[i], ctas[i]);
+    return out[i].cost >= 0;
   };
-  int lo = (int)std::max<int64_t>(1, total * g.n_slabs / sm_count), hi = lo;
-  while (!fits(hi)) {
-    if (hi > 16 * lo + 64) return false;
-    lo = hi;
-    hi += hi / 4 + 1;
+  for (int i = 0; i < n; ++i)
+    if (!fit(i)) out[i].cost = 1e30;                                 // not with so few: the moves below give it more
+  for (int step = 0; step < 32; ++step) {
+    int slow = 0, quick = -1;
+    for (int i = 1; i < n; ++i)
+      if (out[i].cost > out[slow].cost) slow = i;
+    if (left <= 0) {
+      for (int i = 0; i < n; ++i)
+        if (i != slow && ctas[i] > 1 && (quick < 0 || out[i].cost < out[quick].cost)) quick = i;
+      if (quick < 0 || (out[quick].cost > 0.9 * out[slow].cost && left == 0)) break;
+    }
+    const Split slow_was = out[slow], quick_was = quick >= 0 ? out[quick] : Split{};
+    if (quick >= 0) {
+      --ctas[quick];
+      if (!fit(quick)) out[quick].cost = 1e30;
+    } else {
+      --left;
+    }
+    if (left >= 0) {
+      ++ctas[slow];
+      if (!fit(slow)) out[slow].cost = 1e30;
+    } else {
+      ++left;                                                        // the proportional shares had handed out too many
+    }
+    if (quick >= 0 && left >= 0 && out[quick].cost >= slow_was.cost) {   // no better: take the move back and stop
+      ++ctas[quick];
+      --ctas[slow];
+      out[quick] = quick_was;
+      out[slow] = slow_was;
+      break;
+    }
   }
-  while (hi - lo > std::max(1, hi / 64)) {
-    const int mid = lo + (hi - lo) / 2;
-    if (fits(mid)) hi = mid;
-    else lo = mid;
+  int64_t used = 0;
+  for (int i = 0; i < n; ++i) {
+    if (out[i].cost >= 1e30) return false;
+    used += (int64_t)out[i].parts * out[i].per_part;
   }
-  return fits(hi);
+  return used <= sm_count;
 }
 
-// How many prompts, from the first on, go into one launch: as many as leave each CTA room for its tiles between the visits.
+// How many prompts, from the first on, go into one launch.
 int group_size(const Geometry& g, const int64_t* n_tiles, int n, int sm_count) {
-  int per_cta = 1;                                                   // tiles a CTA and slab
-  while (g.wanted(per_cta + 1) <= g.room(per_cta + 1)) ++per_cta;
+  const double most = (double)g.comfortable_tiles() * sm_count;
   double tiles = 0;
   int count = 0;
   while (count < n && count < sm_count) {
     tiles += (double)n_tiles[count];
-    if (count > 0 && tiles > (double)per_cta * sm_count && tiles * g.n_slabs > (double)g.room(per_cta) * sm_count) break;
+    if (count > 0 && tiles > most) break;
     ++count;
   }
   return count;
@@ -586,7 +614,7 @@ int32_t score_fused_launch(const ScoreProblem* p, int n_prompts, void* workspace
     Split split[kFusedMaxBatch];
     if (!split_group(g, n_tiles, n, sm_count, split)) {
       n = 1;
-      split_group(g, n_tiles, 1, sm_count, split);
+      if (!split_group(g, n_tiles, 1, sm_count, split)) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
     }
     const int32_t st = n == 1 ? launch_group<1>(p + first, n, g, split, base, sm_count, dev_status, stream, mode, lse_in)
                               : launch_group<kFusedMaxBatch>(p + first, n, g, split, base, sm_count, dev_status, stream, mode, lse_in);
