@@ -141,6 +141,7 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+from . import _native  # noqa: E402  (linked against the library loaded above)
 
 
 def _check(status: int, where: str) -> None:
@@ -715,69 +716,33 @@ class Selector:
             self.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
         return self.workspace
 
+    def _run(self, kind: int, q, keys, aux, n_tokens: int, token_ids, char_start, char_end, keep: float, stream) -> Selection:
+        """Scoring, pooling, top-k and compaction enqueued by one native call (kind 0: contiguous, 1: paged, 2: 8-bit keys)."""
+        status, where, results = _native.select(self, kind, q, keys, aux, n_tokens, token_ids, char_start, char_end, keep, stream)
+        _check(status, where)
+        importance, lse, chunk_scores, k = results[0]
+        return Selection(importance, lse, chunk_scores, k, self.kept, self.out_ids, self.out_pos, self.tok_spans, self.char_spans,
+                         self.counts)
+
     def run(self, q: torch.Tensor, k_layers: Sequence[torch.Tensor], token_ids: torch.Tensor,
             char_start: torch.Tensor, char_end: torch.Tensor, keep: float,
             stream: Optional[torch.cuda.Stream] = None) -> Selection:
         """Enqueues the whole path for one prompt whose tensors are already on the device.  Nothing is synchronised:
         device-side conditions (see spf_score) accumulate in ``self.dev_status``, which the caller zeroes and reads
         (run_checked does both)."""
-        n = k_layers[0].shape[1]
-        if n > self.max_tokens:
-            raise ValueError(f"prompt has {n} tokens, selector was sized for {self.max_tokens}")
-        bufs = PromptBuffers(q, k_layers, self.importance[:n], self.lse)
-        spf_score([bufs], self._workspace(bufs), self.softmax_scale, self.dev_status, stream)
-        return self._select(n, token_ids, char_start, char_end, keep, stream)
+        return self._run(0, q, k_layers, None, 0, token_ids, char_start, char_end, keep, stream)
 
     def run_paged(self, q: torch.Tensor, k_pools: Sequence[torch.Tensor], block_table: torch.Tensor, n_tokens: int,
                   token_ids: torch.Tensor, char_start: torch.Tensor, char_end: torch.Tensor, keep: float,
                   stream: Optional[torch.cuda.Stream] = None) -> Selection:
         """run() for a prompt whose keys sit in a block pool (see PagedPromptBuffers)."""
-        n = n_tokens
-        if n > self.max_tokens:
-            raise ValueError(f"prompt has {n} tokens, selector was sized for {self.max_tokens}")
-        bufs = PagedPromptBuffers(q, k_pools, block_table, n, self.importance[:n], self.lse)
-        need = spf_score_paged_workspace_bytes([bufs], self.softmax_scale)
-        if self.workspace is None or self.workspace.numel() < need:
-            self.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
-        spf_score_paged([bufs], self.workspace, self.softmax_scale, self.dev_status, stream)
-        return self._select(n, token_ids, char_start, char_end, keep, stream)
+        return self._run(1, q, k_pools, block_table, n_tokens, token_ids, char_start, char_end, keep, stream)
 
     def run_fp8(self, q: torch.Tensor, k_layers: Sequence[torch.Tensor], k_scale: torch.Tensor, token_ids: torch.Tensor,
                 char_start: torch.Tensor, char_end: torch.Tensor, keep: float,
                 stream: Optional[torch.cuda.Stream] = None) -> Selection:
         """run() for a prompt whose key cache is held as E4M3 bytes (see Fp8PromptBuffers)."""
-        n = k_layers[0].shape[1]
-        if n > self.max_tokens:
-            raise ValueError(f"prompt has {n} tokens, selector was sized for {self.max_tokens}")
-        bufs = Fp8PromptBuffers(q, k_layers, k_scale, self.importance[:n], self.lse)
-        need = spf_score_fp8_workspace_bytes([bufs], self.softmax_scale)
-        if self.workspace is None or self.workspace.numel() < need:
-            self.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
-        spf_score_fp8([bufs], self.workspace, self.softmax_scale, self.dev_status, stream)
-        return self._select(n, token_ids, char_start, char_end, keep, stream)
-
-    def _select(self, n: int, token_ids: torch.Tensor, char_start: torch.Tensor, char_end: torch.Tensor, keep: float,
-                stream: Optional[torch.cuda.Stream]) -> Selection:
-        """Pooling, top-k and compaction on the importance scores already in self.importance[:n]."""
-        n_chunks = (n + self.chunk - 1) // self.chunk
-        k = spf_keep_count(n_chunks, keep)
-        if self.pool_edge_rule:
-            spf_chunk_pool_edge(self.importance[:n], self.pool_kernel, self.chunk, self.pool_edge_rule,
-                                self.chunk_scores[:n_chunks], stream)
-        else:
-            spf_chunk_pool(self.importance[:n], self.pool_kernel, self.chunk, self.chunk_scores[:n_chunks], stream)
-        if self.force_first or self.force_last:
-            k = max(k, len({0} if self.force_first else set()) + (1 if self.force_last and (n_chunks > 1 or not self.force_first) else 0))
-            spf_select_topk_forced(self.chunk_scores, n_chunks, k, self.force_first, self.force_last, self.kept, stream)
-            spf_compact_spans(self.kept, k, self.chunk, n, token_ids, char_start, char_end, self.out_ids, self.out_pos,
-                              self.tok_spans, self.char_spans, self.counts, stream)
-        else:
-            # top-k and compaction chained in one launch
-            spf_select_compact(self.chunk_scores, n_chunks, k, self.chunk, n, token_ids, char_start, char_end, self.kept,
-                               self.out_ids, self.out_pos, self.tok_spans, self.char_spans, self.counts, stream)
-        L, Hq, _, _, m = self.geom
-        return Selection(self.importance[:n], self.lse.view(L, Hq, m), self.chunk_scores[:n_chunks], k, self.kept,
-                         self.out_ids, self.out_pos, self.tok_spans, self.char_spans, self.counts)
+        return self._run(2, q, k_layers, k_scale, 0, token_ids, char_start, char_end, keep, stream)
 
     # device conditions after which the general path is tried: a row sum beyond fp32 (-6), a bounded wait that ran
     # out (-5); and the host refusal of a grid that cannot be co-resident (-2, raised as SpfError)
@@ -860,24 +825,7 @@ class BatchSelector:
     def run(self, prompts, keep: float, stream: Optional[torch.cuda.Stream] = None):
         """prompts: objects with q, k (list), token_ids, char_start, char_end, n_tokens (device tensors).  Returns one
         Selection per prompt; nothing is synchronised."""
-        if len(prompts) > len(self.slots):
-            raise ValueError("more prompts than slots")
-        slots = self.slots[:len(prompts)]
-        bufs = [PromptBuffers(p.q, p.k, s.importance[:p.n_tokens], s.lse) for p, s in zip(prompts, slots)]
-        need = spf_score_workspace_bytes(bufs, self.softmax_scale)
-        if self.workspace is None or self.workspace.numel() < need:
-            self.workspace = torch.empty(need, dtype=torch.uint8, device=self.device)
-        spf_score(bufs, self.workspace, self.softmax_scale, self.dev_status, stream)
-        ns = [p.n_tokens for p in prompts]
-        ncs = [(n + self.chunk - 1) // self.chunk for n in ns]
-        ks = [spf_keep_count(c, keep) for c in ncs]
-        spf_chunk_pool_batch([s.importance[:n] for s, n in zip(slots, ns)], self.pool_kernel, self.chunk,
-                             [s.chunk_scores[:c] for s, c in zip(slots, ncs)], stream)
-        spf_select_topk_batch([s.chunk_scores for s in slots], ncs, ks, [s.kept for s in slots], stream)
-        spf_compact_spans_batch([s.kept for s in slots], ks, self.chunk, ns, [p.token_ids for p in prompts],
-                                [p.char_start for p in prompts], [p.char_end for p in prompts], [s.out_ids for s in slots],
-                                [s.out_pos for s in slots], [s.tok_spans for s in slots], [s.char_spans for s in slots],
-                                [s.counts for s in slots], stream)
-        L, Hq, _, _, m = self.geom
-        return [Selection(s.importance[:n], s.lse.view(L, Hq, m), s.chunk_scores[:c], k, s.kept, s.out_ids, s.out_pos,
-                          s.tok_spans, s.char_spans, s.counts) for s, n, c, k in zip(slots, ns, ncs, ks)]
+        status, where, results = _native.select_batch(self, prompts, keep, stream)
+        _check(status, where)
+        return [Selection(importance, lse, chunk_scores, k, s.kept, s.out_ids, s.out_pos, s.tok_spans, s.char_spans, s.counts)
+                for s, (importance, lse, chunk_scores, k) in zip(self.slots, results)]

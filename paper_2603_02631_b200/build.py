@@ -1,4 +1,5 @@
-"""Compiles the CUDA sources into ``libspf.so`` next to this file (sm_100a only).
+"""Compiles the CUDA sources into ``libspf.so`` (sm_100a only) and the native part of the Python binding into
+``_native.so``, both next to this file.
 
 Usage: ``python -m paper_2603_02631_b200.build [--force] [--verbose]``.
 nvcc cross-compiles without a GPU, so this also runs on a CPU-only machine.
@@ -11,12 +12,15 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 import tempfile
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libspf.so")
+NATIVE_SRC = os.path.join(CSRC, "python", "native.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -35,16 +39,29 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _older(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
-        return True
-    built = os.path.getmtime(LIB_PATH)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return any(os.path.getmtime(p) > built for p in deps)
+    headers = glob.glob(os.path.join(ROOT, "include", "*.h"))
+    return _older(LIB_PATH, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers) or _older(NATIVE_PATH, [NATIVE_SRC, *headers])
+
+
+def _native_command() -> list:
+    """g++ command for the binding's native part, against the headers and libraries of the installed torch."""
+    import torch
+    torch_dir = os.path.dirname(os.path.abspath(torch.__file__))
+    include = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+               os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), sysconfig.get_paths()["include"],
+               os.path.join(ROOT, "include")]
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *[f"-I{d}" for d in include], NATIVE_SRC, "-o", NATIVE_PATH, f"-L{os.path.join(torch_dir, 'lib')}", "-ltorch_python", "-ltorch_cpu",
+            "-lc10_cuda", "-lc10", LIB_PATH, "-Wl,-rpath,$ORIGIN"]
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Builds libspf.so if it is missing or older than its sources; returns its path."""
+    """Builds libspf.so and _native.so if one of them is missing or older than its sources; returns the path of libspf.so."""
     if not force and not is_stale():
         return LIB_PATH
     include = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -54,14 +71,16 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         if verbose or proc.returncode != 0:
             sys.stderr.write(proc.stdout + proc.stderr)
         if proc.returncode != 0:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError("compilation failed: " + " ".join(cmd))
         return proc.stdout + proc.stderr
 
     with tempfile.TemporaryDirectory() as tmp:
         objects = [os.path.join(tmp, os.path.basename(src) + ".o") for src in sources()]
         with concurrent.futures.ThreadPoolExecutor(os.cpu_count() or 1) as pool:
             log = "".join(pool.map(lambda so: run([_nvcc(), *NVCC_FLAGS, *include, "-c", so[0], "-o", so[1]]), zip(sources(), objects)))
-        run([_nvcc(), *NVCC_FLAGS, "--shared", "-o", LIB_PATH, *objects])
+        run([_nvcc(), *NVCC_FLAGS, "--shared", "-o", LIB_PATH, "-Xlinker", "-soname=libspf.so", *objects])
+    if force or _older(NATIVE_PATH, [NATIVE_SRC, *glob.glob(os.path.join(ROOT, "include", "*.h"))]):
+        run(_native_command())
     with open(os.path.join(PKG_DIR, "libspf.ptxas.log"), "w") as f:
         f.write(log)
     return LIB_PATH
