@@ -46,14 +46,14 @@
 // detected (the sum is inf) and reported as SPF_ERR_RANGE; the caller can then use the general path.
 //
 // Cross-CTA step.  All CTAs use the same reference for a slab, so their partial sums can simply be added.  Each CTA stores
-// its sums as plain words, [slab][four rows][CTA of the group], zero meaning "not there yet".  Every four rows of a slab
-// have an owner among the CTAs, which reads everybody's words, adds them up in double in a fixed order and stores the
-// log-sum-exps as 64-bit words {value, 1}; every CTA polls those.  No atomics, no fences, no counters: two stores and two
-// polls, about 3 us from a slab's last sum to its log-sum-exps everywhere, and every run arrives at the same bits.  (Exact
-// atomic sums with an arrival counter took 5.4 us; every CTA reading everybody's sums 2 us, but 7 us of a slab's time.)
-// How far visit 2 trails visit 1 is what has to fit in L2, so this latency is what the split is built around.  Visit 1
-// waits for other CTAs only through its lead over visit 2, which covers at least one whole slab, so every slab's sums
-// complete and the words always arrive.
+// its sums as plain words, [slab][CTA of the group][four rows], zero meaning "not there yet".  In a group of few CTAs
+// everybody reads everybody's words and adds them up; in a larger one every four rows of a slab have an owner, which does
+// that and stores the log-sum-exps as 64-bit words {value, 1} that every CTA polls.  Sums are taken in double and in a fixed
+// order, so every run arrives at the same bits.  No atomics, no fences, no counters: 2 or 3 us from a slab's last sum to its
+// log-sum-exps everywhere, where exact atomic sums with an arrival counter took 5.4.  This latency is what the split over
+// the SMs is built around: how far visit 2 trails visit 1 is what has to fit in tensor memory (or in L2).  Visit 1 waits for
+// other CTAs only through that room, which covers at least one whole slab, so every slab's sums complete and the words
+// always arrive.
 //
 // Every wait on a barrier, word or flag in this file is bounded: on expiry the kernel records SPF_ERR_TIMEOUT, drains and
 // returns normally.  The one wait that has no limit is the hardware's own: tcgen05.alloc blocks while another resident CTA
@@ -68,11 +68,16 @@ namespace spf {
 constexpr int kFusedThreads = 768;
 constexpr int kVisitWarps = 8;         // epilogue warps per visit
 constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
+// Groups of up to this many CTAs add up everybody's row sums in every CTA (see fused_publish): one hop instead of two, about
+// 2 us instead of 3, for reading 16 * CTAs * NCOLS / 4 bytes a slab and CTA.
+constexpr int kGatherCtas = 40;
+__host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return ncols <= 32 && n_ctas <= kGatherCtas; }
 constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
 constexpr int kMaxQStages = 4;         // query tiles in flight per visit (two-pass: 2)
 constexpr int kMaxKeyStages = 16;      // key tiles in flight per visit
 constexpr int kMaxTmemStages = 4;      // two-pass: accumulator stages per visit and set
 constexpr int kMaxResident = 32;       // resident: tiles in tensor memory
+constexpr int kRegTiles = 8, kRegSlots = 8;   // running maxima stay in registers up to this many tiles a CTA and lookahead slots a key
 constexpr int kTmemColsAll = 512;      // the CTA takes all of its SM's tensor memory
 constexpr int kOffSlots = 4;           // slabs whose log-sum-exps may be in shared memory at once
 constexpr int kSumSlots = 8;           // slabs whose row sums may be on their way to the publishers at once
@@ -88,7 +93,7 @@ __host__ __device__ constexpr int sum_rows(int ncols) { return ncols <= 32 ? 32 
 struct FusedPrompt {
   const CUtensorMap* k_maps;   // [n_layers] (element of a sub-row, key, sub-tile, kv-head[, pool block])
   const unsigned char* q_tiles;   // [slab] query operands as the tensor cores read them (swizzled, padding rows zero)
-  float4* row_sums;            // [slab][NCOLS / 4][per_part] each CTA's sums of exp2(c*q.k - ref) for four rows; 0: not there yet
+  float4* row_sums;            // [slab][per_part][NCOLS / 4] each CTA's sums of exp2(c*q.k - ref) for four rows; 0: not there yet
   unsigned long long* lse;     // [slab][NCOLS] {log-sum-exp in base-2 units, 1} once known
   const float* refs;           // [slab] reference of visit 1
   const float* slab_c;         // [slab] 8-bit keys: accumulated dot product -> base-2 logit; null: FusedArgs::c for all
@@ -111,7 +116,8 @@ struct FusedArgs {
   int table_tiles;             // tiles per CTA for which there is a table (paged key cache), else 0
   int mode;                    // 0: the whole computation; 1: visit 1 alone (row log-sum-exps of these keys); 2: visit 2 alone
   int k_stages[2], t_stages[2];   // per visit: key tiles; accumulator stages per set (resident: [0] alone, tiles in tensor memory)
-  int max_tiles_per_stage;     // tiles per accumulator stage of visit 2 (visit 1: one)
+  int max_tiles_per_stage;     // two-pass: tiles per accumulator stage of visit 2 (visit 1: one)
+  int max_in_regs;             // resident: no CTA has more than kRegTiles tiles
   float c;                     // softmax scale * log2(e)
   int32_t* dev_status;         // optional
 };
@@ -403,36 +409,40 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
 }
 
 // ---------------------------------------------------------------------------------------------- publishers
-// Rows 4q .. 4q + 3 of a slab: adds up all CTAs' words and stores the log-sum-exps.
-template <class T, int NCOLS, int G>
-__device__ __forceinline__ bool reduce_rows(const FusedArgs& a, const FusedShare& sh, int slab, int q, int n_ctas, int lane, const Abort& ab) {
-  const FusedPrompt& p = *sh.p;
-  constexpr int Q = NCOLS / 4;
-  constexpr int MAXW = (kFusedMaxCtas + 31) / 32;                  // words per lane
-  const int per_part = p.per_part;
-  const float4* in = p.row_sums + ((int64_t)slab * Q + q) * per_part;
+// Waits for and adds up CTAs' row sums of a slab.  LANES = 1: the four rows of quad `q`, a CTA per lane; LANES = NCOLS / 4:
+// all rows, lane mod LANES being the quad.  On return lane (with lane mod 8 < LANES) has the log-sum-exp, in base-2 units,
+// of row 4 * quad + lane / 8 in `lse2`; false if the wait was given up.
+template <int NCOLS, int G, int LANES, int MAXW>
+__device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPrompt& p, int slab, int q, int n_ctas, int lane, bool report,
+                                            float& lse2, const Abort& ab) {
+  constexpr int Q = NCOLS / 4, STEP = 32 / LANES;                  // CTAs per load of the warp
+  if (LANES > 1) q = lane % Q;
+  const int first = lane / LANES;
+  const float4* in = p.row_sums + ((int64_t)slab * p.per_part + first) * Q + q;
   float4 v[MAXW];
 #pragma unroll
   for (int i = 0; i < MAXW; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto missing = [&](int i) {
+    return first + STEP * i < n_ctas && (v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f);
+  };
   unsigned long long t0 = 0;
   for (uint32_t it = 1;; ++it) {
     // whatever is not there yet is asked for again (a word may also be caught half written)
 #pragma unroll
     for (int i = 0; i < MAXW; ++i)
-      if (lane + 32 * i < n_ctas && (v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f))
+      if (missing(i))
         asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w)
-                     : "l"(in + lane + 32 * i)
+                     : "l"(in + (int64_t)STEP * i * Q)
                      : "memory");
     bool there = true;
 #pragma unroll
-    for (int i = 0; i < MAXW; ++i)
-      there = there && (lane + 32 * i >= n_ctas || !(v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f));
+    for (int i = 0; i < MAXW; ++i) there = there && !missing(i);
     if (__all_sync(0xffffffffu, there)) break;
     if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return false;
-    __nanosleep(100);
+    if (LANES == 1) __nanosleep(100);
   }
-  double t[4] = {0.0, 0.0, 0.0, 0.0};                            // the CTAs' shares are fp32: exact to 2^-53
+  double t[4] = {0.0, 0.0, 0.0, 0.0};                              // the CTAs' shares are fp32: exact to 2^-53
 #pragma unroll
   for (int i = 0; i < MAXW; ++i) {
     t[0] += (double)v[i].x;
@@ -440,7 +450,7 @@ __device__ __forceinline__ bool reduce_rows(const FusedArgs& a, const FusedShare
     t[2] += (double)v[i].z;
     t[3] += (double)v[i].w;
   }
-  // two transposing steps leave one row per eight lanes: row 4q + (lane >> 3 & 3), with the bits exchanged
+  // two transposing steps leave one row per lane: lanes 8.. have t[1], 16.. t[2], 24.. t[3]
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const double send = (lane & 16) ? t[e] : t[e + 2], keep = (lane & 16) ? t[e + 2] : t[e];
@@ -451,46 +461,45 @@ __device__ __forceinline__ bool reduce_rows(const FusedArgs& a, const FusedShare
     t[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
   }
 #pragma unroll
-  for (int off = 4; off >= 1; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
-  if ((lane & 7) == 0) {
-    const int row = 4 * q + (lane >> 3);                         // lane 8: t[1], lane 16: t[2], lane 24: t[3]
-    float lse2 = INFINITY;                                       // rows that do not exist: exp2(x - lse2) = 0
-    if (row % G < a.group && row / G < a.n_lookahead) {
-      // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision; an empty (below every
-      // normal number) or overflowed row sum has none
-      const long long tb = __double_as_longlong(t[0]);
-      const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-      lse2 = __ldg(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
-      if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
-      const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
-      if (p.extra_lse != nullptr) {
-        // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
-        const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
-        const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
-        lse2 = hi + log2f(1.f + exp2f(lo - hi));
-      }
+  for (int off = 4; off >= LANES; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
+  const int row = 4 * q + (lane >> 3);
+  lse2 = INFINITY;                                                 // rows that do not exist: exp2(x - lse2) = 0
+  if ((lane & 7) < LANES && row % G < a.group && row / G < a.n_lookahead) {
+    // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision; an empty (below every
+    // normal number) or overflowed row sum has none
+    const long long tb = __double_as_longlong(t[0]);
+    const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+    lse2 = __ldg(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
+    if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
+    const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
+    if (p.extra_lse != nullptr) {
+      // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
+      const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
+      const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
+      lse2 = hi + log2f(1.f + exp2f(lo - hi));
+    }
+    if (report) {
       if (!(lse2 > -INFINITY && lse2 < INFINITY) && a.dev_status != nullptr) atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
       if (p.lse_out != nullptr) p.lse_out[out_idx] = lse2 * kLn2;
     }
-    const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + row), "l"(word) : "memory");
   }
-  __syncwarp();
   return true;
 }
 
 // Publisher w takes slabs w, w + 3, ...: stores this CTA's row sums (a row that does not exist gets its meaningless sum
-// stored too: everybody waits for every word) and then adds up everybody's sums of the rows that this CTA owns.  Item
-// n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab, belongs to CTA (item mod CTAs).  Only now: polling for words that
-// cannot be there yet slowed the key copies down.
-template <class T, int NCOLS, int G>
-__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums,
-                                              const FusedBars& bars, const Abort& ab) {
+// stored too: everybody waits for every word).  Then either this CTA adds up everybody's sums for itself (few CTAs to a
+// group: one hop), or only those of the rows that it owns -- item n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab,
+// belongs to CTA (item mod CTAs) -- and stores their log-sum-exps for all.  Not before its own sums are out: polling for
+// words that cannot be there yet slowed the key copies down.
+template <class T, int NCOLS, int G, bool FP8>
+__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums, float* off,
+                                              float* off_c, const FusedBars& bars, const Abort& ab) {
   constexpr int Q = NCOLS / 4;                                     // lane q has rows 4q .. 4q + 3
-  float4* const row_sums = sh.p->row_sums;
-  const int per_part = sh.p->per_part, n_ctas = min(per_part, sh.p->n_tiles);
+  const FusedPrompt& p = *sh.p;
+  const int per_part = p.per_part, n_ctas = min(per_part, p.n_tiles);
+  const bool alone = gather_alone(NCOLS, n_ctas);
   for (int n = which; n < sh.n_slabs; n += kPublisherWarps) {
-    const int slot = n % kSumSlots;
+    const int slot = n % kSumSlots, slab = sh.slab(n);
     if (!mbar_wait_warp(bars.sums_ready(slot), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
     float t[4] = {0.f, 0.f, 0.f, 0.f};
     if (lane < Q) {
@@ -514,11 +523,35 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
 #pragma unroll
       for (int e = 0; e < 4; ++e) w[e] = max(__float_as_uint(t[e]), 1u);   // never "not there yet"; 2^-149 is nothing to a row's sum
       asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};"
-                   ::"l"(row_sums + ((int64_t)sh.slab(n) * Q + lane) * per_part + sh.first), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                   ::"l"(p.row_sums + ((int64_t)slab * per_part + sh.first) * Q + lane), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
                    : "memory");
     }
-    for (int q = (int)(((unsigned)(n + 1) * (unsigned)n_ctas * Q + sh.first - n * Q) % (unsigned)n_ctas); q < Q; q += n_ctas)
-      if (!reduce_rows<T, NCOLS, G>(a, sh, sh.slab(n), q, n_ctas, lane, ab)) return;
+    float lse2;
+    if constexpr (NCOLS <= 32) {
+      if (alone) {
+        if (a.mode == 1 && sh.first != 0) continue;                // nobody reads the offsets
+        if (!sum_rows_of<NCOLS, G, Q, kGatherCtas * Q / 32>(a, p, slab, 0, n_ctas, lane, sh.first == 0, lse2, ab)) return;
+        if (a.mode == 1) continue;
+        const int x = n % kOffSlots;
+        if (n >= kOffSlots)
+          if (!mbar_wait_warp(bars.off_free(x), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
+        if ((lane & 7) < Q) off[x * 64 + 4 * (lane % Q) + (lane >> 3)] = -lse2;
+        if constexpr (FP8) {
+          if (lane == 0) off_c[x] = __ldg(p.slab_c + slab);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.off_ready(x));
+        continue;
+      }
+    }
+    for (int q = (int)(((unsigned)(n + 1) * (unsigned)n_ctas * Q + sh.first - n * Q) % (unsigned)n_ctas); q < Q; q += n_ctas) {
+      if (!sum_rows_of<NCOLS, G, 1, (kFusedMaxCtas + 31) / 32>(a, p, slab, q, n_ctas, lane, true, lse2, ab)) return;
+      if ((lane & 7) == 0) {
+        const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + 4 * q + (lane >> 3)), "l"(word) : "memory");
+      }
+      __syncwarp();
+    }
   }
 }
 
@@ -582,6 +615,53 @@ __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedS
   }
 }
 
+// ---------------------------------------------------------------------------------------------- importance
+// Mean over the lookahead of exp2(running max) for a tile's keys.  One group of CTAs (parts = 1): straight from the maxima.
+// Several: the groups' maxima meet in global memory, and whichever warp brings the last contribution for 32 keys reads the
+// result.
+template <int NI>
+__device__ __forceinline__ void finish_tile(const FusedArgs& a, const FusedPrompt& p, int tile, int quad, int lane, const uint32_t (&v)[NI]) {
+  const float inv_m = 1.f / (float)a.n_lookahead;
+  const int64_t key = (int64_t)tile * kTileKeys + quad * 32 + lane;
+  float sum = 0.f;
+  if (p.parts == 1) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if (i < a.n_lookahead) sum += fast_exp2(__uint_as_float(v[i]));
+  } else {
+    const int64_t n_pad = (int64_t)p.n_tiles * kTileKeys;
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if (i < a.n_lookahead) atomicMax(p.amax + (int64_t)i * n_pad + key, order_bits(__uint_as_float(v[i])));
+    __threadfence();
+    __syncwarp();
+    unsigned before = 0;
+    if (lane == 0) before = atomicAdd(p.finished + tile * 4 + quad, 1u);
+    if (__shfl_sync(0xffffffffu, before, 0) + 1u != (unsigned)p.parts) return;
+    __threadfence();
+#pragma unroll 8
+    for (int i = 0; i < a.n_lookahead; ++i) sum += fast_exp2(from_order_bits(__ldcg(p.amax + (int64_t)i * n_pad + key)));
+  }
+  if (key < p.n_tokens) p.importance[key] = sum * inv_m;
+}
+
+// The tiles of a max warp's set, from the maxima in tensor memory.
+template <class T>
+__device__ __forceinline__ void fused_finish(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t amax_tmem) {
+  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
+  const uint32_t lane_addr = amax_tmem + ((uint32_t)(quad * 32) << 16);
+  for (int lt = set; lt < sh.n_tiles; lt += 2) {
+    constexpr int LD = T::NI < 32 ? T::NI : 32;                    // columns per load
+    uint32_t v[T::NI];
+#pragma unroll
+    for (int i = 0; i < T::NI; i += LD)
+      tmem_issue<LD>(lane_addr + (uint32_t)(lt * T::NI + i), *reinterpret_cast<uint32_t(*)[LD]>(v + i));
+    tmem_load_wait();
+    tmem_ready<T::NI>(v);
+    finish_tile<T::NI>(a, *sh.p, sh.tile(lt), quad, lane, v);
+  }
+}
+
 // ---------------------------------------------------------------------------------------------- visit 2: maxima
 // Folds one load's accumulators into the running maxima over (layer, head) of the base-2 logits less their rows'
 // log-sum-exps (slots past n_lookahead hold padding and are never read).
@@ -619,7 +699,7 @@ __device__ __forceinline__ void clear_maxima(uint32_t amax_addr, int set, int n_
 }
 
 template <class T, int NCOLS, int G, bool FP8>
-__device__ __forceinline__ bool fused_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, uint32_t amax_tmem,
+__device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, uint32_t amax_tmem,
                                           const float* off, const float* off_c, const FusedBars& bars, const Abort& ab) {
   constexpr int CW = T::CW, NCH = T::NCH, NIW = T::NIW;
   const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
@@ -631,12 +711,12 @@ __device__ __forceinline__ bool fused_max(const FusedArgs& a, const FusedShare& 
   clear_maxima<T>(amax_addr, set, sh.n_tiles);
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
-    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return false;
+    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
     const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
     const float c = FP8 ? off_c[slot] : a.c;
     const uint64_t cc = pack2(c, c);
     for (int lt = set; lt < sh.n_tiles;) {
-      if (!mbar_wait_warp(bars.t_full(1, set, tr.stage), tr.phase, ab)) return false;
+      if (!mbar_wait_warp(bars.t_full(1, set, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
       tmem_store_wait();                                           // the maxima read below may be this warp's last stores
       const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * tps * NCOLS);
@@ -691,7 +771,7 @@ __device__ __forceinline__ bool fused_max(const FusedArgs& a, const FusedShare& 
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
   tmem_store_wait();
-  return true;
+  fused_finish<T>(a, sh, warp, lane, amax_tmem);
 }
 
 // ---------------------------------------------------------------------------------------------- resident form
@@ -842,93 +922,73 @@ __device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShar
 }
 
 // The maxima, once the slab's log-sum-exps are there.  A tile's maxima always belong to the same warps (lt mod 2 == set).
-template <class T, int NCOLS, int G, bool FP8>
-__device__ __forceinline__ bool resident_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem,
+// REGS: up to kRegTiles tiles, whose maxima stay in registers and leave all of tensor memory to the logits.
+template <class T, int NCOLS, int G, bool FP8, bool REGS>
+__device__ __forceinline__ void resident_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem,
                                              uint32_t amax_tmem, const float* off, const float* off_c, const FusedBars& bars,
                                              const Abort& ab) {
-  constexpr int NI = T::NI;
+  constexpr int NI = T::NI, MINE = REGS ? kRegTiles / 2 : 1;
   const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
   const int n_tiles = sh.n_tiles;
   const uint32_t lane_bits = (uint32_t)(quad * 32) << 16;
   const uint32_t lane_addr = tmem + lane_bits, amax_addr = amax_tmem + lane_bits;
-  clear_maxima<T>(amax_addr, set, n_tiles);
+  uint32_t am[MINE][NI];
+  if constexpr (REGS) {
+#pragma unroll
+    for (int u = 0; u < MINE; ++u)
+#pragma unroll
+      for (int j = 0; j < NI; ++j) am[u][j] = 0xff800000u;         // -inf
+  } else {
+    clear_maxima<T>(amax_addr, set, n_tiles);
+  }
   ResidentRing first(a.t_stages[0]);                               // the stage of the slab's first tile
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
-    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return false;
+    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
     const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
     const float c = FP8 ? off_c[slot] : a.c;
     const uint64_t cc = pack2(c, c);
     ResidentRing tr = first;
     tr.advance(set);
-    for (int lt = set; lt < n_tiles; lt += 2) {
+    auto fold = [&](int lt, uint32_t (&m)[NI]) -> bool {
       // complete long since (the log-sum-exps contain it), except where visit 2 runs alone
       if (!mbar_wait_warp(bars.t_full(0, 0, tr.stage), tr.phase, ab)) return false;
       tc_fence_after();
-      tmem_store_wait();                                           // the maxima read below may be this warp's last stores
-      uint32_t r[NCOLS], am[NI];
+      if (!REGS) tmem_store_wait();                                // the maxima read below may be this warp's last stores
+      uint32_t r[NCOLS];
       tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
-      tmem_issue<NI>(amax_addr + (uint32_t)(lt * NI), am);
+      if (!REGS) tmem_issue<NI>(amax_addr + (uint32_t)(lt * NI), m);
       tmem_load_wait();
       tmem_ready<NCOLS>(r);
-      tmem_ready<NI>(am);
+      if (!REGS) tmem_ready<NI>(m);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bars.t_empty(0, 0, tr.stage));
       tr.advance(2);
-      fold_maxima<T, G>(r, am, off2, cc);
-      tmem_store<NI>(amax_addr + (uint32_t)(lt * NI), am);
+      fold_maxima<T, G>(r, m, off2, cc);
+      if (!REGS) tmem_store<NI>(amax_addr + (uint32_t)(lt * NI), m);
+      return true;
+    };
+    if constexpr (REGS) {
+#pragma unroll
+      for (int u = 0; u < MINE; ++u)
+        if (set + 2 * u < n_tiles)
+          if (!fold(set + 2 * u, am[u])) return;
+    } else {
+      for (int lt = set; lt < n_tiles; lt += 2)
+        if (!fold(lt, am[0])) return;
     }
     first.advance(n_tiles);
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
-  tmem_store_wait();
-  return true;
-}
-
-// ---------------------------------------------------------------------------------------------- importance
-// Mean over the lookahead of exp2(running max).  One group of CTAs (parts = 1): straight from tensor memory.  Several: the
-// groups' maxima meet in global memory, and whichever warp brings the last contribution for 32 keys reads the result.
-template <class T, int NCOLS, int G>
-__device__ __forceinline__ void fused_finish(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t amax_tmem) {
-  constexpr int NI = T::NI, FC = NI < 16 ? NI : 16;
-  const FusedPrompt& p = *sh.p;
-  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
-  const uint32_t lane_addr = amax_tmem + ((uint32_t)(quad * 32) << 16);
-  const float inv_m = 1.f / (float)a.n_lookahead;
-  const bool meet = p.parts > 1;
-  const int64_t n_pad = (int64_t)p.n_tiles * kTileKeys;
-  for (int lt = set; lt < sh.n_tiles; lt += 2) {
-    const int tile = sh.tile(lt);
-    const int64_t key = (int64_t)tile * kTileKeys + quad * 32 + lane;
-    float sum = 0.f;
+  if constexpr (REGS) {
 #pragma unroll
-    for (int q = 0; q < NI / FC; ++q) {
-      uint32_t v[FC];
-      tmem_issue<FC>(lane_addr + (uint32_t)(lt * NI + q * FC), v);
-      tmem_load_wait();
-      tmem_ready<FC>(v);
-#pragma unroll
-      for (int j = 0; j < FC; ++j) {
-        const int i = q * FC + j;
-        if (i < a.n_lookahead) {
-          if (meet) atomicMax(p.amax + (int64_t)i * n_pad + key, order_bits(__uint_as_float(v[j])));
-          else sum += fast_exp2(__uint_as_float(v[j]));
-        }
-      }
-    }
-    if (meet) {
-      __threadfence();
-      __syncwarp();
-      unsigned before = 0;
-      if (lane == 0) before = atomicAdd(p.finished + tile * 4 + quad, 1u);
-      if (__shfl_sync(0xffffffffu, before, 0) + 1u != (unsigned)p.parts) continue;
-      __threadfence();
-#pragma unroll 8
-      for (int i = 0; i < a.n_lookahead; ++i) sum += fast_exp2(from_order_bits(__ldcg(p.amax + (int64_t)i * n_pad + key)));
-    }
-    if (key < p.n_tokens) p.importance[key] = sum * inv_m;
+    for (int u = 0; u < MINE; ++u)
+      if (set + 2 * u < n_tiles) finish_tile<NI>(a, *sh.p, sh.tile(set + 2 * u), quad, lane, am[u]);
+  } else {
+    tmem_store_wait();
+    fused_finish<T>(a, sh, warp, lane, amax_tmem);
   }
 }
 
@@ -1025,8 +1085,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   grid_wait();                                                     // what the preparing kernel wrote is visible from here on
 
   // ------------------------------------------------------------------ roles
+  // resident, 32 rows: 768 threads start with 80 registers each; 256 x 64 + 512 x 88 is the same sum
+  constexpr bool kMoveRegs = ONCE && NCOLS == 32;
   const bool visit1 = a.mode != 2, visit2 = a.mode != 1;
   if (warp < 4) {
+    if constexpr (kMoveRegs) reg_dec<64>();
     const int v = warp & 1;
     if (ONCE ? v == 0 : (v == 0 ? visit1 : visit2)) {
       unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
@@ -1041,21 +1104,29 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
       }
     }
   } else if (warp < kSumWarp0) {
+    if constexpr (kMoveRegs) reg_dec<64>();
     if (warp == kFetchWarp) {
-      if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
+      if (visit2 && !(visit1 && gather_alone(NCOLS, min(sh.p->per_part, sh.p->n_tiles)))) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
     } else if (visit1) {
-      fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
+      fused_publish<T, NCOLS, G, FP8>(a, sh, warp - kPublisherWarp0, lane, sums, off, off_c, bars, ab);
     }
   } else if (warp < kMaxWarp0) {
+    if constexpr (kMoveRegs) reg_inc<88>();
     if (visit1) {
       if constexpr (ONCE) resident_sum<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
       else fused_sum<T, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
     }
-  } else if (visit2) {
-    bool ok;
-    if constexpr (ONCE) ok = resident_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
-    else ok = fused_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_v2, amax_tmem, off, off_c, bars, ab);
-    if (ok && misc[0] == 0) fused_finish<T, NCOLS, G>(a, sh, warp, lane, amax_tmem);
+  } else {
+    if constexpr (kMoveRegs) reg_inc<88>();
+    if (!visit2) {
+    } else if constexpr (ONCE && T::NI <= kRegSlots) {
+      if (a.max_in_regs) resident_max<T, NCOLS, G, FP8, true>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
+      else resident_max<T, NCOLS, G, FP8, false>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
+    } else if constexpr (ONCE) {
+      resident_max<T, NCOLS, G, FP8, false>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
+    } else {
+      fused_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_v2, amax_tmem, off, off_c, bars, ab);
+    }
   }
 
   // ------------------------------------------------------------------ teardown

@@ -214,8 +214,9 @@ struct Geometry {
   int handover = 0;       // two-pass: tiles that arrive while a slab's sums travel to the other SMs and come back
   // Resident form: tiles whose logits fit tensor memory next to the running maxima of `tiles` tiles.
   int resident(int tiles) const {
-    return std::min(kMaxResident, (kTmemColsAll - tiles * (ncols / padded_group)) / ncols);
+    return std::min(kMaxResident, (kTmemColsAll - (max_in_regs(tiles) ? 0 : tiles * (ncols / padded_group))) / ncols);
   }
+  bool max_in_regs(int tiles) const { return tiles <= kRegTiles && ncols / padded_group <= kRegSlots; }
   // Most tiles a CTA and slab that leave the two visits room to overlap.
   int comfortable_tiles() const {
     if (!once) return std::max(1, (lead - handover) / 2);           // visit 2 takes as long as visit 1
@@ -373,6 +374,7 @@ bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, 
   const int amax_cols = tiles * (g.ncols / g.padded_group), sr = sum_rows(g.ncols);
   a->table_tiles = paged ? tiles : 0;
   if (g.once) {
+    a->max_in_regs = g.max_in_regs(tiles);
     a->t_stages[0] = g.resident(tiles);
     a->t_stages[1] = 0;
     a->max_tiles_per_stage = 1;
