@@ -202,9 +202,9 @@ constexpr int kSmemBudget = 227 * 1024 - 1024;   // dynamic shared memory we may
 constexpr double kL2KeyBytes = 80e6;
 // What an SM's share of the memory bandwidth brings in a microsecond (6.5 TB/s over 148 SMs).
 constexpr double kSmBytesPerUs = 44e3;
-// Microseconds from a slab's last key to its log-sum-exps having freed the slab's tiles; and what a tile of the next slab
-// takes when its keys are there already.
-constexpr double kHandoverUs = 5.5, kBurstUs = 0.3;
+// Microseconds from a slab's last key to its log-sum-exps having freed the slab's tiles, in one hop between the CTAs of a
+// group or in two; and what a tile of the next slab takes when its keys are there already.
+constexpr double kHandoverUs1 = 4.3, kHandoverUs2 = 5.5, kBurstUs = 0.3;
 
 struct Geometry {
   bool ok = false, fp8 = false, once = false;
@@ -261,7 +261,7 @@ struct Split {
 
 // Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 4k to 250k tokens.
 // Three things can bound it, and near a tie they add up:
-//   memory: half the CTA with the most tiles, half the average (a CTA with more than its share gets more bandwidth);
+//   memory: the average rather than the CTA with the most tiles (one with more than its share gets more bandwidth);
 //   latency (resident): a tile's place is taken until its slab's log-sum-exps are back, and there is room for `held` slabs;
 //   the sum warps, which every slab costs a reduction over the warp on top of its tiles.
 // Two-pass: the tiles, stretched where L2 does not hold the lead that the hand-over takes.
@@ -274,8 +274,9 @@ double split_cost(const Geometry& g, int64_t n_tiles, int tiles, int parts, int 
   }
   const double us = g.tile_bytes / kSmBytesPerUs, per_tile = (double)g.resident(tiles) / tiles;
   const double held = std::max(1.0, 0.5 * (per_tile + std::floor(per_tile)));
-  const double memory = 0.5 * (units + fair);
-  const double latency = std::max(kHandoverUs / us + tiles, slabs / held * (kHandoverUs + tiles * kBurstUs) / us);
+  const double memory = 0.85 * fair + 0.15 * units;
+  const double handover = gather_alone(g.ncols, per_part) ? kHandoverUs1 : kHandoverUs2;
+  const double latency = std::max(handover / us + tiles, slabs / held * (handover + tiles * kBurstUs) / us);
   const double sums = slabs * (g.ncols == 32 ? 0.9 + 0.24 * ((tiles + 1) / 2) : 0.5 + 0.16 * ((tiles + 1) / 2)) / us;
   return std::cbrt(memory * memory * memory + latency * latency * latency + sums * sums * sums) + 2.0 * tiles;
 }
