@@ -335,9 +335,10 @@ SPF_API int32_t spf_compact_spans(const int32_t* kept_chunks, int64_t k, int32_t
 
 /*
  * spf_select_topk followed by spf_compact_spans in ONE launch (Algorithm 1, TopKChunks ... MapDraftChunksToTextSpans):
- * both steps are latency-bound, and chaining them inside one CTA saves a launch per prompt.  Arguments, layouts and
+ * both steps are latency-bound, and chaining them saves a launch per prompt.  Arguments, layouts and
  * results are those of the two calls (kept_chunks receives the k indices as spf_select_topk writes them); n_chunks must
- * equal ceil(n_tokens / chunk).  Results are identical to the two separate calls.
+ * equal ceil(n_tokens / chunk).  Results are identical to the two separate calls.  Prompts of more than 32768 chunks take
+ * the two calls' launches.
  */
 SPF_API int32_t spf_select_compact(const float* chunk_scores, int64_t n_chunks, int64_t k, int32_t chunk, int64_t n_tokens,
                                    const int32_t* token_ids, const int32_t* char_start, const int32_t* char_end,
@@ -383,6 +384,32 @@ SPF_API int32_t spf_chunk_pool_batch(const spf_pool_item* items, int32_t n_items
                                      void* cuda_stream);
 SPF_API int32_t spf_select_topk_batch(const spf_topk_item* items, int32_t n_items, void* cuda_stream);
 SPF_API int32_t spf_compact_spans_batch(const spf_compact_item* items, int32_t n_items, int32_t chunk, void* cuda_stream);
+
+/*
+ * spf_chunk_pool, spf_select_topk and spf_compact_spans (Algorithm 1, AvgPool1D ... MapDraftChunksToTextSpans) of one or more
+ * prompts in ONE launch per 24 prompts; prompts of more than 32768 chunks take the three calls' launches.  `items` is a HOST
+ * array, read during the call only; the pointers in it are DEVICE memory with the layouts that the three calls state.
+ * edge_rule, force_first and force_last as in spf_chunk_pool_edge and spf_select_topk_forced.  Results are identical to the
+ * separate calls.
+ */
+typedef struct {
+  const float* importance; /* fp32 [n_tokens]                    */
+  int64_t n_tokens;
+  float* chunk_scores;     /* out: fp32 [ceil(n_tokens / chunk)] */
+  int64_t k;
+  const int32_t* token_ids;
+  const int32_t* char_start;
+  const int32_t* char_end;
+  int32_t* kept_chunks;    /* out: int32 [k], ascending */
+  int32_t* out_ids;
+  int32_t* out_pos;        /* may be NULL */
+  int32_t* out_tok_spans;
+  int32_t* out_char_spans;
+  int64_t* out_counts;
+} spf_path_item;
+
+SPF_API int32_t spf_pool_select_compact(const spf_path_item* items, int32_t n_items, int32_t pool_kernel, int32_t chunk,
+                                        int32_t edge_rule, int32_t force_first, int32_t force_last, void* cuda_stream);
 
 /*
  * Variants for two points the paper leaves open (Algorithm 1 names the operations, Appendix A.3 gives kernel 13 and

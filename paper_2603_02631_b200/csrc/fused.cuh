@@ -1083,6 +1083,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   const uint32_t amax_tmem = ONCE ? tmem_base + (uint32_t)(a.t_stages[0] * NCOLS)
                                   : tmem_v2 + (uint32_t)(2 * a.t_stages[1] * a.max_tiles_per_stage * NCOLS);
   grid_wait();                                                     // what the preparing kernel wrote is visible from here on
+  grid_launch_dependents();                                        // the next kernel starts where SMs are free, and waits there
 
   // ------------------------------------------------------------------ roles
   // resident, 32 rows: 768 threads start with 80 registers each; 256 x 64 + 512 x 88 is the same sum
@@ -1168,11 +1169,14 @@ int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream
   cfg.blockDim = dim3(kFusedThreads);
   cfg.dynamicSmemBytes = (size_t)l.smem_bytes;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  // the launch overlaps the preparing kernel; grid_wait() orders what reads its results
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, args);
   if (err == cudaErrorCooperativeLaunchTooLarge) {
     (void)cudaGetLastError();

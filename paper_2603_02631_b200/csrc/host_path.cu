@@ -132,15 +132,21 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
     int32_t st = attempt == 0 ? spf_score(shape, &pr, 1, base + a.workspace, ws_bytes, dev_status, stream)
                               : score_on_path(shape, &pr, 1, base + a.workspace, ws_bytes, dev_status, stream, 1);
     if (st != SPF_OK) return st;
-    st = spf_chunk_pool(pr.importance, n_tokens, params->pool_kernel, params->chunk, reinterpret_cast<float*>(base + a.scores), stream);
-    if (st != SPF_OK) return st;
-    st = spf_select_topk(reinterpret_cast<const float*>(base + a.scores), n_chunks, k, reinterpret_cast<int32_t*>(base + a.kept), stream);
-    if (st != SPF_OK) return st;
-    st = spf_compact_spans(reinterpret_cast<const int32_t*>(base + a.kept), k, params->chunk, n_tokens,
-                           reinterpret_cast<const int32_t*>(base + a.ids), reinterpret_cast<const int32_t*>(base + a.cs),
-                           reinterpret_cast<const int32_t*>(base + a.ce), reinterpret_cast<int32_t*>(base + a.out_ids),
-                           reinterpret_cast<int32_t*>(base + a.out_pos), reinterpret_cast<int32_t*>(base + a.tok),
-                           reinterpret_cast<int32_t*>(base + a.ch), reinterpret_cast<int64_t*>(base + a.counts), stream);
+    spf_path_item item{};
+    item.importance = pr.importance;
+    item.n_tokens = n_tokens;
+    item.chunk_scores = reinterpret_cast<float*>(base + a.scores);
+    item.k = k;
+    item.token_ids = reinterpret_cast<const int32_t*>(base + a.ids);
+    item.char_start = reinterpret_cast<const int32_t*>(base + a.cs);
+    item.char_end = reinterpret_cast<const int32_t*>(base + a.ce);
+    item.kept_chunks = reinterpret_cast<int32_t*>(base + a.kept);
+    item.out_ids = reinterpret_cast<int32_t*>(base + a.out_ids);
+    item.out_pos = reinterpret_cast<int32_t*>(base + a.out_pos);
+    item.out_tok_spans = reinterpret_cast<int32_t*>(base + a.tok);
+    item.out_char_spans = reinterpret_cast<int32_t*>(base + a.ch);
+    item.out_counts = reinterpret_cast<int64_t*>(base + a.counts);
+    st = spf_pool_select_compact(&item, 1, params->pool_kernel, params->chunk, 0, 0, 0, stream);
     if (st != SPF_OK) return st;
     SPF_CUDA_CHECK(cudaMemcpyAsync(counts, base + a.counts, 16, cudaMemcpyDeviceToHost, stream));
     SPF_CUDA_CHECK(cudaMemcpyAsync(&device_status, dev_status, 4, cudaMemcpyDeviceToHost, stream));

@@ -211,6 +211,11 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   b->char_end = ce.data_ptr<int32_t>();
 }
 
+spf_path_item path_item(const Buffers& b, int64_t n) {
+  return spf_path_item{b.importance_ptr, n, b.scores_ptr, b.k, b.ids, b.char_start, b.char_end, b.kept, b.out_ids, b.out_pos, b.tok_spans, b.char_spans,
+                       b.counts};
+}
+
 // The selector's workspace, grown where it is too small.
 at::Tensor workspace_of(PyObject* selector, size_t need, const at::Tensor& like) {
   Ref now = attr(selector, N.workspace);
@@ -283,22 +288,9 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
          : kind == kPaged ? spf_score_paged(&shape, &paged, 1, ws_ptr, ws_bytes, status, stream)
                           : spf_score_fp8(&shape, &fp8, 1, ws_ptr, ws_bytes, status, stream);
     if (st == SPF_OK) {
-      where = edge != 0 ? "spf_chunk_pool_edge" : "spf_chunk_pool";
-      st = edge != 0 ? spf_chunk_pool_edge(b.importance_ptr, in.n, pool, chunk, edge, b.scores_ptr, stream)
-                     : spf_chunk_pool(b.importance_ptr, in.n, pool, chunk, b.scores_ptr, stream);
-    }
-    if (st == SPF_OK && (force_first || force_last)) {
-      where = "spf_select_topk_forced";
-      st = spf_select_topk_forced(b.scores_ptr, b.n_chunks, b.k, force_first, force_last, b.kept, stream);
-      if (st == SPF_OK) {
-        where = "spf_compact_spans";
-        st = spf_compact_spans(b.kept, b.k, chunk, in.n, b.ids, b.char_start, b.char_end, b.out_ids, b.out_pos, b.tok_spans, b.char_spans,
-                               b.counts, stream);
-      }
-    } else if (st == SPF_OK) {
-      where = "spf_select_compact";                            // top-k and compaction chained in one launch
-      st = spf_select_compact(b.scores_ptr, b.n_chunks, b.k, chunk, in.n, b.ids, b.char_start, b.char_end, b.kept, b.out_ids, b.out_pos,
-                              b.tok_spans, b.char_spans, b.counts, stream);
+      where = "spf_pool_select_compact";
+      const spf_path_item item = path_item(b, in.n);
+      st = spf_pool_select_compact(&item, 1, pool, chunk, edge, force_first, force_last, stream);
     }
     Py_END_ALLOW_THREADS;
     return result_tuple(st, where, &b, 1);
@@ -329,9 +321,7 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     std::vector<Inputs> in(count);
     std::vector<Buffers> b(count);
     std::vector<spf_prompt> p(count);
-    std::vector<spf_pool_item> pools(count);
-    std::vector<spf_topk_item> topk(count);
-    std::vector<spf_compact_item> compact(count);
+    std::vector<spf_path_item> items(count);
     for (size_t i = 0; i < count; ++i) {
       PyObject* prompt = PySequence_Fast_GET_ITEM(prompts.p, (Py_ssize_t)i);
       Ref q(attr(prompt, N.q)), k(attr(prompt, N.k));
@@ -341,10 +331,7 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
       Ref ids(attr(prompt, N.token_ids)), cs(attr(prompt, N.char_start)), ce(attr(prompt, N.char_end));
       read_buffers(PySequence_Fast_GET_ITEM(slot_items.p, (Py_ssize_t)i), shape, n, chunk, keep, false, false, ids.p, cs.p, ce.p, &b[i]);
       p[i] = spf_prompt{n, in[i].layers.data(), in[i].stride_head, in[i].stride_tok, in[i].q, b[i].importance_ptr, b[i].lse_ptr};
-      pools[i] = spf_pool_item{b[i].importance_ptr, n, b[i].scores_ptr};
-      topk[i] = spf_topk_item{b[i].scores_ptr, b[i].n_chunks, b[i].k, b[i].kept};
-      compact[i] = spf_compact_item{b[i].kept, b[i].k, n, b[i].ids, b[i].char_start, b[i].char_end, b[i].out_ids, b[i].out_pos, b[i].tok_spans,
-                                    b[i].char_spans, b[i].counts};
+      items[i] = path_item(b[i], n);
     }
     int32_t* status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status").data_ptr<int32_t>();
     void* stream = stream_of(args[3], b[0].importance);
@@ -359,16 +346,8 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     where = "spf_score";
     st = spf_score(&shape, p.data(), (int32_t)count, ws_ptr, ws_bytes, status, stream);
     if (st == SPF_OK) {
-      where = "spf_chunk_pool_batch";
-      st = spf_chunk_pool_batch(pools.data(), (int32_t)count, pool, chunk, stream);
-    }
-    if (st == SPF_OK) {
-      where = "spf_select_topk_batch";
-      st = spf_select_topk_batch(topk.data(), (int32_t)count, stream);
-    }
-    if (st == SPF_OK) {
-      where = "spf_compact_spans_batch";
-      st = spf_compact_spans_batch(compact.data(), (int32_t)count, chunk, stream);
+      where = "spf_pool_select_compact";
+      st = spf_pool_select_compact(items.data(), (int32_t)count, pool, chunk, 0, 0, 0, stream);
     }
     Py_END_ALLOW_THREADS;
     return result_tuple(st, where, b.data(), count);

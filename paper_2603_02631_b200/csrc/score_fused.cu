@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
   __shared__ float red[kPrepThreads / 32];
   __shared__ float s_scale;
 
+  grid_launch_dependents();                                         // the scoring kernel sets itself up meanwhile
   for (int i = 0; i < 2; ++i)
     for (int64_t w = (int64_t)slab * kPrepThreads + threadIdx.x; w < p.clear_words[i]; w += (int64_t)n_slabs * kPrepThreads)
       p.clear[i][w] = make_uint4(0, 0, 0, 0);

@@ -3,41 +3,82 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace spf {
 namespace {
 
 // ------------------------------------------------------------------------------------------------
-// spf_chunk_pool: one warp per chunk.  Each lane sums the w-wide windows of its tokens, the warp adds
-// them up in a fixed order, so the result does not depend on scheduling.
+// Pooling: one warp per chunk, BATCH chunks of a warp at a time.  The mean over a chunk of the w-wide window sums is a sum
+// over the tokens in reach, each times the number of the chunk's windows that it lies in, so a chunk of 32 with w = 13 reads
+// 44 values once instead of 13 values for each of 32 tokens: bound by the latency of those loads, hence several chunks at a
+// time.  A warp adds up in a fixed order, so the result does not depend on scheduling.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPoolWarps = 8;
 
-__device__ __forceinline__ void chunk_pool_body(const float* __restrict__ importance, int64_t n_tokens, int half, float inv_w,
-                                                int chunk, bool in_range_divisor, float* __restrict__ chunk_scores,
-                                                int64_t n_chunks) {
-  const int lane = threadIdx.x & 31;
-  const int64_t j = (int64_t)blockIdx.x * kPoolWarps + (threadIdx.x >> 5);
-  if (j >= n_chunks) return;
-  const int64_t lo = j * chunk;
-  const int64_t hi = min(lo + (int64_t)chunk, n_tokens);
-  float sum = 0.f;
-  for (int64_t s = lo + lane; s < hi; s += 32) {
-    const int64_t a = max(s - half, (int64_t)0), b = min(s + half, n_tokens - 1);
-    float win = 0.f;
-    for (int64_t t = a; t <= b; ++t) win += __ldg(importance + t);
-    // the window's divisor: always w (zeros beyond the ends), or the number of tokens it really covers
-    sum += in_range_divisor ? win / (float)(b - a + 1) : win * inv_w;
-  }
+struct PoolRule {
+  int half, chunk;
+  float inv_w;
+  bool in_range_divisor;      // the window's divisor: always w (zeros beyond the ends), or the number of tokens it covers
+};
+
+__device__ __forceinline__ float warp_total(float x) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-  if (lane == 0) chunk_scores[j] = sum / (float)(hi - lo);
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
 }
 
-__global__ void __launch_bounds__(kPoolWarps * 32) chunk_pool_kernel(const float* __restrict__ importance, int64_t n_tokens,
-                                                                      int half, float inv_w, int chunk, bool in_range_divisor,
+// Scores of chunks j, j + step, ... (those below n_chunks), in every lane.
+template <int BATCH>
+__device__ __forceinline__ void pool_chunks(const float* __restrict__ importance, int64_t n_tokens, const PoolRule& r, int64_t j, int64_t step,
+                                            int64_t n_chunks, float (&score)[BATCH]) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo[BATCH], size[BATCH], most = 0;
+#pragma unroll
+  for (int u = 0; u < BATCH; ++u) {
+    lo[u] = (j + u * step) * r.chunk;
+    size[u] = j + u * step < n_chunks ? min((int64_t)r.chunk, n_tokens - lo[u]) : 0;
+    most = max(most, size[u]);
+    score[u] = 0.f;
+  }
+  for (int64_t x = lane - r.half; x < most + r.half; x += 32) {        // position relative to the chunk's first token
+#pragma unroll
+    for (int u = 0; u < BATCH; ++u) {
+      const int64_t t = lo[u] + x;
+      if (x < size[u] + r.half && size[u] > 0 && t >= 0 && t < n_tokens)
+        score[u] = fmaf(__ldcg(importance + t), (float)(min(x + r.half, size[u] - 1) - max(x - r.half, (int64_t)0) + 1), score[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < BATCH; ++u) {
+    score[u] = warp_total(score[u]) * r.inv_w;
+    if (r.in_range_divisor && size[u] > 0 && (lo[u] < r.half || lo[u] + size[u] + r.half > n_tokens)) {
+      // windows that reach beyond the prompt's ends have divisors of their own
+      float sum = 0.f;
+      for (int64_t s = lo[u] + lane; s < lo[u] + size[u]; s += 32) {
+        const int64_t a = max(s - r.half, (int64_t)0), b = min(s + r.half, n_tokens - 1);
+        float win = 0.f;
+        for (int64_t t = a; t <= b; ++t) win += __ldcg(importance + t);
+        sum += win / (float)(b - a + 1);
+      }
+      score[u] = warp_total(sum);
+    }
+    score[u] /= (float)size[u];
+  }
+}
+
+__device__ __forceinline__ void chunk_pool_body(const float* __restrict__ importance, int64_t n_tokens, const PoolRule& r,
+                                                float* __restrict__ chunk_scores, int64_t n_chunks) {
+  const int64_t j = (int64_t)blockIdx.x * kPoolWarps + (threadIdx.x >> 5);
+  if (j >= n_chunks) return;
+  float score[1];
+  pool_chunks<1>(importance, n_tokens, r, j, 0, n_chunks, score);
+  if ((threadIdx.x & 31) == 0) chunk_scores[j] = score[0];
+}
+
+__global__ void __launch_bounds__(kPoolWarps * 32) chunk_pool_kernel(const float* __restrict__ importance, int64_t n_tokens, PoolRule r,
                                                                       float* __restrict__ chunk_scores, int64_t n_chunks) {
-  chunk_pool_body(importance, n_tokens, half, inv_w, chunk, in_range_divisor, chunk_scores, n_chunks);
+  chunk_pool_body(importance, n_tokens, r, chunk_scores, n_chunks);
 }
 
 // Batched calls: up to kBatchItems prompts per launch, their descriptors passed by value; blockIdx.y picks the prompt.
@@ -52,10 +93,9 @@ struct CompactBatch {
   spf_compact_item item[kBatchItems];
 };
 
-__global__ void __launch_bounds__(kPoolWarps * 32) chunk_pool_batch_kernel(const __grid_constant__ PoolBatch b, int half, float inv_w,
-                                                                            int chunk) {
+__global__ void __launch_bounds__(kPoolWarps * 32) chunk_pool_batch_kernel(const __grid_constant__ PoolBatch b, PoolRule r) {
   const spf_pool_item& it = b.item[blockIdx.y];
-  chunk_pool_body(it.importance, it.n_tokens, half, inv_w, chunk, false, it.chunk_scores, (it.n_tokens + chunk - 1) / chunk);
+  chunk_pool_body(it.importance, it.n_tokens, r, it.chunk_scores, (it.n_tokens + r.chunk - 1) / r.chunk);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -309,71 +349,258 @@ __global__ void __launch_bounds__(kCompactThreads) compact_spans_kernel(
 }
 
 // ------------------------------------------------------------------------------------------------
-// spf_select_compact: top-k and compaction of one prompt in ONE CTA (the two steps are latency-bound and the second
-// only needs the first's k indices, so a second launch costs more than the work).  After the selection the same
-// 1024 threads find the runs of consecutive kept chunks (a prefix count of run starts, as compact_spans_kernel's
-// block 0 does) and copy ids and positions, one warp per kept chunk.
+// spf_pool_select_compact, spf_select_compact: the whole path behind the scores in one launch, a cluster of CTAs per prompt.
+//
+// Nothing here is much work; what costs is the chain of dependent steps, so there are as few as possible between one load
+// and the next.  Each CTA pools its share of the chunks and stores the scores' keys into every CTA's shared memory; after
+// the cluster's barrier (the only one) every CTA makes the same selection by itself and writes its own share of the results.
+//   selection: the keys' range is cut into 2048 equal bins (about 300 to 1000 of them hold something, whatever the scores'
+//     distribution), one histogram finds the k-th key's bin, and its few entries are ranked against each other; only a bin
+//     of more than kRankMost entries is cut again.  Ties go to the lower index.
+//   compaction: the selection is a bitmap, one word per warp and step by ballot.  Kept chunks and starts of runs are counted
+//     by population counts, in one scan over the words, instead of a scan per 1024 chunks.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTopkThreads) select_compact_kernel(
-    const float* __restrict__ scores, int n, int k, int chunk, int64_t n_tokens, const int32_t* __restrict__ token_ids,
-    const int32_t* __restrict__ char_start, const int32_t* __restrict__ char_end, int32_t* __restrict__ kept,
-    int32_t* __restrict__ out_ids, int32_t* __restrict__ out_pos, int32_t* __restrict__ out_tok_spans,
-    int32_t* __restrict__ out_char_spans, int64_t* __restrict__ out_counts) {
-  select_topk_body(scores, n, k, 0, kept);
-  __threadfence_block();
-  __syncthreads();                                          // kept[0..k) is complete and visible to the whole CTA
-  __shared__ int warp_counts[kTopkThreads / 32];
+constexpr int kTailThreads = 1024;
+constexpr int kTailChunks = 32768;     // keys of this many chunks fit shared memory (128 KB)
+constexpr int kTailBins = 2 * kTailThreads;
+constexpr int kRankMost = 512;
+constexpr int kTailItems = 24;         // prompts per launch: their descriptors are kernel arguments
+
+struct TailBatch {
+  spf_path_item item[kTailItems];
+  PoolRule rule;
+  int force;                           // bit 0: the first chunk is kept whatever its score, bit 1: the last
+};
+
+struct TailShared {
+  int hist[kTailBins];
+  uint32_t cand_key[kRankMost];
+  int cand_at[kRankMost];
+  uint32_t bits[kTailChunks / 32 + 2];    // kept chunks; a zero word on either side
+  uint32_t before[kTailChunks / 32];      // kept chunks (high half) and starts of runs (low half) ahead of a word
+  uint32_t warp_lo[32], warp_hi[32];
+  int found_bin, found_left, found_count, n_cand;
+  uint32_t last_key;                      // kept: keys above last_key, and those equal to it up to index last_at
+  int last_at;
+};
+
+// Exclusive prefix sum over the CTA in thread order; *all: the sum of every thread's x.  `scratch` is free again once all
+// threads have passed the caller's next barrier.
+__device__ __forceinline__ uint32_t block_exclusive(uint32_t x, uint32_t* scratch, uint32_t* all) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t* kv = kept;                                 // written by other threads of this CTA a moment ago: read past L1
-  int span_base = 0;
-  for (int r0 = 0; r0 < k; r0 += kTopkThreads) {
-    const int r = r0 + threadIdx.x;
-    int64_t j = -1;
-    bool starts = false, ends = false;
-    if (r < k) {
-      j = __ldcg(kv + r);
-      starts = r == 0 || __ldcg(kv + r - 1) + 1 != j;
-      ends = r == k - 1 || __ldcg(kv + r + 1) != j + 1;
-    }
-    const unsigned ballot = __ballot_sync(0xffffffffu, starts);
-    const int within = __popc(ballot & ((2u << lane) - 1u));  // inclusive
-    __syncthreads();
-    if (lane == 0) warp_counts[warp] = __popc(ballot);
-    __syncthreads();
-    int before = 0, all = 0;
-    for (int w = 0; w < kTopkThreads / 32; ++w) {
-      before += w < warp ? warp_counts[w] : 0;
-      all += warp_counts[w];
-    }
-    const int span = span_base + before + within - 1;      // index of the run this chunk belongs to
-    if (r < k) {
-      if (starts) {
-        const int64_t a = j * chunk;
-        out_tok_spans[2 * span] = (int32_t)a;
-        out_char_spans[2 * span] = char_start[a];
-      }
-      if (ends) {
-        const int64_t b = min((j + 1) * chunk, n_tokens);
-        out_tok_spans[2 * span + 1] = (int32_t)b;
-        out_char_spans[2 * span + 1] = char_end[b - 1];
-      }
-    }
-    span_base += all;
+  uint32_t incl = x;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
   }
-  const int64_t last = __ldcg(kv + k - 1);
-  const int64_t n_kept = (int64_t)(k - 1) * chunk + (min((last + 1) * chunk, n_tokens) - last * chunk);
-  if (threadIdx.x == 0) {
-    out_counts[0] = n_kept;
-    out_counts[1] = span_base;
+  if (lane == 31) scratch[warp] = incl;
+  __syncthreads();
+  const uint32_t w = scratch[lane];                        // every warp scans the 32 warp totals by itself
+  *all = __reduce_add_sync(0xffffffffu, w);
+  return incl - x + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+}
+
+// Finds the `left`-th largest of the n keys that are not forced: its key and index go to sh.last_key, sh.last_at.
+__device__ __forceinline__ void select_last(TailShared& sh, const uint32_t* keys, int n, int left, int force) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int first = force & 1, end = n - ((force >> 1) & 1);
+  uint32_t lo = 0xFFFFFFFFu, hi = 0;
+  for (int j = first + tid; j < end; j += kTailThreads) {
+    lo = min(lo, keys[j]);
+    hi = max(hi, keys[j]);
   }
-  // kept chunk r (ascending) starts at output offset r * chunk: only the prompt's last chunk can be short.  The
-  // output is walked as one flat array so that every thread has several independent loads in flight
-#pragma unroll 4
-  for (int64_t o = threadIdx.x; o < n_kept; o += kTopkThreads) {
-    const int64_t r = o / chunk;
-    const int64_t t = (int64_t)__ldcg(kv + r) * chunk + (o - r * chunk);
-    out_ids[o] = __ldg(token_ids + t);
-    if (out_pos != nullptr) out_pos[o] = (int32_t)t;
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    sh.warp_lo[warp] = lo;
+    sh.warp_hi[warp] = hi;
+  }
+  __syncthreads();
+  lo = __reduce_min_sync(0xffffffffu, sh.warp_lo[lane]);
+  hi = __reduce_max_sync(0xffffffffu, sh.warp_hi[lane]);
+  while (true) {
+    // bins of 2^shift keys, from `lo` on; the histogram is zero here
+    const int shift = max(0, 21 - __clz(hi - lo));
+    for (int j = first + tid; j < end; j += kTailThreads)
+      if (keys[j] >= lo && keys[j] <= hi) atomicAdd(&sh.hist[(keys[j] - lo) >> shift], 1);
+    __syncthreads();
+    const int top = kTailBins - 1 - 2 * tid;               // each thread owns two bins, the first thread the highest
+    const int h1 = sh.hist[top], h0 = sh.hist[top - 1];
+    sh.hist[top] = sh.hist[top - 1] = 0;
+    uint32_t all;
+    const int above = (int)block_exclusive((uint32_t)(h0 + h1), sh.warp_lo, &all);
+    if (above < left && above + h0 + h1 >= left) {
+      const bool upper = above + h1 >= left;
+      sh.found_bin = upper ? top : top - 1;
+      sh.found_left = upper ? left - above : left - above - h1;
+      sh.found_count = upper ? h1 : h0;
+      sh.n_cand = 0;
+    }
+    __syncthreads();
+    lo += (uint32_t)sh.found_bin << shift;
+    hi = lo + min(hi - lo, (1u << shift) - 1u);
+    left = sh.found_left;
+    const int count = sh.found_count;
+    if (count <= kRankMost) {
+      for (int j = first + tid; j < end; j += kTailThreads)
+        if (keys[j] >= lo && keys[j] <= hi) {
+          const int at = atomicAdd(&sh.n_cand, 1);
+          sh.cand_key[at] = keys[j];
+          sh.cand_at[at] = j;
+        }
+      __syncthreads();
+      for (int c = warp; c < count; c += kTailThreads / 32) {
+        const uint32_t key = sh.cand_key[c];
+        const int at = sh.cand_at[c];
+        uint32_t better = 0;
+        for (int o = lane; o < count; o += 32) better += sh.cand_key[o] > key || (sh.cand_key[o] == key && sh.cand_at[o] < at);
+        better = __reduce_add_sync(0xffffffffu, better);
+        if (lane == 0 && (int)better == left - 1) {
+          sh.last_key = key;
+          sh.last_at = at;
+        }
+      }
+      __syncthreads();
+      return;
+    }
+    if (shift == 0) {                                      // that many equal keys: the left-th of them by index
+      const int words = (n + 31) / 32;
+      for (int w = warp; w < words; w += kTailThreads / 32) {
+        const int j = w * 32 + lane;
+        const uint32_t same = __ballot_sync(0xffffffffu, j >= first && j < end && keys[min(j, n - 1)] == lo);
+        if (lane == 0) sh.bits[1 + w] = same;
+      }
+      __syncthreads();
+      const uint32_t mine = tid < words ? sh.bits[1 + tid] : 0u;
+      const int ahead = (int)block_exclusive(__popc(mine), sh.warp_hi, &all);
+      if (ahead < left && ahead + __popc(mine) >= left) {
+        uint32_t rest = mine;
+        for (int i = ahead + 1; i < left; ++i) rest &= rest - 1u;
+        sh.last_key = lo;
+        sh.last_at = tid * 32 + __ffs(rest) - 1;
+      }
+      __syncthreads();
+      return;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kTailThreads) pool_select_compact_kernel(const __grid_constant__ TailBatch b) {
+  extern __shared__ uint32_t keys[];                       // the chunks' keys, then the kept chunks' indices
+  __shared__ TailShared sh;
+  const spf_path_item& it = b.item[blockIdx.y];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = blockIdx.x, ctas = gridDim.x;           // the grid's x extent is one cluster
+  const int64_t n_tokens = it.n_tokens;
+  const int chunk = b.rule.chunk, n = (int)((n_tokens + chunk - 1) / chunk), k = (int)it.k;
+
+  sh.hist[tid] = sh.hist[tid + kTailThreads] = 0;
+  cluster_arrive();
+  grid_wait();                                             // the scores are complete from here on
+  cluster_wait();                                          // every CTA has started: its shared memory may be written
+  if (it.importance != nullptr) {
+    constexpr int kBatch = 4;
+    for (int j = rank * 32 + warp; j < n; j += ctas * 32 * kBatch) {
+      float score[kBatch];
+      pool_chunks<kBatch>(it.importance, n_tokens, b.rule, j, ctas * 32, n, score);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int ju = j + u * ctas * 32;
+        if (ju < n) {
+          if (lane < ctas) store_cluster(smem_u32(keys + ju), lane, order_key(score[u]));
+          if (lane == 0) it.chunk_scores[ju] = score[u];
+        }
+      }
+    }
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    for (int j = tid; j < n; j += kTailThreads) keys[j] = order_key(__ldcg(it.chunk_scores + j));
+    __syncthreads();
+  }
+
+  const int first = b.force & 1, end = n - ((b.force >> 1) & 1);
+  const int left = k - first - (end < n && end >= first ? 1 : 0);
+  if (left > 0) {
+    select_last(sh, keys, n, left, b.force);
+  } else {
+    if (tid == 0) {
+      sh.last_key = 0xFFFFFFFFu;
+      sh.last_at = -1;
+    }
+    __syncthreads();
+  }
+  const uint32_t last_key = sh.last_key;
+  const int last_at = sh.last_at, words = (n + 31) / 32;
+  for (int w = warp; w < words; w += kTailThreads / 32) {
+    const int j = w * 32 + lane;
+    const uint32_t key = keys[min(j, n - 1)];
+    const bool kept = j < n && (j < first || j >= end || key > last_key || (key == last_key && j <= last_at));
+    const uint32_t ballot = __ballot_sync(0xffffffffu, kept);
+    if (lane == 0) sh.bits[1 + w] = ballot;
+  }
+  if (tid == 0) sh.bits[0] = sh.bits[1 + words] = 0u;
+  __syncthreads();
+  uint32_t total = 0;
+  {
+    const uint32_t mine = tid < words ? sh.bits[1 + tid] : 0u;
+    const uint32_t starts = tid < words ? mine & ~((mine << 1) | (sh.bits[tid] >> 31)) : 0u;
+    const uint32_t ahead = block_exclusive((uint32_t)__popc(mine) << 16 | (uint32_t)__popc(starts), sh.warp_lo, &total);
+    if (tid < words) sh.before[tid] = ahead;
+  }
+  __syncthreads();
+  // every CTA lists the kept chunks for itself; indices and spans are written by one of them, word by word
+  for (int w = warp; w < words; w += kTailThreads / 32) {
+    const uint32_t mine = sh.bits[1 + w], prev = sh.bits[w], next = sh.bits[2 + w], ahead = sh.before[w];
+    if (!(mine >> lane & 1u)) continue;
+    const int j = w * 32 + lane;
+    const uint32_t upto = (2u << lane) - 1u;               // this chunk and those ahead of it in the word
+    const uint32_t starts = mine & ~((mine << 1) | (prev >> 31));
+    const int r = (int)(ahead >> 16) + __popc(mine & upto) - 1, span = (int)(ahead & 0xFFFFu) + __popc(starts & upto) - 1;
+    keys[r] = (uint32_t)j;
+    if (w % ctas != rank) continue;
+    it.kept_chunks[r] = j;
+    if (starts >> lane & 1u) {
+      const int64_t a = (int64_t)j * chunk;
+      it.out_tok_spans[2 * span] = (int32_t)a;
+      it.out_char_spans[2 * span] = __ldg(it.char_start + a);
+    }
+    if (!((lane < 31 ? mine >> (lane + 1) : next) & 1u)) {
+      const int64_t e = min((int64_t)(j + 1) * chunk, n_tokens);
+      it.out_tok_spans[2 * span + 1] = (int32_t)e;
+      it.out_char_spans[2 * span + 1] = __ldg(it.char_end + e - 1);
+    }
+  }
+  __syncthreads();
+  if (rank == 0 && tid == 0) {
+    const int64_t last = (int64_t)keys[k - 1] * chunk;
+    it.out_counts[0] = (int64_t)(k - 1) * chunk + min((int64_t)chunk, n_tokens - last);
+    it.out_counts[1] = (int64_t)(total & 0xFFFFu);
+  }
+  // Kept chunk r starts at output r * chunk: only the prompt's last chunk can be short, and it is the last one kept.  A warp
+  // copies whole chunks, several at a time.
+  constexpr int kRows = 4;
+  for (int r0 = rank * 32 + warp; r0 < k; r0 += ctas * 32 * kRows) {
+    int64_t from[kRows], size[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      const int r = r0 + u * ctas * 32;
+      from[u] = r < k ? (int64_t)keys[r] * chunk : 0;
+      size[u] = r < k ? min((int64_t)chunk, n_tokens - from[u]) : 0;
+    }
+    for (int64_t s = lane; s < chunk; s += 32) {
+      int32_t id[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) id[u] = s < size[u] ? __ldg(it.token_ids + from[u] + s) : 0;
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        if (s < size[u]) {
+          const int64_t o = (int64_t)(r0 + u * ctas * 32) * chunk + s;
+          it.out_ids[o] = id[u];
+          if (it.out_pos != nullptr) it.out_pos[o] = (int32_t)(from[u] + s);
+        }
+    }
   }
 }
 
@@ -401,7 +628,7 @@ static int32_t chunk_pool_launch(const float* importance, int64_t n_tokens, int3
   const int64_t blocks = ceil_div(n_chunks, kPoolWarps);
   if (blocks > 0x7fffffff) return fail(SPF_ERR_UNSUPPORTED, "spf_chunk_pool: too many chunks");
   chunk_pool_kernel<<<(unsigned)blocks, kPoolWarps * 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      importance, n_tokens, pool_kernel / 2, 1.0f / (float)pool_kernel, chunk, in_range_divisor, chunk_scores, n_chunks);
+      importance, n_tokens, PoolRule{pool_kernel / 2, chunk, 1.0f / (float)pool_kernel, in_range_divisor}, chunk_scores, n_chunks);
   SPF_CUDA_CHECK(cudaGetLastError());
   return SPF_OK;
 }
@@ -495,7 +722,7 @@ extern "C" int32_t spf_chunk_pool_batch(const spf_pool_item* items, int32_t n_it
       blocks = std::max(blocks, ceil_div(ceil_div(items[i0 + i].n_tokens, chunk), kPoolWarps));
     }
     chunk_pool_batch_kernel<<<dim3((unsigned)blocks, (unsigned)cnt), kPoolWarps * 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        b, pool_kernel / 2, 1.0f / (float)pool_kernel, chunk);
+        b, PoolRule{pool_kernel / 2, chunk, 1.0f / (float)pool_kernel, false});
     SPF_CUDA_CHECK(cudaGetLastError());
   }
   return SPF_OK;
@@ -549,6 +776,95 @@ extern "C" int32_t spf_compact_spans_batch(const spf_compact_item* items, int32_
   return SPF_OK;
 }
 
+// ------------------------------------------------------------------------------------------------ the path in one launch
+namespace {
+
+// CTAs per prompt: pooling and copying shrink with their number, while a larger cluster takes longer to start and to meet.
+int tail_ctas(int64_t n_tokens) { return n_tokens <= 2048 ? 1 : n_tokens <= 4096 ? 2 : n_tokens <= 8192 ? 4 : 8; }
+
+int32_t tail_launch(const spf_path_item* items, int n, const PoolRule& rule, int force, cudaStream_t stream) {
+  for (int i0 = 0; i0 < n; i0 += kTailItems) {
+    const int cnt = std::min(kTailItems, n - i0);
+    TailBatch b{};
+    b.rule = rule;
+    b.force = force;
+    int64_t longest = 1, chunks = 1;
+    for (int i = 0; i < cnt; ++i) {
+      b.item[i] = items[i0 + i];
+      longest = std::max(longest, items[i0 + i].n_tokens);
+      chunks = std::max(chunks, ceil_div(items[i0 + i].n_tokens, rule.chunk));
+    }
+    const int ctas = tail_ctas(longest);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas, (unsigned)cnt);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = (size_t)chunks * sizeof(uint32_t);
+    cfg.stream = stream;
+    // beyond 48 KB with the static part (about 21 KB), shared memory has to be asked for
+    if (cfg.dynamicSmemBytes > 24 * 1024)
+      SPF_CUDA_CHECK(cudaFuncSetAttribute(pool_select_compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          kTailChunks * (int)sizeof(uint32_t)));
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {(unsigned)ctas, 1, 1};
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    SPF_CUDA_CHECK(cudaLaunchKernelEx(&cfg, pool_select_compact_kernel, b));
+  }
+  return SPF_OK;
+}
+
+}  // namespace
+
+extern "C" int32_t spf_pool_select_compact(const spf_path_item* items, int32_t n_items, int32_t pool_kernel, int32_t chunk, int32_t edge_rule,
+                                           int32_t force_first, int32_t force_last, void* cuda_stream) {
+  clear_error();
+  if (items == nullptr || n_items < 1) return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: null items or n_items < 1");
+  if (pool_kernel < 1 || pool_kernel > 255 || pool_kernel % 2 == 0)
+    return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: pool_kernel must be odd and in [1, 255] (got %d)", pool_kernel);
+  if (edge_rule != 0 && edge_rule != 1)
+    return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: edge_rule must be 0 or 1 (got %d)", edge_rule);
+  if (chunk < 1) return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: chunk must be >= 1 (got %d)", chunk);
+  const int force = (force_first ? 1 : 0) | (force_last ? 2 : 0);
+  for (int32_t i = 0; i < n_items; ++i) {
+    const spf_path_item& it = items[i];
+    if (it.importance == nullptr || it.chunk_scores == nullptr || it.kept_chunks == nullptr || it.token_ids == nullptr ||
+        it.char_start == nullptr || it.char_end == nullptr || it.out_ids == nullptr || it.out_tok_spans == nullptr ||
+        it.out_char_spans == nullptr || it.out_counts == nullptr)
+      return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: item %d: null pointer", i);
+    if (it.n_tokens < 1 || it.n_tokens > 0x7fffffff)
+      return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: item %d: n_tokens must be in [1, 2^31)", i);
+    const int64_t n_chunks = ceil_div(it.n_tokens, chunk);
+    const int n_forced = (force & 1) + ((force & 2) && (n_chunks > 1 || !(force & 1)) ? 1 : 0);
+    if (it.k < 1 || it.k > n_chunks || it.k < n_forced)
+      return fail(SPF_ERR_INVALID_ARG, "spf_pool_select_compact: item %d: k must be in [1, n_chunks] and cover the forced chunks", i);
+  }
+  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  const PoolRule rule{pool_kernel / 2, chunk, 1.0f / (float)pool_kernel, edge_rule == 1};
+  for (int32_t i = 0; i < n_items;) {
+    int32_t j = i;
+    while (j < n_items && ceil_div(items[j].n_tokens, chunk) <= kTailChunks) ++j;
+    if (j > i) {
+      const int32_t st = tail_launch(items + i, j - i, rule, force, stream);
+      if (st != SPF_OK) return st;
+      i = j;
+      continue;
+    }
+    // too many chunks for one SM's shared memory: the three steps one by one
+    const spf_path_item& it = items[i++];
+    int32_t st = spf_chunk_pool_edge(it.importance, it.n_tokens, pool_kernel, chunk, edge_rule, it.chunk_scores, cuda_stream);
+    if (st == SPF_OK)
+      st = spf_select_topk_forced(it.chunk_scores, ceil_div(it.n_tokens, chunk), it.k, force_first, force_last, it.kept_chunks, cuda_stream);
+    if (st == SPF_OK)
+      st = spf_compact_spans(it.kept_chunks, it.k, chunk, it.n_tokens, it.token_ids, it.char_start, it.char_end, it.out_ids, it.out_pos,
+                             it.out_tok_spans, it.out_char_spans, it.out_counts, cuda_stream);
+    if (st != SPF_OK) return st;
+  }
+  return SPF_OK;
+}
+
 extern "C" int32_t spf_select_compact(const float* chunk_scores, int64_t n_chunks, int64_t k, int32_t chunk, int64_t n_tokens,
                                       const int32_t* token_ids, const int32_t* char_start, const int32_t* char_end,
                                       int32_t* kept_chunks, int32_t* out_ids, int32_t* out_pos, int32_t* out_tok_spans,
@@ -566,9 +882,24 @@ extern "C" int32_t spf_select_compact(const float* chunk_scores, int64_t n_chunk
   if (k < 1 || k > n_chunks)
     return fail(SPF_ERR_INVALID_ARG, "spf_select_compact: k must be in [1, n_chunks] (got k=%lld, n_chunks=%lld)", (long long)k,
                 (long long)n_chunks);
-  select_compact_kernel<<<1, kTopkThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      chunk_scores, (int)n_chunks, (int)k, chunk, n_tokens, token_ids, char_start, char_end, kept_chunks, out_ids, out_pos,
-      out_tok_spans, out_char_spans, out_counts);
-  SPF_CUDA_CHECK(cudaGetLastError());
-  return SPF_OK;
+  if (n_chunks > kTailChunks) {
+    const int32_t st = spf_select_topk(chunk_scores, n_chunks, k, kept_chunks, cuda_stream);
+    return st != SPF_OK ? st
+                        : spf_compact_spans(kept_chunks, k, chunk, n_tokens, token_ids, char_start, char_end, out_ids, out_pos,
+                                            out_tok_spans, out_char_spans, out_counts, cuda_stream);
+  }
+  spf_path_item it{};
+  it.n_tokens = n_tokens;
+  it.chunk_scores = const_cast<float*>(chunk_scores);   // importance is null: the scores are read
+  it.k = k;
+  it.token_ids = token_ids;
+  it.char_start = char_start;
+  it.char_end = char_end;
+  it.kept_chunks = kept_chunks;
+  it.out_ids = out_ids;
+  it.out_pos = out_pos;
+  it.out_tok_spans = out_tok_spans;
+  it.out_char_spans = out_char_spans;
+  it.out_counts = out_counts;
+  return tail_launch(&it, 1, PoolRule{0, chunk, 1.f, false}, 0, static_cast<cudaStream_t>(cuda_stream));
 }

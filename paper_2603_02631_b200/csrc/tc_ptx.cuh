@@ -39,17 +39,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// A look at the barrier that never waits (try_wait suspends the warp for a while when the phase is not complete).
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Every wait of the kernel is bounded: on expiry it records SPF_ERR_TIMEOUT and raises the CTA's abort flag, after which
 // every other wait of the CTA gives up too.
 struct Abort {
@@ -144,6 +133,14 @@ __device__ __forceinline__ uint64_t l2_policy_drop() {
 // and let the next one start its prologue.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// The cluster's barrier, and a store into the shared memory of one of its CTAs (visible there after the barrier).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void store_cluster(uint32_t addr, int rank, uint32_t value) {
+  asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, %1;\nst.shared::cluster.u32 [r], %2;\n}" ::"r"(addr), "r"(rank), "r"(value)
+               : "memory");
+}
 
 // Moves registers between the warpgroups of a CTA (all four warps of one execute it).
 template <int N>
