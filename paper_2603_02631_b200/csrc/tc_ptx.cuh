@@ -134,13 +134,9 @@ __device__ __forceinline__ uint64_t l2_policy_drop() {
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// The cluster's barrier, and a store into the shared memory of one of its CTAs (visible there after the barrier).
+// The cluster's barrier (orders memory accesses, to shared and to global memory, across its CTAs).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void store_cluster(uint32_t addr, int rank, uint32_t value) {
-  asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, %1;\nst.shared::cluster.u32 [r], %2;\n}" ::"r"(addr), "r"(rank), "r"(value)
-               : "memory");
-}
 
 // Moves registers between the warpgroups of a CTA (all four warps of one execute it).
 template <int N>
