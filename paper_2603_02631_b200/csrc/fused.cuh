@@ -10,7 +10,7 @@
 //   Resident (template ONCE): the logits wait in tensor memory.  A tile's 128 x NCOLS accumulators are summed by the sum
 //   warps and stay where they are until the slab's log-sum-exps arrive; then the max warps fold them and free the columns.
 //   Keys are copied and multiplied once.  This needs room for a CTA's tiles of one slab plus those that arrive during the
-//   hand-over: up to 32 query rows, and prompts of up to a few hundred thousand tokens (see resident_tiles).
+//   hand-over: up to 32 query rows, and prompts of up to a few hundred thousand tokens (see Geometry::resident).
 //   Two-pass: the logits are recomputed.  The two visits are two independent pipelines (TMA warp -> key ring -> MMA warp ->
 //   tensor-memory ring -> epilogue warps) that share the SM and meet only in the log-sum-exps.  Visit 2 follows visit 1 over
 //   the same list of tiles as soon as a slab's log-sum-exps are there; visit 1 may be at most `lead` tiles ahead of it, so
@@ -75,7 +75,9 @@ __host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return 
 constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
 constexpr int kMaxQStages = 4;         // query tiles in flight per visit (two-pass: 2)
 constexpr int kMaxKeyStages = 16;      // key tiles in flight per visit
-constexpr int kMaxTmemStages = 4;      // two-pass: accumulator stages per visit and set
+// Two-pass: accumulator stages per visit.  64 rows at 131072 tokens have three for each visit; with two for each set of visit 1
+// and one for each of visit 2 (as many in all) a pass took 559 instead of 519 us, with 8-bit keys 581 instead of 530.
+constexpr int kMaxTmemStages = 16;
 constexpr int kMaxResident = 32;       // resident: tiles in tensor memory
 constexpr int kRegTiles = 8, kRegSlots = 8;   // running maxima stay in registers up to this many tiles a CTA and lookahead slots a key
 constexpr int kTmemColsAll = 512;      // the CTA takes all of its SM's tensor memory
@@ -87,7 +89,7 @@ constexpr float kRefMargin = 60.f;     // base-2 units added to the sampled refe
 // swizzle span: 128 bytes of the row (128-byte swizzle), or the whole row where it has only 64 bytes (64-byte swizzle).
 __host__ __device__ constexpr int row_bytes(int d, bool fp8) { return fp8 ? d : 2 * d; }
 __host__ __device__ constexpr int sub_row_bytes(int rowb) { return rowb > 128 ? 128 : rowb; }
-// Query rows of a visit-1 instruction (its M), and its accumulator columns per tile: 32 x 32 or 64 x 64.
+// Query rows of a two-pass visit-1 instruction (its M), and its accumulator columns per tile: 32 x 32 or 64 x 64.
 __host__ __device__ constexpr int sum_rows(int ncols) { return ncols <= 32 ? 32 : 64; }
 
 struct FusedPrompt {
@@ -115,8 +117,7 @@ struct FusedArgs {
   int n_prompts, n_layers, n_kv_heads, group, n_lookahead;
   int table_tiles;             // tiles per CTA for which there is a table (paged key cache), else 0
   int mode;                    // 0: the whole computation; 1: visit 1 alone (row log-sum-exps of these keys); 2: visit 2 alone
-  int k_stages[2], t_stages[2];   // per visit: key tiles; accumulator stages per set (resident: [0] alone, tiles in tensor memory)
-  int max_tiles_per_stage;     // two-pass: tiles per accumulator stage of visit 2 (visit 1: one)
+  int k_stages[2], t_stages[2];   // per visit: key tiles in shared memory, tiles' logits in tensor memory (resident: [0] alone)
   int max_in_regs;             // resident: no CTA has more than kRegTiles tiles
   float c;                     // softmax scale * log2(e)
   int32_t* dev_status;         // optional
@@ -131,16 +132,15 @@ struct FusedBars {
   __device__ uint32_t k_empty(int v, int s) const { return base + 8u * (v * kVisit + kMaxKeyStages + s); }
   __device__ uint32_t q_full(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + s); }
   __device__ uint32_t q_empty(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + kMaxQStages + s); }
-  // two-pass: stage s of a visit's set; resident: stage s (v = set = 0)
-  __device__ uint32_t t_full(int v, int set, int s) const { return base + 8u * (kTmem + (v * 2 + set) * kMaxTmemStages + s); }
-  __device__ uint32_t t_empty(int v, int set, int s) const { return t_full(v, set, s) + 8u * kMaxResident; }
+  __device__ uint32_t t_full(int v, int s) const { return base + 8u * (kTmem + v * kMaxTmemStages + s); }   // resident: v = 0 alone
+  __device__ uint32_t t_empty(int v, int s) const { return t_full(v, s) + 8u * kMaxResident; }
   __device__ uint32_t off_ready(int x) const { return base + 8u * (kShared + x); }
   __device__ uint32_t off_free(int x) const { return base + 8u * (kShared + kOffSlots + x); }
   __device__ uint32_t sums_ready(int x) const { return base + 8u * (kShared + 2 * kOffSlots + x); }
   __device__ uint32_t sums_free(int x) const { return base + 8u * (kShared + 2 * kOffSlots + kSumSlots + x); }
   __device__ uint32_t mma_done(int v) const { return base + 8u * (kShared + 2 * kOffSlots + 2 * kSumSlots + v); }
 };
-static_assert(4 * kMaxTmemStages <= kMaxResident, "the two-pass stages use the same barriers");
+static_assert(2 * kMaxTmemStages <= kMaxResident, "the two-pass stages use the same barriers");
 
 struct FusedSmem {
   uint32_t k_off[2], q_off[2], sums_off, off_off, offc_off, bar_off, misc_off, tile_off, total;
@@ -173,6 +173,9 @@ struct Ring {
       phase ^= 1u;
     }
   }
+  __device__ void advance(int by) {
+    for (stage += by; stage >= n; stage -= n) phase ^= 1u;
+  }
 };
 
 // fp32 <-> unsigned bits whose integer order is the float order (0 is below every float).
@@ -187,7 +190,7 @@ __device__ __forceinline__ float from_order_bits(unsigned u) {
 template <int D, int NCOLS, int G, bool FP8, bool ONCE>
 struct FusedTraits {
   static constexpr int QS = ONCE ? kMaxQStages : 2;                // query tiles in flight per visit
-  static constexpr int SR = sum_rows(NCOLS);                       // two-pass visit 1: query rows per instruction = accumulator columns per tile
+  static constexpr int SR = sum_rows(NCOLS);
   static constexpr int CW = NCOLS < 32 ? NCOLS : 32;               // visit 2: accumulators per tensor-memory load
   static constexpr int NCH = NCOLS / CW;                           // loads per tile: 1 or 2
   static constexpr int NI = NCOLS / G;                             // lookahead slots per key in the running-max columns
@@ -212,10 +215,6 @@ struct FusedShare {
   __device__ int slab(int n) const { return part + n * parts; }
   __device__ int tile(int lt) const { return first + lt * step; }
 };
-
-// Which set of epilogue warps takes local tile lt of the CTA's n-th slab.  The sums take turns from slab to slab too, so
-// that slabs of a single tile are shared out; a tile's maxima always belong to the same warps.
-__device__ __forceinline__ int fused_set(int v, int n, int lt) { return (v == 0 ? lt + n : lt) & 1; }
 
 // ---------------------------------------------------------------------------------------------- TMA producer of one visit
 template <class T, bool ONCE>
@@ -274,64 +273,58 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
 }
 
 // ---------------------------------------------------------------------------------------------- MMA issuer of one visit
-// The whole warp walks the loop (addresses and descriptors stay warp-uniform); one elected lane issues.
-template <class T, int NCOLS, bool FP8, int V>
-__device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedShare& sh, const unsigned char* k_tiles,
+// Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.  The whole warp walks the loop
+// (addresses and descriptors stay warp-uniform); one elected lane issues.
+// ROWS: query rows are the accumulator's lanes (weight-stationary instructions), else the keys.  SETS: a ring of stages for
+// each of the two sets of epilogue warps, the odd tiles' behind the even tiles': a tile's maxima belong to one set, so with an
+// odd number of tiles a set skips two, and in a common ring of two stages it could take the tile before the one that it
+// skipped for its own (a barrier's parity tells one round from the next only).
+template <class T, int NCOLS, bool FP8, bool ROWS, bool SETS>
+__device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedShare& sh, int v, const unsigned char* k_tiles,
                                                const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
-  constexpr uint32_t idesc = V == 0 ? instr_desc(T::SR, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
-  constexpr int kTileCols = V == 0 ? T::SR : NCOLS;
+  constexpr uint32_t idesc = ROWS ? instr_desc(T::SR, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
   const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
   const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
-  const int tps = V == 0 ? 1 : a.max_tiles_per_stage, stages = a.t_stages[V];
-  Ring kr(a.k_stages[V]), qr(T::QS), tr0(stages), tr1(stages);
-  for (int n = 0; n < sh.n_slabs; ++n) {
-    if (!mbar_wait_warp(bars.q_full(V, qr.stage), qr.phase, ab)) return;
+  Ring kr(a.k_stages[v]), qr(T::QS), even(SETS ? (a.t_stages[v] + 1) / 2 : a.t_stages[v]), odd(a.t_stages[v] / 2);
+  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+  for (int n = 0; n < n_slabs; ++n) {
+    if (!mbar_wait_warp(bars.q_full(v, qr.stage), qr.phase, ab)) return;
     const uint64_t qd0 = q_desc0 + (uint64_t)((qr.stage * T::kQBytes) >> 4);
-    int fill0 = 0, fill1 = 0;                                      // tiles in the sets' current stages
-    auto tile = [&](int lt, int set, Ring& tr, int& fill) -> bool {
-      if (fill == 0) {
-        if (!mbar_wait2_warp(bars.k_full(V, kr.stage), kr.phase, bars.t_empty(V, set, tr.stage), tr.phase ^ 1u, ab)) return false;
-      } else {
-        if (!mbar_wait_warp(bars.k_full(V, kr.stage), kr.phase, ab)) return false;
-      }
+    auto tile = [&](Ring& tr, int stage0) -> bool {
+      const int stage = stage0 + tr.stage;
+      if (!mbar_wait2_warp(bars.k_full(v, kr.stage), kr.phase, bars.t_empty(v, stage), tr.phase ^ 1u, ab)) return false;
       tc_fence_after();
-      const uint32_t d_tmem = tmem + (uint32_t)(((set * stages + tr.stage) * tps + fill) * kTileCols);
+      const uint32_t d_tmem = tmem + (uint32_t)(stage * (ROWS ? T::SR : NCOLS));
       const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
-      const bool last = ++fill == tps || lt + 2 >= sh.n_tiles;     // of this stage: it is full, or the set has no tile left
       if (elect_one()) {
-        // 8-bit keys: the two query terms accumulate into the same columns
 #pragma unroll
-        for (int part = 0; part < T::QPARTS; ++part)
+        for (int part = 0; part < T::QPARTS; ++part)               // 8-bit keys: the two query terms accumulate into the same columns
 #pragma unroll
           for (int h = 0; h < T::KSUB; ++h)
 #pragma unroll
             for (int ks = 0; ks < T::KSTEPS; ++ks) {
               const uint64_t kd = kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks;
               const uint64_t qd = qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks;
-              if constexpr (V == 0) tc_mma<FP8, true>(d_tmem, qd, kd, idesc, (uint32_t)((part | h | ks) != 0));
-              else tc_mma<FP8, false>(d_tmem, kd, qd, idesc, (uint32_t)((part | h | ks) != 0));
+              tc_mma<FP8, ROWS>(d_tmem, ROWS ? qd : kd, ROWS ? kd : qd, idesc, (uint32_t)((part | h | ks) != 0));
             }
-        tc_commit(bars.k_empty(V, kr.stage));
-        if (last) tc_commit(bars.t_full(V, set, tr.stage));
+        tc_commit(bars.k_empty(v, kr.stage));
+        tc_commit(bars.t_full(v, stage));
       }
       __syncwarp();
       kr.advance();
-      if (last) {
-        tr.advance();
-        fill = 0;
-      }
+      tr.advance();
       return true;
     };
-    for (int lt = 0; lt < sh.n_tiles; ++lt)
-      if (!(fused_set(V, n, lt) == 0 ? tile(lt, 0, tr0, fill0) : tile(lt, 1, tr1, fill1))) return;
-    if (elect_one()) tc_commit(bars.q_empty(V, qr.stage));         // arrives once the slab's MMAs are done
+    for (int lt = 0; lt < n_tiles; ++lt)
+      if (!(SETS && (lt & 1) ? tile(odd, even.n) : tile(even, 0))) return;
+    if (elect_one()) tc_commit(bars.q_empty(v, qr.stage));
     __syncwarp();
     qr.advance();
   }
   // leave only after everything issued has completed and signalled its barriers
-  if (elect_one()) tc_commit(bars.mma_done(V));
+  if (elect_one()) tc_commit(bars.mma_done(v));
   __syncwarp();
-  mbar_wait_warp(bars.mma_done(V), 0u, ab);
+  mbar_wait_warp(bars.mma_done(v), 0u, ab);
 }
 
 // ---------------------------------------------------------------------------------------------- visit 1: sums
@@ -348,10 +341,12 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
   const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
   const float* const refs = p.refs;
   const float* const slab_c = p.slab_c;
-  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(set * a.t_stages[0] * T::SR);
+  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) ;
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
   const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - (T::SR == 64 ? (quad >> 1) * 64 : quad * 32);
   Ring tr(a.t_stages[0]);
+  tr.advance(set);
+  int lt = set;                                                    // this set's next tile, counted from the slab's first
   float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
   for (int n = 0; n < n_slabs; ++n) {
     const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
@@ -360,12 +355,12 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
       if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
     }
     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-    for (int lt = fused_set(0, n, 0) == set ? 0 : 1; lt < n_tiles; lt += 2) {
-      if (!mbar_wait_warp(bars.t_full(0, set, tr.stage), tr.phase, ab)) return;
+    for (; lt < n_tiles; lt += 2) {
+      if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
       const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * T::SR);
-      const uint32_t empty = bars.t_empty(0, set, tr.stage);
-      tr.advance();
+      const uint32_t empty = bars.t_empty(0, tr.stage);
+      tr.advance(2);
 #pragma unroll
       for (int load = 0; load < NL; ++load) {
         uint32_t r[32];
@@ -397,12 +392,105 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
         }
       }
     }
+    lt -= n_tiles;
     const int slot = n % kSumSlots;
     if (n >= kSumSlots)
       if (!mbar_wait_warp(bars.sums_free(slot), (uint32_t)(n / kSumSlots - 1) & 1u, ab)) return;
     float x, y;
     unpack2(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), x, y);
     sums[((slot * 2 + set) * 4 + quad) * 32 + lane] = x + y;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.sums_ready(slot));
+  }
+}
+
+// The sums of the resident form.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it
+// shares out over the warp at the end of a slab.  (The two-pass form with its 64 rows took 10 to 20 % longer this way, whether
+// a warp had all rows of every other tile or half the rows of each.)
+template <class T, int NCOLS, bool FP8>
+__device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
+                                             const FusedBars& bars, const Abort& ab) {
+  const FusedPrompt& p = *sh.p;
+  const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
+  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+  const float* const refs = p.refs;
+  const float* const slab_c = p.slab_c;
+  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
+  const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
+  const int tail_lanes = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32;   // real keys of this quadrant in the last tile
+  const bool frees = a.mode == 1;                         // no visit 2: nobody else frees the stages
+  Ring tr(a.t_stages[0]);
+  tr.advance(set);
+  int lt = set;                                                    // this set's next tile, counted from the slab's first
+  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
+  for (int n = 0; n < n_slabs; ++n) {
+    const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
+    if (n + 1 < n_slabs) {
+      next_ref = __ldg(refs + sh.slab(n + 1));
+      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
+    }
+    uint64_t acc[NCOLS / 2];
+#pragma unroll
+    for (int j = 0; j < NCOLS / 2; ++j) acc[j] = 0ull;
+    const bool any = lt < n_tiles;
+    for (; lt < n_tiles; lt += 2) {
+      if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
+      tc_fence_after();
+      uint32_t r[NCOLS];
+      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
+      tmem_load_wait();
+      tmem_ready<NCOLS>(r);
+      if (frees) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
+      }
+      tr.advance(2);
+      if (sh.tile(lt) < full_tiles || lane < tail_lanes) {
+#pragma unroll
+        for (int j = 0; j < NCOLS / 2; ++j) {
+          float x, y;
+          unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
+          acc[j] = add2(acc[j], pack2(fast_exp2(x), fast_exp2(y)));
+        }
+      }
+    }
+    lt -= n_tiles;
+    // Sum over the warp's 32 keys: transposing butterfly steps, each of which halves the columns a lane holds, then (16
+    // columns) one plain step.  The publishers add up quadrants and sets.
+    float s[NCOLS];
+    s[0] = 0.f;
+    if (any) {
+#pragma unroll
+      for (int j = 0; j < NCOLS / 2; ++j) unpack2(acc[j], s[2 * j], s[2 * j + 1]);
+      int width = NCOLS;
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) {
+        if (width > 1) {
+          width >>= 1;
+          const bool upper = (lane & off) != 0;
+#pragma unroll
+          for (int j = 0; j < NCOLS / 2; ++j) {
+            if (j < width) {
+              const float send = upper ? s[j] : s[j + width];
+              const float keep = upper ? s[j + width] : s[j];
+              s[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+          }
+        } else {
+          s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
+        }
+      }
+    }
+    const int slot = n % kSumSlots;
+    if (n >= kSumSlots)
+      if (!mbar_wait_warp(bars.sums_free(slot), (uint32_t)(n / kSumSlots - 1) & 1u, ab)) return;
+    float* out = sums + ((slot * 2 + set) * 4 + quad) * 32;
+    if constexpr (NCOLS == 32) {
+      out[lane] = s[0];
+    } else {
+      if ((lane & 1) == 0) out[lane >> 1] = s[0];
+    }
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.sums_ready(slot));
   }
@@ -698,275 +786,62 @@ __device__ __forceinline__ void clear_maxima(uint32_t amax_addr, int set, int n_
     for (int ch = 0; ch < T::NCH; ++ch) tmem_store<T::NIW>(amax_addr + (uint32_t)(lt * T::NI + ch * T::NIW), ninf);
 }
 
-template <class T, int NCOLS, int G, bool FP8>
+// ---------------------------------------------------------------------------------------------- visit 2: maxima of the tiles
+// Begins a slab once its log-sum-exps are there.  A tile's maxima always belong to the same warps (lt mod 2 == set).  REGS: up
+// to kRegTiles tiles, whose maxima stay in registers and leave all of tensor memory to the logits.
+template <class T, int NCOLS, int G, bool FP8, bool ONCE, bool REGS>
 __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, uint32_t amax_tmem,
                                           const float* off, const float* off_c, const FusedBars& bars, const Abort& ab) {
-  constexpr int CW = T::CW, NCH = T::NCH, NIW = T::NIW;
-  const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
-  const int tps = a.max_tiles_per_stage, stages = a.t_stages[1];
-  const uint32_t lane_bits = (uint32_t)(quad * 32) << 16;
-  const uint32_t lane_addr = tmem + lane_bits + (uint32_t)(set * stages * tps * NCOLS);
-  const uint32_t amax_addr = amax_tmem + lane_bits;
-  Ring tr(stages);
-  clear_maxima<T>(amax_addr, set, sh.n_tiles);
-  for (int n = 0; n < sh.n_slabs; ++n) {
-    const int slot = n % kOffSlots;
-    if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
-    const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
-    const float c = FP8 ? off_c[slot] : a.c;
-    const uint64_t cc = pack2(c, c);
-    for (int lt = set; lt < sh.n_tiles;) {
-      if (!mbar_wait_warp(bars.t_full(1, set, tr.stage), tr.phase, ab)) return;
-      tc_fence_after();
-      tmem_store_wait();                                           // the maxima read below may be this warp's last stores
-      const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * tps * NCOLS);
-      const uint32_t empty = bars.t_empty(1, set, tr.stage);
-      tr.advance();
-      uint32_t r[CW], am[NIW];
-      if constexpr (NCOLS == 16) {
-        uint32_t r1[CW], am1[NIW];
-        const bool two = tps > 1 && lt + 2 < sh.n_tiles;
-        tmem_issue<CW>(taddr, r);
-        tmem_issue<NIW>(amax_addr + (uint32_t)(lt * T::NI), am);
-        if (two) {
-          tmem_issue<CW>(taddr + NCOLS, r1);
-          tmem_issue<NIW>(amax_addr + (uint32_t)((lt + 2) * T::NI), am1);
-        }
-        tmem_load_wait();
-        tmem_ready<CW>(r);
-        tmem_ready<NIW>(am);
-        tmem_ready<CW>(r1);
-        tmem_ready<NIW>(am1);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty);
-        fold_maxima<T, G>(r, am, off2, cc);
-        tmem_store<NIW>(amax_addr + (uint32_t)(lt * T::NI), am);
-        if (two) {
-          fold_maxima<T, G>(r1, am1, off2, cc);
-          tmem_store<NIW>(amax_addr + (uint32_t)((lt + 2) * T::NI), am1);
-        }
-        lt += 2 * tps;
-      } else {
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-          const uint32_t am_addr = amax_addr + (uint32_t)(lt * T::NI + ch * NIW);
-          tmem_issue<CW>(taddr + (uint32_t)(ch * CW), r);
-          tmem_issue<NIW>(am_addr, am);
-          tmem_load_wait();
-          tmem_ready<CW>(r);
-          tmem_ready<NIW>(am);
-          if (ch + 1 == NCH) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty);
-          }
-          fold_maxima<T, G>(r, am, off2 + ch * (CW / 4), cc);
-          tmem_store<NIW>(am_addr, am);
-        }
-        lt += 2;
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bars.off_free(slot));
-  }
-  tmem_store_wait();
-  fused_finish<T>(a, sh, warp, lane, amax_tmem);
-}
-
-// ---------------------------------------------------------------------------------------------- resident form
-// Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.
-struct ResidentRing {
-  int stage = 0, n;
-  uint32_t phase = 0;
-  __device__ explicit ResidentRing(int n_) : n(n_) {}
-  __device__ void advance(int by) {                                // by <= n
-    stage += by;
-    if (stage >= n) {
-      stage -= n;
-      phase ^= 1u;
-    }
-  }
-};
-
-template <class T, int NCOLS, bool FP8>
-__device__ __forceinline__ void resident_multiply(const FusedArgs& a, const FusedShare& sh, const unsigned char* k_tiles,
-                                                  const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
-  constexpr uint32_t idesc = instr_desc(kTileKeys, NCOLS, FP8);
-  const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
-  const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
-  Ring kr(a.k_stages[0]), qr(T::QS), tr(a.t_stages[0]);
-  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
-  for (int n = 0; n < n_slabs; ++n) {
-    if (!mbar_wait_warp(bars.q_full(0, qr.stage), qr.phase, ab)) return;
-    const uint64_t qd0 = q_desc0 + (uint64_t)((qr.stage * T::kQBytes) >> 4);
-    for (int lt = 0; lt < n_tiles; ++lt) {
-      if (!mbar_wait2_warp(bars.k_full(0, kr.stage), kr.phase, bars.t_empty(0, 0, tr.stage), tr.phase ^ 1u, ab)) return;
-      tc_fence_after();
-      const uint32_t d_tmem = tmem + (uint32_t)(tr.stage * NCOLS);
-      const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
-      if (elect_one()) {
-#pragma unroll
-        for (int part = 0; part < T::QPARTS; ++part)               // 8-bit keys: the two query terms accumulate into the same columns
-#pragma unroll
-          for (int h = 0; h < T::KSUB; ++h)
-#pragma unroll
-            for (int ks = 0; ks < T::KSTEPS; ++ks)
-              tc_mma<FP8, false>(d_tmem, kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks,
-                                 qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks, idesc, (uint32_t)((part | h | ks) != 0));
-        tc_commit(bars.k_empty(0, kr.stage));
-        tc_commit(bars.t_full(0, 0, tr.stage));
-      }
-      __syncwarp();
-      kr.advance();
-      tr.advance();
-    }
-    if (elect_one()) tc_commit(bars.q_empty(0, qr.stage));
-    __syncwarp();
-    qr.advance();
-  }
-  if (elect_one()) tc_commit(bars.mma_done(0));
-  __syncwarp();
-  mbar_wait_warp(bars.mma_done(0), 0u, ab);
-}
-
-// The sums.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it shares out over the
-// warp at the end of a slab.
-template <class T, int NCOLS, bool FP8>
-__device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
-                                             const FusedBars& bars, const Abort& ab) {
-  const FusedPrompt& p = *sh.p;
-  const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
-  const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
-  const float* const refs = p.refs;
-  const float* const slab_c = p.slab_c;
-  const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-  const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
-  const int tail_lanes = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32;   // real keys of this quadrant in the last tile
-  const bool frees = a.mode == 1;                                  // no visit 2: nobody else frees the stages
-  ResidentRing tr(a.t_stages[0]);
-  tr.advance(set);
-  int lt = set;                                                    // this set's next tile, counted from the slab's first
-  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
-  for (int n = 0; n < n_slabs; ++n) {
-    const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
-    if (n + 1 < n_slabs) {
-      next_ref = __ldg(refs + sh.slab(n + 1));
-      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
-    }
-    uint64_t acc[NCOLS / 2];
-#pragma unroll
-    for (int j = 0; j < NCOLS / 2; ++j) acc[j] = 0ull;
-    const bool any = lt < n_tiles;
-    for (; lt < n_tiles; lt += 2) {
-      if (!mbar_wait_warp(bars.t_full(0, 0, tr.stage), tr.phase, ab)) return;
-      tc_fence_after();
-      uint32_t r[NCOLS];
-      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
-      tmem_load_wait();
-      tmem_ready<NCOLS>(r);
-      if (frees) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars.t_empty(0, 0, tr.stage));
-      }
-      tr.advance(2);
-      if (sh.tile(lt) < full_tiles || lane < tail_lanes) {
-#pragma unroll
-        for (int j = 0; j < NCOLS / 2; ++j) {
-          float x, y;
-          unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
-          acc[j] = add2(acc[j], pack2(fast_exp2(x), fast_exp2(y)));
-        }
-      }
-    }
-    lt -= n_tiles;
-    // Sum over the warp's 32 keys: transposing butterfly steps, each of which halves the columns a lane holds, then (16
-    // columns) one plain step.  The publishers add up quadrants and sets.
-    float s[NCOLS];
-    s[0] = 0.f;
-    if (any) {
-#pragma unroll
-      for (int j = 0; j < NCOLS / 2; ++j) unpack2(acc[j], s[2 * j], s[2 * j + 1]);
-      int width = NCOLS;
-#pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) {
-        if (width > 1) {
-          width >>= 1;
-          const bool upper = (lane & off) != 0;
-#pragma unroll
-          for (int j = 0; j < NCOLS / 2; ++j) {
-            if (j < width) {
-              const float send = upper ? s[j] : s[j + width];
-              const float keep = upper ? s[j + width] : s[j];
-              s[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-            }
-          }
-        } else {
-          s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
-        }
-      }
-    }
-    const int slot = n % kSumSlots;
-    if (n >= kSumSlots)
-      if (!mbar_wait_warp(bars.sums_free(slot), (uint32_t)(n / kSumSlots - 1) & 1u, ab)) return;
-    float* out = sums + ((slot * 2 + set) * 4 + quad) * 32;
-    if constexpr (NCOLS == 32) {
-      out[lane] = s[0];
-    } else {
-      if ((lane & 1) == 0) out[lane >> 1] = s[0];
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bars.sums_ready(slot));
-  }
-}
-
-// The maxima, once the slab's log-sum-exps are there.  A tile's maxima always belong to the same warps (lt mod 2 == set).
-// REGS: up to kRegTiles tiles, whose maxima stay in registers and leave all of tensor memory to the logits.
-template <class T, int NCOLS, int G, bool FP8, bool REGS>
-__device__ __forceinline__ void resident_max(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem,
-                                             uint32_t amax_tmem, const float* off, const float* off_c, const FusedBars& bars,
-                                             const Abort& ab) {
-  constexpr int NI = T::NI, MINE = REGS ? kRegTiles / 2 : 1;
+  constexpr int V = ONCE ? 0 : 1;                                  // whose logits: resident: those that were summed
+  constexpr int CW = T::CW, NCH = T::NCH, NIW = T::NIW, MINE = REGS ? kRegTiles / 2 : 1;
+  static_assert(!REGS || NCH == 1, "one load per tile");
   const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
   const int n_tiles = sh.n_tiles;
   const uint32_t lane_bits = (uint32_t)(quad * 32) << 16;
   const uint32_t lane_addr = tmem + lane_bits, amax_addr = amax_tmem + lane_bits;
-  uint32_t am[MINE][NI];
+  uint32_t am[MINE][NIW];
   if constexpr (REGS) {
 #pragma unroll
     for (int u = 0; u < MINE; ++u)
 #pragma unroll
-      for (int j = 0; j < NI; ++j) am[u][j] = 0xff800000u;         // -inf
+      for (int j = 0; j < NIW; ++j) am[u][j] = 0xff800000u;        // -inf
   } else {
     clear_maxima<T>(amax_addr, set, n_tiles);
   }
-  ResidentRing first(a.t_stages[0]);                               // the stage of the slab's first tile
+  // resident: the stage of the slab's first tile; two-pass: a ring per set, this one's first stage and the next to be read
+  Ring first(ONCE ? a.t_stages[V] : (a.t_stages[V] + 1 - set) / 2);
+  const int stage0 = ONCE ? 0 : set * ((a.t_stages[V] + 1) / 2);
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
     if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
     const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
     const float c = FP8 ? off_c[slot] : a.c;
     const uint64_t cc = pack2(c, c);
-    ResidentRing tr = first;
-    tr.advance(set);
-    auto fold = [&](int lt, uint32_t (&m)[NI]) -> bool {
-      // complete long since (the log-sum-exps contain it), except where visit 2 runs alone
-      if (!mbar_wait_warp(bars.t_full(0, 0, tr.stage), tr.phase, ab)) return false;
+    Ring tr = first;
+    if (ONCE) tr.advance(set);
+    auto fold = [&](int lt, uint32_t (&m)[NIW]) -> bool {
+      // resident: complete long since (the log-sum-exps contain it), except where visit 2 runs alone
+      if (!mbar_wait_warp(bars.t_full(V, stage0 + tr.stage), tr.phase, ab)) return false;
       tc_fence_after();
       if (!REGS) tmem_store_wait();                                // the maxima read below may be this warp's last stores
-      uint32_t r[NCOLS];
-      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
-      if (!REGS) tmem_issue<NI>(amax_addr + (uint32_t)(lt * NI), m);
-      tmem_load_wait();
-      tmem_ready<NCOLS>(r);
-      if (!REGS) tmem_ready<NI>(m);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars.t_empty(0, 0, tr.stage));
-      tr.advance(2);
-      fold_maxima<T, G>(r, m, off2, cc);
-      if (!REGS) tmem_store<NI>(amax_addr + (uint32_t)(lt * NI), m);
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        const uint32_t m_addr = amax_addr + (uint32_t)(lt * T::NI + ch * NIW);
+        uint32_t r[CW];
+        tmem_issue<CW>(lane_addr + (uint32_t)((stage0 + tr.stage) * NCOLS + ch * CW), r);
+        if (!REGS) tmem_issue<NIW>(m_addr, m);
+        tmem_load_wait();
+        tmem_ready<CW>(r);
+        if (!REGS) tmem_ready<NIW>(m);
+        if (ch + 1 == NCH) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bars.t_empty(V, stage0 + tr.stage));
+        }
+        fold_maxima<T, G>(r, m, off2 + ch * (CW / 4), cc);
+        if (!REGS) tmem_store<NIW>(m_addr, m);
+      }
+      tr.advance(ONCE ? 2 : 1);
       return true;
     };
     if constexpr (REGS) {
@@ -978,14 +853,15 @@ __device__ __forceinline__ void resident_max(const FusedArgs& a, const FusedShar
       for (int lt = set; lt < n_tiles; lt += 2)
         if (!fold(lt, am[0])) return;
     }
-    first.advance(n_tiles);
+    if (ONCE) first.advance(n_tiles);
+    else first = tr;
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
   if constexpr (REGS) {
 #pragma unroll
     for (int u = 0; u < MINE; ++u)
-      if (set + 2 * u < n_tiles) finish_tile<NI>(a, *sh.p, sh.tile(set + 2 * u), quad, lane, am[u]);
+      if (set + 2 * u < n_tiles) finish_tile<NIW>(a, *sh.p, sh.tile(set + 2 * u), quad, lane, am[u]);
   } else {
     tmem_store_wait();
     fused_finish<T>(a, sh, warp, lane, amax_tmem);
@@ -1042,11 +918,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
         mbar_init(bars.q_full(v, s), 1);
         mbar_init(bars.q_empty(v, s), 1);
       }
-      for (int set = 0; set < (ONCE ? 1 : 2); ++set)
-        for (int s = 0; s < a.t_stages[v]; ++s) {
-          mbar_init(bars.t_full(v, set, s), 1);
-          mbar_init(bars.t_empty(v, set, s), kVisitWarps / 2);
-        }
+      for (int s = 0; s < a.t_stages[v]; ++s) {
+        mbar_init(bars.t_full(v, s), 1);
+        mbar_init(bars.t_empty(v, s), kVisitWarps / 2);
+      }
       mbar_init(bars.mma_done(v), 1);
     }
     for (int x = 0; x < kOffSlots; ++x) {
@@ -1079,9 +954,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   tc_fence_after();
   const uint32_t tmem_base = (uint32_t)misc[1];
   // tensor memory: the accumulator stages, then the running maxima, [local tile][NI] columns (lane = key)
-  const uint32_t tmem_v2 = tmem_base + (uint32_t)(2 * a.t_stages[0] * T::SR);
-  const uint32_t amax_tmem = ONCE ? tmem_base + (uint32_t)(a.t_stages[0] * NCOLS)
-                                  : tmem_v2 + (uint32_t)(2 * a.t_stages[1] * a.max_tiles_per_stage * NCOLS);
+  const uint32_t tmem_v2 = tmem_base + (uint32_t)(a.t_stages[0] * (ONCE ? NCOLS : T::SR));
+  const uint32_t amax_tmem = tmem_v2 + (uint32_t)(ONCE ? 0 : a.t_stages[1] * NCOLS);
   grid_wait();                                                     // what the preparing kernel wrote is visible from here on
   grid_launch_dependents();                                        // the next kernel starts where SMs are free, and waits there
 
@@ -1096,12 +970,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
       unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
       if (warp < 2) {
         if (lane == 0) fused_produce<T, ONCE>(a, sh, v, k_tiles, q_tiles, tile_at, bars, misc + 2, ab);
-      } else if constexpr (ONCE) {
-        resident_multiply<T, NCOLS, FP8>(a, sh, k_tiles, q_tiles, tmem_base, bars, ab);
-      } else if (v == 0) {
-        fused_multiply<T, NCOLS, FP8, 0>(a, sh, k_tiles, q_tiles, tmem_base, bars, ab);
       } else {
-        fused_multiply<T, NCOLS, FP8, 1>(a, sh, k_tiles, q_tiles, tmem_v2, bars, ab);
+        if (v == 0) fused_multiply<T, NCOLS, FP8, !ONCE, false>(a, sh, 0, k_tiles, q_tiles, tmem_base, bars, ab);
+        else fused_multiply<T, NCOLS, FP8, false, true>(a, sh, 1, k_tiles, q_tiles, tmem_v2, bars, ab);
       }
     }
   } else if (warp < kSumWarp0) {
@@ -1119,14 +990,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
     }
   } else {
     if constexpr (kMoveRegs) reg_inc<88>();
+    const uint32_t logits = ONCE ? tmem_base : tmem_v2;
     if (!visit2) {
     } else if constexpr (ONCE && T::NI <= kRegSlots) {
-      if (a.max_in_regs) resident_max<T, NCOLS, G, FP8, true>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
-      else resident_max<T, NCOLS, G, FP8, false>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
-    } else if constexpr (ONCE) {
-      resident_max<T, NCOLS, G, FP8, false>(a, sh, warp, lane, tmem_base, amax_tmem, off, off_c, bars, ab);
+      if (a.max_in_regs) fused_max<T, NCOLS, G, FP8, ONCE, true>(a, sh, warp, lane, logits, amax_tmem, off, off_c, bars, ab);
+      else fused_max<T, NCOLS, G, FP8, ONCE, false>(a, sh, warp, lane, logits, amax_tmem, off, off_c, bars, ab);
     } else {
-      fused_max<T, NCOLS, G, FP8>(a, sh, warp, lane, tmem_v2, amax_tmem, off, off_c, bars, ab);
+      fused_max<T, NCOLS, G, FP8, ONCE, false>(a, sh, warp, lane, logits, amax_tmem, off, off_c, bars, ab);
     }
   }
 

@@ -373,13 +373,11 @@ int group_size(const Geometry& g, const int64_t* n_tiles, int n, int sm_count) {
 
 // Shared-memory and tensor-memory stages for CTAs that hold the running maxima of `tiles` tiles.
 bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, int* smem_bytes) {
-  const int amax_cols = tiles * (g.ncols / g.padded_group), sr = sum_rows(g.ncols);
   a->table_tiles = paged ? tiles : 0;
   if (g.once) {
     a->max_in_regs = g.max_in_regs(tiles);
     a->t_stages[0] = g.resident(tiles);
     a->t_stages[1] = 0;
-    a->max_tiles_per_stage = 1;
     for (int ks = kMaxKeyStages; ks >= 2; --ks) {
       a->k_stages[0] = ks;
       a->k_stages[1] = 0;
@@ -391,20 +389,16 @@ bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, 
     }
     return false;
   }
-  a->max_tiles_per_stage = 0;
-  // visit 2 takes two tiles per stage where they have 16 columns each (fewer barriers per tile); then as many stages as fit,
-  // visit 1 first (its epilogue is the longer one)
-  for (int tps = g.ncols == 16 && tiles > 2 ? 2 : 1; tps >= 1 && a->max_tiles_per_stage == 0; --tps)
-    for (int stages = 2 * kMaxTmemStages; stages >= 2; --stages) {
-      const int s1 = (stages + 1) / 2, s2 = stages / 2;
-      if (2 * (s1 * sr + s2 * tps * g.ncols) + amax_cols <= kTmemColsAll) {
-        a->max_tiles_per_stage = tps;
-        a->t_stages[0] = s1;
-        a->t_stages[1] = s2;
-        break;
-      }
+  // as many accumulator stages as fit, visit 1 first (its epilogue is the longer one)
+  const int columns = kTmemColsAll - tiles * (g.ncols / g.padded_group), sr = sum_rows(g.ncols);
+  a->t_stages[0] = a->t_stages[1] = 0;
+  for (int stages = 2 * kMaxTmemStages; stages >= 4; --stages)
+    if ((stages + 1) / 2 * sr + stages / 2 * g.ncols <= columns) {
+      a->t_stages[0] = (stages + 1) / 2;
+      a->t_stages[1] = stages / 2;
+      break;
     }
-  if (a->max_tiles_per_stage == 0) return false;
+  if (a->t_stages[0] == 0) return false;
   for (int ks = 20; ks >= 4; --ks) {
     a->k_stages[0] = (ks + 1) / 2;
     a->k_stages[1] = ks / 2;
