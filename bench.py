@@ -395,20 +395,19 @@ def run_ours(args):
             if want == 2:
                 raise
     spf.spf_set_score_path(2 if fused else 1)
-    # kernels per step: scoring per prompt (fused: score_fused; general: pack_q, score_lse, merge_lse, score_max), then
-    # chunk_pool and select_compact (top-k + compaction) per prompt, or the three batched calls once per batch
-    score_launches = 1 if fused else 4
-    score_kernels = "score_fused_kernel" if fused else "pack_q + score_lse + merge_lse + score_max"
+    # kernels per step: scoring (fused: fused_prep and score_fused, once for several prompts; general: pack_q, score_lse,
+    # merge_lse, score_max per prompt), then pool_select_compact for up to 24 prompts.  A batch may take more launches
+    score_launches = 2 if fused else 4 * n_prompts
+    score_kernels = "fused_prep + score_fused_kernel" if fused else "pack_q + score_lse + merge_lse + score_max"
+    launches_per_step = score_launches + 1
     if n_prompts > 1:
         bsel = spf.BatchSelector(cfg.n_layers, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.n_lookahead, cfg.lengths,
                                  chunk=cfg.chunk, pool_kernel=cfg.pool_kernel, device=dev)
-        launches_per_step = score_launches * n_prompts + 3
 
         def step():
             bsel.run(prompts, keep)
     else:
         bsel = None
-        launches_per_step = score_launches + 2           # chunk_pool, then top-k and compaction in one launch
 
         def step():
             p = prompts[0]
@@ -649,7 +648,7 @@ def run_keys(args, ops=None, device=None, backend="nccl", cfg=None):
 
 def run_fp8_line(args):
     """`--workload <name>_fp8`: the whole path on one prompt of <name> whose key cache is held as E4M3 bytes
-    (Selector.run_fp8: spf_score_fp8 -> spf_chunk_pool -> spf_select_compact), device-resident, one GPU.  The roofline's
+    (Selector.run_fp8: spf_score_fp8 -> spf_pool_select_compact), device-resident, one GPU.  The roofline's
     bytes are this format's own: the 8-bit cache read once + scales + Q + importance + lse."""
     import torch
     import paper_2603_02631_b200 as spf
@@ -708,7 +707,7 @@ def run_fp8_line(args):
                    "l2": "inputs larger than L2 (key cache streamed every step)"},
         "clocks": {"sm_mhz": clocks["sm_mhz"], "sm_max_mhz": clocks["sm_max_mhz"], "reasons": clocks["reasons"],
                    "samples": clocks["samples"]},
-        "gpu_launches": 4 * args.steps, "e2e": None,
+        "gpu_launches": 3 * args.steps, "e2e": None,
         "roofline": {"bound": "hbm", "kernel": "spf_score_fp8", "achieved": gbs, "peak": peak, "peak_kind": f"of {peak_kind}",
                      "unit": "GB/s", "frac": gbs / peak, "traffic": None, "ms_per_launch": ms_score, "algorithmic_bytes": nbytes},
     }), flush=True)

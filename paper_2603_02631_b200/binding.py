@@ -682,7 +682,7 @@ class Selection:
 
 
 class Selector:
-    """Chains spf_score -> spf_chunk_pool -> spf_select_topk -> spf_compact_spans for prompts of one geometry.
+    """Chains spf_score -> spf_pool_select_compact (pooling, top-k and compaction) for prompts of one geometry.
 
     Buffers are allocated once for ``max_tokens`` and reused, so that a call enqueues kernels only.
     """
@@ -808,8 +808,8 @@ class Selector:
 
 
 class BatchSelector:
-    """The path for a batch of prompts of one geometry: one spf_score call for the batch, then ONE launch each of
-    pooling, top-k and compaction for all prompts (the batched calls).  Buffers are allocated once per prompt slot."""
+    """The path for a batch of prompts of one geometry: one spf_score call and one spf_pool_select_compact call for all of
+    them.  Buffers are allocated once per prompt slot."""
 
     def __init__(self, n_layers: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_lookahead: int,
                  max_tokens: Sequence[int], chunk: int = 32, pool_kernel: int = 13, softmax_scale: float = 0.0,

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 
@@ -32,18 +33,23 @@ struct LayerPtrs {
   const __nv_bfloat16* p[kMaxLayers];
 };
 
+// Lets a kernel use `bytes` of dynamic shared memory on the current device; asked for once per device (`done`), not per launch.
+constexpr int kMaxDevices = 64;
+inline int32_t allow_shared_memory(const void* kernel, int bytes, std::atomic<bool> (&done)[kMaxDevices]) {
+  int dev = 0;
+  SPF_CUDA_CHECK(cudaGetDevice(&dev));
+  if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return SPF_OK;
+  SPF_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  if (dev >= 0 && dev < kMaxDevices) done[dev].store(true, std::memory_order_release);
+  return SPF_OK;
+}
+
 static inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float fast_log2(float x) {
-  float y;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 

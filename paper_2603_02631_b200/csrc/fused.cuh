@@ -66,6 +66,7 @@
 namespace spf {
 
 constexpr int kFusedThreads = 768;
+constexpr int kFusedSmemMost = 227 * 1024;   // dynamic shared memory of a CTA
 constexpr int kVisitWarps = 8;         // epilogue warps per visit
 constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
 // Groups of up to this many CTAs add up everybody's row sums in every CTA (see fused_publish): one hop instead of two, about
@@ -1033,7 +1034,9 @@ int32_t fused_launch_d128_fp8(const FusedArgs& args, const FusedLaunch& l, cudaS
 template <int D, int NCOLS, int G, bool FP8, bool ONCE>
 int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
   auto kern = score_fused_kernel<D, NCOLS, G, FP8, ONCE>;
-  SPF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem_bytes));
+  static std::atomic<bool> allowed[kMaxDevices];
+  const int32_t st = allow_shared_memory(reinterpret_cast<const void*>(kern), kFusedSmemMost, allowed);
+  if (st != SPF_OK) return st;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)l.n_cta);
   cfg.blockDim = dim3(kFusedThreads);

@@ -198,7 +198,7 @@ int32_t launch_prep(const PrepArgs<N>& args, int d, bool fp8, int n_slabs, int n
 }
 
 // ---------------------------------------------------------------------------------------------- the split over the SMs
-constexpr int kSmemBudget = 227 * 1024 - 1024;   // dynamic shared memory we may ask for, minus alignment slack
+constexpr int kSmemBudget = kFusedSmemMost - 1024;   // minus alignment slack
 // Key bytes between the first and the second read of a tile that still sit in L2 (126 MB, in two halves).
 constexpr double kL2KeyBytes = 80e6;
 // What an SM's share of the memory bandwidth brings in a microsecond (6.5 TB/s over 148 SMs).

@@ -824,8 +824,11 @@ int32_t tail_launch(const spf_path_item* items, int n, const PoolRule& rule, int
     cfg.stream = stream;
     // beyond 48 KB with the static part (about 21 KB), shared memory has to be asked for
     if (cfg.dynamicSmemBytes > 24 * 1024)
-      SPF_CUDA_CHECK(cudaFuncSetAttribute(pool_select_compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kTailChunks * (int)sizeof(uint32_t)));
+    {
+      static std::atomic<bool> allowed[kMaxDevices];
+      const int32_t st = allow_shared_memory(reinterpret_cast<const void*>(pool_select_compact_kernel), kTailChunks * (int)sizeof(uint32_t), allowed);
+      if (st != SPF_OK) return st;
+    }
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim = {(unsigned)ctas, 1, 1};
