@@ -602,12 +602,6 @@ def spf_compact_spans_batch(kept_chunks: Sequence[torch.Tensor], ks: Sequence[in
     _check(lib.spf_compact_spans_batch(items, n_items, chunk, _stream_ptr(stream)), "spf_compact_spans_batch")
 
 
-def _host(t: torch.Tensor, dtype: torch.dtype, name: str) -> torch.Tensor:
-    if t.is_cuda or t.dtype != dtype or not t.is_contiguous():
-        raise TypeError(f"{name} must be a contiguous host tensor of dtype {dtype}")
-    return t
-
-
 def spf_compress_host_arena_bytes(n_layers: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_lookahead: int,
                                   n_tokens: int, chunk: int, pool_kernel: int, keep: float, softmax_scale: float = 0.0) -> int:
     shape = _Shape(n_layers, n_q_heads, n_kv_heads, head_dim, n_lookahead, float(softmax_scale))
@@ -625,35 +619,8 @@ def spf_compress_host(q: torch.Tensor, k_layers: Sequence[torch.Tensor], token_i
                       stream: Optional[torch.cuda.Stream] = None) -> None:
     """The whole path for one prompt in HOST tensors (inputs and outputs); ``arena`` is device scratch.  Synchronises the
     stream.  See spf_compress_host in include/spf.h for sizes."""
-    L, Hq, m, d = q.shape
-    Hkv, n, _ = k_layers[0].shape
-    _host(q, torch.bfloat16, "q")
-    for kl in k_layers:
-        _host(kl, torch.bfloat16, "k_layers[l]")
-        if tuple(kl.shape) != (Hkv, n, d):
-            raise ValueError("every k_layers[l] must be [Hkv, N, d]")
-    for name, t in (("token_ids", token_ids), ("char_start", char_start), ("char_end", char_end), ("out_ids", out_ids),
-                    ("out_tok_spans", out_tok_spans), ("out_char_spans", out_char_spans)):
-        _host(t, torch.int32, name)
-    if out_pos is not None:
-        _host(out_pos, torch.int32, "out_pos")
-    _host(out_counts, torch.int64, "out_counts")
-    if not arena.is_cuda:
-        raise TypeError("arena must be a CUDA tensor")
-    k = spf_keep_count((n + chunk - 1) // chunk, keep)
-    need = min(k * chunk, n)
-    if len(k_layers) != L or min(token_ids.numel(), char_start.numel(), char_end.numel()) < n or out_ids.numel() < need or \
-            (out_pos is not None and out_pos.numel() < need) or out_tok_spans.numel() < 2 * k or \
-            out_char_spans.numel() < 2 * k or out_counts.numel() < 2:
-        raise ValueError("a buffer is smaller than include/spf.h requires")
-    shape = _Shape(L, Hq, Hkv, d, m, float(softmax_scale))
-    prm = _SelectParams(chunk, pool_kernel, float(keep))
-    ptrs = (ctypes.c_void_p * L)(*[kl.data_ptr() for kl in k_layers])
-    _check(lib.spf_compress_host(ctypes.byref(shape), n, ctypes.cast(ptrs, ctypes.POINTER(ctypes.c_void_p)), q.data_ptr(),
-                                 token_ids.data_ptr(), char_start.data_ptr(), char_end.data_ptr(), ctypes.byref(prm),
-                                 arena.data_ptr(), arena.numel() * arena.element_size(), out_ids.data_ptr(), _ptr(out_pos),
-                                 out_tok_spans.data_ptr(), out_char_spans.data_ptr(), out_counts.data_ptr(),
-                                 _stream_ptr(stream)), "spf_compress_host")
+    _check(_native.compress_host(q, k_layers, token_ids, char_start, char_end, chunk, pool_kernel, keep, arena, out_ids, out_pos,
+                                 out_tok_spans, out_char_spans, out_counts, softmax_scale, stream), "spf_compress_host")
 
 
 @dataclasses.dataclass

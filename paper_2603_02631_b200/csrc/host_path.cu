@@ -1,5 +1,6 @@
 // spf_compress_host: the four calls of the path chained for a prompt whose inputs and results are host buffers.
 #include <algorithm>
+#include <cstddef>
 
 #include "common.cuh"
 #include "score.cuh"
@@ -9,6 +10,11 @@ namespace {
 
 struct Arena {
   size_t k, q, ids, cs, ce, importance, lse, scores, kept, out_ids, out_pos, tok, ch, counts, status, workspace, total;
+};
+
+struct Verdict {
+  int64_t counts[2];
+  int32_t status;
 };
 
 size_t take(size_t* pos, size_t bytes) {
@@ -59,8 +65,8 @@ bool layout(const spf_shape* shape, int64_t n, const spf_select_params* prm, Are
   a->out_pos = take(&pos, kept_tokens * 4);
   a->tok = take(&pos, (size_t)k * 8);
   a->ch = take(&pos, (size_t)k * 8);
-  a->counts = take(&pos, 16);
-  a->status = take(&pos, 4);
+  a->counts = take(&pos, sizeof(Verdict));                 // counts and status come back in one copy
+  a->status = a->counts + offsetof(Verdict, status);
   a->workspace = take(&pos, *ws_bytes);
   a->total = pos;
   return true;
@@ -124,8 +130,9 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
   pr.importance = reinterpret_cast<float*>(base + a.importance);
   pr.lse = reinterpret_cast<float*>(base + a.lse);
   int32_t* dev_status = reinterpret_cast<int32_t*>(base + a.status);
-  int64_t counts[2] = {0, 0};
-  int32_t device_status = 0;
+  Verdict v{};
+  // Rows that are kept whichever chunks are: all chunks but the last are full.  They are copied without waiting for the counts.
+  const size_t sure = (size_t)(k - 1) * params->chunk + (size_t)(n_tokens - (n_chunks - 1) * params->chunk);
   for (int attempt = 0; attempt < 2; ++attempt) {
     // attempt 0: the kernels spf_score would pick; attempt 1 (after a device-side range or timeout report): the general ones
     SPF_CUDA_CHECK(cudaMemsetAsync(dev_status, 0, 4, stream));
@@ -148,20 +155,24 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
     item.out_counts = reinterpret_cast<int64_t*>(base + a.counts);
     st = spf_pool_select_compact(&item, 1, params->pool_kernel, params->chunk, 0, 0, 0, stream);
     if (st != SPF_OK) return st;
-    SPF_CUDA_CHECK(cudaMemcpyAsync(counts, base + a.counts, 16, cudaMemcpyDeviceToHost, stream));
-    SPF_CUDA_CHECK(cudaMemcpyAsync(&device_status, dev_status, 4, cudaMemcpyDeviceToHost, stream));
+    SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host, base + a.out_ids, sure * 4, cudaMemcpyDeviceToHost, stream));
+    if (out_pos_host != nullptr)
+      SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host, base + a.out_pos, sure * 4, cudaMemcpyDeviceToHost, stream));
+    SPF_CUDA_CHECK(cudaMemcpyAsync(&v, base + a.counts, sizeof(v), cudaMemcpyDeviceToHost, stream));
     SPF_CUDA_CHECK(cudaStreamSynchronize(stream));
-    if (device_status != SPF_ERR_RANGE && device_status != SPF_ERR_TIMEOUT) break;
+    if (v.status != SPF_ERR_RANGE && v.status != SPF_ERR_TIMEOUT) break;
   }
-  if (device_status != 0) return fail(device_status, "spf_compress_host: device status %d (%s)", device_status, spf_status_string(device_status));
-  const size_t n_kept = (size_t)counts[0], n_spans = (size_t)counts[1];
-  SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host, base + a.out_ids, n_kept * 4, cudaMemcpyDeviceToHost, stream));
-  if (out_pos_host != nullptr)
-    SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host, base + a.out_pos, n_kept * 4, cudaMemcpyDeviceToHost, stream));
+  if (v.status != 0) return fail(v.status, "spf_compress_host: device status %d (%s)", v.status, spf_status_string(v.status));
+  const size_t n_kept = (size_t)v.counts[0], n_spans = (size_t)v.counts[1];
+  if (n_kept > sure) {
+    SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host + sure, base + a.out_ids + sure * 4, (n_kept - sure) * 4, cudaMemcpyDeviceToHost, stream));
+    if (out_pos_host != nullptr)
+      SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host + sure, base + a.out_pos + sure * 4, (n_kept - sure) * 4, cudaMemcpyDeviceToHost, stream));
+  }
   SPF_CUDA_CHECK(cudaMemcpyAsync(out_tok_spans_host, base + a.tok, n_spans * 8, cudaMemcpyDeviceToHost, stream));
   SPF_CUDA_CHECK(cudaMemcpyAsync(out_char_spans_host, base + a.ch, n_spans * 8, cudaMemcpyDeviceToHost, stream));
   SPF_CUDA_CHECK(cudaStreamSynchronize(stream));
-  out_counts_host[0] = counts[0];
-  out_counts_host[1] = counts[1];
+  out_counts_host[0] = v.counts[0];
+  out_counts_host[1] = v.counts[1];
   return SPF_OK;
 }

@@ -359,9 +359,81 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
   }
 }
 
+const at::Tensor& host_tensor(PyObject* o, at::ScalarType dtype, const char* name) {
+  if (THPVariable_Check(o)) {
+    const at::Tensor& t = THPVariable_Unpack(o);
+    if (!t.is_cuda() && t.scalar_type() == dtype && t.is_contiguous()) return t;
+  }
+  raise(PyExc_TypeError, std::string(name) + " must be a contiguous host tensor of dtype " + dtype_name(dtype));
+}
+
+// compress_host(q, layers, token_ids, char_start, char_end, chunk, pool_kernel, keep, arena, out_ids, out_pos, tok_spans, char_spans,
+//               counts, softmax_scale, stream) -> status
+PyObject* compress_host(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
+  try {
+    if (n_args != 16) raise(PyExc_TypeError, "compress_host takes 16 arguments");
+    const at::Tensor& q = host_tensor(args[0], at::kBFloat16, "q");
+    if (q.dim() != 4) raise(PyExc_ValueError, "q must be [L, Hq, m, d]");
+    Ref layers(PySequence_Fast(args[1], "k_layers must be a sequence"));
+    const Py_ssize_t count = PySequence_Fast_GET_SIZE(layers.p);
+    if (count < 1) raise(PyExc_ValueError, "k_layers must hold one tensor per layer");
+    std::vector<const void*> ptrs((size_t)count);
+    int64_t hkv = 0, n = 0;
+    for (Py_ssize_t l = 0; l < count; ++l) {
+      const at::Tensor& k = host_tensor(PySequence_Fast_GET_ITEM(layers.p, l), at::kBFloat16, "k_layers[l]");
+      if (l == 0 && k.dim() == 3) {
+        hkv = k.size(0);
+        n = k.size(1);
+      }
+      if (k.dim() != 3 || k.size(0) != hkv || k.size(1) != n || k.size(2) != q.size(3))
+        raise(PyExc_ValueError, "every k_layers[l] must be [Hkv, N, d]");
+      ptrs[(size_t)l] = k.data_ptr();
+    }
+    const at::Tensor& ids = host_tensor(args[2], at::kInt, "token_ids");
+    const at::Tensor& cs = host_tensor(args[3], at::kInt, "char_start");
+    const at::Tensor& ce = host_tensor(args[4], at::kInt, "char_end");
+    spf_select_params params{};
+    params.chunk = (int32_t)PyLong_AsLong(args[5]);
+    params.pool_kernel = (int32_t)PyLong_AsLong(args[6]);
+    params.keep_ratio = PyFloat_AsDouble(args[7]);
+    const double scale = PyFloat_AsDouble(args[14]);
+    if (PyErr_Occurred()) throw PyFailure{};
+    const at::Tensor& arena = tensor(args[8], "arena");
+    if (!arena.is_cuda()) raise(PyExc_TypeError, "arena must be a CUDA tensor");
+    const at::Tensor& out_ids = host_tensor(args[9], at::kInt, "out_ids");
+    const at::Tensor* out_pos = args[10] == Py_None ? nullptr : &host_tensor(args[10], at::kInt, "out_pos");
+    const at::Tensor& tok = host_tensor(args[11], at::kInt, "out_tok_spans");
+    const at::Tensor& ch = host_tensor(args[12], at::kInt, "out_char_spans");
+    const at::Tensor& counts = host_tensor(args[13], at::kLong, "out_counts");
+    if (params.chunk >= 1) {
+      const int64_t k = spf_keep_count((n + params.chunk - 1) / params.chunk, params.keep_ratio), need = std::min(k * params.chunk, n);
+      if (count != q.size(0) || std::min(std::min(ids.numel(), cs.numel()), ce.numel()) < n || out_ids.numel() < need ||
+          (out_pos != nullptr && out_pos->numel() < need) || tok.numel() < 2 * k || ch.numel() < 2 * k || counts.numel() < 2)
+        raise(PyExc_ValueError, "a buffer is smaller than include/spf.h requires");
+    }
+    const spf_shape shape{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)hkv, (int32_t)q.size(3), (int32_t)q.size(2), (float)scale};
+    void* stream = stream_of(args[15], arena);
+    void* arena_ptr = arena.data_ptr();
+    const size_t arena_bytes = (size_t)arena.numel() * arena.element_size();
+    int32_t st;
+    Py_BEGIN_ALLOW_THREADS;
+    st = spf_compress_host(&shape, n, ptrs.data(), q.data_ptr(), ids.data_ptr<int32_t>(), cs.data_ptr<int32_t>(), ce.data_ptr<int32_t>(), &params,
+                           arena_ptr, arena_bytes, out_ids.data_ptr<int32_t>(), out_pos != nullptr ? out_pos->data_ptr<int32_t>() : nullptr,
+                           tok.data_ptr<int32_t>(), ch.data_ptr<int32_t>(), counts.data_ptr<int64_t>(), stream);
+    Py_END_ALLOW_THREADS;
+    return PyLong_FromLong(st);
+  } catch (const PyFailure&) {
+    return nullptr;
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
 PyMethodDef kMethods[] = {
     {"select", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(select_one)), METH_FASTCALL, "The path for one prompt."},
     {"select_batch", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(select_batch)), METH_FASTCALL, "The path for a batch of prompts."},
+    {"compress_host", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(compress_host)), METH_FASTCALL, "The path for one prompt in host tensors."},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_native", "Native marshalling of the Selector classes.", -1, kMethods, nullptr, nullptr, nullptr, nullptr};
