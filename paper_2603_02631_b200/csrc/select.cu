@@ -386,6 +386,7 @@ constexpr int kTailThreads = 1024;
 constexpr int kTailChunks = 32768;     // keys of this many chunks fit shared memory (128 KB)
 constexpr int kTailBins = 2 * kTailThreads;
 constexpr int kRankMost = 512;
+constexpr int kRankAll = 128;          // so few chunks are ranked without a histogram and its four barriers (64: 7.9 -> 7.1 us in all)
 constexpr int kTailItems = 24;         // prompts per launch: their descriptors are kernel arguments
 
 struct TailBatch {
@@ -427,6 +428,30 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t x, uint32_t* scratc
 __device__ __forceinline__ void select_last(TailShared& sh, const uint32_t* keys, int n, int left, int force) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int first = force & 1, end = n - ((force >> 1) & 1);
+  if (n <= kRankAll) {
+    constexpr int kEach = kRankAll / 32;
+    uint32_t other[kEach];
+#pragma unroll
+    for (int o = 0; o < kEach; ++o) other[o] = keys[min(first + lane + 32 * o, n - 1)];
+#pragma unroll
+    for (int c = 0; c < kEach; ++c) {
+      const int j = first + warp + 32 * c;
+      const uint32_t key = keys[min(j, n - 1)];
+      uint32_t better = 0;
+#pragma unroll
+      for (int o = 0; o < kEach; ++o) {
+        const int at = first + lane + 32 * o;
+        better += at < end && (other[o] > key || (other[o] == key && at < j));
+      }
+      better = __reduce_add_sync(0xffffffffu, better);
+      if (lane == 0 && j < end && (int)better == left - 1) {
+        sh.last_key = key;
+        sh.last_at = j;
+      }
+    }
+    __syncthreads();
+    return;
+  }
   uint32_t lo = 0xFFFFFFFFu, hi = 0;
   for (int j = first + tid; j < end; j += kTailThreads) {
     lo = min(lo, keys[j]);
