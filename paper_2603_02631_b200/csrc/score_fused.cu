@@ -199,8 +199,11 @@ int32_t launch_prep(const PrepArgs<N>& args, int d, bool fp8, int n_slabs, int n
 
 // ---------------------------------------------------------------------------------------------- the split over the SMs
 constexpr int kSmemBudget = kFusedSmemMost - 1024;   // minus alignment slack
-// Key bytes between the first and the second read of a tile that still sit in L2 (126 MB, in two halves).
-constexpr double kL2KeyBytes = 80e6;
+// Key bytes between the first and the second read of a tile (two-pass): what still sits in L2 (126 MB, in two halves).  A
+// slab of more than kLongSlab tiles a CTA is far enough ahead of its hand-over with less, and more of it is still there
+// (sustained, 64 rows at 131072 tokens 627 -> 605 us, 32 rows at 262000 507 -> 471); with 4 tiles less lead costs 3 %.
+constexpr double kL2KeyBytes = 80e6, kL2KeyBytesLong = 60e6;
+constexpr int kLongSlab = 5;
 // What an SM's share of the memory bandwidth brings in a microsecond (6.5 TB/s over 148 SMs).
 constexpr double kSmBytesPerUs = 44e3;
 // Microseconds from a slab's last key to its log-sum-exps having freed the slab's tiles, in one hop between the CTAs of a
@@ -245,9 +248,9 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
   g.ncols = rows <= 16 ? 16 : rows <= 32 ? 32 : 64;
   g.n_slabs = p.n_layers * p.n_kv_heads;
   g.tile_bytes = kTileKeys * row_bytes(p.head_dim, g.fp8);
-  g.lead = std::max(2, (int)(kL2KeyBytes / ((double)sm_count * g.tile_bytes)));
   g.handover = std::max(2, (int)(3.0 * kSmBytesPerUs / g.tile_bytes));
   const int tiles = (int)std::min<int64_t>(ceil_div(ceil_div(p.n_tokens, kTileKeys), std::min(sm_count, kFusedMaxCtas)), 1 << 20);
+  g.lead = std::max(2, (int)((tiles > kLongSlab ? kL2KeyBytesLong : kL2KeyBytes) / ((double)sm_count * g.tile_bytes)));
   // the resident form wants a slab's tiles and a few more in tensor memory
   g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + 3;
   g.max_tiles = (kTmemColsAll - 2 * (sum_rows(g.ncols) + g.ncols)) / (g.ncols / g.padded_group);
