@@ -66,8 +66,8 @@ struct Names {
 Names N;
 
 Ref attr(PyObject* o, PyObject* name) { return Ref(PyObject_GetAttr(o, name)); }
-// The tensor stays alive: the object that has it as an attribute holds it for the length of the call.
-const at::Tensor& attr_tensor(PyObject* o, PyObject* name, at::ScalarType dtype, const char* what) {
+// A reference of its own: the attribute may be computed, or be replaced by another thread during the call.
+at::Tensor attr_tensor(PyObject* o, PyObject* name, at::ScalarType dtype, const char* what) {
   return device_tensor(attr(o, name).p, dtype, what);
 }
 int64_t attr_int(PyObject* o, PyObject* name) {
@@ -88,8 +88,11 @@ bool attr_true(PyObject* o, PyObject* name) {
 
 enum Kind { kPlain = 0, kPaged = 1, kFp8 = 2 };
 
-// One prompt's scoring inputs in the form of its kind.
+// One prompt's scoring inputs in the form of its kind.  `held` keeps the tensors behind the pointers until the kernels are
+// enqueued: what the caller handed over may be temporary (a property that casts, a sequence that makes its items), and memory
+// given back before that could be the workspace's, or the next prompt's, when the kernels run.
 struct Inputs {
+  std::vector<at::Tensor> held;
   std::vector<const void*> layers;
   int64_t n = 0;
   const void *q = nullptr, *aux = nullptr;     // aux: block table or key scales
@@ -102,6 +105,7 @@ void read_inputs(Kind kind, PyObject* q_obj, PyObject* layers_obj, PyObject* aux
                  spf_shape* shape, Inputs* in) {
   const at::Tensor& q = device_tensor(q_obj, at::kBFloat16, "q");
   if (q.dim() != 4) raise(PyExc_ValueError, "q must be [L, Hq, m, d]");
+  if (PyIter_Check(layers_obj)) raise(PyExc_TypeError, "the key tensors must be a sequence");   // an iterator is used up by one look
   Ref layers(PySequence_Fast(layers_obj, "the key tensors must be a sequence"));
   const Py_ssize_t count = PySequence_Fast_GET_SIZE(layers.p);
   PyObject** items = PySequence_Fast_ITEMS(layers.p);
@@ -124,8 +128,11 @@ void read_inputs(Kind kind, PyObject* q_obj, PyObject* layers_obj, PyObject* aux
     raise(PyExc_ValueError, "q must be contiguous [L, Hq, m, d], the same shape for all prompts");
   if (count != shape->n_layers) raise(PyExc_ValueError, "k_layers must hold one tensor per layer");
   in->layers.resize((size_t)count);
+  in->held.reserve((size_t)count + 2);
+  in->held.push_back(q);
   for (Py_ssize_t l = 0; l < count; ++l) {
     const at::Tensor& kl = device_tensor(items[l], dtype, "k_layers[l]");
+    in->held.push_back(kl);
     bool fine = kl.dim() == dims && kl.sizes() == k0.sizes() && kl.size(dims - 1) == shape->head_dim && hkv == shape->n_kv_heads;
     if (kind == kPaged) fine = fine && kl.is_contiguous();
     else fine = fine && kl.stride(2) == 1 && kl.strides() == k0.strides();
@@ -144,6 +151,7 @@ void read_inputs(Kind kind, PyObject* q_obj, PyObject* layers_obj, PyObject* aux
     if (in->block_tokens < 1 || table.numel() < (in->n + in->block_tokens - 1) / in->block_tokens)
       raise(PyExc_ValueError, "block_table or importance has the wrong size");
     in->aux = table.data_ptr();
+    in->held.push_back(table);
   } else {
     in->n = k0.size(1);
     in->stride_head = k0.stride(0);
@@ -153,12 +161,14 @@ void read_inputs(Kind kind, PyObject* q_obj, PyObject* layers_obj, PyObject* aux
       if (scales.numel() != (int64_t)shape->n_layers * hkv || !scales.is_contiguous())
         raise(PyExc_ValueError, "k_scale must be contiguous fp32 [L, Hkv] and importance fp32 [N]");
       in->aux = scales.data_ptr();
+      in->held.push_back(scales);
     }
   }
 }
 
-// What a Selector brings for one prompt, and the prompt's token arrays.
+// What a Selector brings for one prompt, and the prompt's token arrays (`held`: as in Inputs).
 struct Buffers {
+  std::vector<at::Tensor> held;
   at::Tensor importance, lse, scores;      // trimmed to the prompt, for the result
   float *importance_ptr, *scores_ptr, *lse_ptr;
   int32_t *kept, *out_ids, *out_pos, *tok_spans, *char_spans;
@@ -175,18 +185,18 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   b->n_chunks = (n + chunk - 1) / chunk;
   b->k = spf_keep_count(b->n_chunks, keep);
   if (force_first || force_last) b->k = std::max(b->k, (int64_t)(force_first ? 1 : 0) + (force_last && (b->n_chunks > 1 || !force_first) ? 1 : 0));
-  const at::Tensor& importance = attr_tensor(slot, N.importance, at::kFloat, "importance");
-  const at::Tensor& lse = attr_tensor(slot, N.lse, at::kFloat, "lse");
-  const at::Tensor& scores = attr_tensor(slot, N.chunk_scores, at::kFloat, "chunk_scores");
+  const at::Tensor importance = attr_tensor(slot, N.importance, at::kFloat, "importance");
+  const at::Tensor lse = attr_tensor(slot, N.lse, at::kFloat, "lse");
+  const at::Tensor scores = attr_tensor(slot, N.chunk_scores, at::kFloat, "chunk_scores");
   if (importance.numel() < n || !importance.is_contiguous()) raise(PyExc_ValueError, "importance must be contiguous fp32 [N]");
   if (lse.numel() != (int64_t)shape.n_layers * shape.n_q_heads * shape.n_lookahead || !lse.is_contiguous())
     raise(PyExc_ValueError, "lse must be contiguous fp32 [L, Hq, m]");
-  const at::Tensor& kept = attr_tensor(slot, N.kept, at::kInt, "kept_chunks");
-  const at::Tensor& out_ids = attr_tensor(slot, N.out_ids, at::kInt, "out_ids");
-  const at::Tensor& out_pos = attr_tensor(slot, N.out_pos, at::kInt, "out_pos");
-  const at::Tensor& tok = attr_tensor(slot, N.tok_spans, at::kInt, "out_tok_spans");
-  const at::Tensor& ch = attr_tensor(slot, N.char_spans, at::kInt, "out_char_spans");
-  const at::Tensor& counts = attr_tensor(slot, N.counts, at::kLong, "out_counts");
+  const at::Tensor kept = attr_tensor(slot, N.kept, at::kInt, "kept_chunks");
+  const at::Tensor out_ids = attr_tensor(slot, N.out_ids, at::kInt, "out_ids");
+  const at::Tensor out_pos = attr_tensor(slot, N.out_pos, at::kInt, "out_pos");
+  const at::Tensor tok = attr_tensor(slot, N.tok_spans, at::kInt, "out_tok_spans");
+  const at::Tensor ch = attr_tensor(slot, N.char_spans, at::kInt, "out_char_spans");
+  const at::Tensor counts = attr_tensor(slot, N.counts, at::kLong, "out_counts");
   const at::Tensor& i = device_tensor(ids, at::kInt, "token_ids");
   const at::Tensor& cs = device_tensor(char_start, at::kInt, "char_start");
   const at::Tensor& ce = device_tensor(char_end, at::kInt, "char_end");
@@ -209,6 +219,7 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   b->ids = i.data_ptr<int32_t>();
   b->char_start = cs.data_ptr<int32_t>();
   b->char_end = ce.data_ptr<int32_t>();
+  b->held = {importance, lse, scores, kept, out_ids, out_pos, tok, ch, counts, i, cs, ce};
 }
 
 spf_path_item path_item(const Buffers& b, int64_t n) {
@@ -266,7 +277,8 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     const bool force_first = attr_true(selector, N.force_first), force_last = attr_true(selector, N.force_last);
     Buffers b;
     read_buffers(selector, shape, in.n, chunk, keep, force_first, force_last, args[6], args[7], args[8], &b);
-    int32_t* status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status").data_ptr<int32_t>();
+    const at::Tensor dev_status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status");
+    int32_t* status = dev_status.data_ptr<int32_t>();
     void* stream = stream_of(args[10], b.importance);
 
     spf_prompt plain{in.n, in.layers.data(), in.stride_head, in.stride_tok, in.q, b.importance_ptr, b.lse_ptr};
@@ -333,7 +345,8 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
       p[i] = spf_prompt{n, in[i].layers.data(), in[i].stride_head, in[i].stride_tok, in[i].q, b[i].importance_ptr, b[i].lse_ptr};
       items[i] = path_item(b[i], n);
     }
-    int32_t* status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status").data_ptr<int32_t>();
+    const at::Tensor dev_status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status");
+    int32_t* status = dev_status.data_ptr<int32_t>();
     void* stream = stream_of(args[3], b[0].importance);
     const size_t need = spf_score_workspace_bytes(&shape, p.data(), (int32_t)count);
     if (need == 0) return result_tuple(SPF_ERR_INVALID_ARG, "spf_score_workspace_bytes", nullptr, 0);

@@ -1,0 +1,61 @@
+"""What callers may rely on beyond the numbers: which tensors a call holds, which buffers it takes, what it leaves alone."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+GEOM = (2, 4, 2, 64, 8)                # L, Hq, Hkv, d, m
+
+
+def make(n, seed=0, geom=GEOM):
+    L, Hq, Hkv, d, m = geom
+    gen = torch.Generator(device="cuda").manual_seed(seed + 131 * n)
+    q = torch.randn(L, Hq, m, d, generator=gen, device="cuda").to(torch.bfloat16)
+    return q, [torch.randn(Hkv, n, d, generator=gen, device="cuda").to(torch.bfloat16) for _ in range(L)]
+
+
+def text(n):
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    return ids * 7 % 32000, ids * 3, ids * 3 + 2
+
+
+class Fresh:
+    """A prompt that keeps its tensors in another form and makes those of the call when it is asked for them."""
+
+    def __init__(self, n, seed):
+        q, k = make(n, seed)
+        self.n_tokens, self._q, self._k, self._text = n, q.cpu(), [x.cpu() for x in k], [t.cpu() for t in text(n)]
+
+    q = property(lambda self: self._q.cuda())
+    k = property(lambda self: [x.cuda() for x in self._k])
+    token_ids = property(lambda self: self._text[0].cuda())
+    char_start = property(lambda self: self._text[1].cuda())
+    char_end = property(lambda self: self._text[2].cuda())
+
+
+def test_tensors_made_for_the_call_live_until_it_is_enqueued():
+    """Each prompt's tensors are dropped by their maker at once; the next prompt's, or the workspace, would get their memory."""
+    import paper_2603_02631_b200 as spf
+    prompts = [Fresh(3000, seed) for seed in range(4)]
+    batch = spf.BatchSelector(*GEOM, [3000] * 4)
+    got = batch.run(prompts, 0.3)
+    torch.cuda.synchronize()
+    for p, s in zip(prompts, got):
+        one = spf.Selector(*GEOM, 3000).run(p.q, p.k, p.token_ids, p.char_start, p.char_end, 0.3)
+        torch.testing.assert_close(s.importance, one.importance, rtol=1e-5, atol=0)
+        assert torch.equal(s.out_ids[:int(s.counts[0])], one.out_ids[:int(one.counts[0])])
+    # a sequence that makes its items, and a workspace that has to be allocated after them
+    class Lazy:
+        def __init__(self, host):
+            self.host = host
+
+        def __len__(self):
+            return len(self.host)
+
+        def __getitem__(self, i):
+            return self.host[i].cuda()
+
+    p = prompts[0]
+    s = spf.Selector(*GEOM, 3000).run(p.q, Lazy(p._k), p.token_ids, p.char_start, p.char_end, 0.3)
+    torch.testing.assert_close(s.importance, got[0].importance, rtol=1e-5, atol=0)
+    with pytest.raises(TypeError):                         # one pass over an iterator is all there is: refused
+        spf.Selector(*GEOM, 3000).run(p.q, iter(p.k), p.token_ids, p.char_start, p.char_end, 0.3)
