@@ -70,6 +70,11 @@ Ref attr(PyObject* o, PyObject* name) { return Ref(PyObject_GetAttr(o, name)); }
 at::Tensor attr_tensor(PyObject* o, PyObject* name, at::ScalarType dtype, const char* what) {
   return device_tensor(attr(o, name).p, dtype, what);
 }
+// The same for a buffer that may be None: an undefined tensor.
+at::Tensor attr_tensor_or_none(PyObject* o, PyObject* name, at::ScalarType dtype, const char* what) {
+  const Ref value = attr(o, name);
+  return value.p == Py_None ? at::Tensor() : device_tensor(value.p, dtype, what);
+}
 int64_t attr_int(PyObject* o, PyObject* name) {
   const int64_t v = PyLong_AsLongLong(attr(o, name).p);
   if (v == -1 && PyErr_Occurred()) throw PyFailure{};
@@ -193,7 +198,7 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
     raise(PyExc_ValueError, "lse must be contiguous fp32 [L, Hq, m]");
   const at::Tensor kept = attr_tensor(slot, N.kept, at::kInt, "kept_chunks");
   const at::Tensor out_ids = attr_tensor(slot, N.out_ids, at::kInt, "out_ids");
-  const at::Tensor out_pos = attr_tensor(slot, N.out_pos, at::kInt, "out_pos");
+  const at::Tensor out_pos = attr_tensor_or_none(slot, N.out_pos, at::kInt, "out_pos");
   const at::Tensor tok = attr_tensor(slot, N.tok_spans, at::kInt, "out_tok_spans");
   const at::Tensor ch = attr_tensor(slot, N.char_spans, at::kInt, "out_char_spans");
   const at::Tensor counts = attr_tensor(slot, N.counts, at::kLong, "out_counts");
@@ -201,7 +206,7 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   const at::Tensor& cs = device_tensor(char_start, at::kInt, "char_start");
   const at::Tensor& ce = device_tensor(char_end, at::kInt, "char_end");
   const int64_t need = std::min(b->k * chunk, n);
-  if (scores.numel() < b->n_chunks || kept.numel() < b->k || out_ids.numel() < need || out_pos.numel() < need || tok.numel() < 2 * b->k ||
+  if (scores.numel() < b->n_chunks || kept.numel() < b->k || out_ids.numel() < need || (out_pos.defined() && out_pos.numel() < need) || tok.numel() < 2 * b->k ||
       ch.numel() < 2 * b->k || counts.numel() < 2 || std::min(std::min(i.numel(), cs.numel()), ce.numel()) < n)
     raise(PyExc_ValueError, "a buffer is smaller than include/spf.h requires");
   b->importance = importance.narrow(0, 0, n);
@@ -212,7 +217,7 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   b->lse_ptr = lse.data_ptr<float>();
   b->kept = kept.data_ptr<int32_t>();
   b->out_ids = out_ids.data_ptr<int32_t>();
-  b->out_pos = out_pos.data_ptr<int32_t>();
+  b->out_pos = out_pos.defined() ? out_pos.data_ptr<int32_t>() : nullptr;
   b->tok_spans = tok.data_ptr<int32_t>();
   b->char_spans = ch.data_ptr<int32_t>();
   b->counts = counts.data_ptr<int64_t>();
@@ -277,8 +282,8 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     const bool force_first = attr_true(selector, N.force_first), force_last = attr_true(selector, N.force_last);
     Buffers b;
     read_buffers(selector, shape, in.n, chunk, keep, force_first, force_last, args[6], args[7], args[8], &b);
-    const at::Tensor dev_status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status");
-    int32_t* status = dev_status.data_ptr<int32_t>();
+    const at::Tensor dev_status = attr_tensor_or_none(selector, N.dev_status, at::kInt, "dev_status");
+    int32_t* status = dev_status.defined() ? dev_status.data_ptr<int32_t>() : nullptr;
     void* stream = stream_of(args[10], b.importance);
 
     spf_prompt plain{in.n, in.layers.data(), in.stride_head, in.stride_tok, in.q, b.importance_ptr, b.lse_ptr};
@@ -345,8 +350,8 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
       p[i] = spf_prompt{n, in[i].layers.data(), in[i].stride_head, in[i].stride_tok, in[i].q, b[i].importance_ptr, b[i].lse_ptr};
       items[i] = path_item(b[i], n);
     }
-    const at::Tensor dev_status = attr_tensor(selector, N.dev_status, at::kInt, "dev_status");
-    int32_t* status = dev_status.data_ptr<int32_t>();
+    const at::Tensor dev_status = attr_tensor_or_none(selector, N.dev_status, at::kInt, "dev_status");
+    int32_t* status = dev_status.defined() ? dev_status.data_ptr<int32_t>() : nullptr;
     void* stream = stream_of(args[3], b[0].importance);
     const size_t need = spf_score_workspace_bytes(&shape, p.data(), (int32_t)count);
     if (need == 0) return result_tuple(SPF_ERR_INVALID_ARG, "spf_score_workspace_bytes", nullptr, 0);

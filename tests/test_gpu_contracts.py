@@ -59,3 +59,18 @@ def test_tensors_made_for_the_call_live_until_it_is_enqueued():
     torch.testing.assert_close(s.importance, got[0].importance, rtol=1e-5, atol=0)
     with pytest.raises(TypeError):                         # one pass over an iterator is all there is: refused
         spf.Selector(*GEOM, 3000).run(p.q, iter(p.k), p.token_ids, p.char_start, p.char_end, 0.3)
+
+
+def test_positions_and_status_are_optional():
+    """spf_compact_spans takes no positions and spf_score no status; a selector whose buffer is None asks for neither."""
+    import paper_2603_02631_b200 as spf
+    q, k = make(700)
+    full, bare = spf.Selector(*GEOM, 700), spf.Selector(*GEOM, 700)
+    bare.out_pos = bare.dev_status = None
+    want, got = full.run(q, k, *text(700), 0.3), bare.run(q, k, *text(700), 0.3)
+    kept = int(want.counts[0])
+    assert torch.equal(want.out_ids[:kept], got.out_ids[:kept]) and got.out_pos is None
+    batch, p = spf.BatchSelector(*GEOM, [700]), Fresh(700, 0)
+    batch.slots[0].out_pos = batch.dev_status = None
+    got = batch.run([p], 0.3)[0]
+    assert torch.equal(want.out_ids[:kept], got.out_ids[:kept])
