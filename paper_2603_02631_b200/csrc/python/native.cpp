@@ -187,6 +187,7 @@ void read_buffers(PyObject* slot, const spf_shape& shape, int64_t n, int64_t chu
   const int64_t max_tokens = attr_int(slot, N.max_tokens);
   if (n > max_tokens)
     raise(PyExc_ValueError, "prompt has " + std::to_string(n) + " tokens, selector was sized for " + std::to_string(max_tokens));
+  if (chunk < 1 || chunk > INT32_MAX || n < 0) raise(PyExc_ValueError, "chunk must be in [1, 2^31) and n_tokens not negative");
   b->n_chunks = (n + chunk - 1) / chunk;
   b->k = spf_keep_count(b->n_chunks, keep);
   if (force_first || force_last) b->k = std::max(b->k, (int64_t)(force_first ? 1 : 0) + (force_last && (b->n_chunks > 1 || !force_first) ? 1 : 0));
@@ -277,7 +278,8 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     spf_shape shape{};
     Inputs in;
     read_inputs(kind, args[2], args[3], args[4], n_paged, attr_float(selector, N.softmax_scale), true, &shape, &in);
-    const int32_t chunk = (int32_t)attr_int(selector, N.chunk), pool = (int32_t)attr_int(selector, N.pool_kernel);
+    const int64_t chunk = attr_int(selector, N.chunk);
+    const int32_t pool = (int32_t)attr_int(selector, N.pool_kernel);
     const int32_t edge = (int32_t)attr_int(selector, N.pool_edge_rule);
     const bool force_first = attr_true(selector, N.force_first), force_last = attr_true(selector, N.force_last);
     Buffers b;
@@ -307,7 +309,7 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     if (st == SPF_OK) {
       where = "spf_pool_select_compact";
       const spf_path_item item = path_item(b, in.n);
-      st = spf_pool_select_compact(&item, 1, pool, chunk, edge, force_first, force_last, stream);
+      st = spf_pool_select_compact(&item, 1, pool, (int32_t)chunk, edge, force_first, force_last, stream);
     }
     Py_END_ALLOW_THREADS;
     return result_tuple(st, where, &b, 1);
@@ -332,7 +334,8 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     Ref slot_items(PySequence_Fast(slots.p, "slots must be a sequence"));
     if (count > (size_t)PySequence_Fast_GET_SIZE(slot_items.p)) raise(PyExc_ValueError, "more prompts than slots");
     if (count == 0) raise(PyExc_IndexError, "no prompts");
-    const int32_t chunk = (int32_t)attr_int(selector, N.chunk), pool = (int32_t)attr_int(selector, N.pool_kernel);
+    const int64_t chunk = attr_int(selector, N.chunk);
+    const int32_t pool = (int32_t)attr_int(selector, N.pool_kernel);
     const double scale = attr_float(selector, N.softmax_scale);
     spf_shape shape{};
     std::vector<Inputs> in(count);
@@ -365,7 +368,7 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     st = spf_score(&shape, p.data(), (int32_t)count, ws_ptr, ws_bytes, status, stream);
     if (st == SPF_OK) {
       where = "spf_pool_select_compact";
-      st = spf_pool_select_compact(items.data(), (int32_t)count, pool, chunk, 0, 0, 0, stream);
+      st = spf_pool_select_compact(items.data(), (int32_t)count, pool, (int32_t)chunk, 0, 0, 0, stream);
     }
     Py_END_ALLOW_THREADS;
     return result_tuple(st, where, b.data(), count);

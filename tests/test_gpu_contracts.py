@@ -74,3 +74,16 @@ def test_positions_and_status_are_optional():
     batch.slots[0].out_pos = batch.dev_status = None
     got = batch.run([p], 0.3)[0]
     assert torch.equal(want.out_ids[:kept], got.out_ids[:kept])
+
+
+@pytest.mark.parametrize("chunk", [0, -3, 1 << 32, (1 << 32) + 32])
+def test_selector_refuses_chunks_that_make_no_sense(chunk):
+    """Read on every call: the attribute can be set after construction.  2^32 is zero in 32 bits, 2^32 + 32 is 32."""
+    import paper_2603_02631_b200 as spf
+    q, k = make(300)
+    sel, batch = spf.Selector(*GEOM, 300), spf.BatchSelector(*GEOM, [300])
+    sel.chunk = batch.chunk = chunk
+    with pytest.raises(ValueError):
+        sel.run(q, k, *text(300), 0.3)
+    with pytest.raises(ValueError):
+        batch.run([Fresh(300, 0)], 0.3)
