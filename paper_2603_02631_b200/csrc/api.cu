@@ -4,7 +4,6 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include "common.cuh"
 #include "score.cuh"
@@ -87,46 +86,83 @@ int32_t device_sm_count(int* out) {
   return SPF_OK;
 }
 
-// Scratch that a call with these prompts may use: the general path works on one prompt at a time, the fused path on up to
+// Scratch that a call with some prompts may use: the general path works on one prompt at a time, the fused path on up to
 // kFusedMaxBatch consecutive ones.
-size_t workspace_need(const ScoreProblem* p, int32_t n) {
-  size_t need = 0, window = 0;
-  for (int32_t i = 0; i < n; ++i) {
-    window += score_fused_workspace_bytes(p[i]);
-    if (i >= kFusedMaxBatch) window -= score_fused_workspace_bytes(p[i - kFusedMaxBatch]);
-    need = std::max(need, std::max(score_mma_workspace_bytes(p[i]), window));
+class ScratchNeed {
+ public:
+  void add(const ScoreProblem& p) {
+    const size_t fused = score_fused_workspace_bytes(p);
+    window_ += fused - recent_[count_ % kFusedMaxBatch];
+    recent_[count_++ % kFusedMaxBatch] = fused;
+    most_ = std::max(most_, std::max(score_mma_workspace_bytes(p), window_));
   }
-  return need;
-}
+  size_t most() const { return most_; }
 
-int32_t check_workspace(const char* who, const ScoreProblem* p, int32_t n, const void* workspace, size_t workspace_bytes) {
-  const size_t need = workspace_need(p, n);
+ private:
+  size_t recent_[kFusedMaxBatch] = {}, window_ = 0, most_ = 0;
+  int64_t count_ = 0;
+};
+
+int32_t check_workspace(const char* who, const ScratchNeed& need, const void* workspace, size_t workspace_bytes) {
   if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
     return fail(SPF_ERR_WORKSPACE, "%s: workspace is null or not 256-byte aligned", who);
-  if (workspace_bytes < need) return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need);
+  if (workspace_bytes < need.most())
+    return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need.most());
   return SPF_OK;
 }
 
-// Scores validated prompts: runs of consecutive prompts that the fused kernel takes go to it together, the others one by
-// one to the general kernels.
-int32_t score_problems(const char* who, const ScoreProblem* p, int32_t n, int path, void* workspace, size_t workspace_bytes,
-                       int32_t* dev_status, cudaStream_t stream) {
-  int32_t st = check_workspace(who, p, n, workspace, workspace_bytes);
+// The three forms of a prompt (contiguous, paged, 8-bit keys) differ in how they become a ScoreProblem; everything else is
+// shared.  Problems are made where they are needed, a launch's worth at a time: a call allocates nothing on the host, however
+// many prompts it has.
+template <class Prompt>
+using MakeProblem = int32_t (*)(const spf_shape*, const Prompt&, int32_t index, ScoreProblem*);
+
+template <class Prompt>
+int32_t check_problems(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n, MakeProblem<Prompt> make, ScratchNeed* need) {
+  clear_error();
+  if (shape == nullptr || prompts == nullptr || n < 1) return fail(SPF_ERR_INVALID_ARG, "%s: null argument or n_prompts < 1", who);
+  for (int32_t i = 0; i < n; ++i) {
+    ScoreProblem p;
+    const int32_t st = make(shape, prompts[i], i, &p);
+    if (st != SPF_OK) return st;
+    need->add(p);
+  }
+  return SPF_OK;
+}
+
+template <class Prompt>
+size_t workspace_bytes_for(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n, MakeProblem<Prompt> make) {
+  ScratchNeed need;
+  return check_problems(who, shape, prompts, n, make, &need) == SPF_OK ? need.most() : 0;
+}
+
+// Validates the prompts, then scores them: consecutive prompts that the fused kernel takes go to it together, the others one
+// by one to the general kernels.
+template <class Prompt>
+int32_t score_prompts(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n, MakeProblem<Prompt> make, int path,
+                      const float* const* extra_lse, void* workspace, size_t workspace_bytes, int32_t* dev_status, cudaStream_t stream) {
+  ScratchNeed need;
+  int32_t st = check_problems(who, shape, prompts, n, make, &need);
+  if (st != SPF_OK) return st;
+  st = check_workspace(who, need, workspace, workspace_bytes);
   if (st != SPF_OK) return st;
   int sm_count = 0;
   st = device_sm_count(&sm_count);
   if (st != SPF_OK) return st;
   for (int32_t i = 0; i < n;) {
-    int32_t j = i;
-    while (j < n && (path == 2 || (path == 0 && score_fused_supported(p[j], sm_count)))) ++j;
-    if (j > i) {
-      st = score_fused_launch(p + i, j - i, workspace, sm_count, dev_status, stream);
-      i = j;
-    } else {
-      st = score_mma_launch(p[i], workspace, sm_count, stream);
-      ++i;
+    ScoreProblem p[kFusedMaxBatch];
+    int count = 0;                                       // prompts from i on that the fused kernel takes
+    bool fused = true;
+    for (; fused && count < kFusedMaxBatch && i + count < n; count += fused) {
+      make(shape, prompts[i + count], i + count, &p[count]);
+      if (extra_lse != nullptr) p[count].extra_lse = extra_lse[i + count];
+      fused = path == 2 || (path == 0 && score_fused_supported(p[count], sm_count));
     }
+    int done = 1;
+    st = count > 0 ? score_fused_launch(p, count, workspace, sm_count, dev_status, stream, &done)
+                   : score_mma_launch(p[0], workspace, sm_count, stream);
     if (st != SPF_OK) return st;
+    i += done;
   }
   return SPF_OK;
 }
@@ -147,41 +183,19 @@ void clear_error() { g_error[0] = '\0'; }
 
 using namespace spf;
 
-// The three forms of a prompt (contiguous, paged, 8-bit keys) differ in how they become a ScoreProblem; everything else is
-// shared.
-template <class Prompt, class Make>
-static int32_t make_problems(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n_prompts, Make make,
-                             std::vector<ScoreProblem>* out) {
-  clear_error();
-  if (shape == nullptr || prompts == nullptr || n_prompts < 1)
-    return fail(SPF_ERR_INVALID_ARG, "%s: null argument or n_prompts < 1", who);
-  out->resize((size_t)n_prompts);
-  for (int32_t i = 0; i < n_prompts; ++i) {
-    const int32_t st = make(shape, prompts[i], i, &(*out)[i]);
-    if (st != SPF_OK) return st;
-  }
-  return SPF_OK;
-}
-
 static int32_t make_flat_problem(const spf_shape* shape, const spf_prompt& pr, int32_t index, ScoreProblem* out) {
   return make_problem(shape, pr, index, out);
 }
 
 extern "C" size_t spf_score_workspace_bytes(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts) {
-  std::vector<ScoreProblem> p;
-  if (make_problems("spf_score_workspace_bytes", shape, prompts, n_prompts, make_flat_problem, &p) != SPF_OK) return 0;
-  return workspace_need(p.data(), n_prompts);
+  return workspace_bytes_for("spf_score_workspace_bytes", shape, prompts, n_prompts, make_flat_problem);
 }
 
 static int32_t score_impl(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts, const float* const* extra_lse,
                           void* workspace, size_t workspace_bytes, int32_t* dev_status, void* cuda_stream, int path_override = -1) {
-  std::vector<ScoreProblem> p;
-  const int32_t st = make_problems("spf_score", shape, prompts, n_prompts, make_flat_problem, &p);
-  if (st != SPF_OK) return st;
-  for (int32_t i = 0; i < n_prompts && extra_lse != nullptr; ++i) p[i].extra_lse = extra_lse[i];
   const int path = path_override >= 0 ? path_override : g_score_path.load(std::memory_order_relaxed);
-  return score_problems("spf_score", p.data(), n_prompts, path, workspace, workspace_bytes, dev_status,
-                        static_cast<cudaStream_t>(cuda_stream));
+  return score_prompts("spf_score", shape, prompts, n_prompts, make_flat_problem, path, extra_lse, workspace, workspace_bytes, dev_status,
+                       static_cast<cudaStream_t>(cuda_stream));
 }
 
 namespace spf {
@@ -228,18 +242,13 @@ static int32_t make_paged_problem(const spf_shape* shape, const spf_paged_prompt
 }
 
 extern "C" size_t spf_score_paged_workspace_bytes(const spf_shape* shape, const spf_paged_prompt* prompts, int32_t n_prompts) {
-  std::vector<ScoreProblem> p;
-  if (make_problems("spf_score_paged_workspace_bytes", shape, prompts, n_prompts, make_paged_problem, &p) != SPF_OK) return 0;
-  return workspace_need(p.data(), n_prompts);
+  return workspace_bytes_for("spf_score_paged_workspace_bytes", shape, prompts, n_prompts, make_paged_problem);
 }
 
 extern "C" int32_t spf_score_paged(const spf_shape* shape, const spf_paged_prompt* prompts, int32_t n_prompts, void* workspace,
                                    size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
-  std::vector<ScoreProblem> p;
-  const int32_t st = make_problems("spf_score_paged", shape, prompts, n_prompts, make_paged_problem, &p);
-  if (st != SPF_OK) return st;
-  return score_problems("spf_score_paged", p.data(), n_prompts, g_score_path.load(std::memory_order_relaxed), workspace, workspace_bytes,
-                        dev_status, static_cast<cudaStream_t>(cuda_stream));
+  return score_prompts("spf_score_paged", shape, prompts, n_prompts, make_paged_problem, g_score_path.load(std::memory_order_relaxed), nullptr,
+                       workspace, workspace_bytes, dev_status, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // 8-bit key cache: described as a bf16 prompt over the same pointers (the checks are the same: strides count elements,
@@ -261,18 +270,13 @@ static int32_t make_fp8_problem(const spf_shape* shape, const spf_fp8_prompt& fp
 }
 
 extern "C" size_t spf_score_fp8_workspace_bytes(const spf_shape* shape, const spf_fp8_prompt* prompts, int32_t n_prompts) {
-  std::vector<ScoreProblem> p;
-  if (make_problems("spf_score_fp8_workspace_bytes", shape, prompts, n_prompts, make_fp8_problem, &p) != SPF_OK) return 0;
-  return workspace_need(p.data(), n_prompts);
+  return workspace_bytes_for("spf_score_fp8_workspace_bytes", shape, prompts, n_prompts, make_fp8_problem);
 }
 
 extern "C" int32_t spf_score_fp8(const spf_shape* shape, const spf_fp8_prompt* prompts, int32_t n_prompts, void* workspace,
                                    size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
-  std::vector<ScoreProblem> p;
-  const int32_t st = make_problems("spf_score_fp8", shape, prompts, n_prompts, make_fp8_problem, &p);
-  if (st != SPF_OK) return st;
-  return score_problems("spf_score_fp8", p.data(), n_prompts, g_score_path.load(std::memory_order_relaxed), workspace, workspace_bytes,
-                        dev_status, static_cast<cudaStream_t>(cuda_stream));
+  return score_prompts("spf_score_fp8", shape, prompts, n_prompts, make_fp8_problem, g_score_path.load(std::memory_order_relaxed), nullptr,
+                       workspace, workspace_bytes, dev_status, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // Key-sharded scoring: the two sweeps of the general path as separate calls.
@@ -294,14 +298,16 @@ static int32_t score_shard(const spf_shape* shape, const spf_prompt* prompt, int
   if (st != SPF_OK) return st;
   if (phase == 1) p.importance = nullptr;
   if (phase == 2) p.lse_out = nullptr;
-  const int32_t ws = check_workspace(who, &p, 1, workspace, workspace_bytes);
+  ScratchNeed need;
+  need.add(p);
+  const int32_t ws = check_workspace(who, need, workspace, workspace_bytes);
   if (ws != SPF_OK) return ws;
   int sm_count = 0;
   const int32_t sc = device_sm_count(&sm_count);
   if (sc != SPF_OK) return sc;
   const int path = g_score_path.load(std::memory_order_relaxed);
   if (allow_fused && (path == 2 || (path == 0 && score_fused_supported(p, sm_count))))
-    return score_fused_launch(&p, 1, workspace, sm_count, dev_status, static_cast<cudaStream_t>(cuda_stream), phase, lse_in);
+    return score_fused_launch(&p, 1, workspace, sm_count, dev_status, static_cast<cudaStream_t>(cuda_stream), nullptr, phase, lse_in);
   return score_mma_launch_phase(p, workspace, sm_count, phase, lse_in, static_cast<cudaStream_t>(cuda_stream));
 }
 

@@ -595,34 +595,29 @@ bool score_fused_supported(const ScoreProblem& p, int sm_count) { return geometr
 
 size_t score_fused_workspace_bytes(const ScoreProblem& p) { return fused_workspace(p).total; }
 
-// Scores prompts of one geometry, as many per launch as L2 holds; a launch's workspace is its prompts' one after the other.
 int32_t score_fused_launch(const ScoreProblem* p, int n_prompts, void* workspace, int sm_count, int32_t* dev_status, cudaStream_t stream,
-                           int mode, const float* lse_in) {
+                           int* done, int mode, const float* lse_in) {
   sm_count = std::min(sm_count, kFusedMaxCtas);
-  char* base = static_cast<char*>(workspace);
-  for (int first = 0; first < n_prompts;) {
-    Geometry g;
-    int64_t n_tiles[kFusedMaxBatch];
-    int n = 0;
-    for (; n < kFusedMaxBatch && first + n < n_prompts; ++n) {
-      const Geometry gi = geometry(p[first + n], sm_count);
-      if (!gi.ok) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
-      if (n > 0 && gi.once != g.once) break;          // a prompt too long for the resident form goes by itself
-      g = gi;
-      n_tiles[n] = ceil_div(p[first + n].n_tokens, kTileKeys);
-    }
-    n = group_size(g, n_tiles, n, sm_count);
-    Split split[kFusedMaxBatch];
-    if (!split_group(g, n_tiles, n, sm_count, split)) {
-      n = 1;
-      if (!split_group(g, n_tiles, 1, sm_count, split)) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
-    }
-    const int32_t st = n == 1 ? launch_group<1>(p + first, n, g, split, base, sm_count, dev_status, stream, mode, lse_in)
-                              : launch_group<kFusedMaxBatch>(p + first, n, g, split, base, sm_count, dev_status, stream, mode, lse_in);
-    if (st != SPF_OK) return st;
-    first += n;                                       // the next launch runs after this one and may use the same scratch
+  Geometry g;
+  int64_t n_tiles[kFusedMaxBatch];
+  int n = 0;
+  for (; n < std::min(n_prompts, kFusedMaxBatch); ++n) {
+    const Geometry gi = geometry(p[n], sm_count);
+    if (n > 0 && (!gi.ok || gi.once != g.once)) break;  // refused, or scored in the other form, when its turn comes
+    if (!gi.ok) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
+    g = gi;
+    n_tiles[n] = ceil_div(p[n].n_tokens, kTileKeys);
   }
-  return SPF_OK;
+  n = group_size(g, n_tiles, n, sm_count);
+  Split split[kFusedMaxBatch];
+  if (!split_group(g, n_tiles, n, sm_count, split)) {
+    n = 1;
+    if (!split_group(g, n_tiles, 1, sm_count, split)) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
+  }
+  if (done != nullptr) *done = n;
+  char* base = static_cast<char*>(workspace);
+  return n == 1 ? launch_group<1>(p, n, g, split, base, sm_count, dev_status, stream, mode, lse_in)
+                : launch_group<kFusedMaxBatch>(p, n, g, split, base, sm_count, dev_status, stream, mode, lse_in);
 }
 
 }  // namespace spf
