@@ -83,9 +83,10 @@ typedef struct {
 } spf_prompt;
 
 /*
- * Bytes of scratch spf_score needs for these prompts (0 on invalid arguments; the reason is left in
- * spf_last_error()).  The scratch holds packed queries, per-split softmax partials and row
- * log-sum-exps; one buffer serves all prompts of the call in turn.
+ * Bytes of scratch with which spf_score scores these prompts at full speed (0 on invalid arguments; the reason is left in
+ * spf_last_error()): up to 16 consecutive prompts share a launch of the fused path, each with scratch of its own (queries as
+ * the tensor cores read them, row sums and log-sum-exps, running maxima).  spf_score also takes less, down to the bytes
+ * that this call gives for each prompt alone: then fewer prompts share a launch, and one buffer serves them in turn.
  */
 SPF_API size_t spf_score_workspace_bytes(const spf_shape* shape, const spf_prompt* prompts, int32_t n_prompts);
 
@@ -99,9 +100,9 @@ SPF_API size_t spf_score_workspace_bytes(const spf_shape* shape, const spf_promp
  * bf16 inputs, fp32 accumulation and softmax.  The attention tensor itself is never stored.
  *
  * `shape`, `prompts` and the k_layers arrays are HOST memory, read during the call only.
- * `workspace`: device, 256-byte aligned, at least spf_score_workspace_bytes(...) bytes; contents on
- * entry are irrelevant, contents on exit unspecified.  Calls that share a workspace must be ordered
- * on one stream.
+ * `workspace`: device, 256-byte aligned, spf_score_workspace_bytes(...) bytes, or at least what that call
+ * gives for the most demanding prompt alone; contents on entry are irrelevant, contents on exit
+ * unspecified.  Calls that share a workspace must be ordered on one stream.
  * `dev_status`: device int32, may be NULL (device-side conditions then go unreported).  Kernels store a
  * negative spf_status there when a device-side condition occurs; they never trap.  The caller zeroes it
  * before the call and reads it after synchronising.  Conditions:

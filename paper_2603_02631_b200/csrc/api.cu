@@ -86,28 +86,31 @@ int32_t device_sm_count(int* out) {
   return SPF_OK;
 }
 
-// Scratch that a call with some prompts may use: the general path works on one prompt at a time, the fused path on up to
-// kFusedMaxBatch consecutive ones.
+// Scratch for a call with some prompts.  The general path works on one prompt at a time, the fused path on up to kFusedMaxBatch
+// consecutive ones: `most` is what lets it.  `least` is enough: fewer prompts then share a launch, down to one.
 class ScratchNeed {
  public:
   void add(const ScoreProblem& p) {
     const size_t fused = score_fused_workspace_bytes(p);
     window_ += fused - recent_[count_ % kFusedMaxBatch];
     recent_[count_++ % kFusedMaxBatch] = fused;
-    most_ = std::max(most_, std::max(score_mma_workspace_bytes(p), window_));
+    const size_t alone = std::max(score_mma_workspace_bytes(p), fused);
+    least_ = std::max(least_, alone);
+    most_ = std::max(most_, std::max(alone, window_));
   }
+  size_t least() const { return least_; }
   size_t most() const { return most_; }
 
  private:
-  size_t recent_[kFusedMaxBatch] = {}, window_ = 0, most_ = 0;
+  size_t recent_[kFusedMaxBatch] = {}, window_ = 0, least_ = 0, most_ = 0;
   int64_t count_ = 0;
 };
 
 int32_t check_workspace(const char* who, const ScratchNeed& need, const void* workspace, size_t workspace_bytes) {
   if (workspace == nullptr || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)
     return fail(SPF_ERR_WORKSPACE, "%s: workspace is null or not 256-byte aligned", who);
-  if (workspace_bytes < need.most())
-    return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need.most());
+  if (workspace_bytes < need.least())
+    return fail(SPF_ERR_WORKSPACE, "%s: workspace has %zu bytes, %zu needed", who, workspace_bytes, need.least());
   return SPF_OK;
 }
 
@@ -136,8 +139,8 @@ size_t workspace_bytes_for(const char* who, const spf_shape* shape, const Prompt
   return check_problems(who, shape, prompts, n, make, &need) == SPF_OK ? need.most() : 0;
 }
 
-// Validates the prompts, then scores them: consecutive prompts that the fused kernel takes go to it together, the others one
-// by one to the general kernels.
+// Validates the prompts, then scores them: consecutive prompts that the fused kernel takes go to it together, as many as the
+// workspace holds, the others one by one to the general kernels.
 template <class Prompt>
 int32_t score_prompts(const char* who, const spf_shape* shape, const Prompt* prompts, int32_t n, MakeProblem<Prompt> make, int path,
                       const float* const* extra_lse, void* workspace, size_t workspace_bytes, int32_t* dev_status, cudaStream_t stream) {
@@ -152,11 +155,12 @@ int32_t score_prompts(const char* who, const spf_shape* shape, const Prompt* pro
   for (int32_t i = 0; i < n;) {
     ScoreProblem p[kFusedMaxBatch];
     int count = 0;                                       // prompts from i on that the fused kernel takes
-    bool fused = true;
-    for (; fused && count < kFusedMaxBatch && i + count < n; count += fused) {
+    size_t used = 0;
+    for (bool next = true; next && count < kFusedMaxBatch && i + count < n; count += next) {
       make(shape, prompts[i + count], i + count, &p[count]);
       if (extra_lse != nullptr) p[count].extra_lse = extra_lse[i + count];
-      fused = path == 2 || (path == 0 && score_fused_supported(p[count], sm_count));
+      used += score_fused_workspace_bytes(p[count]);     // the first always fits
+      next = (path == 2 || (path == 0 && score_fused_supported(p[count], sm_count))) && used <= workspace_bytes;
     }
     int done = 1;
     st = count > 0 ? score_fused_launch(p, count, workspace, sm_count, dev_status, stream, &done)

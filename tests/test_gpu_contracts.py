@@ -87,3 +87,30 @@ def test_selector_refuses_chunks_that_make_no_sense(chunk):
         sel.run(q, k, *text(300), 0.3)
     with pytest.raises(ValueError):
         batch.run([Fresh(300, 0)], 0.3)
+
+
+def test_a_batch_is_scored_with_a_workspace_for_its_longest_prompt():
+    """Fewer prompts share a launch, at every size of the workspace between that and the whole batch's."""
+    import paper_2603_02631_b200 as spf
+    lens = [300, 5000, 17, 2500, 5000, 128, 1, 900, 64, 3000, 700, 31, 4000, 222, 1500, 90, 2047, 640]
+    bufs = []
+    for i, n in enumerate(lens):
+        q, k = make(n, i)
+        bufs.append(spf.PromptBuffers(q, k, torch.empty(n, device="cuda"), torch.empty(2 * 4 * 8, device="cuda")))
+    want = []
+    for b in bufs:
+        spf.spf_score([b], torch.empty(spf.spf_score_workspace_bytes([b]), dtype=torch.uint8, device="cuda"))
+        want.append((b.importance.clone(), b.lse.clone()))
+    least, most = max(spf.spf_score_workspace_bytes([b]) for b in bufs), spf.spf_score_workspace_bytes(bufs)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for size in (least, least + 256, (least + most) // 2, most):
+        for b in bufs:
+            b.importance.fill_(-1)
+            b.lse.fill_(-1)
+        ws = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        ws[size:] = 77
+        spf.spf_score(bufs, ws[:size], dev_status=status)
+        assert int(status) == 0 and bool((ws[size:] == 77).all())
+        for b, (importance, lse) in zip(bufs, want):
+            torch.testing.assert_close(b.importance, importance, rtol=1e-5, atol=0)
+            torch.testing.assert_close(b.lse, lse, rtol=1e-5, atol=1e-5)

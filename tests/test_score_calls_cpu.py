@@ -28,3 +28,33 @@ def test_a_batch_of_any_size_is_refused_with_a_status():
     an exception that left the C entry would end it.)"""
     proc = subprocess.run([sys.executable, "-c", HUGE], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert proc.returncode == 0, proc.stderr[-2000:]
+
+
+WORKSPACE = """
+import ctypes, paper_2603_02631_b200 as spf
+from paper_2603_02631_b200 import binding as b
+L = 4
+shape = b._Shape(L, 16, 4, 64, 8, 0.0)
+layers = (ctypes.c_void_p * L)(*([1 << 20] * L))
+lp = ctypes.cast(layers, ctypes.POINTER(ctypes.c_void_p))
+p = 1 << 20
+make = {"": lambda n: b._Prompt(n, lp, n * 64, 64, p, p, None), "_paged": lambda n: b._PagedPrompt(n, lp, 4096, 128, p, p, p, None),
+        "_fp8": lambda n: b._Fp8Prompt(n, lp, n * 64, 64, p, p, p, None)}
+lens = [300, 40000, 17, 25000, 40000, 128] * 5
+for form, one in make.items():
+    score, size = getattr(spf.lib, "spf_score" + form), getattr(spf.lib, "spf_score" + form + "_workspace_bytes")
+    batch = (type(one(1)) * len(lens))(*[one(n) for n in lens])
+    alone = max(size(ctypes.byref(shape), (type(one(1)) * 1)(one(n)), 1) for n in set(lens))
+    together = size(ctypes.byref(shape), batch, len(lens))
+    assert 0 < alone < together
+    # without a device a call that gets past the checks ends with SPF_ERR_CUDA
+    assert score(ctypes.byref(shape), batch, len(lens), 256, together, None, None) == -4
+    assert score(ctypes.byref(shape), batch, len(lens), 256, alone, None, None) == -4, form
+    assert score(ctypes.byref(shape), batch, len(lens), 256, alone - 1, None, None) == -3
+"""
+
+
+def test_a_workspace_for_the_longest_prompt_is_enough_for_a_batch():
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="")       # the pointers are made up: no device may be reached
+    proc = subprocess.run([sys.executable, "-c", WORKSPACE], cwd=ROOT, env=env, capture_output=True, text=True, timeout=300)
+    assert proc.returncode == 0, proc.stderr[-2000:]
