@@ -221,6 +221,12 @@ struct Geometry {
     return std::min(kMaxResident, (kTmemColsAll - (max_in_regs(tiles) ? 0 : tiles * (ncols / padded_group))) / ncols);
   }
   bool max_in_regs(int tiles) const { return tiles <= kRegTiles && ncols / padded_group <= kRegSlots; }
+  bool holds(int64_t tiles) const { return tiles <= max_tiles && (!once || resident((int)tiles) > tiles); }   // of a CTA and slab
+  int most_tiles() const {
+    int t = 1;
+    while (holds(t + 1)) ++t;
+    return t;
+  }
   // Most tiles a CTA and slab that leave the two visits room to overlap.
   int comfortable_tiles() const {
     if (!once) return std::max(1, (lead - handover) / 2);           // visit 2 takes as long as visit 1
@@ -293,7 +299,7 @@ Split best_split(const Geometry& g, int64_t n_tiles, int ctas, int share) {
   for (int parts = 1; parts <= std::min(ctas, g.n_slabs); ++parts) {
     const int most = (int)std::min<int64_t>(ctas / parts, n_tiles);
     const int64_t tiles = ceil_div(n_tiles, most);
-    if (tiles > g.max_tiles || (g.once && g.resident((int)tiles) < tiles + 1)) break;
+    if (!g.holds(tiles)) break;
     const int per_part = (int)ceil_div(n_tiles, tiles);              // no more CTAs than these tiles need
     const double cost = split_cost(g, n_tiles, (int)tiles, parts, per_part, share);
     if (best.cost < 0 || cost < best.cost * 0.999) {
@@ -306,69 +312,70 @@ Split best_split(const Geometry& g, int64_t n_tiles, int ctas, int share) {
   return best;
 }
 
-// Splits a group of prompts over the SMs, each on CTAs of its own: CTAs in proportion to the tiles, then a few moves from
+// Splits a group of prompts, as group_size made it, over the SMs, each on CTAs of its own: CTAs in proportion to the tiles, but
+// as many as hold them (what that hands out too many comes from the prompts with the most to spare), then a few moves from
 // the prompt that would be done first to the one that would be done last.
 bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count, Split* out) {
   if (n == 1) {
     out[0] = best_split(g, n_tiles[0], sm_count, sm_count);
     return out[0].cost >= 0;
   }
+  const int most = g.most_tiles();
   int64_t total = 0;
   for (int i = 0; i < n; ++i) total += n_tiles[i];
-  int ctas[kFusedMaxBatch], left = sm_count;
-  for (int i = 0; i < n; ++i) left -= ctas[i] = std::max(1, (int)(n_tiles[i] * sm_count / total));
-  auto fit = [&](int i) {
-    out[i] = best_split(g, n_tiles[i], ctas[i], ctas[i]);
-    return out[i].cost >= 0;
-  };
-  for (int i = 0; i < n; ++i)
-    if (!fit(i)) out[i].cost = 1e30;                                 // not with so few: the moves below give it more
+  int least[kFusedMaxBatch], ctas[kFusedMaxBatch], left = sm_count;
+  for (int i = 0; i < n; ++i) {
+    least[i] = (int)ceil_div(n_tiles[i], most);
+    left -= ctas[i] = std::max(least[i], (int)(n_tiles[i] * sm_count / total));
+  }
+  for (; left < 0; ++left) {
+    int rich = 0;
+    for (int i = 1; i < n; ++i)
+      if (ctas[i] - least[i] > ctas[rich] - least[rich]) rich = i;
+    --ctas[rich];
+  }
+  for (int i = 0; i < n; ++i) out[i] = best_split(g, n_tiles[i], ctas[i], ctas[i]);
   for (int step = 0; step < 32; ++step) {
     int slow = 0, quick = -1;
     for (int i = 1; i < n; ++i)
       if (out[i].cost > out[slow].cost) slow = i;
-    if (left <= 0) {
+    if (left == 0) {
       for (int i = 0; i < n; ++i)
-        if (i != slow && ctas[i] > 1 && (quick < 0 || out[i].cost < out[quick].cost)) quick = i;
-      if (quick < 0 || (out[quick].cost > 0.9 * out[slow].cost && left == 0)) break;
+        if (i != slow && ctas[i] > least[i] && (quick < 0 || out[i].cost < out[quick].cost)) quick = i;
+      if (quick < 0 || out[quick].cost > 0.9 * out[slow].cost) break;
     }
     const Split slow_was = out[slow], quick_was = quick >= 0 ? out[quick] : Split{};
     if (quick >= 0) {
       --ctas[quick];
-      if (!fit(quick)) out[quick].cost = 1e30;
+      out[quick] = best_split(g, n_tiles[quick], ctas[quick], ctas[quick]);
     } else {
       --left;
     }
-    if (left >= 0) {
-      ++ctas[slow];
-      if (!fit(slow)) out[slow].cost = 1e30;
-    } else {
-      ++left;                                                        // the proportional shares had handed out too many
-    }
-    if (quick >= 0 && left >= 0 && out[quick].cost >= slow_was.cost) {   // no better: take the move back and stop
-      ++ctas[quick];
-      --ctas[slow];
+    ++ctas[slow];
+    out[slow] = best_split(g, n_tiles[slow], ctas[slow], ctas[slow]);
+    if (quick >= 0 && out[quick].cost >= slow_was.cost) {            // no better: take the move back and stop
       out[quick] = quick_was;
       out[slow] = slow_was;
       break;
     }
   }
-  int64_t used = 0;
-  for (int i = 0; i < n; ++i) {
-    if (out[i].cost >= 1e30) return false;
-    used += (int64_t)out[i].parts * out[i].per_part;
-  }
-  return used <= sm_count;
+  for (int i = 0; i < n; ++i)
+    if (out[i].cost < 0) return false;
+  return true;
 }
 
-// How many prompts, from the first on, go into one launch.
+// How many prompts, from the first on, go into one launch: while their tiles leave the visits room to overlap, and while there
+// are CTAs that hold them.
 int group_size(const Geometry& g, const int64_t* n_tiles, int n, int sm_count) {
   const double most = (double)g.comfortable_tiles() * sm_count;
+  const int held = g.most_tiles();
   double tiles = 0;
+  int64_t ctas = 0;
   int count = 0;
-  while (count < n && count < sm_count) {
+  while (count < n) {
     tiles += (double)n_tiles[count];
-    if (count > 0 && tiles > most) break;
+    ctas += ceil_div(n_tiles[count], held);
+    if (count > 0 && (tiles > most || ctas > sm_count)) break;
     ++count;
   }
   return count;
@@ -610,10 +617,7 @@ int32_t score_fused_launch(const ScoreProblem* p, int n_prompts, void* workspace
   }
   n = group_size(g, n_tiles, n, sm_count);
   Split split[kFusedMaxBatch];
-  if (!split_group(g, n_tiles, n, sm_count, split)) {
-    n = 1;
-    if (!split_group(g, n_tiles, 1, sm_count, split)) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
-  }
+  if (!split_group(g, n_tiles, n, sm_count, split)) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
   if (done != nullptr) *done = n;
   char* base = static_cast<char*>(workspace);
   return n == 1 ? launch_group<1>(p, n, g, split, base, sm_count, dev_status, stream, mode, lse_in)
