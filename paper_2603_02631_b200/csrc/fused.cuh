@@ -26,9 +26,10 @@
 // Tensor-core tiles.  The operands in shared memory are 128 keys x d (TMA) and the slab's query rows x d (row j = i * G + g:
 // lookahead i, head g of the GQA group, the group padded to a power of two).  Resident, and visit 2 of the two-pass form:
 // keys are the tensor-memory lanes, so the max over the heads of a group is in-thread; the sum over keys ends every slab
-// with a 32-lane reduction of up to 32 columns.  Visit 1 of the two-pass form: query rows are the lanes (weight-stationary
-// instructions, which fill all 128 lanes with 32 or 64 rows), so the sum over keys stays inside a thread too; with 64
-// columns the reduction cost 1000 to 2900 cycles per slab and CTA.  The running maxima live in tensor memory next to the
+// with a 32-lane reduction of up to 32 columns.  Visit 1 of the two-pass form, 32 rows and more: query rows are the lanes
+// (weight-stationary instructions, which fill all 128 lanes with 32 or 64 rows), so the sum over keys stays inside a thread
+// too; with 64 columns the reduction cost 1000 to 2900 cycles per slab and CTA.  With 16 rows half of those lanes would be
+// padding, and twice the tensor memory: keys are the lanes there.  The running maxima live in tensor memory next to the
 // accumulators.
 //
 // Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each).  4: fetches log-sum-exps
@@ -90,8 +91,9 @@ constexpr float kRefMargin = 60.f;     // base-2 units added to the sampled refe
 // swizzle span: 128 bytes of the row (128-byte swizzle), or the whole row where it has only 64 bytes (64-byte swizzle).
 __host__ __device__ constexpr int row_bytes(int d, bool fp8) { return fp8 ? d : 2 * d; }
 __host__ __device__ constexpr int sub_row_bytes(int rowb) { return rowb > 128 ? 128 : rowb; }
-// Query rows of a two-pass visit-1 instruction (its M), and its accumulator columns per tile: 32 x 32 or 64 x 64.
-__host__ __device__ constexpr int sum_rows(int ncols) { return ncols <= 32 ? 32 : 64; }
+// Two-pass, visit 1: query rows are the accumulator's lanes, 32 rows x 32 columns or 64 x 64 a tile.  Else keys x query rows;
+// either way a tile has as many columns as query rows.
+__host__ __device__ constexpr bool sums_by_rows(bool once, int ncols) { return !once && ncols >= 32; }
 
 struct FusedPrompt {
   const CUtensorMap* k_maps;   // [n_layers] (element of a sub-row, key, sub-tile, kv-head[, pool block])
@@ -150,7 +152,7 @@ struct FusedSmem {
 __host__ __device__ inline FusedSmem fused_smem(int d, bool fp8, int ncols, bool once, int tiles, const int k_stages[2]) {
   FusedSmem s;
   uint32_t o = 0;
-  const uint32_t rowb = (uint32_t)row_bytes(d, fp8), q_rows = ncols < 32 ? 32 : ncols;
+  const uint32_t rowb = (uint32_t)row_bytes(d, fp8), q_rows = (uint32_t)ncols;
   for (int v = 0; v < 2; ++v) { s.k_off[v] = o; o += (uint32_t)k_stages[v] * kTileKeys * rowb; }
   for (int v = 0; v < 2; ++v) { s.q_off[v] = o; o += (uint32_t)(once ? (v == 0 ? kMaxQStages : 0) : 2) * (fp8 ? 2 : 1) * q_rows * rowb; }
   s.sums_off = o;  o += kSumSlots * 256 * 4;            // [slot][set][quadrant][lane]
@@ -191,7 +193,6 @@ __device__ __forceinline__ float from_order_bits(unsigned u) {
 template <int D, int NCOLS, int G, bool FP8, bool ONCE>
 struct FusedTraits {
   static constexpr int QS = ONCE ? kMaxQStages : 2;                // query tiles in flight per visit
-  static constexpr int SR = sum_rows(NCOLS);
   static constexpr int CW = NCOLS < 32 ? NCOLS : 32;               // visit 2: accumulators per tensor-memory load
   static constexpr int NCH = NCOLS / CW;                           // loads per tile: 1 or 2
   static constexpr int NI = NCOLS / G;                             // lookahead slots per key in the running-max columns
@@ -204,7 +205,7 @@ struct FusedTraits {
   static constexpr int kSubTileBytes = kTileKeys * SUBROW;
   static constexpr int kTileBytes = KSUB * kSubTileBytes;
   static constexpr int QPARTS = FP8 ? 2 : 1;                       // 8-bit keys: the queries come as two E4M3 terms
-  static constexpr int kQSub = (NCOLS < 32 ? 32 : NCOLS) * SUBROW; // the weight-stationary form multiplies at least 32 rows; unused ones are zero
+  static constexpr int kQSub = NCOLS * SUBROW;
   static constexpr int kQBytes = QPARTS * KSUB * kQSub;
 };
 
@@ -283,7 +284,7 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
 template <class T, int NCOLS, bool FP8, bool ROWS, bool SETS>
 __device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedShare& sh, int v, const unsigned char* k_tiles,
                                                const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
-  constexpr uint32_t idesc = ROWS ? instr_desc(T::SR, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
+  constexpr uint32_t idesc = ROWS ? instr_desc(NCOLS, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
   const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
   const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
   Ring kr(a.k_stages[v]), qr(T::QS), even(SETS ? (a.t_stages[v] + 1) / 2 : a.t_stages[v]), odd(a.t_stages[v] / 2);
@@ -295,7 +296,7 @@ __device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedSh
       const int stage = stage0 + tr.stage;
       if (!mbar_wait2_warp(bars.k_full(v, kr.stage), kr.phase, bars.t_empty(v, stage), tr.phase ^ 1u, ab)) return false;
       tc_fence_after();
-      const uint32_t d_tmem = tmem + (uint32_t)(stage * (ROWS ? T::SR : NCOLS));
+      const uint32_t d_tmem = tmem + (uint32_t)(stage * NCOLS);
       const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
       if (elect_one()) {
 #pragma unroll
@@ -333,10 +334,10 @@ __device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedSh
 // half; 32 rows: a quarter of the keys per quadrant).  Bound by the exp2 unit (16 results a cycle and SM: 512 cycles per
 // tile of 64 rows; the loop alone with its MMAs takes 645).  One load of 32 columns at a time, computed before the next is
 // asked for: the other set's warps fill the gap, and keeping a load in flight across the arithmetic measured 8 to 15 % slower.
-template <class T, bool FP8>
-__device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
+template <class T, int NCOLS, bool FP8>
+__device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
                                           const FusedBars& bars, const Abort& ab) {
-  constexpr int NL = T::SR / 32;                                   // tensor-memory loads of 32 columns per tile
+  constexpr int NL = NCOLS / 32;                                   // tensor-memory loads of 32 columns per tile
   const FusedPrompt& p = *sh.p;
   const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
   const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
@@ -344,7 +345,7 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
   const float* const slab_c = p.slab_c;
   const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) ;
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
-  const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - (T::SR == 64 ? (quad >> 1) * 64 : quad * 32);
+  const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - (NCOLS == 64 ? (quad >> 1) * 64 : quad * 32);
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
@@ -359,7 +360,7 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
     for (; lt < n_tiles; lt += 2) {
       if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
-      const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * T::SR);
+      const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * NCOLS);
       const uint32_t empty = bars.t_empty(0, tr.stage);
       tr.advance(2);
 #pragma unroll
@@ -405,11 +406,13 @@ __device__ __forceinline__ void fused_sum(const FusedArgs& a, const FusedShare& 
   }
 }
 
-// The sums of the resident form.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it
+// The sums where keys are the lanes.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it
 // shares out over the warp at the end of a slab.  (The two-pass form with its 64 rows took 10 to 20 % longer this way, whether
-// a warp had all rows of every other tile or half the rows of each.)
-template <class T, int NCOLS, bool FP8>
-__device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
+// a warp had all rows of every other tile or half the rows of each.  With 16 rows it is the quicker one, 960 -> 910 us for
+// 16 layers x 8 heads at 340942 tokens, and its columns are half as many: 28 tiles a CTA at 16 slots a key instead of 26, where
+// the general path takes 152 us for two layers at 511438 tokens and this one 105.)
+template <class T, int NCOLS, bool FP8, bool ONCE>
+__device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
                                              const FusedBars& bars, const Abort& ab) {
   const FusedPrompt& p = *sh.p;
   const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
@@ -419,7 +422,7 @@ __device__ __forceinline__ void resident_sum(const FusedArgs& a, const FusedShar
   const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
   const int tail_lanes = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32;   // real keys of this quadrant in the last tile
-  const bool frees = a.mode == 1;                         // no visit 2: nobody else frees the stages
+  const bool frees = !ONCE || a.mode == 1;                // the accumulators wait for no visit 2
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
@@ -955,7 +958,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   tc_fence_after();
   const uint32_t tmem_base = (uint32_t)misc[1];
   // tensor memory: the accumulator stages, then the running maxima, [local tile][NI] columns (lane = key)
-  const uint32_t tmem_v2 = tmem_base + (uint32_t)(a.t_stages[0] * (ONCE ? NCOLS : T::SR));
+  const uint32_t tmem_v2 = tmem_base + (uint32_t)(a.t_stages[0] * NCOLS);
   const uint32_t amax_tmem = tmem_v2 + (uint32_t)(ONCE ? 0 : a.t_stages[1] * NCOLS);
   grid_wait();                                                     // what the preparing kernel wrote is visible from here on
   grid_launch_dependents();                                        // the next kernel starts where SMs are free, and waits there
@@ -972,7 +975,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
       if (warp < 2) {
         if (lane == 0) fused_produce<T, ONCE>(a, sh, v, k_tiles, q_tiles, tile_at, bars, misc + 2, ab);
       } else {
-        if (v == 0) fused_multiply<T, NCOLS, FP8, !ONCE, false>(a, sh, 0, k_tiles, q_tiles, tmem_base, bars, ab);
+        if (v == 0) fused_multiply<T, NCOLS, FP8, sums_by_rows(ONCE, NCOLS), false>(a, sh, 0, k_tiles, q_tiles, tmem_base, bars, ab);
         else fused_multiply<T, NCOLS, FP8, false, true>(a, sh, 1, k_tiles, q_tiles, tmem_v2, bars, ab);
       }
     }
@@ -986,8 +989,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   } else if (warp < kMaxWarp0) {
     if constexpr (kMoveRegs) reg_inc<88>();
     if (visit1) {
-      if constexpr (ONCE) resident_sum<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
-      else fused_sum<T, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+      if constexpr (sums_by_rows(ONCE, NCOLS)) sum_by_rows<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+      else sum_by_keys<T, NCOLS, FP8, ONCE>(a, sh, warp, lane, tmem_base, sums, bars, ab);
     }
   } else {
     if constexpr (kMoveRegs) reg_inc<88>();

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
   // the slab's query operand, 16 bytes of the swizzled image per thread and step: sub-tiles of `image_rows` rows x one
   // swizzle span, the 16-byte chunks of a row permuted by the row's index (mod 8; 64-byte rows: by half of it, mod 4)
   constexpr int ROWB = row_bytes(D, FP8), SUBROW = sub_row_bytes(ROWB), CH = SUBROW / 16, KSUB = ROWB / SUBROW, EL = FP8 ? 16 : 8;
-  const int image_rows = a.ncols < 32 ? 32 : a.ncols, chunks = KSUB * image_rows * CH;
+  const int image_rows = a.ncols, chunks = KSUB * image_rows * CH;
   uint4* image = reinterpret_cast<uint4*>(p.q_tiles) + (int64_t)slab * (FP8 ? 2 : 1) * chunks;
   const float S = FP8 ? s_scale : 1.f;
   for (int idx = threadIdx.x; idx < chunks; idx += kPrepThreads) {
@@ -259,7 +259,7 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
   g.lead = std::max(2, (int)((tiles > kLongSlab ? kL2KeyBytesLong : kL2KeyBytes) / ((double)sm_count * g.tile_bytes)));
   // the resident form wants a slab's tiles and a few more in tensor memory
   g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + 3;
-  g.max_tiles = (kTmemColsAll - 2 * (sum_rows(g.ncols) + g.ncols)) / (g.ncols / g.padded_group);
+  g.max_tiles = (kTmemColsAll - 4 * g.ncols) / (g.ncols / g.padded_group);
   g.ok = tiles <= g.max_tiles;
   return g;
 }
@@ -400,15 +400,10 @@ bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, 
     return false;
   }
   // as many accumulator stages as fit, visit 1 first (its epilogue is the longer one)
-  const int columns = kTmemColsAll - tiles * (g.ncols / g.padded_group), sr = sum_rows(g.ncols);
-  a->t_stages[0] = a->t_stages[1] = 0;
-  for (int stages = 2 * kMaxTmemStages; stages >= 4; --stages)
-    if ((stages + 1) / 2 * sr + stages / 2 * g.ncols <= columns) {
-      a->t_stages[0] = (stages + 1) / 2;
-      a->t_stages[1] = stages / 2;
-      break;
-    }
-  if (a->t_stages[0] == 0) return false;
+  const int stages = std::min(2 * kMaxTmemStages, (kTmemColsAll - tiles * (g.ncols / g.padded_group)) / g.ncols);
+  if (stages < 4) return false;
+  a->t_stages[0] = (stages + 1) / 2;
+  a->t_stages[1] = stages / 2;
   for (int ks = 20; ks >= 4; --ks) {
     a->k_stages[0] = (ks + 1) / 2;
     a->k_stages[1] = ks / 2;

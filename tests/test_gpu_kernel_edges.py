@@ -66,6 +66,26 @@ def test_scores_at_the_edges_of_tiles_and_rings(L, Hq, Hkv, d, m, n):
     assert (s.lse.double().reshape(-1) - lse).abs().max() < 1e-4
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,d,m,tiles", [
+    *[(2, 1, 1, 64, 8, t) for t in (14, 15, 16, 27, 28)], (1, 2, 1, 64, 8, 20), (1, 2, 1, 64, 8, 56), (3, 1, 1, 128, 16, 28), (1, 8, 1, 64, 2, 57)])
+def test_sixteen_rows_on_the_fused_path_up_to_its_longest_prompts(L, Hq, Hkv, d, m, tiles):
+    """Running maxima of 28 tiles a CTA at 16 slots a key, or of 56 at 8, leave room for four accumulators of 16 columns.
+    Tolerance as above."""
+    import paper_2603_02631_b200 as spf
+    n = tiles * SPAN - 50
+    q, k = make(L, Hq, Hkv, d, m, n)
+    sel = spf.Selector(L, Hq, Hkv, d, m, n)
+    before = spf.spf_set_score_path(2)
+    try:
+        s = sel.run(q, k, *text(n), keep=0.2)
+    finally:
+        spf.spf_set_score_path(before)
+    want, lse = reference(q, k)
+    assert int(sel.dev_status) == 0
+    assert ((s.importance.double() - want).abs() / want).max() < 2e-4
+    assert (s.lse.double().reshape(-1) - lse).abs().max() < 1e-4
+
+
 def test_batch_of_more_prompts_than_one_launch_takes():
     """Lengths from one token to several tiles per SM, together and one by one: only the order of sums differs (a row sum of
     n terms in fp32, at most n * 2^-24 apart, far less in practice)."""
