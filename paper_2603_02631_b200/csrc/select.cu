@@ -533,6 +533,28 @@ __device__ __forceinline__ void select_last(TailShared& sh, const uint32_t* keys
   }
 }
 
+// Copies the kept chunks' tokens in pieces of 128, dealt out to `warps` warps of which this is number `at`: however long the
+// chunks are, all warps share them (one kept chunk of 16384 tokens: 2 us, and 190 as the work of one warp).
+constexpr int kPiece = 128;
+
+__device__ __forceinline__ void copy_pieces(const spf_path_item& it, const uint32_t* keys, int k, int chunk, int at, int warps) {
+  const int per = (chunk + kPiece - 1) / kPiece, lane = threadIdx.x & 31;
+  for (int i = at; i < k * per; i += warps) {
+    const int r = i / per;
+    const int64_t within = (int64_t)(i - r * per) * kPiece, a = (int64_t)keys[r] * chunk + within, o = (int64_t)r * chunk + within;
+    const int size = (int)min(min((int64_t)kPiece, chunk - within), it.n_tokens - a);
+    int32_t id[kPiece / 32];
+#pragma unroll
+    for (int u = 0; u < kPiece / 32; ++u) id[u] = 32 * u + lane < size ? __ldg(it.token_ids + a + 32 * u + lane) : 0;
+#pragma unroll
+    for (int u = 0; u < kPiece / 32; ++u)
+      if (32 * u + lane < size) {
+        it.out_ids[o + 32 * u + lane] = id[u];
+        if (it.out_pos != nullptr) it.out_pos[o + 32 * u + lane] = (int32_t)a + 32 * u + lane;
+      }
+  }
+}
+
 __global__ void __launch_bounds__(kTailThreads) pool_select_compact_kernel(const __grid_constant__ TailBatch b) {
   extern __shared__ uint32_t keys[];                       // the chunks' keys, then the kept chunks' indices
   __shared__ TailShared sh;
@@ -624,31 +646,36 @@ __global__ void __launch_bounds__(kTailThreads) pool_select_compact_kernel(const
     it.out_counts[1] = (int64_t)(total & 0xFFFFu);
   }
   // Kept chunk r starts at output r * chunk: only the prompt's last chunk can be short, and it is the last one kept.  A warp
-  // copies whole chunks, several at a time.
+  // copies whole chunks, several at a time ...
   constexpr int kRows = 8;
-  for (int r0 = rank * 32 + warp; r0 < k; r0 += ctas * 32 * kRows) {
-    const int32_t* from[kRows];
-    int size[kRows];
+  if (chunk <= kPiece) {
+    for (int r0 = rank * 32 + warp; r0 < k; r0 += ctas * 32 * kRows) {
+      const int32_t* from[kRows];
+      int size[kRows];
 #pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      const int r = r0 + u * ctas * 32;
-      const int64_t a = r < k ? (int64_t)keys[r] * chunk : 0;
-      from[u] = it.token_ids + a;
-      size[u] = r < k ? (int)min((int64_t)chunk, n_tokens - a) : 0;
+      for (int u = 0; u < kRows; ++u) {
+        const int r = r0 + u * ctas * 32;
+        const int64_t a = r < k ? (int64_t)keys[r] * chunk : 0;
+        from[u] = it.token_ids + a;
+        size[u] = r < k ? (int)min((int64_t)chunk, n_tokens - a) : 0;
+      }
+      const int64_t o = (int64_t)r0 * chunk;
+      for (int s = lane; s < chunk; s += 32) {
+        int32_t id[kRows];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) id[u] = s < size[u] ? __ldg(from[u] + s) : 0;
+#pragma unroll
+        for (int u = 0; u < kRows; ++u)
+          if (s < size[u]) {
+            it.out_ids[o + (int64_t)u * ctas * 32 * chunk + s] = id[u];
+            if (it.out_pos != nullptr) it.out_pos[o + (int64_t)u * ctas * 32 * chunk + s] = (int32_t)(from[u] - it.token_ids) + s;
+          }
+      }
     }
-    const int64_t o = (int64_t)r0 * chunk;
-    for (int s = lane; s < chunk; s += 32) {
-      int32_t id[kRows];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) id[u] = s < size[u] ? __ldg(from[u] + s) : 0;
-#pragma unroll
-      for (int u = 0; u < kRows; ++u)
-        if (s < size[u]) {
-          it.out_ids[o + (int64_t)u * ctas * 32 * chunk + s] = id[u];
-          if (it.out_pos != nullptr) it.out_pos[o + (int64_t)u * ctas * 32 * chunk + s] = (int32_t)(from[u] - it.token_ids) + s;
-        }
-    }
+    return;
   }
+  // ... or pieces of longer ones
+  copy_pieces(it, keys, k, chunk, rank * 32 + warp, ctas * 32);
 }
 
 __global__ void __launch_bounds__(kCompactThreads) compact_spans_batch_kernel(const __grid_constant__ CompactBatch b, int chunk) {

@@ -125,6 +125,8 @@ class Item(ctypes.Structure):
     ([32768, 32769, 40000], 1, 3, 0, (0, 0), 0),                       # 32768 chunks in shared memory, more in three launches
     ([131071], 32, 13, 0, (0, 0), 3), ([30000], 1, 1, 0, (1, 1), 1),   # hundreds and thousands of equal scores
     ([64] * 30, 16, 5, 0, (0, 0), 0),                                  # more prompts than one launch takes
+    ([100001, 70000], 33, 13, 0, (0, 0), 0), ([100001], 1000, 13, 0, (0, 1), 0),   # chunks of more than one row of a warp
+    ([100001], 16384, 13, 0, (0, 1), 0), ([100001], 100001, 13, 0, (0, 0), 0), ([9000], 20000, 13, 0, (0, 0), 0),
 ])
 @pytest.mark.parametrize("keep", [0.001, 0.3, 1.0])
 def test_pool_select_compact_equals_the_separate_calls(lens, chunk, pool, edge, force, levels, keep):
