@@ -139,31 +139,6 @@ __device__ __forceinline__ uint32_t chunk_key(const float* __restrict__ scores, 
   return order_key(scores[j]);
 }
 
-// Exclusive prefix count of `flag` over the CTA (thread order); *total gets the CTA-wide count.  The 32 warp totals
-// are scanned by warp 0 with shuffles (slot 32 of warp_counts receives the CTA-wide total).
-__device__ __forceinline__ int block_exclusive_count(bool flag, int* warp_counts, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned ballot = __ballot_sync(0xffffffffu, flag);
-  const int within = __popc(ballot & ((1u << lane) - 1u));
-  __syncthreads();  // warp_counts may still be read from the previous use
-  if (lane == 0) warp_counts[warp] = __popc(ballot);
-  __syncthreads();
-  if (warp == 0) {
-    const int own = warp_counts[lane];
-    int incl = own;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += v;
-    }
-    warp_counts[lane] = incl - own;                      // exclusive offset of warp `lane`
-    if (lane == 31) warp_counts[32] = incl;
-  }
-  __syncthreads();
-  *total = warp_counts[32];
-  return warp_counts[warp] + within;
-}
-
 // One histogram increment per distinct bin of a warp instead of one per thread: scores share their top bits, so the
 // first passes would otherwise send thousands of atomics to a handful of shared-memory words.
 __device__ __forceinline__ void hist_add_aggregated(int* hist, bool take, uint32_t bin) {
@@ -174,7 +149,7 @@ __device__ __forceinline__ void hist_add_aggregated(int* hist, bool take, uint32
 __device__ __forceinline__ void select_topk_body(const float* __restrict__ scores, int n, int k, int force,
                                                  int32_t* __restrict__ kept) {
   __shared__ int hist[256];
-  __shared__ int warp_counts[kTopkThreads / 32 + 1];
+  __shared__ uint32_t warp_counts[2][kTopkThreads / 32];
   __shared__ uint32_t sh_prefix;
   __shared__ int sh_remaining;
 
@@ -253,8 +228,12 @@ __device__ __forceinline__ void select_topk_body(const float* __restrict__ score
     mask |= 255u << shift;
     __syncthreads();
   }
-  // `prefix` is now the k-th largest key; `remaining` of the entries equal to it are kept (lowest indices).
-  int out_base = 0, eq_base = 0;
+  // `prefix` is now the k-th largest key; `remaining` of the entries equal to it are kept (lowest indices).  Larger and equal
+  // keys are counted together (high and low half of a word), with one barrier per 1024 keys: the counts of a step and of the
+  // next have scratch of their own.
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lower = (1u << lane) - 1u;
+  int gt_base = 0, eq_base = 0;
   for (int j0 = 0, it = 0; j0 < n; j0 += kTopkThreads, ++it) {
     const int j = j0 + threadIdx.x;
     uint32_t key = 0u;
@@ -265,15 +244,16 @@ __device__ __forceinline__ void select_topk_body(const float* __restrict__ score
     } else if (j < n) {
       key = chunk_key(scores, j, n, force);
     }
-    const bool gt = j < n && key > prefix;
-    const bool eq = j < n && key == prefix;
-    int eq_total, sel_total;
-    const int eq_rank = eq_base + block_exclusive_count(eq, warp_counts, &eq_total);
-    const bool sel = gt || (eq && eq_rank < remaining);
-    const int pos = out_base + block_exclusive_count(sel, warp_counts, &sel_total);
-    if (sel && pos < k) kept[pos] = j;
-    out_base += sel_total;
-    eq_base += eq_total;
+    const bool gt = j < n && key > prefix, eq = j < n && key == prefix;
+    const uint32_t gts = __ballot_sync(0xffffffffu, gt), eqs = __ballot_sync(0xffffffffu, eq);
+    if (lane == 0) warp_counts[it & 1][warp] = (uint32_t)__popc(gts) << 16 | (uint32_t)__popc(eqs);
+    __syncthreads();
+    const uint32_t w = warp_counts[it & 1][lane], all = __reduce_add_sync(0xffffffffu, w);
+    const uint32_t ahead = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+    const int gt_rank = gt_base + (int)(ahead >> 16) + __popc(gts & lower), eq_rank = eq_base + (int)(ahead & 0xFFFFu) + __popc(eqs & lower);
+    if (gt || (eq && eq_rank < remaining)) kept[gt_rank + min(eq_rank, remaining)] = j;
+    gt_base += (int)(all >> 16);
+    eq_base += (int)(all & 0xFFFFu);
   }
 }
 
@@ -294,7 +274,11 @@ __global__ void __launch_bounds__(kTopkThreads) select_topk_batch_kernel(const _
 // other blocks copy ids and positions, one warp per kept chunk.
 // ------------------------------------------------------------------------------------------------
 constexpr int kCompactThreads = 256;
+// From so many kept chunks on block 0's walk over them is what takes the time (13108 chunks of one token: 54 us in all with 256
+// threads, 29 with 1024), below the copy, which wants to be spread over the SMs (128 chunks of 1024 tokens: 18 and 21 us).
+constexpr int kCompactMany = 1025, kCompactManyThreads = 1024;
 
+template <int THREADS>
 __device__ __forceinline__ void compact_spans_body(
     const int32_t* __restrict__ kept, int k, int chunk, int64_t n_tokens, const int32_t* __restrict__ token_ids,
     const int32_t* __restrict__ char_start, const int32_t* __restrict__ char_end, int32_t* __restrict__ out_ids,
@@ -302,42 +286,53 @@ __device__ __forceinline__ void compact_spans_body(
     int64_t* __restrict__ out_counts) {
   const int64_t n_chunks = (n_tokens + chunk - 1) / chunk;
   if (blockIdx.x == 0) {
-    __shared__ int warp_counts[kCompactThreads / 32];
+    // 1024 chunks a step: the 32 counts of a step are read by every warp at once, and those of the next have
+    // scratch of their own
+    constexpr int kEach = 1024 / THREADS, kWarps = THREADS / 32;
+    static_assert(kEach * kWarps == 32, "a count per lane");
+    __shared__ int counts[2][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int span_base = 0;
-    for (int r0 = 0; r0 < k; r0 += kCompactThreads) {
-      const int r = r0 + threadIdx.x;
-      int64_t j = -1;
-      bool starts = false, ends = false;
-      if (r < k) {
-        j = kept[r];
-        starts = r == 0 || kept[r - 1] + 1 != j;
-        ends = r == k - 1 || kept[r + 1] != j + 1;
+    for (int r0 = 0, it = 0; r0 < k; r0 += kEach * THREADS, ++it) {
+      int64_t j[kEach];
+      bool starts[kEach], ends[kEach];
+      int within[kEach];
+#pragma unroll
+      for (int u = 0; u < kEach; ++u) {
+        const int r = r0 + u * THREADS + threadIdx.x;
+        j[u] = -1;
+        starts[u] = ends[u] = false;
+        if (r < k) {
+          j[u] = kept[r];
+          starts[u] = r == 0 || kept[r - 1] + 1 != j[u];
+          ends[u] = r == k - 1 || kept[r + 1] != j[u] + 1;
+        }
       }
-      const unsigned ballot = __ballot_sync(0xffffffffu, starts);
-      const int within = __popc(ballot & ((2u << lane) - 1u));  // inclusive
-      __syncthreads();
-      if (lane == 0) warp_counts[warp] = __popc(ballot);
-      __syncthreads();
-      int before = 0, all = 0;
-      for (int w = 0; w < kCompactThreads / 32; ++w) {
-        before += w < warp ? warp_counts[w] : 0;
-        all += warp_counts[w];
+#pragma unroll
+      for (int u = 0; u < kEach; ++u) {
+        const unsigned ballot = __ballot_sync(0xffffffffu, starts[u]);
+        within[u] = __popc(ballot & ((2u << lane) - 1u));        // inclusive
+        if (lane == 0) counts[it & 1][u * kWarps + warp] = __popc(ballot);
       }
-      const int span = span_base + before + within - 1;  // index of the run this chunk belongs to
-      if (r < k && j >= 0 && j < n_chunks) {
-        if (starts) {
-          const int64_t a = j * chunk;
+      __syncthreads();
+      const int count = counts[it & 1][lane];
+#pragma unroll
+      for (int u = 0; u < kEach; ++u) {
+        const int before = __reduce_add_sync(0xffffffffu, lane < u * kWarps + warp ? count : 0);
+        const int span = span_base + before + within[u] - 1;     // index of the run this chunk belongs to
+        if (j[u] < 0 || j[u] >= n_chunks) continue;
+        if (starts[u]) {
+          const int64_t a = j[u] * chunk;
           out_tok_spans[2 * span] = (int32_t)a;
           out_char_spans[2 * span] = char_start[a];
         }
-        if (ends) {
-          const int64_t b = min((j + 1) * chunk, n_tokens);
+        if (ends[u]) {
+          const int64_t b = min((j[u] + 1) * chunk, n_tokens);
           out_tok_spans[2 * span + 1] = (int32_t)b;
           out_char_spans[2 * span + 1] = char_end[b - 1];
         }
       }
-      span_base += all;
+      span_base += __reduce_add_sync(0xffffffffu, count);
     }
     if (threadIdx.x == 0) {
       const int64_t last = kept[k - 1];
@@ -347,7 +342,7 @@ __device__ __forceinline__ void compact_spans_body(
     }
     return;
   }
-  const int warps = kCompactThreads / 32;
+  const int warps = THREADS / 32;
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)(blockIdx.x - 1) * warps + (threadIdx.x >> 5);
   if (r >= k) return;
@@ -361,12 +356,13 @@ __device__ __forceinline__ void compact_spans_body(
   }
 }
 
-__global__ void __launch_bounds__(kCompactThreads) compact_spans_kernel(
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) compact_spans_kernel(
     const int32_t* __restrict__ kept, int k, int chunk, int64_t n_tokens, const int32_t* __restrict__ token_ids,
     const int32_t* __restrict__ char_start, const int32_t* __restrict__ char_end, int32_t* __restrict__ out_ids,
     int32_t* __restrict__ out_pos, int32_t* __restrict__ out_tok_spans, int32_t* __restrict__ out_char_spans,
     int64_t* __restrict__ out_counts) {
-  compact_spans_body(kept, k, chunk, n_tokens, token_ids, char_start, char_end, out_ids, out_pos, out_tok_spans, out_char_spans,
+  compact_spans_body<THREADS>(kept, k, chunk, n_tokens, token_ids, char_start, char_end, out_ids, out_pos, out_tok_spans, out_char_spans,
                      out_counts);
 }
 
@@ -678,10 +674,11 @@ __global__ void __launch_bounds__(kTailThreads) pool_select_compact_kernel(const
   copy_pieces(it, keys, k, chunk, rank * 32 + warp, ctas * 32);
 }
 
-__global__ void __launch_bounds__(kCompactThreads) compact_spans_batch_kernel(const __grid_constant__ CompactBatch b, int chunk) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) compact_spans_batch_kernel(const __grid_constant__ CompactBatch b, int chunk) {
   const spf_compact_item& it = b.item[blockIdx.y];
-  if ((int64_t)blockIdx.x > 1 + (it.k + kCompactThreads / 32 - 1) / (kCompactThreads / 32)) return;
-  compact_spans_body(it.kept_chunks, (int)it.k, chunk, it.n_tokens, it.token_ids, it.char_start, it.char_end, it.out_ids, it.out_pos,
+  if ((int64_t)blockIdx.x > 1 + (it.k + THREADS / 32 - 1) / (THREADS / 32)) return;
+  compact_spans_body<THREADS>(it.kept_chunks, (int)it.k, chunk, it.n_tokens, it.token_ids, it.char_start, it.char_end, it.out_ids, it.out_pos,
                      it.out_tok_spans, it.out_char_spans, it.out_counts);
 }
 
@@ -764,8 +761,11 @@ extern "C" int32_t spf_compact_spans(const int32_t* kept_chunks, int64_t k, int3
   if (k < 1 || k > n_chunks)
     return fail(SPF_ERR_INVALID_ARG, "spf_compact_spans: k must be in [1, n_chunks] (got k=%lld, n_chunks=%lld)", (long long)k,
                 (long long)n_chunks);
-  const int64_t blocks = 1 + ceil_div(k, kCompactThreads / 32);
-  compact_spans_kernel<<<(unsigned)blocks, kCompactThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+  const bool many = k >= kCompactMany;
+  const int threads = many ? kCompactManyThreads : kCompactThreads;
+  const int64_t blocks = 1 + ceil_div(k, threads / 32);
+  auto kernel = many ? compact_spans_kernel<kCompactManyThreads> : compact_spans_kernel<kCompactThreads>;
+  kernel<<<(unsigned)blocks, threads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
       kept_chunks, (int)k, chunk, n_tokens, token_ids, char_start, char_end, out_ids, out_pos, out_tok_spans, out_char_spans,
       out_counts);
   SPF_CUDA_CHECK(cudaGetLastError());
@@ -839,12 +839,15 @@ extern "C" int32_t spf_compact_spans_batch(const spf_compact_item* items, int32_
   for (int32_t i0 = 0; i0 < n_items; i0 += kBatchItems) {
     const int cnt = std::min<int32_t>(kBatchItems, n_items - i0);
     CompactBatch b{};
-    int64_t blocks = 2;
+    int64_t most = 1;
     for (int i = 0; i < cnt; ++i) {
       b.item[i] = items[i0 + i];
-      blocks = std::max(blocks, 1 + ceil_div(items[i0 + i].k, kCompactThreads / 32));
+      most = std::max(most, items[i0 + i].k);
     }
-    compact_spans_batch_kernel<<<dim3((unsigned)blocks, (unsigned)cnt), kCompactThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(b, chunk);
+    const bool many = most >= kCompactMany;
+    const int threads = many ? kCompactManyThreads : kCompactThreads;
+    auto kernel = many ? compact_spans_batch_kernel<kCompactManyThreads> : compact_spans_batch_kernel<kCompactThreads>;
+    kernel<<<dim3((unsigned)(1 + ceil_div(most, threads / 32)), (unsigned)cnt), threads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(b, chunk);
     SPF_CUDA_CHECK(cudaGetLastError());
   }
   return SPF_OK;

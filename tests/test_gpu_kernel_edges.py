@@ -164,6 +164,35 @@ def test_pool_select_compact_equals_the_separate_calls(lens, chunk, pool, edge, 
             assert torch.equal(a[name], b[name]), name
 
 
+@pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 8191, 8192, 8193, 40001])
+@pytest.mark.parametrize("levels", [0, 3])
+def test_separate_selection_where_its_steps_and_block_sizes_change(n, levels):
+    """Keys in registers up to 8192 chunks, 1024 kept chunks and more; all distinct, and thousands of equal ones.  Against a
+    stable sort and a walk over the kept chunks: whole numbers, nothing to tolerate."""
+    import paper_2603_02631_b200 as spf
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    scores = torch.rand(n, generator=gen, device="cuda")
+    if levels:
+        scores = (scores * levels).floor()
+    order = torch.argsort(scores, descending=True, stable=True)
+    ids, start, end = text(n)
+    for k in sorted({1, min(n, 1024), min(n, 1025), -(-n // 3), n}):
+        i32 = lambda *size: torch.full(size, -1, dtype=torch.int32, device="cuda")
+        kept, out, pos, tok, ch = i32(k), i32(n), i32(n), i32(k, 2), i32(k, 2)
+        counts = torch.zeros(2, dtype=torch.int64, device="cuda")
+        spf.spf_select_topk(scores, n, k, kept)
+        want = order[:k].sort().values.int()
+        assert torch.equal(kept, want)
+        spf.spf_compact_spans(kept, k, 1, n, ids, start, end, out, pos, tok, ch, counts)
+        first = torch.cat([torch.ones(1, dtype=torch.bool, device="cuda"), want[1:] != want[:-1] + 1])
+        a = want[first]
+        b = torch.cat([want[:-1][first[1:]], want[-1:]]) + 1
+        spans = len(a)
+        assert counts.tolist() == [k, spans]
+        assert torch.equal(tok[:spans], torch.stack([a, b], 1)) and torch.equal(pos[:k], want) and torch.equal(out[:k], ids[want.long()])
+        assert torch.equal(ch[:spans], torch.stack([start[a.long()], end[b.long() - 1]], 1)) and bool((tok[spans:] == -1).all())
+
+
 def test_selector_refuses_what_does_not_fit():
     import paper_2603_02631_b200 as spf
     q, k = make(2, 4, 2, 64, 8, 300)
