@@ -27,17 +27,20 @@ __device__ __forceinline__ float warp_total(float x) {
   return x;
 }
 
-// Score of a chunk that windows reach beyond the prompt's ends from, where each window has a divisor of its own.
-__device__ __noinline__ float pool_edge_chunk(const float* importance, int64_t n_tokens, int half, int64_t lo, int64_t hi) {
+// Score of a chunk window by window: where windows reach beyond the prompt's ends and each has a divisor of its own, and where
+// the weighted sum below, up to min(w, chunk) times larger than the windows' means add up to, is not finite.
+__device__ __noinline__ float pool_by_windows(const float* importance, int64_t n_tokens, const PoolRule& r, int64_t lo, int64_t hi) {
   float sum = 0.f;
   for (int64_t s = lo + (threadIdx.x & 31); s < hi; s += 32) {
-    const int64_t a = max(s - half, (int64_t)0), b = min(s + half, n_tokens - 1);
+    const int64_t a = max(s - r.half, (int64_t)0), b = min(s + r.half, n_tokens - 1);
     float win = 0.f;
     for (int64_t t = a; t <= b; ++t) win += __ldcg(importance + t);
-    sum += win / (float)(b - a + 1);
+    sum += r.in_range_divisor ? win / (float)(b - a + 1) : win * r.inv_w;
   }
   return warp_total(sum) / (float)(hi - lo);
 }
+
+__device__ __forceinline__ bool is_finite(float x) { return fabsf(x) < INFINITY; }
 
 // Score of chunk j, in every lane.  Int counts tokens of a chunk and its surroundings: 32 bits unless the chunk is longer than
 // kShortChunk.
@@ -49,11 +52,12 @@ __device__ __forceinline__ float pool_chunk(const float* __restrict__ importance
   const float* from = importance + lo;
   const Int size = (Int)min((int64_t)r.chunk, rest);
   const Int begin = (Int)max((int64_t)-r.half, -lo), end = (Int)min((int64_t)size + r.half, rest);   // in reach, relative to lo
-  if (r.in_range_divisor && (begin > -r.half || end < size + r.half)) return pool_edge_chunk(importance, n_tokens, r.half, lo, lo + size);
+  if (r.in_range_divisor && (begin > -r.half || end < size + r.half)) return pool_by_windows(importance, n_tokens, r, lo, lo + size);
   float sum = 0.f;
   for (Int x = (Int)(threadIdx.x & 31) - r.half; x < end; x += 32)
     if (x >= begin) sum = fmaf(__ldcg(from + x), (float)(min(x + r.half, size - 1) - max(x - r.half, (Int)0) + 1), sum);
-  return warp_total(sum) * r.inv_w / (float)size;
+  sum = warp_total(sum);
+  return is_finite(sum) ? sum * r.inv_w / (float)size : pool_by_windows(importance, n_tokens, r, lo, lo + size);
 }
 
 // The same for eight chunks from j on, none of them short and none with windows beyond the prompt's ends: what depends on the
@@ -87,7 +91,15 @@ __device__ __forceinline__ float pool_eight(const float* __restrict__ importance
   float total = sum[0];
 #pragma unroll
   for (int off = 2; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
-  return total * r.inv_w / (float)r.chunk;
+  const float score = total * r.inv_w / (float)r.chunk;
+  if (__all_sync(0xffffffffu, is_finite(total))) return score;
+  float mine = score;
+  for (int u = 0; u < kPoolBatch; ++u) {
+    const int64_t lo = (j + u) * r.chunk;
+    const float again = pool_by_windows(importance, lo + r.chunk + r.half, r, lo, lo + r.chunk);
+    if ((lane >> 2) == u && !is_finite(total)) mine = again;
+  }
+  return mine;
 }
 
 __device__ __forceinline__ void chunk_pool_body(const float* __restrict__ importance, int64_t n_tokens, const PoolRule& r,

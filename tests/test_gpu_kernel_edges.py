@@ -193,6 +193,33 @@ def test_separate_selection_where_its_steps_and_block_sizes_change(n, levels):
         assert torch.equal(ch[:spans], torch.stack([start[a.long()], end[b.long() - 1]], 1)) and bool((tok[spans:] == -1).all())
 
 
+@pytest.mark.parametrize("chunk,pool,edge", [(32, 13, 0), (32, 13, 1), (64, 255, 0), (7, 5, 0), (1000, 13, 1)])
+def test_pooling_of_values_near_the_end_of_the_range(chunk, pool, edge):
+    """Scores that are representable come out, whatever the sums on the way to them; infinities and NaN reach the chunks whose
+    windows hold them and no other.  Tolerance: sums of up to chunk + pool terms of one sign in fp32, 2^-24 per addition."""
+    import paper_2603_02631_b200 as spf
+    n, lib = 9001, spf.lib
+    gen = torch.Generator(device="cuda").manual_seed(chunk)
+    imp = (1 + torch.rand(n, generator=gen, device="cuda")) * (1.6e38 / max(chunk, pool))
+    imp[700], imp[4000], imp[4010], imp[8000] = float("inf"), float("inf"), float("-inf"), float("nan")
+    half, chunks = pool // 2, -(-n // chunk)
+    padded = torch.nn.functional.pad(imp.double(), (half, half))
+    windows = padded.unfold(0, pool, 1).sum(1)
+    reach = torch.nn.functional.pad(torch.ones(n, dtype=torch.float64, device="cuda"), (half, half)).unfold(0, pool, 1).sum(1)
+    smooth = windows / (reach if edge else pool)
+    want = torch.stack([x.mean() for x in smooth.split(chunk)])
+    scores = torch.empty(chunks, device="cuda")
+    spf.spf_chunk_pool_edge(imp, pool, chunk, edge, scores)
+    torch.testing.assert_close(scores.double(), want, rtol=(chunk + pool) * 2.0 ** -24, atol=0, equal_nan=True)
+    assert bool(scores.isfinite().any())
+    both, i32 = torch.empty(chunks, device="cuda"), lambda *size: torch.empty(size, dtype=torch.int32, device="cuda")
+    ids, out = text(n), (i32(1), i32(n), i32(n), i32(2), i32(2), torch.empty(2, dtype=torch.int64, device="cuda"))
+    lib.spf_pool_select_compact.argtypes = [ctypes.POINTER(Item)] + [ctypes.c_int32] * 6 + [ctypes.c_void_p]
+    item = (Item * 1)(Item(imp.data_ptr(), n, both.data_ptr(), 1, *[t.data_ptr() for t in (*ids, *out)]))
+    assert lib.spf_pool_select_compact(item, 1, pool, chunk, edge, 0, 0, torch.cuda.current_stream().cuda_stream) == 0
+    torch.testing.assert_close(both, scores, rtol=0, atol=0, equal_nan=True)
+
+
 def test_selector_refuses_what_does_not_fit():
     import paper_2603_02631_b200 as spf
     q, k = make(2, 4, 2, 64, 8, 300)
