@@ -146,14 +146,14 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
     }
     __syncthreads();
   }
-  // the slab's query operand, 16 bytes of the swizzled image per thread and step: sub-tiles of `image_rows` rows x one
+  // the slab's query operand, 16 bytes of the swizzled image per thread and step: sub-tiles of `rows_stored` rows x one
   // swizzle span, the 16-byte chunks of a row permuted by the row's index (mod 8; 64-byte rows: by half of it, mod 4)
   constexpr int ROWB = row_bytes(D, FP8), SUBROW = sub_row_bytes(ROWB), CH = SUBROW / 16, KSUB = ROWB / SUBROW, EL = FP8 ? 16 : 8;
-  const int image_rows = a.ncols, chunks = KSUB * image_rows * CH;
+  const int rows_stored = image_rows(a.ncols), chunks = KSUB * rows_stored * CH;
   uint4* image = reinterpret_cast<uint4*>(p.q_tiles) + (int64_t)slab * (FP8 ? 2 : 1) * chunks;
   const float S = FP8 ? s_scale : 1.f;
   for (int idx = threadIdx.x; idx < chunks; idx += kPrepThreads) {
-    const int h = idx / (image_rows * CH), j = idx / CH % image_rows, pos = idx % CH;
+    const int h = idx / (rows_stored * CH), j = idx / CH % rows_stored, pos = idx % CH;
     const int chunk = pos ^ (CH == 8 ? j & 7 : (j >> 1) & 3);
     const int g = j % a.padded_group, i = j / a.padded_group;
     const bool real = g < a.group && i < a.n_lookahead;
