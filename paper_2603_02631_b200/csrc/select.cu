@@ -28,7 +28,7 @@ __device__ __forceinline__ float warp_total(float x) {
 }
 
 // Score of a chunk window by window: where windows reach beyond the prompt's ends and each has a divisor of its own, and where
-// the weighted sum below, up to min(w, chunk) times larger than the windows' means add up to, is not finite.
+// the weighted sum below, up to min(w, chunk) times larger than what the windows' means add up to, has overflowed.
 __device__ __noinline__ float pool_by_windows(const float* importance, int64_t n_tokens, const PoolRule& r, int64_t lo, int64_t hi) {
   float sum = 0.f;
   for (int64_t s = lo + (threadIdx.x & 31); s < hi; s += 32) {
@@ -56,8 +56,7 @@ __device__ __forceinline__ float pool_chunk(const float* __restrict__ importance
   float sum = 0.f;
   for (Int x = (Int)(threadIdx.x & 31) - r.half; x < end; x += 32)
     if (x >= begin) sum = fmaf(__ldcg(from + x), (float)(min(x + r.half, size - 1) - max(x - r.half, (Int)0) + 1), sum);
-  sum = warp_total(sum);
-  return is_finite(sum) ? sum * r.inv_w / (float)size : pool_by_windows(importance, n_tokens, r, lo, lo + size);
+  return warp_total(sum) * r.inv_w / (float)size;
 }
 
 // The same for eight chunks from j on, none of them short and none with windows beyond the prompt's ends: what depends on the
@@ -91,22 +90,15 @@ __device__ __forceinline__ float pool_eight(const float* __restrict__ importance
   float total = sum[0];
 #pragma unroll
   for (int off = 2; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
-  const float score = total * r.inv_w / (float)r.chunk;
-  if (__all_sync(0xffffffffu, is_finite(total))) return score;
-  float mine = score;
-  for (int u = 0; u < kPoolBatch; ++u) {
-    const int64_t lo = (j + u) * r.chunk;
-    const float again = pool_by_windows(importance, lo + r.chunk + r.half, r, lo, lo + r.chunk);
-    if ((lane >> 2) == u && !is_finite(total)) mine = again;
-  }
-  return mine;
+  return total * r.inv_w / (float)r.chunk;
 }
 
 __device__ __forceinline__ void chunk_pool_body(const float* __restrict__ importance, int64_t n_tokens, const PoolRule& r,
                                                 float* __restrict__ chunk_scores, int64_t n_chunks) {
   const int64_t j = (int64_t)blockIdx.x * kPoolWarps + (threadIdx.x >> 5);
   if (j >= n_chunks) return;
-  const float score = r.chunk <= kShortChunk ? pool_chunk<int>(importance, n_tokens, r, j) : pool_chunk<int64_t>(importance, n_tokens, r, j);
+  float score = r.chunk <= kShortChunk ? pool_chunk<int>(importance, n_tokens, r, j) : pool_chunk<int64_t>(importance, n_tokens, r, j);
+  if (!is_finite(score)) score = pool_by_windows(importance, n_tokens, r, j * r.chunk, min((j + 1) * r.chunk, n_tokens));
   if ((threadIdx.x & 31) == 0) chunk_scores[j] = score;
 }
 
@@ -541,6 +533,18 @@ __device__ __forceinline__ void select_last(TailShared& sh, const uint32_t* keys
   }
 }
 
+// Chunks j0, j0 + step, ... below `end`, `each` in a row: those whose scores are not finite are done window by window.
+__device__ __noinline__ void pool_again(const spf_path_item& it, const PoolRule& r, int j0, int end, int step, int each) {
+  __syncwarp();
+  for (int j = j0; j < end; j += step)
+    for (int i = j; i < j + each; ++i)
+      if (!is_finite(__ldcg(it.chunk_scores + i))) {
+        const int64_t lo = (int64_t)i * r.chunk;
+        const float score = pool_by_windows(it.importance, it.n_tokens, r, lo, min(lo + r.chunk, it.n_tokens));
+        if ((threadIdx.x & 31) == 0) it.chunk_scores[i] = score;
+      }
+}
+
 // Copies the kept chunks' tokens in pieces of 128, dealt out to `warps` warps of which this is number `at`: however long the
 // chunks are, all warps share them (one kept chunk of 16384 tokens: 2 us, and 190 as the work of one warp).
 constexpr int kPiece = 128;
@@ -580,14 +584,18 @@ __global__ void __launch_bounds__(kTailThreads) pool_select_compact_kernel(const
     const int all = (n + kPoolBatch - 1) / kPoolBatch, warps = ctas * 32, at = rank * 32 + warp;
     const int fast = (int)min((b.rule.half + reach - 1) / reach, (int64_t)all);
     const int slow = (int)max(min((n_tokens - b.rule.half) / reach, (int64_t)all), (int64_t)fast);
+    bool fine = true;
     for (int i = fast + at; i < slow; i += warps) {
       const float score = pool_eight(it.importance, b.rule, (int64_t)i * kPoolBatch);
       if ((lane & 3) == 0) it.chunk_scores[i * kPoolBatch + (lane >> 2)] = score;
+      fine = fine && is_finite(score);
     }
+    if (!__all_sync(0xffffffffu, fine)) pool_again(it, b.rule, (fast + at) * kPoolBatch, slow * kPoolBatch, warps * kPoolBatch, kPoolBatch);
     for (int i = warps - 1 - at; i < n - (slow - fast) * kPoolBatch; i += warps) {
       const int j = i < fast * kPoolBatch ? i : i + (slow - fast) * kPoolBatch;
       const float score = pool_chunk<int>(it.importance, n_tokens, b.rule, j);
       if (lane == 0) it.chunk_scores[j] = score;
+      if (!is_finite(score)) pool_again(it, b.rule, j, j + 1, 1, 1);
     }
     cluster_arrive();                                      // orders the stores before the loads below, in all CTAs
     cluster_wait();
