@@ -431,10 +431,9 @@ SPF_API int32_t spf_select_topk_forced(const float* chunk_scores, int64_t n_chun
 
 /*
  * The whole path for ONE prompt whose inputs and results live in HOST memory (Algorithm 1 from AggregateMaxMean to
- * MapDraftChunksToTextSpans): copies the inputs to the device, runs spf_score -> spf_chunk_pool -> spf_select_topk
- * -> spf_compact_spans, copies the selection back.  This is the entry for a caller that holds the draft model's
- * tensors on the host or on another device; a caller whose tensors are already on this GPU chains the four calls
- * itself.  Unlike every other call it SYNCHRONISES `cuda_stream` (twice: once to learn the counts, once at the end).
+ * MapDraftChunksToTextSpans): copies the inputs to the device, runs spf_score -> spf_pool_select_compact, copies the
+ * selection back.  This is the entry for a caller that holds the draft model's tensors on the host or on another
+ * device; a caller whose tensors are already on this GPU chains the two calls itself.  Unlike every other call it SYNCHRONISES `cuda_stream` (twice: once to learn the counts, once at the end).
  *
  *   k_layers_host   HOST array of L HOST pointers, layer l bf16 [Hkv][N][d] contiguous (pinned memory copies at full
  *                   PCIe / NVLink-C2C speed, pageable memory works)
@@ -448,7 +447,7 @@ SPF_API int32_t spf_select_topk_forced(const float* chunk_scores, int64_t n_chun
  *   out_counts_host                             HOST int64 [2]: {n_kept, n_spans}; only that many rows are written
  *
  * If the fused scoring kernel reports SPF_ERR_RANGE or SPF_ERR_TIMEOUT the prompt is scored again with the general
- * kernels before anything is returned.  Errors: as the four calls; SPF_ERR_WORKSPACE for a small or misaligned arena;
+ * kernels before anything is written to the caller's buffers.  Errors: as those calls; SPF_ERR_WORKSPACE for a small or misaligned arena;
  * a device-side status that survives the retry is returned as the call's status.
  */
 typedef struct {

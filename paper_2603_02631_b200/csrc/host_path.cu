@@ -107,8 +107,7 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
   char* base = static_cast<char*>(arena);
   const size_t L = shape->n_layers, Hq = shape->n_q_heads, Hkv = shape->n_kv_heads, d = shape->head_dim, m = shape->n_lookahead;
   const size_t layer_bytes = Hkv * (size_t)n_tokens * d * 2;
-  const int64_t n_chunks = ceil_div(n_tokens, params->chunk);
-  const int64_t k = spf_keep_count(n_chunks, params->keep_ratio);
+  const int64_t k = spf_keep_count(ceil_div(n_tokens, params->chunk), params->keep_ratio);
 
   // inputs to the device (one copy per tensor, in order on the stream)
   const void* dev_layers[kMaxLayers];
@@ -131,8 +130,6 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
   pr.lse = reinterpret_cast<float*>(base + a.lse);
   int32_t* dev_status = reinterpret_cast<int32_t*>(base + a.status);
   Verdict v{};
-  // Rows that are kept whichever chunks are: all chunks but the last are full.  They are copied without waiting for the counts.
-  const size_t sure = (size_t)(k - 1) * params->chunk + (size_t)(n_tokens - (n_chunks - 1) * params->chunk);
   for (int attempt = 0; attempt < 2; ++attempt) {
     // attempt 0: the kernels spf_score would pick; attempt 1 (after a device-side range or timeout report): the general ones
     SPF_CUDA_CHECK(cudaMemsetAsync(dev_status, 0, 4, stream));
@@ -155,20 +152,16 @@ extern "C" int32_t spf_compress_host(const spf_shape* shape, int64_t n_tokens, c
     item.out_counts = reinterpret_cast<int64_t*>(base + a.counts);
     st = spf_pool_select_compact(&item, 1, params->pool_kernel, params->chunk, 0, 0, 0, stream);
     if (st != SPF_OK) return st;
-    SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host, base + a.out_ids, sure * 4, cudaMemcpyDeviceToHost, stream));
-    if (out_pos_host != nullptr)
-      SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host, base + a.out_pos, sure * 4, cudaMemcpyDeviceToHost, stream));
     SPF_CUDA_CHECK(cudaMemcpyAsync(&v, base + a.counts, sizeof(v), cudaMemcpyDeviceToHost, stream));
     SPF_CUDA_CHECK(cudaStreamSynchronize(stream));
     if (v.status != SPF_ERR_RANGE && v.status != SPF_ERR_TIMEOUT) break;
   }
   if (v.status != 0) return fail(v.status, "spf_compress_host: device status %d (%s)", v.status, spf_status_string(v.status));
   const size_t n_kept = (size_t)v.counts[0], n_spans = (size_t)v.counts[1];
-  if (n_kept > sure) {
-    SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host + sure, base + a.out_ids + sure * 4, (n_kept - sure) * 4, cudaMemcpyDeviceToHost, stream));
-    if (out_pos_host != nullptr)
-      SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host + sure, base + a.out_pos + sure * 4, (n_kept - sure) * 4, cudaMemcpyDeviceToHost, stream));
-  }
+  // the caller's buffers are written from here on: an attempt that is given up leaves them alone
+  SPF_CUDA_CHECK(cudaMemcpyAsync(out_ids_host, base + a.out_ids, n_kept * 4, cudaMemcpyDeviceToHost, stream));
+  if (out_pos_host != nullptr)
+    SPF_CUDA_CHECK(cudaMemcpyAsync(out_pos_host, base + a.out_pos, n_kept * 4, cudaMemcpyDeviceToHost, stream));
   SPF_CUDA_CHECK(cudaMemcpyAsync(out_tok_spans_host, base + a.tok, n_spans * 8, cudaMemcpyDeviceToHost, stream));
   SPF_CUDA_CHECK(cudaMemcpyAsync(out_char_spans_host, base + a.ch, n_spans * 8, cudaMemcpyDeviceToHost, stream));
   SPF_CUDA_CHECK(cudaStreamSynchronize(stream));

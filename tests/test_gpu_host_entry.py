@@ -43,3 +43,33 @@ def test_compress_host_reports_a_small_arena():
         spf.spf_compress_host(prompt.q, prompt.k, prompt.token_ids, prompt.char_start, prompt.char_end, cfg.chunk,
                               cfg.pool_kernel, 0.25, arena, *out)
     assert err.value.status == -3
+
+
+def test_compress_host_writes_nothing_of_an_attempt_it_gives_up():
+    """A head that overflows the fused path's row sums: the prompt is scored again with the general kernels, and the buffers hold
+    that result and, beyond its rows, what they held before."""
+    import paper_2603_02631_b200 as spf
+    L, Hq, Hkv, m, d, n, chunk, keep = 1, 4, 1, 8, 64, 3000, 32, 0.3
+    gen = torch.Generator().manual_seed(3)
+    q, k = torch.randn(L, Hq, m, d, generator=gen), torch.randn(Hkv, n, d, generator=gen)
+    q[0, 3] *= 60                                         # logits of several hundred nats against other heads' single digits
+    q, k = q.to(torch.bfloat16), k.to(torch.bfloat16)
+    ids = torch.arange(n, dtype=torch.int32)
+    sel = spf.Selector(L, Hq, Hkv, d, m, n)
+    dev = [t.cuda() for t in (q, k, ids)]
+    sel.run(dev[0], [dev[1]], dev[2], dev[2], dev[2], keep)
+    assert int(sel.dev_status) == -6                      # what the first attempt reports
+    before = spf.spf_set_score_path(1)
+    try:
+        want = sel.run(dev[0], [dev[1]], dev[2], dev[2], dev[2], keep).host()
+    finally:
+        spf.spf_set_score_path(before)
+    out = [torch.full((n,), -7, dtype=torch.int32).pin_memory(), torch.full((n,), -7, dtype=torch.int32).pin_memory(),
+           torch.full((n, 2), -7, dtype=torch.int32).pin_memory(), torch.full((n, 2), -7, dtype=torch.int32).pin_memory(),
+           torch.zeros(2, dtype=torch.int64).pin_memory()]
+    arena = torch.empty(spf.spf_compress_host_arena_bytes(L, Hq, Hkv, d, m, n, chunk, 13, keep), dtype=torch.uint8, device="cuda")
+    spf.spf_compress_host(q, [k], ids, ids, ids, chunk, 13, keep, arena, *out)
+    kept, spans = out[4].tolist()
+    assert out[0][:kept].tolist() == want["ids"].tolist() and out[2][:spans].tolist() == want["tok_spans"].tolist()
+    for t, rows in zip(out, (kept, kept, spans, spans)):
+        assert bool((t[rows:] == -7).all())
