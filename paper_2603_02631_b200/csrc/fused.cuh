@@ -185,6 +185,10 @@ struct Ring {
   }
 };
 
+// Reads what the preparing kernel writes.  This kernel is started while that one still runs, so these are not read-only for its
+// lifetime: __ldg may be moved ahead of the wait for the other kernel, or be answered from the SM's cache.
+__device__ __forceinline__ float produced(const float* at) { return __ldcg(at); }
+
 // fp32 <-> unsigned bits whose integer order is the float order (0 is below every float).
 __device__ __forceinline__ unsigned order_bits(float x) {
   const unsigned b = __float_as_uint(x);
@@ -353,12 +357,12 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
-  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
+  float next_ref = produced(refs + sh.slab(0)), next_c = FP8 ? produced(slab_c + sh.slab(0)) : a.c;
   for (int n = 0; n < n_slabs; ++n) {
     const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
     if (n + 1 < n_slabs) {
-      next_ref = __ldg(refs + sh.slab(n + 1));
-      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
+      next_ref = produced(refs + sh.slab(n + 1));
+      if constexpr (FP8) next_c = produced(slab_c + sh.slab(n + 1));
     }
     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
     for (; lt < n_tiles; lt += 2) {
@@ -430,12 +434,12 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
-  float next_ref = __ldg(refs + sh.slab(0)), next_c = FP8 ? __ldg(slab_c + sh.slab(0)) : a.c;
+  float next_ref = produced(refs + sh.slab(0)), next_c = FP8 ? produced(slab_c + sh.slab(0)) : a.c;
   for (int n = 0; n < n_slabs; ++n) {
     const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
     if (n + 1 < n_slabs) {
-      next_ref = __ldg(refs + sh.slab(n + 1));
-      if constexpr (FP8) next_c = __ldg(slab_c + sh.slab(n + 1));
+      next_ref = produced(refs + sh.slab(n + 1));
+      if constexpr (FP8) next_c = produced(slab_c + sh.slab(n + 1));
     }
     uint64_t acc[NCOLS / 2];
 #pragma unroll
@@ -565,7 +569,7 @@ __device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPromp
     // normal number) or overflowed row sum has none
     const long long tb = __double_as_longlong(t[0]);
     const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-    lse2 = __ldg(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
+    lse2 = produced(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
     if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
     const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
     if (p.extra_lse != nullptr) {
@@ -633,7 +637,7 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
           if (!mbar_wait_warp(bars.off_free(x), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
         if ((lane & 7) < Q) off[x * 64 + 4 * (lane % Q) + (lane >> 3)] = -lse2;
         if constexpr (FP8) {
-          if (lane == 0) off_c[x] = __ldg(p.slab_c + slab);
+          if (lane == 0) off_c[x] = produced(p.slab_c + slab);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bars.off_ready(x));
@@ -702,7 +706,7 @@ __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedS
         for (int r = 0; r < RPL; ++r)
           if (lane + 32 * r < NCOLS) off[slot * 64 + lane + 32 * r] = v[r];
         if constexpr (FP8) {
-          if (lane == 0) off_c[slot] = __ldg(p.slab_c + sh.slab(n));
+          if (lane == 0) off_c[slot] = produced(p.slab_c + sh.slab(n));
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bars.off_ready(slot));
