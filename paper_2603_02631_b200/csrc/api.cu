@@ -1,4 +1,6 @@
 // Host side of the C ABI: argument validation, error text, dispatch of spf_score.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -182,6 +184,18 @@ int32_t fail(int32_t code, const char* fmt, ...) {
 }
 
 void clear_error() { g_error[0] = '\0'; }
+
+unsigned long long context_id() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId get_id = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+    return reinterpret_cast<GetId>(ok ? p : nullptr);
+  }();
+  unsigned long long id = 0;
+  return get_id != nullptr && get_id(nullptr, &id) == CUDA_SUCCESS ? id + 1 : 0;
+}
 
 }  // namespace spf
 

@@ -33,14 +33,16 @@ struct LayerPtrs {
   const __nv_bfloat16* p[kMaxLayers];
 };
 
-// Lets a kernel use `bytes` of dynamic shared memory on the current device; asked for once per device (`done`), not per launch.
-constexpr int kMaxDevices = 64;
-inline int32_t allow_shared_memory(const void* kernel, int bytes, std::atomic<bool> (&done)[kMaxDevices]) {
-  int dev = 0;
-  SPF_CUDA_CHECK(cudaGetDevice(&dev));
-  if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return SPF_OK;
+// Lets a kernel use `bytes` of dynamic shared memory.  The attribute belongs to the kernel as it is loaded in a context, so it
+// is asked for once per context, not per launch (about a microsecond) nor per device (a device can have several contexts, one
+// after the other or at once).  `done` remembers the ids of contexts, which are never reused.
+using ContextSet = std::atomic<unsigned long long>[64];
+unsigned long long context_id();   // of the calling thread's context, 0 if there is none yet
+inline int32_t allow_shared_memory(const void* kernel, int bytes, ContextSet& done) {
+  const unsigned long long id = context_id();
+  if (id != 0 && done[id % 64].load(std::memory_order_acquire) == id) return SPF_OK;
   SPF_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  if (dev >= 0 && dev < kMaxDevices) done[dev].store(true, std::memory_order_release);
+  done[id % 64].store(id, std::memory_order_release);
   return SPF_OK;
 }
 

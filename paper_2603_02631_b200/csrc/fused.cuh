@@ -1045,7 +1045,7 @@ int32_t fused_launch_d128_fp8(const FusedArgs& args, const FusedLaunch& l, cudaS
 template <int D, int NCOLS, int G, bool FP8, bool ONCE>
 int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
   auto kern = score_fused_kernel<D, NCOLS, G, FP8, ONCE>;
-  static std::atomic<bool> allowed[kMaxDevices];
+  static ContextSet allowed;
   const int32_t st = allow_shared_memory(reinterpret_cast<const void*>(kern), kFusedSmemMost, allowed);
   if (st != SPF_OK) return st;
   cudaLaunchConfig_t cfg{};

@@ -900,7 +900,7 @@ int32_t tail_launch(const spf_path_item* items, int n, const PoolRule& rule, int
     // beyond 48 KB with the static part (about 21 KB), shared memory has to be asked for
     if (cfg.dynamicSmemBytes > 24 * 1024)
     {
-      static std::atomic<bool> allowed[kMaxDevices];
+      static ContextSet allowed;
       const int32_t st = allow_shared_memory(reinterpret_cast<const void*>(pool_select_compact_kernel), kTailChunks * (int)sizeof(uint32_t), allowed);
       if (st != SPF_OK) return st;
     }

@@ -1,7 +1,12 @@
 """What callers may rely on beyond the numbers: which tensors a call holds, which buffers it takes, what it leaves alone."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 pytestmark = pytest.mark.gpu
 GEOM = (2, 4, 2, 64, 8)                # L, Hq, Hkv, d, m
 
@@ -114,3 +119,43 @@ def test_a_batch_is_scored_with_a_workspace_for_its_longest_prompt():
         for b, (importance, lse) in zip(bufs, want):
             torch.testing.assert_close(b.importance, importance, rtol=1e-5, atol=0)
             torch.testing.assert_close(b.lse, lse, rtol=1e-5, atol=1e-5)
+
+
+TWO_CONTEXTS = """
+import ctypes, numpy as np, torch
+import paper_2603_02631_b200 as spf
+from paper_2603_02631_b200 import binding as b
+L, Hq, Hkv, m, d, n, chunk, keep = 2, 4, 2, 8, 64, 300000, 32, 0.3
+gen = torch.Generator().manual_seed(1)
+q = torch.randn(L, Hq, m, d, generator=gen).to(torch.bfloat16)
+k = [torch.randn(Hkv, n, d, generator=gen).to(torch.bfloat16) for _ in range(L)]
+ids = torch.arange(n, dtype=torch.int32)
+shape, prm = b._Shape(L, Hq, Hkv, d, m, 0.0), b._SelectParams(chunk, 13, keep)
+layers = (ctypes.c_void_p * L)(*[x.data_ptr() for x in k])
+lp = ctypes.cast(layers, ctypes.POINTER(ctypes.c_void_p))
+size = spf.lib.spf_compress_host_arena_bytes(ctypes.byref(shape), n, ctypes.byref(prm))
+
+def compress(arena):
+    out = [torch.full((n,), -1, dtype=torch.int32), torch.full((n,), -1, dtype=torch.int32), torch.full((n, 2), -1, dtype=torch.int32),
+           torch.full((n, 2), -1, dtype=torch.int32), torch.zeros(2, dtype=torch.int64)]
+    rc = spf.lib.spf_compress_host(ctypes.byref(shape), n, lp, q.data_ptr(), ids.data_ptr(), ids.data_ptr(), ids.data_ptr(), ctypes.byref(prm),
+                                   arena, size, *[t.data_ptr() for t in out], None)
+    return rc, out
+
+first = compress(torch.empty(size, dtype=torch.uint8, device="cuda").data_ptr())
+assert first[0] == 0, spf.spf_last_error()
+cu = ctypes.CDLL("libcuda.so.1")
+ctx, ptr, dev = ctypes.c_void_p(), ctypes.c_uint64(), ctypes.c_int()
+assert cu.cuDeviceGet(ctypes.byref(dev), 0) == 0 and cu.cuCtxCreate_v2(ctypes.byref(ctx), 0, dev) == 0
+assert cu.cuMemAlloc_v2(ctypes.byref(ptr), ctypes.c_size_t(size)) == 0
+second = compress(ptr.value)
+assert second[0] == 0, spf.spf_last_error()
+assert all(torch.equal(x, y) for x, y in zip(first[1], second[1]))
+"""
+
+
+def test_a_second_context_on_the_device():
+    """What a kernel is allowed in one context says nothing about another's.  All device memory of the second call is its own
+    context's; the call either runs or is refused by the host."""
+    proc = subprocess.run([sys.executable, "-c", TWO_CONTEXTS], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert proc.returncode == 0, proc.stderr[-2000:]
