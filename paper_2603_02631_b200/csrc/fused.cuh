@@ -186,8 +186,13 @@ struct Ring {
 };
 
 // Reads what the preparing kernel writes.  This kernel is started while that one still runs, so these are not read-only for its
-// lifetime: __ldg may be moved ahead of the wait for the other kernel, or be answered from the SM's cache.
-__device__ __forceinline__ float produced(const float* at) { return __ldcg(at); }
+// lifetime: __ldg may be moved ahead of the wait for the other kernel, a volatile load stays behind it.  (Through L1, which
+// has nothing of them before: the loads of neighbouring slabs share a line.)
+__device__ __forceinline__ float produced(const float* at) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(at));
+  return x;
+}
 
 // fp32 <-> unsigned bits whose integer order is the float order (0 is below every float).
 __device__ __forceinline__ unsigned order_bits(float x) {
@@ -519,6 +524,7 @@ __device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPromp
   if (LANES > 1) q = lane % Q;
   const int first = lane / LANES;
   const float4* in = p.row_sums + ((int64_t)slab * p.per_part + first) * Q + q;
+  const float ref = produced(p.refs + slab);                        // its way to L2 and back passes during the wait below
   float4 v[MAXW];
 #pragma unroll
   for (int i = 0; i < MAXW; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -569,7 +575,7 @@ __device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPromp
     // normal number) or overflowed row sum has none
     const long long tb = __double_as_longlong(t[0]);
     const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-    lse2 = produced(p.refs + slab) + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
+    lse2 = ref + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
     if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
     const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
     if (p.extra_lse != nullptr) {
@@ -630,6 +636,7 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
     if constexpr (NCOLS <= 32) {
       if (alone) {
         if (a.mode == 1 && sh.first != 0) continue;                // nobody reads the offsets
+        const float c = FP8 ? produced(p.slab_c + slab) : 0.f;
         if (!sum_rows_of<NCOLS, G, Q, kGatherCtas * Q / 32>(a, p, slab, 0, n_ctas, lane, sh.first == 0, lse2, ab)) return;
         if (a.mode == 1) continue;
         const int x = n % kOffSlots;
@@ -637,7 +644,7 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
           if (!mbar_wait_warp(bars.off_free(x), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
         if ((lane & 7) < Q) off[x * 64 + 4 * (lane % Q) + (lane >> 3)] = -lse2;
         if constexpr (FP8) {
-          if (lane == 0) off_c[x] = produced(p.slab_c + slab);
+          if (lane == 0) off_c[x] = c;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bars.off_ready(x));
@@ -686,6 +693,7 @@ __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedS
     for (int i = 0; i < kAhead; ++i) {
       const int n = n0 + i;
       if (n < sh.n_slabs) {
+        const float c = FP8 ? produced(p.slab_c + sh.slab(n)) : 0.f;
         unsigned long long t0 = 0;
         for (uint32_t it = 1;; ++it) {
           bool there = true;
@@ -706,7 +714,7 @@ __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedS
         for (int r = 0; r < RPL; ++r)
           if (lane + 32 * r < NCOLS) off[slot * 64 + lane + 32 * r] = v[r];
         if constexpr (FP8) {
-          if (lane == 0) off_c[slot] = produced(p.slab_c + sh.slab(n));
+          if (lane == 0) off_c[slot] = c;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bars.off_ready(slot));
