@@ -200,7 +200,7 @@ int32_t launch_prep(const PrepArgs<N>& args, int d, bool fp8, int n_slabs, int n
 // ---------------------------------------------------------------------------------------------- the split over the SMs
 constexpr int kSmemBudget = kFusedSmemMost - 1024;   // minus alignment slack
 // Key bytes between the first and the second read of a tile (two-pass): what still sits in L2 (126 MB, in two halves).  A
-// slab of more than kLongSlab tiles a CTA is far enough ahead of its hand-over with less, and more of it is still there
+// slab of more than kLongSlab tiles for every SM of the chip is far enough ahead with less, and more of it is still there
 // (sustained, 64 rows at 131072 tokens 627 -> 605 us, 32 rows at 262000 507 -> 471); with 4 tiles less lead costs 3 %.
 constexpr double kL2KeyBytes = 80e6, kL2KeyBytesLong = 60e6;
 constexpr int kLongSlab = 5;
@@ -315,12 +315,12 @@ Split best_split(const Geometry& g, int64_t n_tiles, int ctas, int share) {
 // Splits a group of prompts, as group_size made it, over the SMs, each on CTAs of its own: CTAs in proportion to the tiles, but
 // as many as hold them (what that hands out too many comes from the prompts with the most to spare), then a few moves from
 // the prompt that would be done first to the one that would be done last.
-bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count, Split* out) {
+bool split_group(const Geometry* g, const int64_t* n_tiles, int n, int sm_count, Split* out) {
   if (n == 1) {
-    out[0] = best_split(g, n_tiles[0], sm_count, sm_count);
+    out[0] = best_split(g[0], n_tiles[0], sm_count, sm_count);
     return out[0].cost >= 0;
   }
-  const int most = g.most_tiles();
+  const int most = g[0].most_tiles();                                // the same for all: they differ in lead alone
   int64_t total = 0;
   for (int i = 0; i < n; ++i) total += n_tiles[i];
   int least[kFusedMaxBatch], ctas[kFusedMaxBatch], left = sm_count;
@@ -334,7 +334,7 @@ bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count,
       if (ctas[i] - least[i] > ctas[rich] - least[rich]) rich = i;
     --ctas[rich];
   }
-  for (int i = 0; i < n; ++i) out[i] = best_split(g, n_tiles[i], ctas[i], ctas[i]);
+  for (int i = 0; i < n; ++i) out[i] = best_split(g[i], n_tiles[i], ctas[i], ctas[i]);
   for (int step = 0; step < 32; ++step) {
     int slow = 0, quick = -1;
     for (int i = 1; i < n; ++i)
@@ -347,12 +347,12 @@ bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count,
     const Split slow_was = out[slow], quick_was = quick >= 0 ? out[quick] : Split{};
     if (quick >= 0) {
       --ctas[quick];
-      out[quick] = best_split(g, n_tiles[quick], ctas[quick], ctas[quick]);
+      out[quick] = best_split(g[quick], n_tiles[quick], ctas[quick], ctas[quick]);
     } else {
       --left;
     }
     ++ctas[slow];
-    out[slow] = best_split(g, n_tiles[slow], ctas[slow], ctas[slow]);
+    out[slow] = best_split(g[slow], n_tiles[slow], ctas[slow], ctas[slow]);
     if (quick >= 0 && out[quick].cost >= slow_was.cost) {            // no better: take the move back and stop
       out[quick] = quick_was;
       out[slow] = slow_was;
@@ -366,14 +366,14 @@ bool split_group(const Geometry& g, const int64_t* n_tiles, int n, int sm_count,
 
 // How many prompts, from the first on, go into one launch: while their tiles leave the visits room to overlap, and while there
 // are CTAs that hold them.
-int group_size(const Geometry& g, const int64_t* n_tiles, int n, int sm_count) {
-  const double most = (double)g.comfortable_tiles() * sm_count;
-  const int held = g.most_tiles();
-  double tiles = 0;
+int group_size(const Geometry* g, const int64_t* n_tiles, int n, int sm_count) {
+  const int held = g[0].most_tiles();
+  double tiles = 0, most = 1e30;
   int64_t ctas = 0;
   int count = 0;
   while (count < n) {
     tiles += (double)n_tiles[count];
+    most = std::min(most, (double)g[count].comfortable_tiles() * sm_count);
     ctas += ceil_div(n_tiles[count], held);
     if (count > 0 && (tiles > most || ctas > sm_count)) break;
     ++count;
@@ -490,11 +490,12 @@ int32_t encode_key_map(const ScoreProblem& p, const Geometry& g, CUtensorMap* ma
 }
 
 template <int N>
-int32_t launch_group(const ScoreProblem* p, int n, const Geometry& g, const Split* split, char* base, int sm_count, int32_t* dev_status,
+int32_t launch_group(const ScoreProblem* p, int n, const Geometry* geometries, const Split* split, char* base, int sm_count, int32_t* dev_status,
                      cudaStream_t stream, int mode, const float* lse_in) {
   PrepArgs<N> prep{};
   FusedArgs args{};
   const ScoreProblem& p0 = p[0];
+  const Geometry& g = geometries[0];                                 // the prompts' differ in lead alone
   prep.n_kv_heads = args.n_kv_heads = p0.n_kv_heads;
   prep.group = args.group = p0.group;
   prep.padded_group = g.padded_group;
@@ -554,7 +555,7 @@ int32_t launch_group(const ScoreProblem* p, int n, const Geometry& g, const Spli
     fp.cta0 = l.n_cta;
     fp.parts = split[i].parts;
     fp.per_part = split[i].per_part;
-    fp.lead = std::max(g.lead, split[i].tiles + g.handover);
+    fp.lead = std::max(geometries[i].lead, split[i].tiles + g.handover);
     l.n_cta += split[i].parts * split[i].per_part;
     if ((int64_t)split[i].tiles * split[i].per_part < fp.n_tiles || l.n_cta > sm_count)
       return fail(SPF_ERR_UNSUPPORTED, "spf_score: no split of %d key tiles over the SMs", fp.n_tiles);
@@ -600,14 +601,13 @@ size_t score_fused_workspace_bytes(const ScoreProblem& p) { return fused_workspa
 int32_t score_fused_launch(const ScoreProblem* p, int n_prompts, void* workspace, int sm_count, int32_t* dev_status, cudaStream_t stream,
                            int* done, int mode, const float* lse_in) {
   sm_count = std::min(sm_count, kFusedMaxCtas);
-  Geometry g;
+  Geometry g[kFusedMaxBatch];
   int64_t n_tiles[kFusedMaxBatch];
   int n = 0;
   for (; n < std::min(n_prompts, kFusedMaxBatch); ++n) {
-    const Geometry gi = geometry(p[n], sm_count);
-    if (n > 0 && (!gi.ok || gi.once != g.once)) break;  // refused, or scored in the other form, when its turn comes
-    if (!gi.ok) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
-    g = gi;
+    g[n] = geometry(p[n], sm_count);
+    if (n > 0 && (!g[n].ok || g[n].once != g[0].once)) break;  // refused, or scored in the other form, when its turn comes
+    if (!g[n].ok) return fail(SPF_ERR_UNSUPPORTED, "spf_score: shape not covered by the fused path");
     n_tiles[n] = ceil_div(p[n].n_tokens, kTileKeys);
   }
   n = group_size(g, n_tiles, n, sm_count);

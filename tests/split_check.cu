@@ -25,21 +25,21 @@ int main() {
     in >> p.n_layers >> p.n_kv_heads >> p.group >> p.head_dim >> p.n_lookahead >> key_bytes;
     p.n_q_heads = p.n_kv_heads * p.group;
     p.k_scale = key_bytes == 1 ? reinterpret_cast<const float*>(4096) : nullptr;
-    Geometry g;
+    std::vector<Geometry> g;
     std::vector<int64_t> tiles;
     bool same = true;
     while (in >> p.n_tokens) {
       p.stride_tok = p.head_dim;
       p.stride_head = p.n_tokens * p.head_dim;
       const Geometry gi = geometry(p, kSms);
-      same = same && gi.ok && (tiles.empty() || gi.once == g.once);
-      g = gi;
+      same = same && gi.ok && (tiles.empty() || gi.once == g[0].once);
+      g.push_back(gi);
       tiles.push_back(ceil_div(p.n_tokens, kTileKeys));
     }
     // which prompts share the first launch, and the CTAs of each: groups, CTAs per group, tiles per CTA
-    const int n = same ? group_size(g, tiles.data(), (int)tiles.size(), kSms) : 0;
+    const int n = same ? group_size(g.data(), tiles.data(), (int)tiles.size(), kSms) : 0;
     Split split[kFusedMaxBatch];
-    const bool ok = n > 0 && split_group(g, tiles.data(), n, kSms, split);
+    const bool ok = n > 0 && split_group(g.data(), tiles.data(), n, kSms, split);
     std::cout << same << ' ' << n << ' ' << ok;
     for (int i = 0; ok && i < n; ++i) std::cout << ' ' << split[i].parts << ' ' << split[i].per_part << ' ' << split[i].tiles;
     std::cout << '\n';
