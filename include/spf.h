@@ -251,8 +251,8 @@ SPF_API int32_t spf_score_shard_apply_ex(const spf_shape* shape, const spf_promp
 /*
  * Chooses the kernels behind spf_score, process-wide: 0 = automatic (the fused single-kernel path when
  * the shape allows it, else the general two-sweep path), 1 = always the general path, 2 = always the
- * fused path (spf_score then returns SPF_ERR_UNSUPPORTED for shapes outside it: G not in {1,2,4,8},
- * more than 64 layers, or a prompt too long for the per-CTA state).  Both compute the same function
+ * fused path (spf_score then returns SPF_ERR_UNSUPPORTED for shapes outside it: G > 8, G rounded up to a
+ * power of two times m > 64, more than 64 layers, or a prompt whose running maxima do not fit tensor memory).  Both compute the same function
  * (Appendix A.1.1).  Meant for tests and measurements.  Returns the previous setting; an invalid value
  * changes nothing.
  */

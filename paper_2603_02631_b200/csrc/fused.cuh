@@ -1081,8 +1081,10 @@ int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream
 
 template <int D, int NCOLS, bool FP8, bool ONCE>
 int32_t fused_launch_group(const FusedArgs& args, const FusedLaunch& l, cudaStream_t stream) {
+  if constexpr (NCOLS <= 32) {                                     // one head per group: at most 32 lookahead queries
+    if (l.padded_group == 1) return fused_launch_one<D, NCOLS, 1, FP8, ONCE>(args, l, stream);
+  }
   switch (l.padded_group) {
-    case 1: return fused_launch_one<D, NCOLS, 1, FP8, ONCE>(args, l, stream);
     case 2: return fused_launch_one<D, NCOLS, 2, FP8, ONCE>(args, l, stream);
     case 4: return fused_launch_one<D, NCOLS, 4, FP8, ONCE>(args, l, stream);
     default: return fused_launch_one<D, NCOLS, 8, FP8, ONCE>(args, l, stream);

@@ -246,7 +246,7 @@ at::Tensor workspace_of(PyObject* selector, size_t need, const at::Tensor& like)
   return t;
 }
 
-void* stream_of(PyObject* stream, const at::Tensor& on) {
+void* stream_of(PyObject* stream) {
   if (stream == Py_None) return c10::cuda::getCurrentCUDAStream(c10::cuda::current_device()).stream();
   Ref handle(PyObject_GetAttrString(stream, "cuda_stream"));
   void* p = PyLong_AsVoidPtr(handle.p);
@@ -286,7 +286,7 @@ PyObject* select_one(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     read_buffers(selector, shape, in.n, chunk, keep, force_first, force_last, args[6], args[7], args[8], &b);
     const at::Tensor dev_status = attr_tensor_or_none(selector, N.dev_status, at::kInt, "dev_status");
     int32_t* status = dev_status.defined() ? dev_status.data_ptr<int32_t>() : nullptr;
-    void* stream = stream_of(args[10], b.importance);
+    void* stream = stream_of(args[10]);
 
     spf_prompt plain{in.n, in.layers.data(), in.stride_head, in.stride_tok, in.q, b.importance_ptr, b.lse_ptr};
     spf_paged_prompt paged{in.n, in.layers.data(), in.pool_blocks, in.block_tokens, static_cast<const int32_t*>(in.aux), in.q, b.importance_ptr, b.lse_ptr};
@@ -355,7 +355,7 @@ PyObject* select_batch(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     }
     const at::Tensor dev_status = attr_tensor_or_none(selector, N.dev_status, at::kInt, "dev_status");
     int32_t* status = dev_status.defined() ? dev_status.data_ptr<int32_t>() : nullptr;
-    void* stream = stream_of(args[3], b[0].importance);
+    void* stream = stream_of(args[3]);
     const size_t need = spf_score_workspace_bytes(&shape, p.data(), (int32_t)count);
     if (need == 0) return result_tuple(SPF_ERR_INVALID_ARG, "spf_score_workspace_bytes", nullptr, 0);
     const at::Tensor ws = workspace_of(selector, need, b[0].importance);
@@ -433,7 +433,7 @@ PyObject* compress_host(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
         raise(PyExc_ValueError, "a buffer is smaller than include/spf.h requires");
     }
     const spf_shape shape{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)hkv, (int32_t)q.size(3), (int32_t)q.size(2), (float)scale};
-    void* stream = stream_of(args[15], arena);
+    void* stream = stream_of(args[15]);
     void* arena_ptr = arena.data_ptr();
     const size_t arena_bytes = (size_t)arena.numel() * arena.element_size();
     int32_t st;

@@ -376,9 +376,9 @@ __global__ void __launch_bounds__(THREADS) compact_spans_kernel(
 // Nothing here is much work; what costs is the chain of dependent steps, so there are as few as possible between one load
 // and the next.  Each CTA pools its share of the chunks; after the cluster's barrier (the only one) every CTA reads all scores,
 // makes the same selection by itself and writes its own share of the results.
-//   selection: the keys' range is cut into 2048 equal bins (about 300 to 1000 of them hold something, whatever the scores'
-//     distribution), one histogram finds the k-th key's bin, and its few entries are ranked against each other; only a bin
-//     of more than kRankMost entries is cut again.  Ties go to the lower index.
+//   selection: the keys' range is cut into 2048 equal bins (4096 log-normal scores fill some 800 of them; one score of zero
+//     among them leaves 70, the fullest with 200 entries), one histogram finds the k-th key's bin, and its few entries are
+//     ranked against each other; a bin of more than kRankMost entries is cut again.  Ties go to the lower index.
 //   compaction: the selection is a bitmap, one word per warp and step by ballot.  Kept chunks and starts of runs are counted
 //     by population counts, in one scan over the words, instead of a scan per 1024 chunks.
 // ------------------------------------------------------------------------------------------------

@@ -151,7 +151,6 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -220,19 +219,6 @@ template <int N>
 __device__ __forceinline__ void tmem_ready(uint32_t (&r)[N]) {
 #pragma unroll
   for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j]) : : "memory");
-}
-template <>
-__device__ __forceinline__ void tmem_issue<1>(uint32_t taddr, uint32_t (&r)[1]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
-               : "=r"(r[0])
-               : "r"(taddr));
-}
-template <>
-__device__ __forceinline__ void tmem_store<1>(uint32_t taddr, const uint32_t (&r)[1]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};"
-               :
-               : "r"(taddr), "r"(r[0])
-               : "memory");
 }
 template <>
 __device__ __forceinline__ void tmem_issue<2>(uint32_t taddr, uint32_t (&r)[2]) {
