@@ -141,7 +141,12 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
-from . import _native  # noqa: E402  (linked against the library loaded above)
+try:
+    from . import _native  # noqa: E402  (linked against the library loaded above)
+except ImportError as err:
+    from .build import _running, native_is_for
+    raise ImportError(f"_native.so does not load ({err}); it was built against {native_is_for() or 'nothing on record'}, this is {_running()}: "
+                      "run python -m paper_2603_02631_b200.build") from err
 
 
 def _check(status: int, where: str) -> None:

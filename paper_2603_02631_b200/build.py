@@ -21,6 +21,7 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libspf.so")
 NATIVE_SRC = os.path.join(CSRC, "python", "native.cpp")
 NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
+NATIVE_FOR_PATH = NATIVE_PATH + ".for"       # the interpreter and the torch that _native.so was built against
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -43,9 +44,27 @@ def _older(target: str, deps) -> bool:
     return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
 
 
+def _running() -> str:
+    import torch
+    return f"python {sys.version_info.major}.{sys.version_info.minor}, torch {torch.__version__}"
+
+
+def native_is_for() -> str:
+    """What _native.so was built against, as _running() names it; empty if that is not known."""
+    try:
+        with open(NATIVE_FOR_PATH) as f:
+            return f.read().strip()
+    except OSError:
+        return ""
+
+
+def _native_is_stale() -> bool:
+    return _older(NATIVE_PATH, [NATIVE_SRC, *glob.glob(os.path.join(ROOT, "include", "*.h"))]) or native_is_for() != _running()
+
+
 def is_stale() -> bool:
     headers = glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return _older(LIB_PATH, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers) or _older(NATIVE_PATH, [NATIVE_SRC, *headers])
+    return _older(LIB_PATH, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers) or _native_is_stale()
 
 
 def _native_command() -> list:
@@ -61,7 +80,8 @@ def _native_command() -> list:
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Builds libspf.so and _native.so if one of them is missing or older than its sources; returns the path of libspf.so."""
+    """Builds libspf.so and _native.so if one of them is missing, older than its sources or (the latter) built against another
+    torch or Python; returns the path of libspf.so."""
     if not force and not is_stale():
         return LIB_PATH
     include = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -79,8 +99,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         with concurrent.futures.ThreadPoolExecutor(os.cpu_count() or 1) as pool:
             log = "".join(pool.map(lambda so: run([_nvcc(), *NVCC_FLAGS, *include, "-c", so[0], "-o", so[1]]), zip(sources(), objects)))
         run([_nvcc(), *NVCC_FLAGS, "--shared", "-o", LIB_PATH, "-Xlinker", "-soname=libspf.so", *objects])
-    if force or _older(NATIVE_PATH, [NATIVE_SRC, *glob.glob(os.path.join(ROOT, "include", "*.h"))]):
+    if force or _native_is_stale():
         run(_native_command())
+        with open(NATIVE_FOR_PATH, "w") as f:
+            f.write(_running() + "\n")
     with open(os.path.join(PKG_DIR, "libspf.ptxas.log"), "w") as f:
         f.write(log)
     return LIB_PATH
