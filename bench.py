@@ -32,10 +32,11 @@ FALLBACK_HBM_GBS = 6650.0
 
 
 # DRAM read + write bytes of one scoring launch, from the ncu capture summarised in profiles/.  Each entry names
-# the SHA-256 of the kernel source it was taken from: once the source changes, the figure is reported as null.
+# the SHA-256 of the sources it depends on (the kernel, and the host code that sets the split and the lead between its
+# visits): once one of them changes, the figure is reported as null.
 NCU_TRAFFIC = {
-    ("long128k", "fused"): {"bytes": 4 * (564846848 + 9958656), "source": "paper_2603_02631_b200/csrc/fused.cuh",
-                            "sha256": "189d61eda44e8aca845d74d559762699370851b3569c8ea69496711d7198852d",
+    ("long128k", "fused"): {"bytes": 4 * (564846848 + 9958656), "sources": ["fused.cuh", "score_fused.cu", "tc_ptx.cuh", "score.cuh"],
+                            "sha256": "9b0f1ebe568c93f52dda8b3a4b01795d9abb9237c9312054c70a1be3f32acacc",
                             "note": "captured on long128k_l4 (4 of 16 layers), scaled x4"},
 }
 
@@ -46,9 +47,12 @@ def ncu_traffic(workload, path):
     if entry is None:
         return None
     try:
-        with open(os.path.join(ROOT, entry["source"]), "rb") as f:
-            if hashlib.sha256(f.read()).hexdigest() != entry["sha256"]:
-                return None
+        digest = hashlib.sha256()
+        for name in entry["sources"]:
+            with open(os.path.join(ROOT, "paper_2603_02631_b200", "csrc", name), "rb") as f:
+                digest.update(f.read())
+        if digest.hexdigest() != entry["sha256"]:
+            return None
     except OSError:
         return None
     return entry["bytes"]
