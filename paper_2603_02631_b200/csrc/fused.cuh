@@ -23,19 +23,21 @@
 // running maxima then meet in global memory (integer max on order-preserving bits, exact and independent of order), and the
 // last group to finish 32 keys turns them into importance.  Several prompts share one launch, each with CTAs of its own.
 //
-// Tensor-core tiles.  The operands in shared memory are 128 keys x d (TMA) and the slab's query rows x d (row j = i * G + g:
-// lookahead i, head g of the GQA group, the group padded to a power of two).  Resident, and visit 2 of the two-pass form:
-// keys are the tensor-memory lanes, so the max over the heads of a group is in-thread; the sum over keys ends every slab
-// with a 32-lane reduction of up to 32 columns.  Visit 1 of the two-pass form, 32 rows and more: query rows are the lanes
+// Tensor-core tiles.  The operands in shared memory are 128 keys x d (TMA) and the slab's query rows x d (query_row: row j
+// is lookahead i and head g of the GQA group, the group padded to a power of two).  Resident, and visit 2 of the two-pass form:
+// keys are the tensor-memory lanes.  A thread has four keys of every fourth column, and the rows are dealt to the columns so that
+// these are all heads of a lookahead: the max over them is in-thread, a thread needs a quarter of the log-sum-exps, and the sum
+// over keys ends every slab with a reduction over eight lanes of up to 8 columns.  Visit 1 of the two-pass form, 32 rows and more: query rows are the lanes
 // (weight-stationary instructions, which fill all 128 lanes with 32 or 64 rows), so the sum over keys stays inside a thread
 // too; with 64 columns the reduction cost 1000 to 2900 cycles per slab and CTA.  With 16 rows half of those lanes would be
 // padding, and twice the tensor memory: keys are the lanes there.  The running maxima live in tensor memory next to the
 // accumulators.
 //
-// Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each).  4: fetches log-sum-exps
-// for visit 2.  5..7: publishers (store this CTA's row sums of a slab; add up all CTAs' sums of the rows this CTA owns).  8..15: "sum" warps.  16..23: "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM
-// lane quadrant and the next bit the `set`: the two sets take turns at the tiles, so that one set's tensor-memory loads and
-// waits run while the other set computes.  (Splitting every tile's columns between the sets kept all eight warps in step,
+// Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each; the spare warp 1 stores row sums
+// for the gathering warps).  4: fetches log-sum-exps for visit 2.  5..7: publishers (store this CTA's row sums of a slab; add up
+// all CTAs' sums of the rows this CTA owns).  In groups of few CTAs 4..7 add up all rows instead.  8..15: "sum" warps.  16..23:
+// "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM lane quadrant and the next bit the `set`: the two sets
+// take turns at the tiles, so that one set's tensor-memory loads and waits run while the other set computes.  (Splitting every tile's columns between the sets kept all eight warps in step,
 // all waiting or all computing.)
 //
 // Reference.  Visit 1 subtracts one reference per slab inside the exp2 argument: the SMALLEST logit of the slab's rows
@@ -70,11 +72,15 @@ constexpr int kFusedThreads = 768;
 constexpr int kFusedSmemMost = 227 * 1024;   // dynamic shared memory of a CTA
 constexpr int kVisitWarps = 8;         // epilogue warps per visit
 constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
-// Groups of up to this many CTAs add up everybody's row sums in every CTA (see fused_publish): one hop instead of two, about
-// 2 us instead of 3, for reading 16 * CTAs * NCOLS / 4 bytes a slab and CTA.
-constexpr int kGatherCtas = 40;
-__host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return ncols <= 32 && n_ctas <= kGatherCtas; }
+// Groups of up to this many CTAs add up everybody's row sums in every CTA (see fused_gather): one hop instead of two, for reading
+// up to 7 KB a slab and CTA.  Three groups of 49 CTAs with 32 rows each: 178 us for 16 layers x 8 heads at 50000 tokens, in two
+// hops 200; two groups of 74 gained nothing.
+__host__ __device__ constexpr int gather_ctas(int ncols) { return ncols == 64 ? 28 : 56; }
+__host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return n_ctas <= gather_ctas(ncols); }
 constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
+constexpr int kGatherWarp0 = 4, kTeamWarps = 2;
+__host__ __device__ constexpr int gather_teams(bool once) { return once ? 2 : 1; }
+__host__ __device__ constexpr int store_warp(bool once) { return once ? 1 : kGatherWarp0 + kTeamWarps; }   // one that has nothing else to do
 constexpr int kMaxQStages = 4;         // query tiles in flight per visit (two-pass: 2)
 constexpr int kMaxKeyStages = 16;      // key tiles in flight per visit
 // Two-pass: accumulator stages per visit.  64 rows at 131072 tokens have three for each visit; with two for each set of visit 1
@@ -84,7 +90,7 @@ constexpr int kMaxResident = 32;       // resident: tiles in tensor memory
 constexpr int kRegTiles = 8, kRegSlots = 8;   // running maxima stay in registers up to this many tiles a CTA and lookahead slots a key
 constexpr int kTmemColsAll = 512;      // the CTA takes all of its SM's tensor memory
 constexpr int kOffSlots = 4;           // slabs whose log-sum-exps may be in shared memory at once
-constexpr int kSumSlots = 8;           // slabs whose row sums may be on their way to the publishers at once
+constexpr int kSumSlots = 4;           // slabs whose row sums may be on their way to the publishers at once
 constexpr float kRefMargin = 60.f;     // base-2 units added to the sampled reference logit
 
 // Key rows are d bf16 (128 or 256 bytes) or d E4M3 bytes (64 or 128).  A tile is stored as sub-tiles of 128 keys x one
@@ -98,6 +104,22 @@ __host__ __device__ constexpr int image_rows(int ncols) { return ncols < 32 ? 32
 // Two-pass, visit 1: query rows are the accumulator's lanes, 32 rows x 32 columns or 64 x 64 a tile.  Else keys x query rows;
 // either way a tile has as many columns as query rows.
 __host__ __device__ constexpr bool sums_by_rows(bool once, int ncols) { return !once && ncols >= 32; }
+
+// Which query row is column j of the logits (row j of the slab's query operand): lookahead i, head g of the GQA group, padded to a
+// power of two.  A thread that has every fourth column of a key has all heads of a lookahead (of two columns' distance where there
+// are only 16 columns for 8 heads).
+struct QueryRow {
+  int i, g;
+};
+__host__ __device__ constexpr QueryRow query_row(int j, int ncols, int padded_group) {
+  const int t = j & 3, c = j >> 2;
+  return ncols == 16 && padded_group == 8 ? QueryRow{t >> 1, 2 * c + (t & 1)} : QueryRow{c / padded_group * 4 + t, c % padded_group};
+}
+
+// Log-sum-exps in shared memory: what a thread of visit 2 needs is in one piece, the four pieces on banks of their own.
+constexpr int kOffFloats = 4 * (64 / 4 + 4);   // per slab
+__host__ __device__ constexpr int off_stride(int ncols) { return ncols / 4 + 4; }
+__device__ __forceinline__ void store_off(float* off, int ncols, int j, float v) { off[(j & 3) * off_stride(ncols) + (j >> 2)] = v; }
 
 struct FusedPrompt {
   const CUtensorMap* k_maps;   // [n_layers] (element of a sub-row, key, sub-tile, kv-head[, pool block])
@@ -134,18 +156,19 @@ struct FusedArgs {
 struct FusedBars {
   uint32_t base;
   static constexpr int kVisit = 2 * (kMaxKeyStages + kMaxQStages), kTmem = 2 * kVisit, kShared = kTmem + 2 * kMaxResident;
-  static constexpr int kCount = kShared + 2 * kOffSlots + 2 * kSumSlots + 2;
+  static constexpr int kOffReady = kShared, kOffFree = kOffReady + kOffSlots, kSumsReady = kOffFree + kOffSlots;
+  static constexpr int kSumsFree = kSumsReady + kSumSlots, kMmaDone = kSumsFree + kSumSlots, kCount = kMmaDone + 2;
   __device__ uint32_t k_full(int v, int s) const { return base + 8u * (v * kVisit + s); }
   __device__ uint32_t k_empty(int v, int s) const { return base + 8u * (v * kVisit + kMaxKeyStages + s); }
   __device__ uint32_t q_full(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + s); }
   __device__ uint32_t q_empty(int v, int s) const { return base + 8u * (v * kVisit + 2 * kMaxKeyStages + kMaxQStages + s); }
   __device__ uint32_t t_full(int v, int s) const { return base + 8u * (kTmem + v * kMaxTmemStages + s); }   // resident: v = 0 alone
   __device__ uint32_t t_empty(int v, int s) const { return t_full(v, s) + 8u * kMaxResident; }
-  __device__ uint32_t off_ready(int x) const { return base + 8u * (kShared + x); }
-  __device__ uint32_t off_free(int x) const { return base + 8u * (kShared + kOffSlots + x); }
-  __device__ uint32_t sums_ready(int x) const { return base + 8u * (kShared + 2 * kOffSlots + x); }
-  __device__ uint32_t sums_free(int x) const { return base + 8u * (kShared + 2 * kOffSlots + kSumSlots + x); }
-  __device__ uint32_t mma_done(int v) const { return base + 8u * (kShared + 2 * kOffSlots + 2 * kSumSlots + v); }
+  __device__ uint32_t off_ready(int x) const { return base + 8u * (kOffReady + x); }
+  __device__ uint32_t off_free(int x) const { return base + 8u * (kOffFree + x); }
+  __device__ uint32_t sums_ready(int x) const { return base + 8u * (kSumsReady + x); }
+  __device__ uint32_t sums_free(int x) const { return base + 8u * (kSumsFree + x); }
+  __device__ uint32_t mma_done(int v) const { return base + 8u * (kMmaDone + v); }
 };
 static_assert(2 * kMaxTmemStages <= kMaxResident, "the two-pass stages use the same barriers");
 
@@ -160,7 +183,7 @@ __host__ __device__ inline FusedSmem fused_smem(int d, bool fp8, int ncols, bool
   for (int v = 0; v < 2; ++v) { s.k_off[v] = o; o += (uint32_t)k_stages[v] * kTileKeys * rowb; }
   for (int v = 0; v < 2; ++v) { s.q_off[v] = o; o += (uint32_t)(once ? (v == 0 ? kMaxQStages : 0) : 2) * (fp8 ? 2 : 1) * q_rows * rowb; }
   s.sums_off = o;  o += kSumSlots * 256 * 4;            // [slot][set][quadrant][lane]
-  s.off_off = o;   o += kOffSlots * 64 * 4;
+  s.off_off = o;   o += kOffSlots * kOffFloats * 4;
   s.offc_off = o;  o += kOffSlots * 4;
   s.bar_off = o;   o += FusedBars::kCount * 8;
   s.misc_off = o;  o += 64;
@@ -210,6 +233,8 @@ struct FusedTraits {
   static constexpr int NCH = NCOLS / CW;                           // loads per tile: 1 or 2
   static constexpr int NI = NCOLS / G;                             // lookahead slots per key in the running-max columns
   static constexpr int NIW = CW / G;                               // of which one load's accumulators hold
+  static constexpr int CT = CW / 4;                                // a thread's columns of a load, each for four keys
+  static constexpr bool PAIRS = G > CT;                            // 8 heads in 16 columns: two lanes share a lookahead's heads
   static constexpr int ROWB = row_bytes(D, FP8);                   // bytes per key row: 64, 128 or 256
   static constexpr int SUBROW = sub_row_bytes(ROWB);               // the swizzle span: 128 bytes, or the whole 64-byte row
   static constexpr int KSUB = ROWB / SUBROW;                       // sub-tiles per key tile
@@ -248,6 +273,7 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
   int layer = sh.part / n_kv_heads, hk = sh.part - layer * n_kv_heads, issued = 0;
   const int layer_step = sh.parts / n_kv_heads, hk_step = sh.parts - layer_step * n_kv_heads;
   map_acquire(maps + layer);
+#pragma unroll 1
   for (int n = 0; n < sh.n_slabs; ++n) {
     const CUtensorMap* map = maps + layer;
     if (!mbar_wait(bars.q_empty(v, qr.stage), qr.phase ^ 1u, ab)) return;
@@ -255,6 +281,7 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
     bulk_load(q_smem + (uint32_t)(qr.stage * T::kQBytes), q_src + (int64_t)sh.slab(n) * T::kQBytes, (uint32_t)T::kQBytes,
               bars.q_full(v, qr.stage));
     qr.advance();
+#pragma unroll 1
     for (int lt = 0; lt < sh.n_tiles; ++lt, ++issued) {
       if (!ONCE && v == 0) {
         // never more than `lead` tiles ahead of visit 2
@@ -288,8 +315,10 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
 }
 
 // ---------------------------------------------------------------------------------------------- MMA issuer of one visit
-// Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.  The whole warp walks the loop
-// (addresses and descriptors stay warp-uniform); one elected lane issues.
+// Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.  One thread walks the
+// loop.  (The whole warp in step, with votes on the barriers and an elected lane at each tile, took 460 cycles to issue a tile's
+// four instructions and 120 for its barriers, 0.34 us a tile in all: more than the sums of 32 rows take.  The tensor cores want
+// 160 cycles for them, and 24 for each of the two commits.)
 // ROWS: query rows are the accumulator's lanes (weight-stationary instructions), else the keys.  SETS: a ring of stages for
 // each of the two sets of epilogue warps, the odd tiles' behind the even tiles': a tile's maxima belong to one set, so with an
 // odd number of tiles a set skips two, and in a common ring of two stages it could take the tile before the one that it
@@ -297,49 +326,47 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
 template <class T, int NCOLS, bool FP8, bool ROWS, bool SETS>
 __device__ __forceinline__ void fused_multiply(const FusedArgs& a, const FusedShare& sh, int v, const unsigned char* k_tiles,
                                                const unsigned char* q_tiles, uint32_t tmem, const FusedBars& bars, const Abort& ab) {
+  if (!elect_one()) return;
   constexpr uint32_t idesc = ROWS ? instr_desc(NCOLS, kTileKeys, FP8) : instr_desc(kTileKeys, NCOLS, FP8);
   const uint64_t k_desc0 = smem_desc<T::SUBROW>(smem_u32(k_tiles));
   const uint64_t q_desc0 = smem_desc<T::SUBROW>(smem_u32(q_tiles));
   Ring kr(a.k_stages[v]), qr(T::QS), even(SETS ? (a.t_stages[v] + 1) / 2 : a.t_stages[v]), odd(a.t_stages[v] / 2);
   const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
+#pragma unroll 1
   for (int n = 0; n < n_slabs; ++n) {
-    if (!mbar_wait_warp(bars.q_full(v, qr.stage), qr.phase, ab)) return;
+    if (!mbar_wait(bars.q_full(v, qr.stage), qr.phase, ab)) return;
     const uint64_t qd0 = q_desc0 + (uint64_t)((qr.stage * T::kQBytes) >> 4);
     auto tile = [&](Ring& tr, int stage0) -> bool {
       const int stage = stage0 + tr.stage;
-      if (!mbar_wait2_warp(bars.k_full(v, kr.stage), kr.phase, bars.t_empty(v, stage), tr.phase ^ 1u, ab)) return false;
+      if (!mbar_wait2(bars.k_full(v, kr.stage), kr.phase, bars.t_empty(v, stage), tr.phase ^ 1u, ab)) return false;
       tc_fence_after();
       const uint32_t d_tmem = tmem + (uint32_t)(stage * NCOLS);
       const uint64_t kd0 = k_desc0 + (uint64_t)((kr.stage * T::kTileBytes) >> 4);
-      if (elect_one()) {
 #pragma unroll
-        for (int part = 0; part < T::QPARTS; ++part)               // 8-bit keys: the two query terms accumulate into the same columns
+      for (int part = 0; part < T::QPARTS; ++part)                 // 8-bit keys: the two query terms accumulate into the same columns
 #pragma unroll
-          for (int h = 0; h < T::KSUB; ++h)
+        for (int h = 0; h < T::KSUB; ++h)
 #pragma unroll
-            for (int ks = 0; ks < T::KSTEPS; ++ks) {
-              const uint64_t kd = kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks;
-              const uint64_t qd = qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks;
-              tc_mma<FP8, ROWS>(d_tmem, ROWS ? qd : kd, ROWS ? kd : qd, idesc, (uint32_t)((part | h | ks) != 0));
-            }
-        tc_commit(bars.k_empty(v, kr.stage));
-        tc_commit(bars.t_full(v, stage));
-      }
-      __syncwarp();
+          for (int ks = 0; ks < T::KSTEPS; ++ks) {
+            const uint64_t kd = kd0 + (uint64_t)((h * T::kSubTileBytes) >> 4) + 2u * ks;
+            const uint64_t qd = qd0 + (uint64_t)(((part * T::KSUB + h) * T::kQSub) >> 4) + 2u * ks;
+            tc_mma<FP8, ROWS>(d_tmem, ROWS ? qd : kd, ROWS ? kd : qd, idesc, (uint32_t)((part | h | ks) != 0));
+          }
+      tc_commit(bars.k_empty(v, kr.stage));
+      tc_commit(bars.t_full(v, stage));
       kr.advance();
       tr.advance();
       return true;
     };
+#pragma unroll 1
     for (int lt = 0; lt < n_tiles; ++lt)
       if (!(SETS && (lt & 1) ? tile(odd, even.n) : tile(even, 0))) return;
-    if (elect_one()) tc_commit(bars.q_empty(v, qr.stage));
-    __syncwarp();
+    tc_commit(bars.q_empty(v, qr.stage));
     qr.advance();
   }
   // leave only after everything issued has completed and signalled its barriers
-  if (elect_one()) tc_commit(bars.mma_done(v));
-  __syncwarp();
-  mbar_wait_warp(bars.mma_done(v), 0u, ab);
+  tc_commit(bars.mma_done(v));
+  mbar_wait(bars.mma_done(v), 0u, ab);
 }
 
 // ---------------------------------------------------------------------------------------------- visit 1: sums
@@ -363,6 +390,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
   float next_ref = produced(refs + sh.slab(0)), next_c = FP8 ? produced(slab_c + sh.slab(0)) : a.c;
+#pragma unroll 1
   for (int n = 0; n < n_slabs; ++n) {
     const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
     if (n + 1 < n_slabs) {
@@ -370,6 +398,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
       if constexpr (FP8) next_c = produced(slab_c + sh.slab(n + 1));
     }
     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
     for (; lt < n_tiles; lt += 2) {
       if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
@@ -419,14 +448,16 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
   }
 }
 
-// The sums where keys are the lanes.  Tiles k with k mod 2 == set; a thread has one key per tile and sums of all rows, which it
-// shares out over the warp at the end of a slab.  (The two-pass form with its 64 rows took 10 to 20 % longer this way, whether
-// a warp had all rows of every other tile or half the rows of each.  With 16 rows it is the quicker one, 960 -> 910 us for
-// 16 layers x 8 heads at 340942 tokens, and its columns are half as many: 28 tiles a CTA at 16 slots a key instead of 26, where
-// the general path takes 152 us for two layers at 511438 tokens and this one 105.)
+// The sums where keys are the lanes.  Tiles k with k mod 2 == set; a thread has four keys of a tile and sums of a quarter of the
+// rows, which the warp's eight groups of lanes share out at the end of a slab (7 shuffles for 32 rows; with one key and all rows
+// to a thread there were 31, and that step took 0.38 us).  (The two-pass form with 64 or 32 rows has query rows as lanes instead.
+// With 16 rows keys are the quicker ones, 960 -> 910 us for 16 layers x 8 heads at 340942 tokens, and its columns are half as many:
+// 28 tiles a CTA at 16 slots a key instead of 26, where the general path takes 152 us for two layers at 511438 tokens and this one
+// 105.)
 template <class T, int NCOLS, bool FP8, bool ONCE>
 __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
                                              const FusedBars& bars, const Abort& ab) {
+  constexpr int CT = NCOLS / 4;
   const FusedPrompt& p = *sh.p;
   const int quad = warp & 3, set = (warp - kSumWarp0) >> 2;
   const int n_slabs = sh.n_slabs, n_tiles = sh.n_tiles;
@@ -434,27 +465,29 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
   const float* const slab_c = p.slab_c;
   const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
-  const int tail_lanes = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32;   // real keys of this quadrant in the last tile
+  // of the last, partial tile: real keys from this thread's first on
+  const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32 - (lane >> 2);
   const bool frees = !ONCE || a.mode == 1;                // the accumulators wait for no visit 2
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
   float next_ref = produced(refs + sh.slab(0)), next_c = FP8 ? produced(slab_c + sh.slab(0)) : a.c;
+#pragma unroll 1
   for (int n = 0; n < n_slabs; ++n) {
     const uint64_t nref = pack2(-next_ref, -next_ref), cc = pack2(next_c, next_c);
     if (n + 1 < n_slabs) {
       next_ref = produced(refs + sh.slab(n + 1));
       if constexpr (FP8) next_c = produced(slab_c + sh.slab(n + 1));
     }
-    uint64_t acc[NCOLS / 2];
+    uint64_t acc[CT];                                              // two keys each
 #pragma unroll
-    for (int j = 0; j < NCOLS / 2; ++j) acc[j] = 0ull;
-    const bool any = lt < n_tiles;
+    for (int j = 0; j < CT; ++j) acc[j] = 0ull;
+#pragma unroll 1
     for (; lt < n_tiles; lt += 2) {
       if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
       uint32_t r[NCOLS];
-      tmem_issue<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
+      tmem_issue_quarters<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
       tmem_load_wait();
       tmem_ready<NCOLS>(r);
       if (frees) {
@@ -463,40 +496,50 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
         if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
       }
       tr.advance(2);
-      if (sh.tile(lt) < full_tiles || lane < tail_lanes) {
+      if (sh.tile(lt) < full_tiles) {
 #pragma unroll
         for (int j = 0; j < NCOLS / 2; ++j) {
           float x, y;
           unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
-          acc[j] = add2(acc[j], pack2(fast_exp2(x), fast_exp2(y)));
+          acc[j % CT] = add2(acc[j % CT], pack2(fast_exp2(x), fast_exp2(y)));
+        }
+      } else {
+        // keys beyond the prompt's end count nothing
+#pragma unroll
+        for (int j = 0; j < NCOLS / 2; ++j) {
+          const int key = j / CT * 16;
+          float x, y;
+          unpack2(fma2(pack2(r[2 * j], r[2 * j + 1]), cc, nref), x, y);
+          acc[j % CT] = add2(acc[j % CT], pack2(key < tail_keys ? fast_exp2(x) : 0.f, key + 8 < tail_keys ? fast_exp2(y) : 0.f));
         }
       }
     }
     lt -= n_tiles;
-    // Sum over the warp's 32 keys: transposing butterfly steps, each of which halves the columns a lane holds, then (16
-    // columns) one plain step.  The publishers add up quadrants and sets.
-    float s[NCOLS];
-    s[0] = 0.f;
-    if (any) {
+    // Transposing butterfly steps over the eight groups of lanes, each of which halves the columns a lane holds, then (16 columns)
+    // one plain step.  The publishers add up quadrants and sets.
+    float s[CT];
 #pragma unroll
-      for (int j = 0; j < NCOLS / 2; ++j) unpack2(acc[j], s[2 * j], s[2 * j + 1]);
-      int width = NCOLS;
+    for (int j = 0; j < CT; ++j) {
+      float x, y;
+      unpack2(acc[j], x, y);
+      s[j] = x + y;
+    }
+    int width = CT;
 #pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) {
-        if (width > 1) {
-          width >>= 1;
-          const bool upper = (lane & off) != 0;
+    for (int off = 16; off >= 4; off >>= 1) {
+      if (width > 1) {
+        width >>= 1;
+        const bool upper = (lane & off) != 0;
 #pragma unroll
-          for (int j = 0; j < NCOLS / 2; ++j) {
-            if (j < width) {
-              const float send = upper ? s[j] : s[j + width];
-              const float keep = upper ? s[j + width] : s[j];
-              s[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-            }
+        for (int j = 0; j < CT / 2; ++j) {
+          if (j < width) {
+            const float send = upper ? s[j] : s[j + width];
+            const float keep = upper ? s[j + width] : s[j];
+            s[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
           }
-        } else {
-          s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
         }
+      } else {
+        s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
       }
     }
     const int slot = n % kSumSlots;
@@ -506,7 +549,7 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
     if constexpr (NCOLS == 32) {
       out[lane] = s[0];
     } else {
-      if ((lane & 1) == 0) out[lane >> 1] = s[0];
+      if ((lane & 4) == 0) out[(lane >> 3) * 4 + (lane & 3)] = s[0];
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.sums_ready(slot));
@@ -514,47 +557,71 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
 }
 
 // ---------------------------------------------------------------------------------------------- publishers
-// Waits for and adds up CTAs' row sums of a slab.  LANES = 1: the four rows of quad `q`, a CTA per lane; LANES = NCOLS / 4:
-// all rows, lane mod LANES being the quad.  On return lane (with lane mod 8 < LANES) has the log-sum-exp, in base-2 units,
-// of row 4 * quad + lane / 8 in `lse2`; false if the wait was given up.
-template <int NCOLS, int G, int LANES, int MAXW>
-__device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPrompt& p, int slab, int q, int n_ctas, int lane, bool report,
-                                            float& lse2, const Abort& ab) {
-  constexpr int Q = NCOLS / 4, STEP = 32 / LANES;                  // CTAs per load of the warp
-  if (LANES > 1) q = lane % Q;
-  const int first = lane / LANES;
-  const float4* in = p.row_sums + ((int64_t)slab * p.per_part + first) * Q + q;
-  const float ref = produced(p.refs + slab);                        // its way to L2 and back passes during the wait below
-  float4 v[MAXW];
+// Everybody's row sums of a slab, as they come in: LANES quads (float4 of rows) q0 .. q0 + LANES - 1, lane mod LANES being the
+// quad, lane / LANES the first CTA.  Whatever is not there yet is asked for again.  A quad is stored and loaded as one 128-bit word.
+template <int NCOLS, int LANES, int MAXW>
+struct RowSums {
+  static constexpr int Q = NCOLS / 4, STEP = 32 / LANES;           // CTAs per load of the warp
+  uint64_t lo[MAXW], hi[MAXW];                                     // rows 0 and 1, 2 and 3 of the quad
+  const float4* in;
+  int left;                                                        // CTAs from this lane's first on
+  __device__ __forceinline__ void begin(const FusedPrompt& p, int slab, int q0, int n_ctas, int lane) {
+    in = p.row_sums + ((int64_t)slab * p.per_part + lane / LANES) * Q + q0 + lane % LANES;
+    left = n_ctas - lane / LANES;
 #pragma unroll
-  for (int i = 0; i < MAXW; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto missing = [&](int i) {
-    return first + STEP * i < n_ctas && (v[i].x == 0.f || v[i].y == 0.f || v[i].z == 0.f || v[i].w == 0.f);
-  };
-  unsigned long long t0 = 0;
-  for (uint32_t it = 1;; ++it) {
-    // whatever is not there yet is asked for again (a word may also be caught half written)
+    for (int i = 0; i < MAXW; ++i) lo[i] = hi[i] = 0ull;
+  }
+  __device__ __forceinline__ bool missing(int i) const { return STEP * i < left && (uint32_t)lo[i] == 0u; }
+  __device__ __forceinline__ void ask() {
 #pragma unroll
     for (int i = 0; i < MAXW; ++i)
       if (missing(i))
-        asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w)
+        asm volatile("{\n.reg .b128 w;\nld.relaxed.gpu.global.b128 w, [%2];\nmov.b128 {%0, %1}, w;\n}"
+                     : "=l"(lo[i]), "=l"(hi[i])
                      : "l"(in + (int64_t)STEP * i * Q)
                      : "memory");
-    bool there = true;
-#pragma unroll
-    for (int i = 0; i < MAXW; ++i) there = there && !missing(i);
-    if (__all_sync(0xffffffffu, there)) break;
-    if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return false;
-    if (LANES == 1) __nanosleep(100);
   }
+  __device__ __forceinline__ bool there() const {
+    bool all = true;
+#pragma unroll
+    for (int i = 0; i < MAXW; ++i) all = all && !missing(i);
+    return __all_sync(0xffffffffu, all);
+  }
+};
+
+// The log-sum-exp, in base-2 units, of one row from its total: reported where it is to be.
+static __device__ __noinline__ float lse_of(double total, float ref, const float* extra, float* out, int32_t* status) {
+  // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision; an empty (below every
+  // normal number) or overflowed row sum has none
+  const long long tb = __double_as_longlong(total);
+  const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+  float lse2 = ref + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
+  if (!(total > 1.2e-38 && total < (double)INFINITY)) lse2 = INFINITY;
+  if (extra != nullptr) {
+    // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
+    const float e = __ldg(extra) * kLog2e;
+    const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
+    lse2 = hi + log2f(1.f + exp2f(lo - hi));
+  }
+  if (status != nullptr && !(lse2 > -INFINITY && lse2 < INFINITY)) atomicCAS(status, 0, (int32_t)SPF_ERR_RANGE);
+  if (out != nullptr) *out = lse2 * kLn2;
+  return lse2;
+}
+
+// The log-sum-exps, in base-2 units, from a complete set of sums: lane (with lane mod 8 < LANES) gets that of row
+// 4 * (q0 + lane mod LANES) + lane / 8.
+template <int NCOLS, int G, int LANES, int MAXW>
+__device__ __forceinline__ float row_lse(const FusedArgs& a, const FusedPrompt& p, const RowSums<NCOLS, LANES, MAXW>& w, int n_ctas, int slab,
+                                         float ref, int q0, int lane, bool report) {
   double t[4] = {0.0, 0.0, 0.0, 0.0};                              // the CTAs' shares are fp32: exact to 2^-53
 #pragma unroll
   for (int i = 0; i < MAXW; ++i) {
-    t[0] += (double)v[i].x;
-    t[1] += (double)v[i].y;
-    t[2] += (double)v[i].z;
-    t[3] += (double)v[i].w;
+    if (i > 0 && RowSums<NCOLS, LANES, MAXW>::STEP * i >= n_ctas) break;
+    float x[4];
+    unpack2(w.lo[i], x[0], x[1]);
+    unpack2(w.hi[i], x[2], x[3]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) t[e] += (double)x[e];
   }
   // two transposing steps leave one row per lane: lanes 8.. have t[1], 16.. t[2], 24.. t[3]
 #pragma unroll
@@ -568,91 +635,131 @@ __device__ __forceinline__ bool sum_rows_of(const FusedArgs& a, const FusedPromp
   }
 #pragma unroll
   for (int off = 4; off >= LANES; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
-  const int row = 4 * q + (lane >> 3);
-  lse2 = INFINITY;                                                 // rows that do not exist: exp2(x - lse2) = 0
-  if ((lane & 7) < LANES && row % G < a.group && row / G < a.n_lookahead) {
-    // log2 of the total: its binary exponent plus the log2 of its mantissa in single precision; an empty (below every
-    // normal number) or overflowed row sum has none
-    const long long tb = __double_as_longlong(t[0]);
-    const float mant = (float)__longlong_as_double((tb & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-    lse2 = ref + ((float)((int)((tb >> 52) & 0x7ff) - 1023) + log2f(mant));
-    if (!(t[0] > 1.2e-38 && t[0] < (double)INFINITY)) lse2 = INFINITY;
-    const int64_t out_idx = ((int64_t)slab * a.group + row % G) * a.n_lookahead + row / G;
-    if (p.extra_lse != nullptr) {
-      // the denominator also holds exp(extra): log2-add, in the order that cannot overflow
-      const float e = __ldg(p.extra_lse + out_idx) * kLog2e;
-      const float hi = fmaxf(lse2, e), lo = fminf(lse2, e);
-      lse2 = hi + log2f(1.f + exp2f(lo - hi));
-    }
-    if (report) {
-      if (!(lse2 > -INFINITY && lse2 < INFINITY) && a.dev_status != nullptr) atomicCAS(a.dev_status, 0, (int32_t)SPF_ERR_RANGE);
-      if (p.lse_out != nullptr) p.lse_out[out_idx] = lse2 * kLn2;
-    }
-  }
-  return true;
+  const QueryRow r = query_row(4 * (q0 + lane % LANES) + (lane >> 3), NCOLS, G);
+  if (!((lane & 7) < LANES && r.g < a.group && r.i < a.n_lookahead)) return INFINITY;   // rows that do not exist: exp2(x - lse2) = 0
+  const int64_t at = ((int64_t)slab * a.group + r.g) * a.n_lookahead + r.i;
+  return lse_of(t[0], ref, p.extra_lse != nullptr ? p.extra_lse + at : nullptr, report && p.lse_out != nullptr ? p.lse_out + at : nullptr,
+                report ? a.dev_status : nullptr);
 }
 
-// Publisher w takes slabs w, w + 3, ...: stores this CTA's row sums (a row that does not exist gets its meaningless sum
-// stored too: everybody waits for every word).  Then either this CTA adds up everybody's sums for itself (few CTAs to a
-// group: one hop), or only those of the rows that it owns -- item n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab,
-// belongs to CTA (item mod CTAs) -- and stores their log-sum-exps for all.  Not before its own sums are out: polling for
-// words that cannot be there yet slowed the key copies down.
-template <class T, int NCOLS, int G, bool FP8>
-__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums, float* off,
-                                              float* off_c, const FusedBars& bars, const Abort& ab) {
-  constexpr int Q = NCOLS / 4;                                     // lane q has rows 4q .. 4q + 3
+// Stores this CTA's sums of quads q0 .. q0 + LANES - 1 of its n-th slab for all to read (a row that does not exist gets its
+// meaningless sum stored too: everybody waits for every word).
+template <int NCOLS, int LANES>
+__device__ __forceinline__ void store_sums(const FusedPrompt& p, const FusedShare& sh, int n, int q0, int lane, const float* sums,
+                                           const FusedBars& bars) {
+  constexpr int Q = NCOLS / 4;
+  const int slot = n % kSumSlots, q = q0 + lane;
+  float t[4] = {0.f, 0.f, 0.f, 0.f};
+  if (lane < LANES) {
+    // [set][quadrant][lane]: 64 rows: quadrants 0 and 2 have rows 0..31, 1 and 3 rows 32..63; else every quadrant all rows
+    const float* in = sums + slot * 256 + (NCOLS == 64 ? (q >> 3) * 32 + (q & 7) * 4 : q * 4);
+#pragma unroll
+    for (int set = 0; set < 2; ++set)
+#pragma unroll
+      for (int quad = 0; quad < (NCOLS == 64 ? 2 : 4); ++quad) {
+        const float4 v = *reinterpret_cast<const float4*>(in + set * 128 + quad * (NCOLS == 64 ? 64 : 32));
+        t[0] += v.x;
+        t[1] += v.y;
+        t[2] += v.z;
+        t[3] += v.w;
+      }
+    unsigned w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = max(__float_as_uint(t[e]), 1u);   // never "not there yet"; 2^-149 is nothing to a row's sum
+    asm volatile("{\n.reg .b128 w;\n.reg .b64 lo, hi;\nmov.b64 lo, {%1, %2};\nmov.b64 hi, {%3, %4};\nmov.b128 w, {lo, hi};\n"
+                 "st.relaxed.gpu.global.b128 [%0], w;\n}"
+                 ::"l"(p.row_sums + ((int64_t)sh.slab(n) * p.per_part + sh.first) * Q + q), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                 : "memory");
+  }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bars.sums_free(slot));
+}
+
+// Few CTAs to a group: every CTA adds up everybody's sums.  One warp stores the CTA's own, slab after slab; two warps (resident:
+// two teams of two that take the slabs in turn) wait for everybody's, half the rows each.  (With the same warps storing and
+// waiting, sums went out up to 2.3 us late: 32 rows at 4001 tokens.)
+template <int NCOLS>
+__device__ __forceinline__ void fused_store(const FusedShare& sh, int lane, const float* sums, volatile int* stored, const FusedBars& bars,
+                                            const Abort& ab) {
+#pragma unroll 1
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    if (!mbar_wait_warp(bars.sums_ready(n % kSumSlots), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
+    store_sums<NCOLS, NCOLS / 4>(*sh.p, sh, n, 0, lane, sums, bars);
+    if (lane == 0) *stored = n + 1;
+  }
+}
+
+template <class T, int NCOLS, int G, bool FP8, int TEAMS>
+__device__ __forceinline__ void fused_gather(const FusedArgs& a, const FusedShare& sh, int which, int lane, volatile int* stored, float* off,
+                                             float* off_c, const FusedBars& bars, const Abort& ab) {
+  constexpr int LANES = NCOLS / 4 / kTeamWarps;                    // quads of this warp
+  constexpr int MAXW = (gather_ctas(NCOLS) * LANES + 31) / 32;
   const FusedPrompt& p = *sh.p;
-  const int per_part = p.per_part, n_ctas = min(per_part, p.n_tiles);
-  const bool alone = gather_alone(NCOLS, n_ctas);
-  for (int n = which; n < sh.n_slabs; n += kPublisherWarps) {
-    const int slot = n % kSumSlots, slab = sh.slab(n);
-    if (!mbar_wait_warp(bars.sums_ready(slot), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
-    float t[4] = {0.f, 0.f, 0.f, 0.f};
-    if (lane < Q) {
-      // [set][quadrant][lane]: 64 rows: quadrants 0 and 2 have rows 0..31, 1 and 3 rows 32..63; else every quadrant all rows
-      const float* in = sums + slot * 256 + (NCOLS == 64 ? (lane >> 3) * 32 + (lane & 7) * 4 : lane * 4);
-#pragma unroll
-      for (int set = 0; set < 2; ++set)
-#pragma unroll
-        for (int q = 0; q < (NCOLS == 64 ? 2 : 4); ++q) {
-          const float4 v = *reinterpret_cast<const float4*>(in + set * 128 + q * (NCOLS == 64 ? 64 : 32));
-          t[0] += v.x;
-          t[1] += v.y;
-          t[2] += v.z;
-          t[3] += v.w;
-        }
+  const int n_ctas = min(p.per_part, p.n_tiles), q0 = which % kTeamWarps * LANES;
+  if (a.mode == 1 && sh.first != 0) return;                        // visit 1 alone: nobody but the one that reports needs the sums
+  RowSums<NCOLS, LANES, MAXW> w;
+#pragma unroll 1
+  for (int n = which / kTeamWarps; n < sh.n_slabs; n += TEAMS) {
+    const int slab = sh.slab(n);
+    w.begin(p, slab, q0, n_ctas, lane);
+    const float ref = produced(p.refs + slab);                     // its way to L2 and back passes during the waits below
+    const float c = FP8 ? produced(p.slab_c + slab) : 0.f;
+    unsigned long long t0 = 0;
+    // not before the own sums are out: polling for words that cannot be there yet slows the key copies down
+#pragma unroll 1
+    for (uint32_t it = 1; __any_sync(0xffffffffu, *stored <= n); ++it) {
+      if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
+      __nanosleep(20);
+    }
+#pragma unroll 1
+    for (uint32_t it = 1;; ++it) {
+      w.ask();
+      if (w.there()) break;
+      if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
+      if (it > 4) __nanosleep(100);                                // CTAs far apart: then there is also time
+    }
+    const float lse2 = row_lse<NCOLS, G, LANES, MAXW>(a, p, w, n_ctas, slab, ref, q0, lane, sh.first == 0);
+    if (a.mode == 1) continue;
+    const int x = n % kOffSlots;
+    if (n >= kOffSlots)
+      if (!mbar_wait_warp(bars.off_free(x), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
+    if ((lane & 7) < LANES) store_off(off + x * kOffFloats, NCOLS, 4 * (q0 + lane % LANES) + (lane >> 3), -lse2);
+    if constexpr (FP8) {
+      if (q0 == 0 && lane == 0) off_c[x] = c;
     }
     __syncwarp();
-    if (lane == 0) mbar_arrive(bars.sums_free(slot));
-    if (lane < Q) {
-      unsigned w[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) w[e] = max(__float_as_uint(t[e]), 1u);   // never "not there yet"; 2^-149 is nothing to a row's sum
-      asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};"
-                   ::"l"(p.row_sums + ((int64_t)slab * per_part + sh.first) * Q + lane), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
-                   : "memory");
-    }
-    float lse2;
-    if constexpr (NCOLS <= 32) {
-      if (alone) {
-        if (a.mode == 1 && sh.first != 0) continue;                // nobody reads the offsets
-        const float c = FP8 ? produced(p.slab_c + slab) : 0.f;
-        if (!sum_rows_of<NCOLS, G, Q, kGatherCtas * Q / 32>(a, p, slab, 0, n_ctas, lane, sh.first == 0, lse2, ab)) return;
-        if (a.mode == 1) continue;
-        const int x = n % kOffSlots;
-        if (n >= kOffSlots)
-          if (!mbar_wait_warp(bars.off_free(x), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
-        if ((lane & 7) < Q) off[x * 64 + 4 * (lane % Q) + (lane >> 3)] = -lse2;
-        if constexpr (FP8) {
-          if (lane == 0) off_c[x] = c;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars.off_ready(x));
-        continue;
-      }
-    }
+    if (lane == 0) mbar_arrive(bars.off_ready(x));
+  }
+}
+
+// Many: publisher w takes slabs w, w + 3, ...: stores this CTA's row sums, then adds up those of the rows that it owns -- item
+// n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab, belongs to CTA (item mod CTAs) -- and stores their log-sum-exps for all.
+// Not before its own sums are out: polling for words that cannot be there yet slowed the key copies down.
+template <class T, int NCOLS, int G>
+__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums,
+                                              const FusedBars& bars, const Abort& ab) {
+  constexpr int Q = NCOLS / 4, MAXW = (kFusedMaxCtas + 31) / 32;   // lane q has rows 4q .. 4q + 3
+  const FusedPrompt& p = *sh.p;
+  const int n_ctas = min(p.per_part, p.n_tiles);
+#pragma unroll 1
+  for (int n = which; n < sh.n_slabs; n += kPublisherWarps) {
+    const int slab = sh.slab(n);
+    if (!mbar_wait_warp(bars.sums_ready(n % kSumSlots), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
+    store_sums<NCOLS, Q>(p, sh, n, 0, lane, sums, bars);
+#pragma unroll 1
     for (int q = (int)(((unsigned)(n + 1) * (unsigned)n_ctas * Q + sh.first - n * Q) % (unsigned)n_ctas); q < Q; q += n_ctas) {
-      if (!sum_rows_of<NCOLS, G, 1, (kFusedMaxCtas + 31) / 32>(a, p, slab, q, n_ctas, lane, true, lse2, ab)) return;
+      RowSums<NCOLS, 1, MAXW> w;
+      w.begin(p, slab, q, n_ctas, lane);
+      const float ref = produced(p.refs + slab);
+      unsigned long long t0 = 0;
+#pragma unroll 1
+      for (uint32_t it = 1;; ++it) {
+        w.ask();
+        if (w.there()) break;
+        if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
+        __nanosleep(100);
+      }
+      const float lse2 = row_lse<NCOLS, G, 1, MAXW>(a, p, w, n_ctas, slab, ref, q, lane, true);
       if ((lane & 7) == 0) {
         const unsigned long long word = (1ull << 32) | __float_as_uint(lse2);
         asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.lse + (int64_t)slab * NCOLS + 4 * q + (lane >> 3)), "l"(word) : "memory");
@@ -663,135 +770,161 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
 }
 
 // ---------------------------------------------------------------------------------------------- log-sum-exps for visit 2
-// Fetches each slab's log-sum-exps in turn, kAhead slabs' words in flight, and hands them to the max warps through shared
-// memory (negated: what visit 2 adds).
+// Fetches each slab's log-sum-exps in turn and hands them to the max warps through shared memory (negated: what visit 2 adds).
 template <class T, int NCOLS, int G, bool FP8>
 __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedShare& sh, int lane, float* off, float* off_c,
                                                 const FusedBars& bars, const Abort& ab) {
   const FusedPrompt& p = *sh.p;
   constexpr int RPL = NCOLS == 64 ? 2 : 1;
-  constexpr int kAhead = 4;
-  unsigned long long w[kAhead][RPL];
-  auto load = [&](unsigned long long (&dst)[RPL], int n) {
+  const bool there_already = a.mode == 2;                          // supplied by the caller
+#pragma unroll 1
+  for (int n = 0; n < sh.n_slabs; ++n) {
+    const int slab = sh.slab(n);
+    const float c = FP8 ? produced(p.slab_c + slab) : 0.f;
+    float v[RPL];
+    if (there_already) {
 #pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-      const int row = min(lane + 32 * r, NCOLS - 1);
-      if (a.mode == 2) {
-        const bool real = row % G < a.group && row / G < a.n_lookahead;
-        const float v = real ? __ldg(p.lse_in + ((int64_t)sh.slab(n) * a.group + row % G) * a.n_lookahead + row / G) * kLog2e : INFINITY;
-        dst[r] = (1ull << 32) | __float_as_uint(v);
-      } else {
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(dst[r]) : "l"(p.lse + (int64_t)sh.slab(n) * NCOLS + row) : "memory");
+      for (int r = 0; r < RPL; ++r) {
+        const QueryRow q = query_row(min(lane + 32 * r, NCOLS - 1), NCOLS, G);
+        v[r] = q.g < a.group && q.i < a.n_lookahead ? -__ldg(p.lse_in + ((int64_t)slab * a.group + q.g) * a.n_lookahead + q.i) * kLog2e : -INFINITY;
       }
-    }
-  };
+    } else {
+      unsigned long long w[RPL], t0 = 0;
+#pragma unroll 1
+      for (uint32_t it = 1;; ++it) {
+        bool there = true;
 #pragma unroll
-  for (int i = 0; i < kAhead; ++i)
-    if (i < sh.n_slabs) load(w[i], i);
-  for (int n0 = 0; n0 < sh.n_slabs; n0 += kAhead) {
-#pragma unroll
-    for (int i = 0; i < kAhead; ++i) {
-      const int n = n0 + i;
-      if (n < sh.n_slabs) {
-        const float c = FP8 ? produced(p.slab_c + sh.slab(n)) : 0.f;
-        unsigned long long t0 = 0;
-        for (uint32_t it = 1;; ++it) {
-          bool there = true;
-#pragma unroll
-          for (int r = 0; r < RPL; ++r) there = there && (w[i][r] >> 32) != 0ull;
-          if (__all_sync(0xffffffffu, there)) break;
-          if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
-          load(w[i], n);
+        for (int r = 0; r < RPL; ++r) {
+          asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w[r]) : "l"(p.lse + (int64_t)slab * NCOLS + min(lane + 32 * r, NCOLS - 1)) : "memory");
+          there = there && (w[r] >> 32) != 0ull;
         }
-        float v[RPL];
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) v[r] = -__uint_as_float((unsigned)w[i][r]);
-        if (n + kAhead < sh.n_slabs) load(w[i], n + kAhead);
-        const int slot = n % kOffSlots;
-        if (n >= kOffSlots)
-          if (!mbar_wait_warp(bars.off_free(slot), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
-#pragma unroll
-        for (int r = 0; r < RPL; ++r)
-          if (lane + 32 * r < NCOLS) off[slot * 64 + lane + 32 * r] = v[r];
-        if constexpr (FP8) {
-          if (lane == 0) off_c[slot] = c;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars.off_ready(slot));
+        if (__all_sync(0xffffffffu, there)) break;
+        if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
       }
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) v[r] = -__uint_as_float((unsigned)w[r]);
     }
+    const int slot = n % kOffSlots;
+    if (n >= kOffSlots)
+      if (!mbar_wait_warp(bars.off_free(slot), (uint32_t)(n / kOffSlots - 1) & 1u, ab)) return;
+#pragma unroll
+    for (int r = 0; r < RPL; ++r)
+      if (lane + 32 * r < NCOLS) store_off(off + slot * kOffFloats, NCOLS, lane + 32 * r, v[r]);
+    if constexpr (FP8) {
+      if (lane == 0) off_c[slot] = c;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bars.off_ready(slot));
   }
 }
 
 // ---------------------------------------------------------------------------------------------- importance
 // Mean over the lookahead of exp2(running max) for a tile's keys.  One group of CTAs (parts = 1): straight from the maxima.
 // Several: the groups' maxima meet in global memory, and whichever warp brings the last contribution for 32 keys reads the
-// result.
-template <int NI>
+// result.  v[x] belongs to key 8 * key_of(x) + lane / 4 of the quadrant and lookahead i_of(x).
+template <int NI, bool PAIRS>
 __device__ __forceinline__ void finish_tile(const FusedArgs& a, const FusedPrompt& p, int tile, int quad, int lane, const uint32_t (&v)[NI]) {
   const float inv_m = 1.f / (float)a.n_lookahead;
-  const int64_t key = (int64_t)tile * kTileKeys + quad * 32 + lane;
+  const int64_t key0 = (int64_t)tile * kTileKeys + quad * 32;
+  const int t = lane & 3;
+  auto key_of = [&](int x) { return PAIRS ? 2 * (t & 1) + x : x & 3; };
+  auto i_of = [&](int x) { return PAIRS ? t >> 1 : (x >> 2) * 4 + t; };
+  int64_t key;
   float sum = 0.f;
   if (p.parts == 1) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};                             // of the thread's keys, over its lookahead slots
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-      if (i < a.n_lookahead) sum += fast_exp2(__uint_as_float(v[i]));
+    for (int x = 0; x < NI; ++x) {
+      const float e = i_of(x) < a.n_lookahead ? fast_exp2(__uint_as_float(v[x])) : 0.f;
+      if constexpr (PAIRS) {
+        s[x] += (t & 1) == 0 ? e : 0.f;
+        s[2 + x] += (t & 1) != 0 ? e : 0.f;
+      } else {
+        s[x & 3] += e;
+      }
+    }
+    // the four lanes of a key's lookahead slots; lane t keeps key 8 * t + lane / 4
+#pragma unroll
+    for (int u = 0; u < 2; ++u) s[u] = ((t & 2) ? s[u + 2] : s[u]) + __shfl_xor_sync(0xffffffffu, (t & 2) ? s[u] : s[u + 2], 2);
+    sum = ((t & 1) ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, (t & 1) ? s[0] : s[1], 1);
+    key = key0 + 8 * t + (lane >> 2);
   } else {
     const int64_t n_pad = (int64_t)p.n_tiles * kTileKeys;
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-      if (i < a.n_lookahead) atomicMax(p.amax + (int64_t)i * n_pad + key, order_bits(__uint_as_float(v[i])));
+    for (int x = 0; x < NI; ++x)
+      if (i_of(x) < a.n_lookahead)
+        atomicMax(p.amax + (int64_t)i_of(x) * n_pad + key0 + 8 * key_of(x) + (lane >> 2), order_bits(__uint_as_float(v[x])));
     __threadfence();
     __syncwarp();
     unsigned before = 0;
     if (lane == 0) before = atomicAdd(p.finished + tile * 4 + quad, 1u);
     if (__shfl_sync(0xffffffffu, before, 0) + 1u != (unsigned)p.parts) return;
     __threadfence();
-#pragma unroll 8
+    key = key0 + lane;
+#pragma unroll 4
     for (int i = 0; i < a.n_lookahead; ++i) sum += fast_exp2(from_order_bits(__ldcg(p.amax + (int64_t)i * n_pad + key)));
   }
   if (key < p.n_tokens) p.importance[key] = sum * inv_m;
 }
 
-// The tiles of a max warp's set, from the maxima in tensor memory.
+// The tiles of a max warp's set, from the maxima in tensor memory: tile lt's in stage (first + lt) mod stages, `cols` columns each.
 template <class T>
-__device__ __forceinline__ void fused_finish(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t amax_tmem) {
+__device__ __forceinline__ void fused_finish(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t lane_addr, Ring first, int cols) {
   const int quad = warp & 3, set = (warp - kMaxWarp0) >> 2;
-  const uint32_t lane_addr = amax_tmem + ((uint32_t)(quad * 32) << 16);
+  first.advance(set);
+#pragma unroll 1
   for (int lt = set; lt < sh.n_tiles; lt += 2) {
     constexpr int LD = T::NI < 32 ? T::NI : 32;                    // columns per load
     uint32_t v[T::NI];
 #pragma unroll
     for (int i = 0; i < T::NI; i += LD)
-      tmem_issue<LD>(lane_addr + (uint32_t)(lt * T::NI + i), *reinterpret_cast<uint32_t(*)[LD]>(v + i));
+      tmem_issue<LD>(lane_addr + (uint32_t)(first.stage * cols + i), *reinterpret_cast<uint32_t(*)[LD]>(v + i));
     tmem_load_wait();
     tmem_ready<T::NI>(v);
-    finish_tile<T::NI>(a, *sh.p, sh.tile(lt), quad, lane, v);
+    finish_tile<T::NI, T::PAIRS>(a, *sh.p, sh.tile(lt), quad, lane, v);
+    first.advance(2);
   }
 }
 
 // ---------------------------------------------------------------------------------------------- visit 2: maxima
 // Folds one load's accumulators into the running maxima over (layer, head) of the base-2 logits less their rows'
-// log-sum-exps (slots past n_lookahead hold padding and are never read).
+// log-sum-exps (slots past n_lookahead hold padding and are never read).  Maximum 4 * ih + k is that of the thread's key k and
+// lookahead 4 * ih + lane % 4; PAIRS: the two lanes of a lookahead's heads keep two keys each.
 template <class T, int G>
-__device__ __forceinline__ void fold_maxima(const uint32_t (&r)[T::CW], uint32_t (&am)[T::NIW], const ulonglong2* off2, uint64_t cc) {
-  float z[T::CW];
+__device__ __forceinline__ void fold_maxima(const uint32_t (&r)[T::CW], uint32_t (&am)[T::NIW], const float* off, float scale, int lane) {
+  float z[4][T::CT];
 #pragma unroll
-  for (int j = 0; j < T::CW / 4; ++j) {
-    const ulonglong2 o = off2[j];
-    unpack2(fma2(pack2(r[4 * j], r[4 * j + 1]), cc, o.x), z[4 * j], z[4 * j + 1]);
-    unpack2(fma2(pack2(r[4 * j + 2], r[4 * j + 3]), cc, o.y), z[4 * j + 2], z[4 * j + 3]);
-  }
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-  for (int i = 0; i < T::NIW; ++i) {
-    float m = __uint_as_float(am[i]);
-    if constexpr (G == 1) {
-      m = fmaxf(m, z[i]);
-    } else {
-#pragma unroll
-      for (int g = 0; g < G; g += 2) m = max3(m, z[i * G + g], z[i * G + g + 1]);
+    for (int c = 0; c < T::CT; ++c) {
+      const int at = h * (T::CW / 2) + 2 * c;
+      z[2 * h][c] = fmaf(__uint_as_float(r[at]), scale, off[c]);
+      z[2 * h + 1][c] = fmaf(__uint_as_float(r[at + 1]), scale, off[c]);
     }
-    am[i] = __float_as_uint(m);
+  if constexpr (T::PAIRS) {
+    float top[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) top[k] = fmaxf(max3(z[k][0], z[k][1], z[k][2]), z[k][3]);
+    const bool odd = lane & 1;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float other = __shfl_xor_sync(0xffffffffu, odd ? top[u] : top[2 + u], 1);
+      am[u] = __float_as_uint(max3(__uint_as_float(am[u]), odd ? top[2 + u] : top[u], other));
+    }
+  } else {
+#pragma unroll
+    for (int ih = 0; ih < T::CT / G; ++ih)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float m = __uint_as_float(am[4 * ih + k]);
+        if constexpr (G == 1) {
+          m = fmaxf(m, z[k][ih]);
+        } else {
+#pragma unroll
+          for (int g = 0; g < G; g += 2) m = max3(m, z[k][ih * G + g], z[k][ih * G + g + 1]);
+        }
+        am[4 * ih + k] = __float_as_uint(m);
+      }
   }
 }
 
@@ -801,6 +934,7 @@ __device__ __forceinline__ void clear_maxima(uint32_t amax_addr, int set, int n_
   uint32_t ninf[T::NIW];
 #pragma unroll
   for (int j = 0; j < T::NIW; ++j) ninf[j] = 0xff800000u;
+#pragma unroll 1
   for (int lt = set; lt < n_tiles; lt += 2)
 #pragma unroll
     for (int ch = 0; ch < T::NCH; ++ch) tmem_store<T::NIW>(amax_addr + (uint32_t)(lt * T::NI + ch * T::NIW), ninf);
@@ -830,25 +964,43 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
   }
   // resident: the stage of the slab's first tile; two-pass: a ring per set, this one's first stage and the next to be read
   Ring first(ONCE ? a.t_stages[V] : (a.t_stages[V] + 1 - set) / 2);
+  Ring last = first;                                               // resident: that of the slab before
   const int stage0 = ONCE ? 0 : set * ((a.t_stages[V] + 1) / 2);
+#pragma unroll 1
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
     if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
-    const ulonglong2* off2 = reinterpret_cast<const ulonglong2*>(off + slot * 64);
+    const float4* my_off = reinterpret_cast<const float4*>(off + slot * kOffFloats + (lane & 3) * off_stride(NCOLS));
+    float o[T::CT];                                                // one load a tile: the same for all tiles
+    auto load_off = [&](int ch) {
+#pragma unroll
+      for (int j = 0; j < T::CT / 4; ++j) *reinterpret_cast<float4*>(o + 4 * j) = my_off[ch * (T::CT / 4) + j];
+    };
+    if (NCH == 1) load_off(0);
     const float c = FP8 ? off_c[slot] : a.c;
-    const uint64_t cc = pack2(c, c);
     Ring tr = first;
     if (ONCE) tr.advance(set);
-    auto fold = [&](int lt, uint32_t (&m)[NIW]) -> bool {
-      // resident: complete long since (the log-sum-exps contain it), except where visit 2 runs alone
-      if (!mbar_wait_warp(bars.t_full(V, stage0 + tr.stage), tr.phase, ab)) return false;
+    if (ONCE) {
+      // all complete long since (the log-sum-exps contain them), except where visit 2 runs alone
+      if (a.mode == 2) {
+        Ring full = tr;
+#pragma unroll 1
+        for (int lt = set; lt < n_tiles; lt += 2, full.advance(2))
+          if (!mbar_wait_warp(bars.t_full(V, full.stage), full.phase, ab)) return;
+      }
       tc_fence_after();
+    }
+    auto fold = [&](int lt, uint32_t (&m)[NIW]) -> bool {
+      if constexpr (!ONCE) {
+        if (!mbar_wait_warp(bars.t_full(V, stage0 + tr.stage), tr.phase, ab)) return false;
+        tc_fence_after();
+      }
       if (!REGS) tmem_store_wait();                                // the maxima read below may be this warp's last stores
 #pragma unroll
       for (int ch = 0; ch < NCH; ++ch) {
         const uint32_t m_addr = amax_addr + (uint32_t)(lt * T::NI + ch * NIW);
         uint32_t r[CW];
-        tmem_issue<CW>(lane_addr + (uint32_t)((stage0 + tr.stage) * NCOLS + ch * CW), r);
+        tmem_issue_quarters<CW>(lane_addr + (uint32_t)((stage0 + tr.stage) * NCOLS + ch * CW), r);
         if (!REGS) tmem_issue<NIW>(m_addr, m);
         tmem_load_wait();
         tmem_ready<CW>(r);
@@ -858,7 +1010,8 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
           __syncwarp();
           if (lane == 0) mbar_arrive(bars.t_empty(V, stage0 + tr.stage));
         }
-        fold_maxima<T, G>(r, m, off2 + ch * (CW / 4), cc);
+        if (NCH > 1) load_off(ch);
+        fold_maxima<T, G>(r, m, o, c, lane);
         if (!REGS) tmem_store<NIW>(m_addr, m);
       }
       tr.advance(ONCE ? 2 : 1);
@@ -870,21 +1023,33 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
         if (set + 2 * u < n_tiles)
           if (!fold(set + 2 * u, am[u])) return;
     } else {
+#pragma unroll 1
       for (int lt = set; lt < n_tiles; lt += 2)
         if (!fold(lt, am[0])) return;
     }
-    if (ONCE) first.advance(n_tiles);
-    else first = tr;
+    if (ONCE) {
+      last = first;
+      first.advance(n_tiles);
+    } else {
+      first = tr;
+    }
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
   if constexpr (REGS) {
+    // to the columns of the last slab's logits, which only this warp would still read
+    Ring to = last;
+    to.advance(set);
 #pragma unroll
-    for (int u = 0; u < MINE; ++u)
-      if (set + 2 * u < n_tiles) finish_tile<NIW>(a, *sh.p, sh.tile(set + 2 * u), quad, lane, am[u]);
+    for (int u = 0; u < MINE; ++u) {
+      if (set + 2 * u < n_tiles) tmem_store<NIW>(lane_addr + (uint32_t)(to.stage * NCOLS), am[u]);
+      to.advance(2);
+    }
+    tmem_store_wait();
+    fused_finish<T>(a, sh, warp, lane, lane_addr, last, NCOLS);
   } else {
     tmem_store_wait();
-    fused_finish<T>(a, sh, warp, lane, amax_tmem);
+    fused_finish<T>(a, sh, warp, lane, amax_addr, Ring(1 << 30), T::NI);
   }
 }
 
@@ -901,7 +1066,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   float* sums = reinterpret_cast<float*>(smem + lay.sums_off);
   float* off = reinterpret_cast<float*>(smem + lay.off_off);
   float* off_c = reinterpret_cast<float*>(smem + lay.offc_off);
-  volatile int* misc = reinterpret_cast<volatile int*>(smem + lay.misc_off);  // [0] abort, [1] tensor-memory base, [2] tiles visit 2 has issued
+  volatile int* misc = reinterpret_cast<volatile int*>(smem + lay.misc_off);  // [0] abort, [1] tensor-memory base, [2] tiles visit 2 has issued, [3] slabs whose sums are stored
   const FusedBars bars{smem_u32(smem + lay.bar_off)};
   const Abort ab{misc, a.dev_status};
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -923,38 +1088,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
     sh.n_tiles = sh.first < min(p.per_part, p.n_tiles) ? (p.n_tiles - sh.first + sh.step - 1) / sh.step : 0;
   }
   if (sh.n_tiles == 0) return;
+  const bool visit1 = a.mode != 2, visit2 = a.mode != 1;
+  const bool gathers = visit1 && gather_alone(NCOLS, min(sh.p->per_part, sh.p->n_tiles));
 
   // ------------------------------------------------------------------ set-up
-  if (threadIdx.x == 0) {
-    misc[0] = 0;
-    misc[1] = 0;
-    misc[2] = 0;
-    for (int v = 0; v < (ONCE ? 1 : 2); ++v) {
-      for (int s = 0; s < a.k_stages[v]; ++s) {
-        mbar_init(bars.k_full(v, s), 1);
-        mbar_init(bars.k_empty(v, s), 1);
-      }
-      for (int s = 0; s < T::QS; ++s) {
-        mbar_init(bars.q_full(v, s), 1);
-        mbar_init(bars.q_empty(v, s), 1);
-      }
-      for (int s = 0; s < a.t_stages[v]; ++s) {
-        mbar_init(bars.t_full(v, s), 1);
-        mbar_init(bars.t_empty(v, s), kVisitWarps / 2);
-      }
-      mbar_init(bars.mma_done(v), 1);
-    }
-    for (int x = 0; x < kOffSlots; ++x) {
-      mbar_init(bars.off_ready(x), 1);
-      mbar_init(bars.off_free(x), kVisitWarps);
-    }
-    for (int x = 0; x < kSumSlots; ++x) {
-      mbar_init(bars.sums_ready(x), kVisitWarps);
-      mbar_init(bars.sums_free(x), 1);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (threadIdx.x < 4) misc[threadIdx.x] = 0;
+  for (int x = (int)threadIdx.x - 32; x >= 0 && x < FusedBars::kCount; x += kFusedThreads) {
+    uint32_t count = 1;
+    if (x >= FusedBars::kTmem + kMaxResident && x < FusedBars::kShared) count = kVisitWarps / 2;   // t_empty
+    else if (x >= FusedBars::kOffReady && x < FusedBars::kOffFree) count = gathers ? kTeamWarps : 1;
+    else if (x >= FusedBars::kOffFree && x < FusedBars::kSumsFree) count = kVisitWarps;            // off_free, sums_ready
+    mbar_init(bars.base + 8u * x, count);
   }
-  // paged key cache: a tile never straddles a block (blocks are multiples of 128 tokens): one lookup per tile for the whole kernel
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   int2* const tile_at = reinterpret_cast<int2*>(smem + lay.tile_off);
   if (sh.p->block_tokens > 0) {
     grid_wait();
@@ -982,25 +1128,32 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   // ------------------------------------------------------------------ roles
   // resident, 32 rows: 768 threads start with 80 registers each; 256 x 64 + 512 x 88 is the same sum
   constexpr bool kMoveRegs = ONCE && NCOLS == 32;
-  const bool visit1 = a.mode != 2, visit2 = a.mode != 1;
   if (warp < 4) {
     if constexpr (kMoveRegs) reg_dec<64>();
     const int v = warp & 1;
-    if (ONCE ? v == 0 : (v == 0 ? visit1 : visit2)) {
-      unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
+    unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
+    if (ONCE && v == 1) {
+      if (gathers && warp == store_warp(ONCE)) fused_store<NCOLS>(sh, lane, sums, misc + 3, bars, ab);
+    } else if (ONCE || (v == 0 ? visit1 : visit2)) {
       if (warp < 2) {
         if (lane == 0) fused_produce<T, ONCE>(a, sh, v, k_tiles, q_tiles, tile_at, bars, misc + 2, ab);
+      } else if (v == 0) {
+        fused_multiply<T, NCOLS, FP8, sums_by_rows(ONCE, NCOLS), false>(a, sh, 0, k_tiles, q_tiles, tmem_base, bars, ab);
       } else {
-        if (v == 0) fused_multiply<T, NCOLS, FP8, sums_by_rows(ONCE, NCOLS), false>(a, sh, 0, k_tiles, q_tiles, tmem_base, bars, ab);
-        else fused_multiply<T, NCOLS, FP8, false, true>(a, sh, 1, k_tiles, q_tiles, tmem_v2, bars, ab);
+        fused_multiply<T, NCOLS, FP8, false, true>(a, sh, 1, k_tiles, q_tiles, tmem_v2, bars, ab);
       }
     }
   } else if (warp < kSumWarp0) {
     if constexpr (kMoveRegs) reg_dec<64>();
-    if (warp == kFetchWarp) {
-      if (visit2 && !(visit1 && gather_alone(NCOLS, min(sh.p->per_part, sh.p->n_tiles)))) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
+    if (gathers) {
+      if (warp < kGatherWarp0 + gather_teams(ONCE) * kTeamWarps)
+        fused_gather<T, NCOLS, G, FP8, gather_teams(ONCE)>(a, sh, warp - kGatherWarp0, lane, misc + 3, off, off_c, bars, ab);
+      else if (warp == store_warp(ONCE))
+        fused_store<NCOLS>(sh, lane, sums, misc + 3, bars, ab);
+    } else if (warp == kFetchWarp) {
+      if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
     } else if (visit1) {
-      fused_publish<T, NCOLS, G, FP8>(a, sh, warp - kPublisherWarp0, lane, sums, off, off_c, bars, ab);
+      fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
     }
   } else if (warp < kMaxWarp0) {
     if constexpr (kMoveRegs) reg_inc<88>();

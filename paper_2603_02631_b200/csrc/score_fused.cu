@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
   for (int idx = threadIdx.x; idx < chunks; idx += kPrepThreads) {
     const int h = idx / (rows_stored * CH), j = idx / CH % rows_stored, pos = idx % CH;
     const int chunk = pos ^ (CH == 8 ? j & 7 : (j >> 1) & 3);
-    const int g = j % a.padded_group, i = j / a.padded_group;
-    const bool real = g < a.group && i < a.n_lookahead;
-    const uint4* src = reinterpret_cast<const uint4*>(q + (int64_t)(g * a.n_lookahead + i) * D + h * (SUBROW / (FP8 ? 1 : 2)) + chunk * EL);
+    const QueryRow r = query_row(j, a.ncols, a.padded_group);
+    const bool real = r.g < a.group && r.i < a.n_lookahead;
+    const uint4* src = reinterpret_cast<const uint4*>(q + (int64_t)(r.g * a.n_lookahead + r.i) * D + h * (SUBROW / (FP8 ? 1 : 2)) + chunk * EL);
     if constexpr (!FP8) {
       image[idx] = real ? __ldg(src) : make_uint4(0, 0, 0, 0);
     } else {
