@@ -204,11 +204,18 @@ constexpr int kSmemBudget = kFusedSmemMost - 1024;   // minus alignment slack
 // (sustained, 64 rows at 131072 tokens 627 -> 605 us, 32 rows at 262000 507 -> 471); with 4 tiles less lead costs 3 %.
 constexpr double kL2KeyBytes = 80e6, kL2KeyBytesLong = 60e6;
 constexpr int kLongSlab = 5;
-// What an SM's share of the memory bandwidth brings in a microsecond (6.5 TB/s over 148 SMs).
-constexpr double kSmBytesPerUs = 44e3;
-// Microseconds from a slab's last key to its log-sum-exps having freed the slab's tiles, in one hop between the CTAs of a
-// group or in two; and what a tile of the next slab takes when its keys are there already.
-constexpr double kHandoverUs1 = 4.3, kHandoverUs2 = 5.5, kBurstUs = 0.3;
+// What an SM's share of the memory bandwidth brings in a microsecond: at the rate of a copy (6.5 TB/s over 148 SMs), and at that of
+// a kernel that only reads (7.2 TB/s), which the resident form comes close to.
+constexpr double kSmBytesPerUs = 44e3, kReadBytesPerUs = 49e3;
+// Resident, fitted to 93 splits of 29 prompts, 1500 to 250003 tokens, timed under a sustained load (mean error 5.5 %; the split that
+// it picks is 0.8 % slower than the best of those measured): microseconds from a slab's last key to its log-sum-exps being back,
+// what a tile of the next slab takes when its keys are there already, what the sums of a slab take on top of their tiles and for
+// two tiles of 32 rows, and what it costs groups to meet in global memory.
+constexpr double kHandoverUs = 2.5, kBurstUs = 0.35, kSlabUs = 0.5, kTwoTilesUs = 0.45, kMeetUs = 4.0;
+// The resident form wants room for the keys of so many microseconds beside a slab's tiles.  Sustained, 32 rows of 64 dimensions:
+// with 10 tiles a CTA and room for 13 a pass over 180000 tokens takes 761 us and 622 in two passes, with 7 and 12 (16 slots a
+// key) 577 and 457, with 7 and 16 441 and 456; 16 rows with 14 and 25: 736 and 767.
+constexpr double kSpareUs = 2.0;
 
 struct Geometry {
   bool ok = false, fp8 = false, once = false;
@@ -257,8 +264,7 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
   g.handover = std::max(2, (int)(3.0 * kSmBytesPerUs / g.tile_bytes));
   const int tiles = (int)std::min<int64_t>(ceil_div(ceil_div(p.n_tokens, kTileKeys), std::min(sm_count, kFusedMaxCtas)), 1 << 20);
   g.lead = std::max(2, (int)((tiles > kLongSlab ? kL2KeyBytesLong : kL2KeyBytes) / ((double)sm_count * g.tile_bytes)));
-  // the resident form wants a slab's tiles and a few more in tensor memory
-  g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + 3;
+  g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + std::max(3, (int)std::ceil(kSpareUs * kSmBytesPerUs / g.tile_bytes));
   g.max_tiles = (kTmemColsAll - 4 * g.ncols) / (g.ncols / g.padded_group);
   g.ok = tiles <= g.max_tiles;
   return g;
@@ -269,26 +275,24 @@ struct Split {
   double cost = 0;                          // time, in tiles that an SM's share of the memory bandwidth brings
 };
 
-// Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 4k to 250k tokens.
+// Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 2k to 250k tokens.
 // Three things can bound it, and near a tie they add up:
-//   memory: the average rather than the CTA with the most tiles (one with more than its share gets more bandwidth);
+//   memory: the average, not the CTA with the most tiles (one with more than its share gets more bandwidth);
 //   latency (resident): a tile's place is taken until its slab's log-sum-exps are back, and there is room for `held` slabs;
-//   the sum warps, which every slab costs a reduction over the warp on top of its tiles.
+//   the sum warps, which every slab costs something on top of its tiles.
 // Two-pass: the tiles, stretched where L2 does not hold the lead that the hand-over takes.
-double split_cost(const Geometry& g, int64_t n_tiles, int tiles, int parts, int per_part, int share) {
+double split_cost(const Geometry& g, int64_t n_tiles, int tiles, int parts, int share) {
   const int slabs = (g.n_slabs + parts - 1) / parts;
   const double units = (double)tiles * slabs, fair = (double)n_tiles * g.n_slabs / share;
   if (!g.once) {
     const double stretch = units > g.lead ? std::max(1.0, (double)(2 * tiles + g.handover) / g.lead) : 1.0;
     return units * stretch + 0.1 * slabs + 2.0 * tiles;
   }
-  const double us = g.tile_bytes / kSmBytesPerUs, per_tile = (double)g.resident(tiles) / tiles;
+  const double us = g.tile_bytes / kReadBytesPerUs, per_tile = (double)g.resident(tiles) / tiles;
   const double held = std::max(1.0, 0.5 * (per_tile + std::floor(per_tile)));
-  const double memory = 0.85 * fair + 0.15 * units;
-  const double handover = gather_alone(g.ncols, per_part) ? kHandoverUs1 : kHandoverUs2;
-  const double latency = std::max(handover / us + tiles, slabs / held * (handover + tiles * kBurstUs) / us);
-  const double sums = slabs * (g.ncols == 32 ? 0.9 + 0.24 * ((tiles + 1) / 2) : 0.5 + 0.16 * ((tiles + 1) / 2)) / us;
-  return std::cbrt(memory * memory * memory + latency * latency * latency + sums * sums * sums) + 2.0 * tiles;
+  const double latency = std::max(kHandoverUs / us + tiles, slabs / held * (kHandoverUs + tiles * kBurstUs) / us);
+  const double sums = slabs * (kSlabUs + kTwoTilesUs * g.ncols / 32 * ((tiles + 1) / 2)) / us;
+  return std::cbrt(fair * fair * fair + latency * latency * latency + sums * sums * sums) + 2.5 * tiles + (parts > 1 ? kMeetUs / us : 0.0);
 }
 
 // The best split over at most `ctas` CTAs; cost < 0 if there is none.  `share`: CTAs among which the memory bandwidth is
@@ -301,7 +305,7 @@ Split best_split(const Geometry& g, int64_t n_tiles, int ctas, int share) {
     const int64_t tiles = ceil_div(n_tiles, most);
     if (!g.holds(tiles)) break;
     const int per_part = (int)ceil_div(n_tiles, tiles);              // no more CTAs than these tiles need
-    const double cost = split_cost(g, n_tiles, (int)tiles, parts, per_part, share);
+    const double cost = split_cost(g, n_tiles, (int)tiles, parts, share);
     if (best.cost < 0 || cost < best.cost * 0.999) {
       best.parts = parts;
       best.per_part = per_part;

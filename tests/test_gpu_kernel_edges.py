@@ -66,6 +66,33 @@ def test_scores_at_the_edges_of_tiles_and_rings(L, Hq, Hkv, d, m, n):
     assert (s.lse.double().reshape(-1) - lse).abs().max() < 1e-4
 
 
+ROWS_AND_GROUPS = [
+    # row sums added up in every CTA up to 56 CTAs to a group (64 rows: 28), by owners beyond
+    *[(1, 4, 1, 64, 8, n) for n in (56 * 128, 56 * 128 + 1)], *[(1, 4, 1, 64, 16, n) for n in (28 * 128, 28 * 128 + 1)],
+    *[(1, 2, 1, 128, 8, n) for n in (56 * 128, 56 * 128 + 1)],
+    # rows dealt to the columns: each padded group with the fewest and the most lookahead queries of 16, 32 and 64 rows
+    *[(2, 2 * g, 2, 64, m, 2500) for g, ms in ((1, (1, 16, 17, 32)), (2, (1, 8, 9, 16, 17, 32)), (4, (1, 4, 5, 8, 9, 16)), (8, (1, 2, 3, 4, 5, 8)))
+      for m in ms],
+    # 8 heads in 16 columns, with the maxima in registers and (9 tiles a CTA) in tensor memory
+    (1, 8, 1, 64, 2, 5 * SPAN - 50), (1, 6, 1, 64, 2, 9 * SPAN - 50),
+    # more slabs than CTAs, and groups of CTAs that meet
+    (40, 8, 4, 64, 8, 600), (40, 8, 4, 64, 8, 3000),
+]
+
+
+@pytest.mark.parametrize("L,Hq,Hkv,d,m,n", ROWS_AND_GROUPS)
+def test_rows_are_dealt_to_columns_and_sums_to_warps(L, Hq, Hkv, d, m, n):
+    """Tolerance as above."""
+    import paper_2603_02631_b200 as spf
+    q, k = make(L, Hq, Hkv, d, m, n)
+    sel = spf.Selector(L, Hq, Hkv, d, m, n)
+    s = sel.run(q, k, *text(n), keep=0.2)
+    want, lse = reference(q, k)
+    assert int(sel.dev_status) == 0
+    assert ((s.importance.double() - want).abs() / want).max() < 2e-4
+    assert (s.lse.double().reshape(-1) - lse).abs().max() < 1e-4
+
+
 @pytest.mark.parametrize("L,Hq,Hkv,d,m,tiles", [
     *[(2, 1, 1, 64, 8, t) for t in (14, 15, 16, 27, 28)], (1, 2, 1, 64, 8, 20), (1, 2, 1, 64, 8, 56), (3, 1, 1, 128, 16, 28), (1, 8, 1, 64, 2, 57)])
 def test_sixteen_rows_on_the_fused_path_up_to_its_longest_prompts(L, Hq, Hkv, d, m, tiles):
