@@ -389,6 +389,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
+  bool ready = false;                                              // that tile's logits are there: asked before this one's arithmetic
   float next_ref = produced(refs + sh.slab(0)), next_c = FP8 ? produced(slab_c + sh.slab(0)) : a.c;
 #pragma unroll 1
   for (int n = 0; n < n_slabs; ++n) {
@@ -400,7 +401,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 1
     for (; lt < n_tiles; lt += 2) {
-      if (!mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
+      if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(bars.t_full(0, tr.stage), tr.phase, ab)) return;
       tc_fence_after();
       const uint32_t taddr = lane_addr + (uint32_t)(tr.stage * NCOLS);
       const uint32_t empty = bars.t_empty(0, tr.stage);
@@ -416,6 +417,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(empty);
+          ready = mbar_test_wait(bars.t_full(0, tr.stage), tr.phase);
         }
         if (sh.tile(lt) < full_tiles) {
 #pragma unroll
@@ -965,6 +967,7 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
   // resident: the stage of the slab's first tile; two-pass: a ring per set, this one's first stage and the next to be read
   Ring first(ONCE ? a.t_stages[V] : (a.t_stages[V] + 1 - set) / 2);
   Ring last = first;                                               // resident: that of the slab before
+  bool ready = false;
   const int stage0 = ONCE ? 0 : set * ((a.t_stages[V] + 1) / 2);
 #pragma unroll 1
   for (int n = 0; n < sh.n_slabs; ++n) {
@@ -992,7 +995,7 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
     }
     auto fold = [&](int lt, uint32_t (&m)[NIW]) -> bool {
       if constexpr (!ONCE) {
-        if (!mbar_wait_warp(bars.t_full(V, stage0 + tr.stage), tr.phase, ab)) return false;
+        if (!__all_sync(0xffffffffu, ready) && !mbar_wait_warp(bars.t_full(V, stage0 + tr.stage), tr.phase, ab)) return false;
         tc_fence_after();
       }
       if (!REGS) tmem_store_wait();                                // the maxima read below may be this warp's last stores
@@ -1009,12 +1012,13 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(bars.t_empty(V, stage0 + tr.stage));
+          tr.advance(ONCE ? 2 : 1);
+          if (!ONCE) ready = mbar_test_wait(bars.t_full(V, stage0 + tr.stage), tr.phase);   // the next tile's, before this one's arithmetic
         }
         if (NCH > 1) load_off(ch);
         fold_maxima<T, G>(r, m, o, c, lane);
         if (!REGS) tmem_store<NIW>(m_addr, m);
       }
-      tr.advance(ONCE ? 2 : 1);
       return true;
     };
     if constexpr (REGS) {
