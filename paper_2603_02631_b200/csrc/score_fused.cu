@@ -59,15 +59,57 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
     for (int64_t w = (int64_t)slab * kPrepThreads + threadIdx.x; w < p.clear_words[i]; w += (int64_t)n_slabs * kPrepThreads)
       p.clear[i][w] = make_uint4(0, 0, 0, 0);
 
+  // What follows is a chain of trips to memory that the scoring kernel waits for, so independent ones go first and none waits for
+  // another's (tensor maps behind a fence and the query operand behind the reference: 41.0 instead of 39.9 us for 16 layers x 8
+  // heads at 4001 tokens, 24.7 instead of 22.7 for one of the shortest prompts).
+  //
   // tensor maps: the first slab of a layer writes the layer's
-  if (hk == 0 && warp == 0) {
-    if (lane < 8) reinterpret_cast<uint4*>(p.k_maps_out + layer)[lane] = reinterpret_cast<const uint4*>(&p.k_map)[lane];
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) map_set_address(p.k_maps_out + layer, p.k_layers[layer]);
-    __syncwarp();
+  // (one thread, whose stores are in order)
+  if (hk == 0 && threadIdx.x == kPrepThreads - 32) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) reinterpret_cast<uint4*>(p.k_maps_out + layer)[i] = reinterpret_cast<const uint4*>(&p.k_map)[i];
+    map_set_address(p.k_maps_out + layer, p.k_layers[layer]);
     map_release();
   }
+
+  // the slab's query operand, 16 bytes of the swizzled image per thread and step: sub-tiles of `rows_stored` rows x one
+  // swizzle span, the 16-byte chunks of a row permuted by the row's index (mod 8; 64-byte rows: by half of it, mod 4)
+  const __nv_bfloat16* q = p.q + (int64_t)slab * (a.group * a.n_lookahead) * D;
+  auto write_image = [&](float S) {
+    constexpr int ROWB = row_bytes(D, FP8), SUBROW = sub_row_bytes(ROWB), CH = SUBROW / 16, KSUB = ROWB / SUBROW, EL = FP8 ? 16 : 8;
+    const int rows_stored = image_rows(a.ncols), chunks = KSUB * rows_stored * CH;
+    uint4* image = reinterpret_cast<uint4*>(p.q_tiles) + (int64_t)slab * (FP8 ? 2 : 1) * chunks;
+    for (int idx = threadIdx.x; idx < chunks; idx += kPrepThreads) {
+      const int h = idx / (rows_stored * CH), j = idx / CH % rows_stored, pos = idx % CH;
+      const int chunk = pos ^ (CH == 8 ? j & 7 : (j >> 1) & 3);
+      const QueryRow r = query_row(j, a.ncols, a.padded_group);
+      const bool real = r.g < a.group && r.i < a.n_lookahead;
+      const uint4* src = reinterpret_cast<const uint4*>(q + (int64_t)(r.g * a.n_lookahead + r.i) * D + h * (SUBROW / (FP8 ? 1 : 2)) + chunk * EL);
+      if constexpr (!FP8) {
+        image[idx] = real ? __ldg(src) : make_uint4(0, 0, 0, 0);
+      } else {
+        uint32_t hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+        if (real) {
+  #pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const uint4 v = __ldg(src + half);
+            const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&v);
+  #pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              const float2 f = __bfloat1622float2(v2[x >> 1]);
+              const float s = ((x & 1) ? f.y : f.x) * S;
+              const uint32_t t = float_to_e4m3(s);
+              hi[2 * half + (x >> 2)] |= t << (8 * (x & 3));
+              lo[2 * half + (x >> 2)] |= float_to_e4m3(s - e4m3_to_float(t)) << (8 * (x & 3));
+            }
+          }
+        }
+        image[idx] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        image[chunks + idx] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
+    }
+  };
+  if constexpr (!FP8) write_image(1.f);                             // (8-bit keys: the scale comes first)
 
   // reference: the smallest logit of the slab's rows against one fixed sample key, plus a margin (see fused.cuh).  A bad
   // block-table entry is clamped: this is a plain load, not a bounds-checked TMA copy
@@ -99,7 +141,6 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
       kf[2 * e + 1] = f.y;
     }
   }
-  const __nv_bfloat16* q = p.q + (int64_t)slab * rows * D;
   float ref = INFINITY, top = 0.f;                                  // smallest logit; largest |q| (8-bit keys)
   for (int r0 = warp * (32 / LPR); r0 < rows; r0 += (kPrepThreads / 32) * (32 / LPR)) {
     const int row = min(r0 + lane / LPR, rows - 1);                 // padding repeats a real row
@@ -146,41 +187,7 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
     }
     __syncthreads();
   }
-  // the slab's query operand, 16 bytes of the swizzled image per thread and step: sub-tiles of `rows_stored` rows x one
-  // swizzle span, the 16-byte chunks of a row permuted by the row's index (mod 8; 64-byte rows: by half of it, mod 4)
-  constexpr int ROWB = row_bytes(D, FP8), SUBROW = sub_row_bytes(ROWB), CH = SUBROW / 16, KSUB = ROWB / SUBROW, EL = FP8 ? 16 : 8;
-  const int rows_stored = image_rows(a.ncols), chunks = KSUB * rows_stored * CH;
-  uint4* image = reinterpret_cast<uint4*>(p.q_tiles) + (int64_t)slab * (FP8 ? 2 : 1) * chunks;
-  const float S = FP8 ? s_scale : 1.f;
-  for (int idx = threadIdx.x; idx < chunks; idx += kPrepThreads) {
-    const int h = idx / (rows_stored * CH), j = idx / CH % rows_stored, pos = idx % CH;
-    const int chunk = pos ^ (CH == 8 ? j & 7 : (j >> 1) & 3);
-    const QueryRow r = query_row(j, a.ncols, a.padded_group);
-    const bool real = r.g < a.group && r.i < a.n_lookahead;
-    const uint4* src = reinterpret_cast<const uint4*>(q + (int64_t)(r.g * a.n_lookahead + r.i) * D + h * (SUBROW / (FP8 ? 1 : 2)) + chunk * EL);
-    if constexpr (!FP8) {
-      image[idx] = real ? __ldg(src) : make_uint4(0, 0, 0, 0);
-    } else {
-      uint32_t hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-      if (real) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const uint4 v = __ldg(src + half);
-          const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&v);
-#pragma unroll
-          for (int x = 0; x < 8; ++x) {
-            const float2 f = __bfloat1622float2(v2[x >> 1]);
-            const float s = ((x & 1) ? f.y : f.x) * S;
-            const uint32_t t = float_to_e4m3(s);
-            hi[2 * half + (x >> 2)] |= t << (8 * (x & 3));
-            lo[2 * half + (x >> 2)] |= float_to_e4m3(s - e4m3_to_float(t)) << (8 * (x & 3));
-          }
-        }
-      }
-      image[idx] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      image[chunks + idx] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    }
-  }
+  if constexpr (FP8) write_image(s_scale);
 }
 
 template <int N>
