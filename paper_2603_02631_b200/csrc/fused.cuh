@@ -456,7 +456,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
 // With 16 rows keys are the quicker ones, 960 -> 910 us for 16 layers x 8 heads at 340942 tokens, and its columns are half as many:
 // 28 tiles a CTA at 16 slots a key instead of 26, where the general path takes 152 us for two layers at 511438 tokens and this one
 // 105.)
-template <class T, int NCOLS, bool FP8, bool ONCE>
+template <class T, int NCOLS, bool FP8>
 __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
                                              const FusedBars& bars, const Abort& ab) {
   constexpr int CT = NCOLS / 4;
@@ -469,7 +469,6 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
   // of the last, partial tile: real keys from this thread's first on
   const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32 - (lane >> 2);
-  const bool frees = !ONCE || a.mode == 1;                // the accumulators wait for no visit 2
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
@@ -492,11 +491,9 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
       tmem_issue_quarters<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
       tmem_load_wait();
       tmem_ready<NCOLS>(r);
-      if (frees) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
-      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
       tr.advance(2);
       if (sh.tile(lt) < full_tiles) {
 #pragma unroll
@@ -966,12 +963,20 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
   }
   // resident: the stage of the slab's first tile; two-pass: a ring per set, this one's first stage and the next to be read
   Ring first(ONCE ? a.t_stages[V] : (a.t_stages[V] + 1 - set) / 2);
-  Ring last = first;                                               // resident: that of the slab before
+  Ring last = first, end = first;                                  // resident: that of the slab before, and the slab's last tile's
   bool ready = false;
   const int stage0 = ONCE ? 0 : set * ((a.t_stages[V] + 1) / 2);
 #pragma unroll 1
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
+    if (ONCE) {
+      // That the log-sum-exps contain these logits orders nothing (they come by way of relaxed words in global memory): the
+      // barrier of the slab's last tile does, whose commit tracks everything issued before it.  Asked ahead of the log-sum-exps,
+      // whose wait hides it.
+      end = first;
+      end.advance(n_tiles - 1);
+      if (!mbar_wait_warp(bars.t_full(V, end.stage), end.phase, ab)) return;
+    }
     if (!mbar_wait_warp(bars.off_ready(slot), (uint32_t)(n / kOffSlots) & 1u, ab)) return;
     const float4* my_off = reinterpret_cast<const float4*>(off + slot * kOffFloats + (lane & 3) * off_stride(NCOLS));
     float o[T::CT];                                                // one load a tile: the same for all tiles
@@ -982,15 +987,8 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
     if (NCH == 1) load_off(0);
     const float c = FP8 ? off_c[slot] : a.c;
     Ring tr = first;
-    if (ONCE) tr.advance(set);
     if (ONCE) {
-      // all complete long since (the log-sum-exps contain them), except where visit 2 runs alone
-      if (a.mode == 2) {
-        Ring full = tr;
-#pragma unroll 1
-        for (int lt = set; lt < n_tiles; lt += 2, full.advance(2))
-          if (!mbar_wait_warp(bars.t_full(V, full.stage), full.phase, ab)) return;
-      }
+      tr.advance(set);
       tc_fence_after();
     }
     auto fold = [&](int lt, uint32_t (&m)[NIW]) -> bool {
@@ -1033,7 +1031,8 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
     }
     if (ONCE) {
       last = first;
-      first.advance(n_tiles);
+      first = end;
+      first.advance();
     } else {
       first = tr;
     }
@@ -1041,12 +1040,16 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
   if constexpr (REGS) {
-    // to the columns of the last slab's logits, which only this warp would still read
+    // to the columns of the last slab's logits, once everybody has read them
     Ring to = last;
     to.advance(set);
 #pragma unroll
     for (int u = 0; u < MINE; ++u) {
-      if (set + 2 * u < n_tiles) tmem_store<NIW>(lane_addr + (uint32_t)(to.stage * NCOLS), am[u]);
+      if (set + 2 * u < n_tiles) {
+        if (!mbar_wait_warp(bars.t_empty(V, to.stage), to.phase, ab)) return;
+        tc_fence_after();
+        tmem_store<NIW>(lane_addr + (uint32_t)(to.stage * NCOLS), am[u]);
+      }
       to.advance(2);
     }
     tmem_store_wait();
@@ -1099,7 +1102,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   if (threadIdx.x < 4) misc[threadIdx.x] = 0;
   for (int x = (int)threadIdx.x - 32; x >= 0 && x < FusedBars::kCount; x += kFusedThreads) {
     uint32_t count = 1;
-    if (x >= FusedBars::kTmem + kMaxResident && x < FusedBars::kShared) count = kVisitWarps / 2;   // t_empty
+    // t_empty: a set of the visit's warps; resident, of both visits' (the MMAs must not overtake either one's loads)
+    if (x >= FusedBars::kTmem + kMaxResident && x < FusedBars::kShared) count = ONCE && a.mode == 0 ? kVisitWarps : kVisitWarps / 2;
     else if (x >= FusedBars::kOffReady && x < FusedBars::kOffFree) count = gathers ? kTeamWarps : 1;
     else if (x >= FusedBars::kOffFree && x < FusedBars::kSumsFree) count = kVisitWarps;            // off_free, sums_ready
     mbar_init(bars.base + 8u * x, count);
@@ -1163,7 +1167,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
     if constexpr (kMoveRegs) reg_inc<88>();
     if (visit1) {
       if constexpr (sums_by_rows(ONCE, NCOLS)) sum_by_rows<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
-      else sum_by_keys<T, NCOLS, FP8, ONCE>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+      else sum_by_keys<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
     }
   } else {
     if constexpr (kMoveRegs) reg_inc<88>();

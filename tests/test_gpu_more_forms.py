@@ -37,6 +37,28 @@ def test_shards_through_many_rounds_of_every_ring(L, Hq, Hkv, d, m, n):
     assert int(status) == 0
 
 
+@pytest.mark.parametrize("L,Hq,Hkv,d,m,n", [
+    (40, 32, 8, 64, 8, 600), (16, 16, 8, 64, 8, 20 * 128),                                # a tile a CTA, 320 and 128 slabs; 32 and 16 rows
+    (16, 32, 8, 64, 8, 50000), (16, 32, 8, 64, 8, 8 * SPAN - 50),                         # maxima in registers; groups that gather, owners
+    (8, 16, 8, 64, 16, 4 * SPAN - 50), (8, 32, 8, 128, 8, 9 * SPAN - 50), (8, 8, 4, 128, 8, 12 * SPAN - 50)])   # in tensor memory
+def test_repeated_passes_bring_the_same_bits(L, Hq, Hkv, d, m, n):
+    """Every stage of tensor memory is filled, summed, folded and filled again many times a pass; sums are taken in a fixed order and
+    maxima are exact, so a load that saw another round's logits shows as a difference."""
+    import paper_2603_02631_b200 as spf
+    q, k = make(L, Hq, Hkv, d, m, n)
+    first, again = out(L, Hq, m, n), out(L, Hq, m, n)
+    p, r = spf.PromptBuffers(q, k, *first), spf.PromptBuffers(q, k, *again)
+    ws, status = scratch(spf.spf_score_workspace_bytes([p])), torch.zeros(1, dtype=torch.int32, device="cuda")
+    spf.spf_score([p], ws, dev_status=status)
+    for _ in range(20):
+        spf.spf_score([r], ws, dev_status=status)
+        assert torch.equal(first[0], again[0]) and torch.equal(first[1], again[1])
+    spf.spf_score_shard_lse_ex(r, ws, status)
+    spf.spf_score_shard_apply_ex(r, again[1], ws, status)            # the log-sum-exps went through base e: half a unit each way
+    torch.testing.assert_close(again[0], first[0], rtol=1e-5, atol=0)
+    assert int(status) == 0
+
+
 LENS = [1, 5000, 130, 700, 2048, 12000, 257]
 
 
