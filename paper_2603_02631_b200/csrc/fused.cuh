@@ -73,9 +73,12 @@ constexpr int kFusedSmemMost = 227 * 1024;   // dynamic shared memory of a CTA
 constexpr int kVisitWarps = 8;         // epilogue warps per visit
 constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
 // Groups of up to this many CTAs add up everybody's row sums in every CTA (see fused_gather): one hop instead of two, for reading
-// up to 7 KB a slab and CTA.  Three groups of 49 CTAs with 32 rows each: 178 us for 16 layers x 8 heads at 50000 tokens, in two
-// hops 200; two groups of 74 gained nothing.
-__host__ __device__ constexpr int gather_ctas(int ncols) { return ncols == 64 ? 28 : 56; }
+// up to 7 KB a slab and CTA.  Up to 56, which are seven words of 128 bits a lane with 32 rows: three groups of 49 CTAs with 32 rows
+// each take 178 us for 16 layers x 8 heads at 50000 tokens, in two hops 200; one prompt of 2 to 56 tiles and 16 or 128 slabs is up to
+// 16 % faster and never more than 2 % slower; two groups of 74 gained nothing.  64 rows have one pair of warps for it, to which a slab
+// of many CTAs is more work than its tiles: 128 slabs of 64 dimensions at 8 CTAs to a group take 0.99 of the time in two hops, at 12
+// 1.02, at 16 1.10, at 28 1.25 (68.8 us for 8 heads x 8 at 3568 tokens, 54.6 in two hops).
+__host__ __device__ constexpr int gather_ctas(int ncols) { return ncols == 64 ? 12 : 56; }
 __host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return n_ctas <= gather_ctas(ncols); }
 constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
 constexpr int kGatherWarp0 = 4, kTeamWarps = 2;

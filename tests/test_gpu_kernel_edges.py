@@ -67,8 +67,8 @@ def test_scores_at_the_edges_of_tiles_and_rings(L, Hq, Hkv, d, m, n):
 
 
 ROWS_AND_GROUPS = [
-    # row sums added up in every CTA up to 56 CTAs to a group (64 rows: 28), by owners beyond
-    *[(1, 4, 1, 64, 8, n) for n in (56 * 128, 56 * 128 + 1)], *[(1, 4, 1, 64, 16, n) for n in (28 * 128, 28 * 128 + 1)],
+    # row sums added up in every CTA up to 56 CTAs to a group (64 rows: 12), by owners beyond
+    *[(1, 4, 1, 64, 8, n) for n in (56 * 128, 56 * 128 + 1)], *[(1, 4, 1, 64, 16, n) for n in (12 * 128, 12 * 128 + 1, 28 * 128 + 1)],
     *[(1, 2, 1, 128, 8, n) for n in (56 * 128, 56 * 128 + 1)],
     # rows dealt to the columns: each padded group with the fewest and the most lookahead queries of 16, 32 and 64 rows
     *[(2, 2 * g, 2, 64, m, 2500) for g, ms in ((1, (1, 16, 17, 32)), (2, (1, 8, 9, 16, 17, 32)), (4, (1, 4, 5, 8, 9, 16)), (8, (1, 2, 3, 4, 5, 8)))
