@@ -219,10 +219,18 @@ constexpr double kSmBytesPerUs = 44e3, kReadBytesPerUs = 49e3;
 // what a tile of the next slab takes when its keys are there already, what the sums of a slab take on top of their tiles and for
 // two tiles of 32 rows, and what it costs groups to meet in global memory.
 constexpr double kHandoverUs = 2.5, kBurstUs = 0.35, kSlabUs = 0.5, kTwoTilesUs = 0.45, kMeetUs = 4.0;
-// The resident form wants room for the keys of so many microseconds beside a slab's tiles.  Sustained, 32 rows of 64 dimensions:
+// 32 rows: the resident form wants room for the keys of so many microseconds beside a slab's tiles.  Sustained, 64 dimensions, bf16:
 // with 10 tiles a CTA and room for 13 a pass over 180000 tokens takes 761 us and 622 in two passes, with 7 and 12 (16 slots a
-// key) 577 and 457, with 7 and 16 441 and 456; 16 rows with 14 and 25: 736 and 767.
+// key) 577 and 457, with 7 and 16 441 and 456.  8-bit keys, 128 slabs: with 9 and 13 622 and 483, with 7 and 12 527 and 399, with 6
+// and 16 334 and 336, with 8 and 16 424 and 433 (48 slabs: the two-pass form is 6 to 9 % quicker); 128 dimensions, with 9 and 13
+// 704 and 726, with 8 and 12 670 and 668.
 constexpr double kSpareUs = 2.0;
+// 16 rows: a slab's keys take longer than their sums, and the resident form is the quicker one with any room to speak of: 128
+// dimensions, bf16, with 18 tiles and room for 23 480 us and 790 in two passes, 8-bit keys 569 and 641.  With 64 dimensions, where
+// products cost half as much, this ends at 8 slots a key (bf16: with 16 and 24 262 and 254; with 4 slots, 17 and 27, 1.03 times as
+// long in two passes; 8-bit keys: 338 and 368) or at 16 (bf16: with 13 and 19 232 and 211; 8-bit keys: 330 and 309): the max warps
+// move as many columns of maxima as of logits, and where tensor memory does not hold two slabs the next one waits for them.
+constexpr int kSpareTiles = 3;
 
 struct Geometry {
   bool ok = false, fp8 = false, once = false;
@@ -271,7 +279,9 @@ Geometry geometry(const ScoreProblem& p, int sm_count) {
   g.handover = std::max(2, (int)(3.0 * kSmBytesPerUs / g.tile_bytes));
   const int tiles = (int)std::min<int64_t>(ceil_div(ceil_div(p.n_tokens, kTileKeys), std::min(sm_count, kFusedMaxCtas)), 1 << 20);
   g.lead = std::max(2, (int)((tiles > kLongSlab ? kL2KeyBytesLong : kL2KeyBytes) / ((double)sm_count * g.tile_bytes)));
-  g.once = g.ncols <= 32 && g.resident(tiles) >= tiles + std::max(3, (int)std::ceil(kSpareUs * kSmBytesPerUs / g.tile_bytes));
+  const int spare = g.resident(tiles) - tiles, slots = g.ncols / g.padded_group;
+  if (g.ncols == 32) g.once = spare >= std::max(kSpareTiles, (int)std::ceil(kSpareUs * kSmBytesPerUs / g.tile_bytes));
+  if (g.ncols == 16) g.once = spare >= (p.head_dim == 64 && slots >= (g.fp8 ? 16 : 8) ? std::max(kSpareTiles, tiles) : kSpareTiles);
   g.max_tiles = (kTmemColsAll - 4 * g.ncols) / (g.ncols / g.padded_group);
   g.ok = tiles <= g.max_tiles;
   return g;

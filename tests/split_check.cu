@@ -1,4 +1,5 @@
-// Prints the split over the SMs of batches read from standard input, one per line: L Hkv group d m key-bytes n_tokens...
+// Prints the split over the SMs of batches read from standard input, one per line: L Hkv group d m key-bytes n_tokens...; called with
+// an argument, the form of their prompts: 2 resident with the maxima in registers, 1 resident, 0 two-pass.
 // Includes the host side of the fused path as it is; nothing of it runs on a device.
 #include <iostream>
 #include <sstream>
@@ -16,7 +17,7 @@ int32_t fused_launch_d128_fp8(const FusedArgs&, const FusedLaunch&, cudaStream_t
 
 using namespace spf;
 
-int main() {
+int main(int argc, char**) {
   constexpr int kSms = 148;
   for (std::string line; std::getline(std::cin, line);) {
     std::istringstream in(line);
@@ -35,6 +36,12 @@ int main() {
       same = same && gi.ok && (tiles.empty() || gi.once == g[0].once);
       g.push_back(gi);
       tiles.push_back(ceil_div(p.n_tokens, kTileKeys));
+    }
+    if (argc > 1) {
+      for (size_t i = 0; i < g.size(); ++i)
+        std::cout << (g[i].ok ? (int)g[i].once + (int)(g[i].once && g[i].max_in_regs((int)ceil_div(tiles[i], kSms))) : -1) << ' ';
+      std::cout << '\n';
+      continue;
     }
     // which prompts share the first launch, and the CTAs of each: groups, CTAs per group, tiles per CTA
     const int n = same ? group_size(g.data(), tiles.data(), (int)tiles.size(), kSms) : 0;

@@ -37,14 +37,18 @@ def text(n):
 EDGES = [
     # one and two tiles, ragged; few CTAs per group, several groups that meet
     *[(3, 8, 2, 64, 8, n) for n in (1, 127, 128, 129, 255, 700, 5000)],
-    # 41 CTAs to a group and more: row sums in two hops instead of one
+    # a tile to each CTA of groups of 40 and more
     *[(1, 2, 1, 128, 8, n) for n in (40 * 128, 40 * 128 + 1, SPAN)],
     # groups that are padded to a power of two
     *[(2, 2 * g, 2, 64, 8, 3001) for g in (3, 5, 6, 7)],
     # maxima in registers up to 8 tiles a CTA, in tensor memory beyond
     *[(2, 2, 1, 128, 8, t * SPAN + more) for t in (7, 8) for more in (-1, 1)],
-    # 32 rows: from logits kept in tensor memory to logits computed twice
+    # 32 rows, 64 dimensions: logits computed twice
     *[(2, 4, 1, 64, 8, t * SPAN - 50) for t in (9, 10, 11, 12)],
+    # from logits kept (maxima in registers, in tensor memory) to logits computed twice: test_split_cpu.py has the edges
+    (2, 4, 1, 64, 8, 8 * SPAN - 50), *[(2, 4, 1, 128, 8, t * SPAN - 50) for t in (8, 9, 10, 11)],
+    *[(2, 2, 1, 64, 16, t * SPAN - 50) for t in (4, 6, 7)], *[(2, 1, 1, 64, 16, t * SPAN - 50) for t in (10, 11)],
+    *[(2, 2, 1, 64, 8, t * SPAN - 50) for t in (12, 13)], *[(1, 4, 1, 64, 4, t * SPAN - 50) for t in (23, 24)],
     # 64 rows: odd and even numbers of tiles, the two-pass form's rings from most to fewest stages
     *[(3, 4, 1, 64, 16, t * SPAN - 50) for t in (1, 2, 3, 6, 7, 11, 12, 15, 16)],
     (2, 8, 1, 128, 8, 3 * SPAN + 5), (2, 8, 2, 64, 5, 9001),

@@ -18,7 +18,8 @@ def scratch(size):
 
 @pytest.mark.parametrize("L,Hq,Hkv,d,m,n", [
     (16, 32, 8, 64, 8, 4001), (16, 32, 8, 64, 8, 60001), (16, 32, 8, 64, 8, 100100),      # groups of 8, 67 and 132 CTAs; 4, 7, 6 tiles
-    (12, 16, 8, 128, 8, 60001), (8, 32, 8, 64, 8, 9 * SPAN - 300), (6, 24, 8, 128, 8, 20011), (8, 16, 4, 64, 16, 30001)])
+    (12, 16, 8, 128, 8, 60001), (8, 32, 8, 64, 8, 9 * SPAN - 300), (6, 24, 8, 128, 8, 20011), (8, 16, 4, 64, 16, 30001),
+    (4, 8, 2, 128, 8, 9 * SPAN - 50), (4, 4, 2, 64, 16, 5 * SPAN - 50), (4, 2, 2, 64, 16, 10 * SPAN - 50)])     # maxima in tensor memory
 def test_shards_through_many_rounds_of_every_ring(L, Hq, Hkv, d, m, n):
     """One visit alone: stages are freed by the sum warps (first call), or waited for without a sum pass (second)."""
     import paper_2603_02631_b200 as spf
@@ -103,7 +104,11 @@ def test_batches_of_every_form_equal_their_prompts(geom, form):
     assert int(status) == 0
 
 
-@pytest.mark.parametrize("L,Hq,Hkv,d,m,tiles", [(4, 8, 2, 64, 8, 3), (4, 4, 2, 64, 8, 9), (2, 2, 1, 128, 8, 12), (2, 4, 1, 128, 8, 14)])
+@pytest.mark.parametrize("L,Hq,Hkv,d,m,tiles", [
+    (4, 8, 2, 64, 8, 3), (4, 4, 2, 64, 8, 9), (2, 2, 1, 128, 8, 12), (2, 4, 1, 128, 8, 14),
+    # either side of the edges between the forms (test_split_cpu.py)
+    *[(2, 4, 1, 64, 8, t) for t in (5, 6)], *[(2, 2, 1, 64, 16, t) for t in (3, 4)], *[(2, 4, 1, 128, 8, t) for t in (9, 10)],
+    *[(2, 2, 1, 64, 8, t) for t in (19, 20)], *[(2, 2, 1, 128, 8, t) for t in (19, 20)], *[(2, 1, 1, 64, 16, t) for t in (10, 11)]])
 def test_eight_bit_keys_of_many_tiles(L, Hq, Hkv, d, m, tiles):
     """Maxima in registers and in tensor memory, logits kept and computed twice."""
     import paper_2603_02631_b200 as spf

@@ -17,10 +17,12 @@ def split(tmp_path_factory):
     subprocess.run([_nvcc(), "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
                     "-o", exe, os.path.join(ROOT, "tests", "split_check.cu")], check=True, capture_output=True, timeout=600)
 
-    def run(batches):
+    def run(batches, forms=False):
         text = "".join(" ".join(map(str, [*geom, *lens])) + "\n" for geom, lens in batches)
-        out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True, timeout=300).stdout.splitlines()
+        out = subprocess.run([exe] + ["forms"] * forms, input=text, capture_output=True, text=True, check=True, timeout=300).stdout.splitlines()
         rows = [[int(x) for x in line.split()] for line in out]
+        if forms:
+            return rows
         return [(bool(r[0]), r[1], bool(r[2]), [tuple(r[i:i + 3]) for i in range(3, len(r), 3)]) for r in rows]
 
     return run
@@ -52,3 +54,18 @@ def test_every_batch_that_is_grouped_is_split(split):
         for length, (parts, per_part, tiles) in zip(lens, prompts):
             assert 1 <= parts <= geom[0] * geom[1] and per_part * tiles >= -(-length // TILE), (geom, lens)
     assert seen > 3000
+
+
+@pytest.mark.parametrize("geom,registers,kept,twice", [
+    # group, d, m, bytes per key element; the most tiles an SM with the maxima in registers, with the logits kept, and the next more
+    ((4, 64, 8, 2), 8, 8, 9), ((2, 64, 16, 2), 0, 6, 7), ((4, 128, 8, 2), 8, 10, 11), ((1, 64, 32, 2), 0, 5, 6),
+    ((4, 64, 8, 1), 5, 5, 6), ((2, 64, 16, 1), 0, 3, 4), ((4, 128, 8, 1), 8, 8, 9), ((1, 64, 32, 1), 0, 2, 3),
+    ((1, 64, 16, 2), 0, 10, 11), ((2, 64, 8, 2), 8, 12, 13), ((4, 64, 4, 2), 8, 23, 24), ((8, 64, 2, 2), 8, 25, 26),
+    ((1, 64, 16, 1), 0, 10, 11), ((2, 64, 8, 1), 8, 19, 20), ((1, 128, 16, 1), 0, 14, 15), ((2, 128, 8, 1), 8, 19, 20), ((2, 128, 8, 2), 8, 19, 20),
+    ((4, 64, 16, 2), 0, 0, 1)])
+def test_form_by_tiles(split, geom, registers, kept, twice):
+    """The edges that the tests on the GPU are placed at."""
+    group, d, m, element = geom
+    for tiles, form in ((registers, 2), (registers + 1, 1 if kept > registers else 0), (kept, 2 if kept == registers else 1), (twice, 0)):
+        if tiles > 0:
+            assert split([((3, 1, group, d, m, element), [(tiles - 1) * SMS * TILE + 1, tiles * SMS * TILE])], forms=True) == [[form, form]], tiles
