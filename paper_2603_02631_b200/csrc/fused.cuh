@@ -459,7 +459,7 @@ __device__ __forceinline__ void sum_by_rows(const FusedArgs& a, const FusedShare
 // With 16 rows keys are the quicker ones, 960 -> 910 us for 16 layers x 8 heads at 340942 tokens, and its columns are half as many:
 // 28 tiles a CTA at 16 slots a key instead of 26, where the general path takes 152 us for two layers at 511438 tokens and this one
 // 105.)
-template <class T, int NCOLS, bool FP8>
+template <class T, int NCOLS, bool FP8, bool ONCE>
 __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare& sh, int warp, int lane, uint32_t tmem, float* sums,
                                              const FusedBars& bars, const Abort& ab) {
   constexpr int CT = NCOLS / 4;
@@ -472,6 +472,7 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
   const int full_tiles = (int)(p.n_tokens / kTileKeys);            // tiles below this index have 128 real keys
   // of the last, partial tile: real keys from this thread's first on
   const int tail_keys = (int)(p.n_tokens - (int64_t)full_tiles * kTileKeys) - quad * 32 - (lane >> 2);
+  const bool frees = !ONCE || a.mode == 1;                // else the max warps do (whose loads come after these: see Stored)
   Ring tr(a.t_stages[0]);
   tr.advance(set);
   int lt = set;                                                    // this set's next tile, counted from the slab's first
@@ -494,9 +495,11 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
       tmem_issue_quarters<NCOLS>(lane_addr + (uint32_t)(tr.stage * NCOLS), r);
       tmem_load_wait();
       tmem_ready<NCOLS>(r);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
+      if (frees) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bars.t_empty(0, tr.stage));
+      }
       tr.advance(2);
       if (sh.tile(lt) < full_tiles) {
 #pragma unroll
@@ -553,6 +556,7 @@ __device__ __forceinline__ void sum_by_keys(const FusedArgs& a, const FusedShare
     } else {
       if ((lane & 4) == 0) out[(lane >> 3) * 4 + (lane & 3)] = s[0];
     }
+    tc_fence_before();                                             // the slab's loads from tensor memory are done (see Stored)
     __syncwarp();
     if (lane == 0) mbar_arrive(bars.sums_ready(slot));
   }
@@ -644,6 +648,33 @@ __device__ __forceinline__ float row_lse(const FusedArgs& a, const FusedPrompt& 
                 report ? a.dev_status : nullptr);
 }
 
+// How many slabs' row sums a warp has stored: what the gathering and the fetching warps wait for before they ask for anybody's.
+// Released and acquired, it carries an order that the words in global memory do not: the sum warps' loads of a slab's logits come
+// before the max warps' work on that slab, hence before the products (or the maxima at the end) that overwrite them.  (An arrival of
+// the sum warps at every tile's barrier instead costs up to 2 %: 16 rows of 64 dimensions, 8-bit keys, 12 layers x 4 heads at 89720
+// tokens 91.1 -> 92.8 us, this way 91.4.)
+struct Stored {
+  uint32_t at;                                                     // one word for each warp that stores
+  __device__ __forceinline__ void release(int which, int n) const {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(at + 4u * which), "r"(n) : "memory");
+  }
+  __device__ __forceinline__ int acquire(int which) const {
+    int n;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(n) : "r"(at + 4u * which) : "memory");
+    return n;
+  }
+  // Until more than n are stored; all lanes of the warp agree.
+  __device__ __forceinline__ bool wait(int which, int n, const Abort& ab) const {
+    unsigned long long t0 = 0;
+#pragma unroll 1
+    for (uint32_t it = 1; __any_sync(0xffffffffu, acquire(which) <= n); ++it) {
+      if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return false;
+      __nanosleep(20);
+    }
+    return true;
+  }
+};
+
 // Stores this CTA's sums of quads q0 .. q0 + LANES - 1 of its n-th slab for all to read (a row that does not exist gets its
 // meaningless sum stored too: everybody waits for every word).
 template <int NCOLS, int LANES>
@@ -681,18 +712,18 @@ __device__ __forceinline__ void store_sums(const FusedPrompt& p, const FusedShar
 // two teams of two that take the slabs in turn) wait for everybody's, half the rows each.  (With the same warps storing and
 // waiting, sums went out up to 2.3 us late: 32 rows at 4001 tokens.)
 template <int NCOLS>
-__device__ __forceinline__ void fused_store(const FusedShare& sh, int lane, const float* sums, volatile int* stored, const FusedBars& bars,
+__device__ __forceinline__ void fused_store(const FusedShare& sh, int lane, const float* sums, const Stored& stored, const FusedBars& bars,
                                             const Abort& ab) {
 #pragma unroll 1
   for (int n = 0; n < sh.n_slabs; ++n) {
     if (!mbar_wait_warp(bars.sums_ready(n % kSumSlots), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
     store_sums<NCOLS, NCOLS / 4>(*sh.p, sh, n, 0, lane, sums, bars);
-    if (lane == 0) *stored = n + 1;
+    if (lane == 0) stored.release(0, n + 1);
   }
 }
 
 template <class T, int NCOLS, int G, bool FP8, int TEAMS>
-__device__ __forceinline__ void fused_gather(const FusedArgs& a, const FusedShare& sh, int which, int lane, volatile int* stored, float* off,
+__device__ __forceinline__ void fused_gather(const FusedArgs& a, const FusedShare& sh, int which, int lane, const Stored& stored, float* off,
                                              float* off_c, const FusedBars& bars, const Abort& ab) {
   constexpr int LANES = NCOLS / 4 / kTeamWarps;                    // quads of this warp
   constexpr int MAXW = (gather_ctas(NCOLS) * LANES + 31) / 32;
@@ -706,13 +737,9 @@ __device__ __forceinline__ void fused_gather(const FusedArgs& a, const FusedShar
     w.begin(p, slab, q0, n_ctas, lane);
     const float ref = produced(p.refs + slab);                     // its way to L2 and back passes during the waits below
     const float c = FP8 ? produced(p.slab_c + slab) : 0.f;
-    unsigned long long t0 = 0;
     // not before the own sums are out: polling for words that cannot be there yet slows the key copies down
-#pragma unroll 1
-    for (uint32_t it = 1; __any_sync(0xffffffffu, *stored <= n); ++it) {
-      if (__any_sync(0xffffffffu, give_up(it, t0, ab))) return;
-      __nanosleep(20);
-    }
+    if (!stored.wait(0, n, ab)) return;
+    unsigned long long t0 = 0;
 #pragma unroll 1
     for (uint32_t it = 1;; ++it) {
       w.ask();
@@ -738,7 +765,7 @@ __device__ __forceinline__ void fused_gather(const FusedArgs& a, const FusedShar
 // n * Q + q, rows 4q .. 4q + 3 of the group's n-th slab, belongs to CTA (item mod CTAs) -- and stores their log-sum-exps for all.
 // Not before its own sums are out: polling for words that cannot be there yet slowed the key copies down.
 template <class T, int NCOLS, int G>
-__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums,
+__device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedShare& sh, int which, int lane, const float* sums, const Stored& stored,
                                               const FusedBars& bars, const Abort& ab) {
   constexpr int Q = NCOLS / 4, MAXW = (kFusedMaxCtas + 31) / 32;   // lane q has rows 4q .. 4q + 3
   const FusedPrompt& p = *sh.p;
@@ -748,6 +775,7 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
     const int slab = sh.slab(n);
     if (!mbar_wait_warp(bars.sums_ready(n % kSumSlots), (uint32_t)(n / kSumSlots) & 1u, ab)) return;
     store_sums<NCOLS, Q>(p, sh, n, 0, lane, sums, bars);
+    if (lane == 0) stored.release(which, n + 1);
 #pragma unroll 1
     for (int q = (int)(((unsigned)(n + 1) * (unsigned)n_ctas * Q + sh.first - n * Q) % (unsigned)n_ctas); q < Q; q += n_ctas) {
       RowSums<NCOLS, 1, MAXW> w;
@@ -774,7 +802,7 @@ __device__ __forceinline__ void fused_publish(const FusedArgs& a, const FusedSha
 // ---------------------------------------------------------------------------------------------- log-sum-exps for visit 2
 // Fetches each slab's log-sum-exps in turn and hands them to the max warps through shared memory (negated: what visit 2 adds).
 template <class T, int NCOLS, int G, bool FP8>
-__device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedShare& sh, int lane, float* off, float* off_c,
+__device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedShare& sh, int lane, const Stored& stored, float* off, float* off_c,
                                                 const FusedBars& bars, const Abort& ab) {
   const FusedPrompt& p = *sh.p;
   constexpr int RPL = NCOLS == 64 ? 2 : 1;
@@ -791,6 +819,7 @@ __device__ __forceinline__ void fused_fetch_lse(const FusedArgs& a, const FusedS
         v[r] = q.g < a.group && q.i < a.n_lookahead ? -__ldg(p.lse_in + ((int64_t)slab * a.group + q.g) * a.n_lookahead + q.i) * kLog2e : -INFINITY;
       }
     } else {
+      if (!stored.wait(n % kPublisherWarps, n, ab)) return;
       unsigned long long w[RPL], t0 = 0;
 #pragma unroll 1
       for (uint32_t it = 1;; ++it) {
@@ -973,9 +1002,9 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
   for (int n = 0; n < sh.n_slabs; ++n) {
     const int slot = n % kOffSlots;
     if (ONCE) {
-      // That the log-sum-exps contain these logits orders nothing (they come by way of relaxed words in global memory): the
-      // barrier of the slab's last tile does, whose commit tracks everything issued before it.  Asked ahead of the log-sum-exps,
-      // whose wait hides it.
+      // That the log-sum-exps contain these logits orders nothing (they come by way of relaxed words in global memory).  For the
+      // products, the barrier of the slab's last tile does, whose commit tracks everything issued before it: asked ahead of the
+      // log-sum-exps, whose wait hides it.  For the sum warps' loads: see Stored.
       end = first;
       end.advance(n_tiles - 1);
       if (!mbar_wait_warp(bars.t_full(V, end.stage), end.phase, ab)) return;
@@ -1043,16 +1072,12 @@ __device__ __forceinline__ void fused_max(const FusedArgs& a, const FusedShare& 
     if (lane == 0) mbar_arrive(bars.off_free(slot));
   }
   if constexpr (REGS) {
-    // to the columns of the last slab's logits, once everybody has read them
+    // to the columns of the last slab's logits, which only this warp would still read
     Ring to = last;
     to.advance(set);
 #pragma unroll
     for (int u = 0; u < MINE; ++u) {
-      if (set + 2 * u < n_tiles) {
-        if (!mbar_wait_warp(bars.t_empty(V, to.stage), to.phase, ab)) return;
-        tc_fence_after();
-        tmem_store<NIW>(lane_addr + (uint32_t)(to.stage * NCOLS), am[u]);
-      }
+      if (set + 2 * u < n_tiles) tmem_store<NIW>(lane_addr + (uint32_t)(to.stage * NCOLS), am[u]);
       to.advance(2);
     }
     tmem_store_wait();
@@ -1076,9 +1101,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   float* sums = reinterpret_cast<float*>(smem + lay.sums_off);
   float* off = reinterpret_cast<float*>(smem + lay.off_off);
   float* off_c = reinterpret_cast<float*>(smem + lay.offc_off);
-  volatile int* misc = reinterpret_cast<volatile int*>(smem + lay.misc_off);  // [0] abort, [1] tensor-memory base, [2] tiles visit 2 has issued, [3] slabs whose sums are stored
+  volatile int* misc = reinterpret_cast<volatile int*>(smem + lay.misc_off);  // [0] abort, [1] tensor-memory base, [2] tiles visit 2 has issued, [3..] slabs whose sums are stored
   const FusedBars bars{smem_u32(smem + lay.bar_off)};
   const Abort ab{misc, a.dev_status};
+  const Stored stored{smem_u32(smem + lay.misc_off) + 12u};
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ------------------------------------------------------------------ this CTA's share
@@ -1102,11 +1128,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   const bool gathers = visit1 && gather_alone(NCOLS, min(sh.p->per_part, sh.p->n_tiles));
 
   // ------------------------------------------------------------------ set-up
-  if (threadIdx.x < 4) misc[threadIdx.x] = 0;
+  if (threadIdx.x < 3 + kPublisherWarps) misc[threadIdx.x] = 0;
   for (int x = (int)threadIdx.x - 32; x >= 0 && x < FusedBars::kCount; x += kFusedThreads) {
     uint32_t count = 1;
-    // t_empty: a set of the visit's warps; resident, of both visits' (the MMAs must not overtake either one's loads)
-    if (x >= FusedBars::kTmem + kMaxResident && x < FusedBars::kShared) count = ONCE && a.mode == 0 ? kVisitWarps : kVisitWarps / 2;
+    if (x >= FusedBars::kTmem + kMaxResident && x < FusedBars::kShared) count = kVisitWarps / 2;   // t_empty
     else if (x >= FusedBars::kOffReady && x < FusedBars::kOffFree) count = gathers ? kTeamWarps : 1;
     else if (x >= FusedBars::kOffFree && x < FusedBars::kSumsFree) count = kVisitWarps;            // off_free, sums_ready
     mbar_init(bars.base + 8u * x, count);
@@ -1144,7 +1169,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
     const int v = warp & 1;
     unsigned char *k_tiles = smem + lay.k_off[v], *q_tiles = smem + lay.q_off[v];
     if (ONCE && v == 1) {
-      if (gathers && warp == store_warp(ONCE)) fused_store<NCOLS>(sh, lane, sums, misc + 3, bars, ab);
+      if (gathers && warp == store_warp(ONCE)) fused_store<NCOLS>(sh, lane, sums, stored, bars, ab);
     } else if (ONCE || (v == 0 ? visit1 : visit2)) {
       if (warp < 2) {
         if (lane == 0) fused_produce<T, ONCE>(a, sh, v, k_tiles, q_tiles, tile_at, bars, misc + 2, ab);
@@ -1158,19 +1183,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
     if constexpr (kMoveRegs) reg_dec<64>();
     if (gathers) {
       if (warp < kGatherWarp0 + gather_teams(ONCE) * kTeamWarps)
-        fused_gather<T, NCOLS, G, FP8, gather_teams(ONCE)>(a, sh, warp - kGatherWarp0, lane, misc + 3, off, off_c, bars, ab);
+        fused_gather<T, NCOLS, G, FP8, gather_teams(ONCE)>(a, sh, warp - kGatherWarp0, lane, stored, off, off_c, bars, ab);
       else if (warp == store_warp(ONCE))
-        fused_store<NCOLS>(sh, lane, sums, misc + 3, bars, ab);
+        fused_store<NCOLS>(sh, lane, sums, stored, bars, ab);
     } else if (warp == kFetchWarp) {
-      if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, off, off_c, bars, ab);
+      if (visit2) fused_fetch_lse<T, NCOLS, G, FP8>(a, sh, lane, stored, off, off_c, bars, ab);
     } else if (visit1) {
-      fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, bars, ab);
+      fused_publish<T, NCOLS, G>(a, sh, warp - kPublisherWarp0, lane, sums, stored, bars, ab);
     }
   } else if (warp < kMaxWarp0) {
     if constexpr (kMoveRegs) reg_inc<88>();
     if (visit1) {
       if constexpr (sums_by_rows(ONCE, NCOLS)) sum_by_rows<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
-      else sum_by_keys<T, NCOLS, FP8>(a, sh, warp, lane, tmem_base, sums, bars, ab);
+      else sum_by_keys<T, NCOLS, FP8, ONCE>(a, sh, warp, lane, tmem_base, sums, bars, ab);
     }
   } else {
     if constexpr (kMoveRegs) reg_inc<88>();
