@@ -219,6 +219,11 @@ constexpr double kSmBytesPerUs = 44e3, kReadBytesPerUs = 49e3;
 // what a tile of the next slab takes when its keys are there already, what the sums of a slab take on top of their tiles and for
 // two tiles of 32 rows, and what it costs groups to meet in global memory.
 constexpr double kHandoverUs = 2.5, kBurstUs = 0.35, kSlabUs = 0.5, kTwoTilesUs = 0.45, kMeetUs = 4.0;
+// What a tile of the next slab takes more where the max warps load and store its maxima in tensor memory, a slot of a key.  Without it
+// 12 layers x 4 heads of 64 dimensions, 2 x 16 rows, went over 382 tiles as two groups of 64 CTAs with six tiles each: 101 us, and 83 as
+// one group of 128 with three.  Of 456 prompts of 5 to 1016 tiles, 4 to 128 slabs, it changes the split of 11, none for the worse; 90
+// others whose split it changes take 0.95 of the time on average (0.71 to 1.11).
+constexpr double kFoldUs = 0.0125;
 // 32 rows: the resident form wants room for the keys of so many microseconds beside a slab's tiles.  Sustained, 64 dimensions, bf16:
 // with 10 tiles a CTA and room for 13 a pass over 180000 tokens takes 761 us and 622 in two passes, with 7 and 12 (16 slots a
 // key) 577 and 457, with 7 and 16 441 and 456.  8-bit keys, 128 slabs: with 9 and 13 622 and 483, with 7 and 12 527 and 399, with 6
@@ -292,7 +297,7 @@ struct Split {
   double cost = 0;                          // time, in tiles that an SM's share of the memory bandwidth brings
 };
 
-// Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 2k to 250k tokens.
+// Time of a prompt of T tiles x S slabs as `parts` groups of `per_part` CTAs, fitted to measurements at 1.5k to 250k tokens.
 // Three things can bound it, and near a tie they add up:
 //   memory: the average, not the CTA with the most tiles (one with more than its share gets more bandwidth);
 //   latency (resident): a tile's place is taken until its slab's log-sum-exps are back, and there is room for `held` slabs;
@@ -307,7 +312,8 @@ double split_cost(const Geometry& g, int64_t n_tiles, int tiles, int parts, int 
   }
   const double us = g.tile_bytes / kReadBytesPerUs, per_tile = (double)g.resident(tiles) / tiles;
   const double held = std::max(1.0, 0.5 * (per_tile + std::floor(per_tile)));
-  const double latency = std::max(kHandoverUs / us + tiles, slabs / held * (kHandoverUs + tiles * kBurstUs) / us);
+  const double burst = kBurstUs + (g.max_in_regs(tiles) ? 0.0 : kFoldUs * g.ncols / g.padded_group);
+  const double latency = std::max(kHandoverUs / us + tiles, slabs / held * (kHandoverUs + tiles * burst) / us);
   const double sums = slabs * (kSlabUs + kTwoTilesUs * g.ncols / 32 * ((tiles + 1) / 2)) / us;
   return std::cbrt(fair * fair * fair + latency * latency * latency + sums * sums * sums) + 2.5 * tiles + (parts > 1 ? kMeetUs / us : 0.0);
 }
