@@ -33,9 +33,9 @@
 // padding, and twice the tensor memory: keys are the lanes there.  The running maxima live in tensor memory next to the
 // accumulators.
 //
-// Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: one of each; the spare warp 1 stores row sums
-// for the gathering warps).  4: fetches log-sum-exps for visit 2.  5..7: publishers (store this CTA's row sums of a slab; add up
-// all CTAs' sums of the rows this CTA owns).  In groups of few CTAs 4..7 add up all rows instead.  8..15: "sum" warps.  16..23:
+// Warps.  0 / 1: TMA producers of visit 1 / visit 2.  2 / 3: MMA issuers (resident: 0 and 2 alone).  4: fetches log-sum-exps for
+// visit 2.  5..7: publishers (store this CTA's row sums of a slab; add up all CTAs' sums of the rows this CTA owns).  In groups of
+// few CTAs one warp stores and others add up all rows instead: resident, 1 and 4..7; two-pass, 6 and 4..5.  8..15: "sum" warps.  16..23:
 // "max" warps.  Of the eight warps of a visit, warp % 4 picks the TMEM lane quadrant and the next bit the `set`: the two sets
 // take turns at the tiles, so that one set's tensor-memory loads and waits run while the other set computes.  (Splitting every tile's columns between the sets kept all eight warps in step,
 // all waiting or all computing.)
@@ -76,8 +76,8 @@ constexpr int kSumWarp0 = 8, kMaxWarp0 = 16;
 // up to 7 KB a slab and CTA.  Up to 56, which are seven words of 128 bits a lane with 32 rows: three groups of 49 CTAs with 32 rows
 // each take 178 us for 16 layers x 8 heads at 50000 tokens, in two hops 200; one prompt of 2 to 56 tiles and 16 or 128 slabs is up to
 // 16 % faster and never more than 2 % slower; two groups of 74 gained nothing.  64 rows have one pair of warps for it, to which a slab
-// of many CTAs is more work than its tiles: 128 slabs of 64 dimensions at 8 CTAs to a group take 0.99 of the time in two hops, at 12
-// 1.02, at 16 1.10, at 28 1.25 (68.8 us for 8 heads x 8 at 3568 tokens, 54.6 in two hops).
+// of many CTAs is more work than its tiles: over 128 slabs, 8 CTAs to a group take 0.99 of the time in two hops, 12 1.01, 16 1.09, 28
+// 1.20 (71.7 us for 8 heads x 8 of 64 dimensions at 3554 tokens, 58.2 in two hops; 54.6 and 68.8 with the keys in L2).
 __host__ __device__ constexpr int gather_ctas(int ncols) { return ncols == 64 ? 12 : 56; }
 __host__ __device__ constexpr bool gather_alone(int ncols, int n_ctas) { return n_ctas <= gather_ctas(ncols); }
 constexpr int kFetchWarp = 4, kPublisherWarp0 = 5, kPublisherWarps = 3;
@@ -211,9 +211,10 @@ struct Ring {
   }
 };
 
-// Reads what the preparing kernel writes.  This kernel is started while that one still runs, so these are not read-only for its
-// lifetime: __ldg may be moved ahead of the wait for the other kernel, a volatile load stays behind it.  (Through L1, which
-// has nothing of them before: the loads of neighbouring slabs share a line.)
+// Reads what the preparing kernel writes.  This kernel may be started while that one still runs (it asks for that; a cooperative
+// launch was not seen to overlap, but nothing here relies on it), so these are not read-only for its lifetime: __ldg may be moved
+// ahead of the wait for the other kernel, a volatile load stays behind it.  (Through L1, which has nothing of them before: the loads
+// of neighbouring slabs share a line.)
 __device__ __forceinline__ float produced(const float* at) {
   float x;
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(at));
@@ -320,8 +321,11 @@ __device__ __forceinline__ void fused_produce(const FusedArgs& a, const FusedSha
 // ---------------------------------------------------------------------------------------------- MMA issuer of one visit
 // Tile k of the CTA (k counts over slabs and tiles) has its logits in stage k mod stages.  One thread walks the
 // loop.  (The whole warp in step, with votes on the barriers and an elected lane at each tile, took 460 cycles to issue a tile's
-// four instructions and 120 for its barriers, 0.34 us a tile in all: more than the sums of 32 rows take.  The tensor cores want
-// 160 cycles for them, and 24 for each of the two commits.)
+// four instructions and 120 for its barriers, 0.34 us a tile in all: more than the sums of 32 rows take.  One thread's loop takes 150,
+// traced at 32768 tokens with 32 rows of 64 dimensions.)
+// It commits tile after tile, so whoever has seen a tile's barrier complete knows those of the tiles before it to be, too.  The
+// warps of visit 1 rely on that: a set asks for every other tile, the ring of stages is common to both sets, and with three stages
+// the barrier's phase before was another set's tile (a parity tells one round from the next only).  It takes at least two stages.
 // ROWS: query rows are the accumulator's lanes (weight-stationary instructions), else the keys.  SETS: a ring of stages for
 // each of the two sets of epilogue warps, the odd tiles' behind the even tiles': a tile's maxima belong to one set, so with an
 // odd number of tiles a set skips two, and in a common ring of two stages it could take the tile before the one that it
@@ -1155,7 +1159,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) score_fused_kernel(const __g
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = (uint32_t)misc[1];
-  // tensor memory: the accumulator stages, then the running maxima, [local tile][NI] columns (lane = key)
+  // tensor memory: the accumulator stages, then the running maxima, [local tile][NI] columns (a lane has four keys of a quarter of the lookahead slots, as fold_maxima has them)
   const uint32_t tmem_v2 = tmem_base + (uint32_t)(a.t_stages[0] * NCOLS);
   const uint32_t amax_tmem = tmem_v2 + (uint32_t)(ONCE ? 0 : a.t_stages[1] * NCOLS);
   grid_wait();                                                     // what the preparing kernel wrote is visible from here on
@@ -1254,7 +1258,8 @@ int32_t fused_launch_one(const FusedArgs& args, const FusedLaunch& l, cudaStream
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
-  // the launch overlaps the preparing kernel; grid_wait() orders what reads its results
+  // The launch may overlap the preparing kernel; grid_wait() orders what reads its results.  (Cooperative, it was seen to start 1.8 to
+  // 2 us after that kernel's end all the same.)
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kPrepThreads) fused_prep_kernel(const __grid_c
   __shared__ float red[kPrepThreads / 32];
   __shared__ float s_scale;
 
-  grid_launch_dependents();                                         // the scoring kernel sets itself up meanwhile
+  grid_launch_dependents();                                         // the scoring kernel may set itself up meanwhile
   for (int i = 0; i < 2; ++i)
     for (int64_t w = (int64_t)slab * kPrepThreads + threadIdx.x; w < p.clear_words[i]; w += (int64_t)n_slabs * kPrepThreads)
       p.clear[i][w] = make_uint4(0, 0, 0, 0);
@@ -428,7 +428,7 @@ bool pick_stages(const Geometry& g, int d, int tiles, bool paged, FusedArgs* a, 
   }
   // as many accumulator stages as fit, visit 1 first (its epilogue is the longer one)
   const int stages = std::min(2 * kMaxTmemStages, (kTmemColsAll - tiles * (g.ncols / g.padded_group)) / g.ncols);
-  if (stages < 4) return false;
+  if (stages < 4) return false;                                      // two for each visit (see fused_multiply)
   a->t_stages[0] = (stages + 1) / 2;
   a->t_stages[1] = stages / 2;
   for (int ks = 20; ks >= 4; --ks) {
